@@ -34,7 +34,7 @@ struct CycCLayout {
     unsigned int *hll, *bump;
     uint2 *Sp, *Tp;
     uint32_t *offS, *offT;
-    uint32_t *items;
+    uint32_t *items, *order;
     void *scan_tmp;
     unsigned int *counter;
     unsigned long long *big_slots, *big_off, *bigset;
@@ -64,6 +64,7 @@ size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, co
     L.Tp = A.take<uint2>(T.n + 2);
     L.offT = A.take<uint32_t>(z + 1);
     L.items = A.take<uint32_t>(z + 1);
+    L.order = A.take<uint32_t>(z + 1);
     L.scan_tmp = A.take<char>(scan_scratch_bytes(z + 1));
     L.counter = A.take<unsigned int>(1);
     L.big_slots = A.take<unsigned long long>(z + 1);
@@ -138,7 +139,7 @@ mwj_status check_cyc_shares(mwj_ctx *ctx, const mwj_shares &sh, CycPlan *p) {
 }  // namespace
 
 // Default shares: (1, 1, z), R whole and grouped by B, C split so that a
-// bucket's T_k averages half of a CTA's on-chip set (cyclic_c.cu).  In the
+// bucket's T_k averages a third of a CTA's on-chip set (cyclic_c.cu).  In the
 // read cost z'|R| + x|S| + y|T| of Section 5.2 (with a third share) R is
 // read once here, through the L2 as b -> [a] lists, and S and T once each;
 // the cube tilings below keep R's buckets in shared memory instead.
@@ -147,7 +148,7 @@ mwj_status plan_cyclic_default(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S,
     (void)ctx;
     (void)R;
     (void)S;
-    const uint64_t want = ((uint64_t)T.n + cyc_c_tcap() / 2 - 1) / (cyc_c_tcap() / 2);
+    const uint64_t want = ((uint64_t)T.n + cyc_c_tavg() - 1) / cyc_c_tavg();
     uint32_t z = pow2_at_least(want ? want : 1);
     if (z > kMaxBuckets) z = kMaxBuckets;
     sh->s[0] = 1;
@@ -271,6 +272,7 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
         g.r = LC.r;
         g.Sp = LC.Sp; g.offS = LC.offS; g.Tp = LC.Tp; g.offT = LC.offT;
         g.z = p.z;
+        g.order = LC.order;
         g.schunk = cyc_c_schunk(S.n, ctx->dev.num_sms);
         g.big_off = LC.big_off;
         g.bigset = LC.bigset;

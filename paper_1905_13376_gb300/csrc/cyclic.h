@@ -41,6 +41,7 @@ struct CycCArgs {
     const uint2 *Tp;            // T grouped by F(c): (c, a)
     const uint32_t *offT;       // z + 1
     uint32_t z;
+    const uint32_t *order;      // z: the buckets in the order they are taken (written by cyc_c_run)
     uint32_t schunk;            // S tuples of a work item at most (cyc_c_schunk)
     const unsigned long long *big_off;   // z + 1: big buckets' set regions (slots), scanned
     const unsigned long long *bigset;    // the regions: one slot per distinct (c, a) pair
@@ -53,8 +54,9 @@ struct CycCArgs {
     DevStatus *st;
 };
 
-// T tuples a bucket's on-chip set holds (larger buckets keep theirs in the L2).
-uint32_t cyc_c_tcap();
+// T tuples of an average bucket under the default shares (a third of a CTA's
+// on-chip set, so that uneven buckets still fit).
+uint32_t cyc_c_tavg();
 // S tuples of a work item at most: S_k is split so that a join with few
 // buckets (a small T) still gives every probe CTA work.
 uint32_t cyc_c_schunk(int64_t nS, int num_sms);

@@ -15,11 +15,10 @@
 // the cube tiling's wedge checks, each wedge of R |x| S once, without the
 // per-tile rebuilds.  A bucket whose T_k exceeds a CTA's shared-memory set
 // is taken in chunks of it, S_k streamed past each (every chunk checks the
-// bucket's wedges again, against its part of T_k), up to kChunkMax chunks; a
-// larger one (a C value with many T tuples: skewed or tiny C domains) keeps
-// its set in an L2-resident region of the workspace instead, built before
-// the probe, so that its wedges are checked once.  Results do not depend on
-// z.
+// bucket's wedges again, against its part of T_k); one above CC_TBIG tuples
+// (a C value with many T tuples: skewed or tiny C domains) keeps its set in an
+// L2-resident region of the workspace instead, built before the probe, so
+// that its wedges are checked once.  Results do not depend on z.
 #include "api_internal.h"
 #include "cyclic.h"
 #include "tables.h"
@@ -27,14 +26,16 @@
 namespace mwj {
 namespace {
 
-constexpr int CC_T = 768;                // threads per probe CTA (two CTAs per SM)
-constexpr uint32_t CC_TCAP = 4096;       // T tuples of an on-chip set: it is at most half full
-constexpr uint32_t kChunkMax = 4;        // on-chip chunks of a bucket before its set moves to the L2
+constexpr int CC_T = 640;                // threads per probe CTA (two CTAs per SM)
+constexpr uint32_t CC_TAVG = 2048;       // T tuples of an average bucket under the default shares
+constexpr uint32_t CC_TCAP = 6144;       // T tuples of an on-chip set: it is at most 3/4 full
+constexpr uint32_t CC_TBIG = 16384;      // T tuples of a bucket above which its set moves to the L2
 constexpr uint32_t CC_TSLOTS = 8192;     // slots of an on-chip (c, a) multiset (64 KB)
+constexpr uint32_t CC_FWORDS = 8192;     // words of the filter in front of it (2^18 bits, 32 KB)
 constexpr int RG_T = 512;                // threads of the grouping kernels
-constexpr uint32_t CC_QCAP = 2048;       // long R lists queued per work item
-constexpr uint32_t CC_CH = 256;          // wedges of a queued list per warp step
-constexpr uint32_t kQueueMin = 128;      // lists this long go to the item's queue
+constexpr uint32_t CC_QCAP = 768;        // long R lists queued per work item
+constexpr uint32_t CC_CH = 1024;         // wedges of a list per warp step (32 per lane, one mask word)
+constexpr uint32_t kQueueMin = 512;      // lists this long go to the item's queue
 constexpr uint32_t CC_SCHUNK_MIN = 32;   // S tuples of a bucket's work item, at least (a warp's batch)
 
 __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
@@ -45,24 +46,43 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
 // bytes, one shared-memory load), one slot per distinct pair.  An insert
 // takes the first slot of its home bucket or of the buckets after it that is
 // free or holds its pair, so the occupied slots of a bucket are a prefix and
-// a lookup can stop at the first bucket with a free slot: with the set at
-// most half full that is nearly always the home bucket.  T is a bag: a chunk
-// that repeats a pair (rare) is rebuilt in the CTA's own region of the
+// a lookup can stop at the first bucket with a free slot.  T is a bag: a
+// chunk that repeats a pair (rare) is rebuilt in the CTA's own region of the
 // workspace with a multiplicity per slot and looked up there like a big
-// bucket's set, so that the lookups of every other chunk stay as they are.
+// bucket's set.
+//
+// Nearly every wedge is open (about 1 in 90 closes on the 2^22-vertex power-law
+// graph), so the set is not looked up per wedge: a filter of 2^18 bits, one
+// bit per (c, a) pair, answers first.  The bit of a wedge is a multiply-add of
+// its a (the hash of c is computed once per list), one 4-byte shared-memory
+// load and a shift, with no probe chain whose longest lane the whole warp
+// waits for; the set is looked up for the 1 to 2 % that pass (2048 pairs
+// leave 0.8 % of the open wedges standing, 6144 pairs 2.3 %).  On the
+// 2^22-vertex graph (2.79e10 wedges, one GB300) the probe took 122 ms when it
+// looked every wedge up in the set and takes 38 ms: 26 ms for the filter's
+// side (issue slots and the 3.5 shared-memory wavefronts of a divergent load)
+// and 12 ms for the lookups of what passes.
 constexpr uint32_t CC_NB = CC_TSLOTS / 2;
 constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); one region each
 // two probe CTAs per SM: each keeps below half of the SM's 228 KB of shared
 // memory less the 1 KB the hardware reserves per CTA and the static arrays
-static_assert(CC_TSLOTS * 8 + CC_QCAP * 16 + (CC_QCAP + 1) * 4 + 1024 <= 228 * 1024 / 2 - 1024,
+static_assert(CC_TSLOTS * 8 + CC_FWORDS * 4 + CC_QCAP * 16 + (CC_QCAP + 1) * 4 + 1024 <= 228 * 1024 / 2 - 1024,
               "the probe's shared memory must leave room for two CTAs per SM");
 
-__device__ __forceinline__ uint32_t cbucket(uint32_t c, uint32_t a, uint32_t seed) {
-    uint32_t h = (c ^ seed) * 0x9E3779B1u ^ a * 0x85EBCA6Bu;
-    h ^= h >> 16;
-    h *= 0x7feb352dU;
-    h ^= h >> 15;
-    return h & (CC_NB - 1);
+// The filter bit of (c, a): word h >> 19, bit (h >> 14) & 31 of
+// h = a * K + chash(c), so that only the multiply-add depends on a.
+constexpr uint32_t CC_FMUL = 0x9E3779B1u;
+static_assert(CC_FWORDS == 1u << 13, "the filter's word index is the top 13 bits");
+__device__ __forceinline__ uint32_t chash(uint32_t c, uint32_t seed) { return mix32(c ^ seed); }
+
+__device__ __forceinline__ uint32_t chash_a(uint32_t a, uint32_t ch) { return a * CC_FMUL + ch; }
+// the home bucket of (c, a) in the on-chip set
+static_assert(CC_NB == 1u << 12, "the home bucket is the top 12 bits");
+__device__ __forceinline__ uint32_t cbucket(uint32_t h) { return h >> 20; }
+
+__device__ __forceinline__ uint32_t fbit(const uint32_t *filt, uint32_t a, uint32_t ch) {
+    const uint32_t h = chash_a(a, ch);
+    return (filt[h >> 19] >> ((h >> 14) & 31u)) & 1u;
 }
 
 // 1: the pair took a free slot; 2: it was there already; 0: the set is full.
@@ -85,14 +105,13 @@ __device__ __forceinline__ int cset_insert(unsigned long long *tk, unsigned long
 
 // 1 when key is in the set, else 0 (key != kEmpty64)
 __device__ __forceinline__ uint32_t cset_count(const unsigned long long *tk, unsigned long long key, uint32_t bk) {
-    uint32_t m = 0;
     for (uint32_t it = 0; it < CC_NB; ++it) {
         const ulonglong2 v = *(const ulonglong2 *)(tk + 2 * bk);
-        m += (v.x == key) + (v.y == key);
+        if (v.x == key || v.y == key) return 1u;
         if (v.y == kEmpty64) break;   // (v.x empty implies v.y empty)
         bk = (bk + 1) & (CC_NB - 1);
     }
-    return m;
+    return 0u;
 }
 
 // Entries of R's grouping: the direct-address layout (key b at b - min) or
@@ -181,7 +200,7 @@ __global__ void __launch_bounds__(RG_T) k_rg_scatter(const int32_t *__restrict__
     }
 }
 
-__host__ __device__ __forceinline__ bool cc_big(uint32_t nt) { return nt > kChunkMax * CC_TCAP; }
+__host__ __device__ __forceinline__ bool cc_big(uint32_t nt) { return nt > CC_TBIG; }
 
 // S chunks of a bucket: S_k in pieces of at most schunk tuples
 __host__ __device__ __forceinline__ uint32_t cc_schunks(uint32_t ns, uint32_t schunk) {
@@ -193,18 +212,59 @@ __host__ __device__ __forceinline__ uint32_t cc_schunks(uint32_t ns, uint32_t sc
 // of its S chunks, item (t, s) at t * S chunks + s; a big bucket also gets a
 // region of 2^k >= 2 |T_k| slots for its set in the workspace (big_slots[k],
 // 0 for the others).
-__global__ void k_cc_plan(const uint32_t *__restrict__ offS, const uint32_t *__restrict__ offT, uint32_t z,
-                          uint32_t schunk, uint32_t *__restrict__ items,
-                          unsigned long long *__restrict__ big_slots) {
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < z; k += gridDim.x * blockDim.x) {
+//
+// Buckets are taken in the order of four classes of |S_k| (4x, 2x, 1.25x the
+// mean and the rest): a hub's C value makes an item of some 3 ms where the
+// mean item takes 0.3 ms (2^22-vertex power-law graph), and one that starts
+// last leaves every other SM idle for as long.  order[p] is the bucket at
+// position p, items[p] its item count.  One CTA (z <= 32768).
+constexpr int CC_PLAN_T = 1024;
+__device__ __forceinline__ uint32_t cc_class(uint32_t ns, uint32_t mean) {
+    return ns >= 4u * mean ? 0u : ns >= 2u * mean ? 1u : 4ull * ns >= 5ull * mean ? 2u : 3u;
+}
+
+__global__ void __launch_bounds__(CC_PLAN_T) k_cc_plan(const uint32_t *__restrict__ offS,
+                                                       const uint32_t *__restrict__ offT, uint32_t z,
+                                                       uint32_t schunk, uint32_t *__restrict__ items,
+                                                       uint32_t *__restrict__ order,
+                                                       unsigned long long *__restrict__ big_slots) {
+    __shared__ uint32_t cursor[4];
+    if (threadIdx.x < 4) cursor[threadIdx.x] = 0u;
+    __syncthreads();
+    const uint32_t mean = (offS[z] - offS[0]) / z + 1u;
+    uint32_t mine[4] = {0u, 0u, 0u, 0u};
+    for (uint32_t k = threadIdx.x; k < z; k += CC_PLAN_T) {
         const uint32_t ns = offS[k + 1] - offS[k], nt = offT[k + 1] - offT[k];
-        items[k] = (ns && nt) ? (cc_big(nt) ? 1u : (nt + CC_TCAP - 1) / CC_TCAP) * cc_schunks(ns, schunk) : 0u;
+        const uint32_t c = cc_class(ns, mean);
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) mine[q] += c == q;
         unsigned long long slots = 0;
         if (ns && cc_big(nt)) {
             slots = 16;
             while (slots < 2ull * nt) slots <<= 1;
         }
         big_slots[k] = slots;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        mine[q] = warp_sum(mine[q]);
+        if ((threadIdx.x & 31) == 0 && mine[q]) atomicAdd(&cursor[q], mine[q]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t at = 0;
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t n = cursor[q];
+            cursor[q] = at;
+            at += n;
+        }
+    }
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < z; k += CC_PLAN_T) {
+        const uint32_t ns = offS[k + 1] - offS[k], nt = offT[k + 1] - offT[k];
+        const uint32_t p = atomicAdd(&cursor[cc_class(ns, mean)], 1u);
+        order[p] = k;
+        items[p] = (ns && nt) ? (cc_big(nt) ? 1u : (nt + CC_TCAP - 1) / CC_TCAP) * cc_schunks(ns, schunk) : 0u;
     }
 }
 
@@ -285,7 +345,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                                                       uint32_t *__restrict__ rep_cnt) {
     extern __shared__ __align__(16) unsigned char smraw[];
     unsigned long long *tk = (unsigned long long *)smraw;                      // CC_TSLOTS
-    uint4 *queue = (uint4 *)(tk + CC_TSLOTS);                                   // CC_QCAP x (b, c, start, n)
+    uint32_t *filt = (uint32_t *)(tk + CC_TSLOTS);                              // CC_FWORDS
+    uint4 *queue = (uint4 *)(filt + CC_FWORDS);                                 // CC_QCAP x (b, c, start, n)
     uint32_t *cpre = (uint32_t *)(queue + CC_QCAP);                             // CC_QCAP + 1 chunk offsets
     __shared__ uint32_t item_s, tneg, batch_ctr, chunk_ctr, qn, carry, tdup;
     // this CTA's region for a chunk that repeats pairs
@@ -304,16 +365,16 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         __syncthreads();
         const uint32_t item = item_s;
         if (item >= total_items) break;
-        // bucket of this item: last k with item_off[k] <= item
+        // bucket of this item: at the last position with item_off <= item
         uint32_t lo = 0, hi = z;
         while (hi - lo > 1) {
             const uint32_t mid = (lo + hi) >> 1;
             if (item_off[mid] <= item) lo = mid; else hi = mid;
         }
-        const uint32_t k = lo;
+        const uint32_t k = g.order[lo];
         // (T chunk, S chunk) of this item
         const uint32_t sch = cc_schunks(g.offS[k + 1] - g.offS[k], g.schunk);
-        const uint32_t li = item - item_off[k];
+        const uint32_t li = item - item_off[lo];
         const uint32_t tci = li / sch, sci = li - tci * sch;
         const uint32_t s0 = g.offS[k] + sci * g.schunk, s1 = min(g.offS[k + 1], s0 + g.schunk);
         // T_k's set: the item's chunk on chip, or for a big bucket its region
@@ -328,7 +389,11 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
 
         // ---- T_k as a (c, a) multiset: a slot per distinct pair ----
         if (!big)
-            for (uint32_t q = threadIdx.x; q < CC_TSLOTS; q += CC_T) tk[q] = kEmpty64;
+            for (uint32_t q = threadIdx.x; q < CC_NB; q += CC_T)
+                ((ulonglong2 *)tk)[q] = make_ulonglong2(kEmpty64, kEmpty64);
+        // (a big bucket's filter passes everything)
+        const uint32_t fw = big ? 0xffffffffu : 0u;
+        for (uint32_t q = threadIdx.x; q < CC_FWORDS / 4; q += CC_T) ((uint4 *)filt)[q] = make_uint4(fw, fw, fw, fw);
         if (threadIdx.x == 0) {
             tdup = 0u;
             tneg = big ? g.big_neg[k] : 0u;
@@ -341,11 +406,13 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         for (uint32_t q = ta + threadIdx.x; !big && q < tz; q += CC_T) {
             const uint2 tu = __ldg(g.Tp + q);   // (c, a)
             const unsigned long long key = cpack(tu.x, tu.y);
+            const uint32_t h = chash_a(tu.y, chash(tu.x, g.seed));
+            atomicOr(filt + (h >> 19), 1u << ((h >> 14) & 31u));
             if (key == kEmpty64) {               // (-1, -1) is the empty marker: counted apart
                 atomicAdd(&tneg, 1u);
                 continue;
             }
-            const int r = cset_insert(tk, key, cbucket(tu.x, tu.y, g.seed));
+            const int r = cset_insert(tk, key, cbucket(h));
             if (r == 2 && !tdup) tdup = 1u;
             if (r == 0) set_status(g.st, MWJ_ERR_CHECK, 24);
         }
@@ -415,10 +482,10 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 }
             }
         };
-        auto count = [&](uint32_t c, uint32_t a) -> uint32_t {
+        auto count = [&](uint32_t c, uint32_t a, uint32_t ch) -> uint32_t {
             const unsigned long long key = cpack(c, a);
             if (key == kEmpty64) return negs;
-            if (!big) return cset_count(tk, key, cbucket(c, a, g.seed));
+            if (!big) return cset_count(tk, key, cbucket(chash_a(a, ch)));
             // a big bucket's set, or this CTA's for a chunk that repeats
             // pairs (written in this kernel: read through the L2)
             uint32_t s = gslot(c, a, g.seed) & gmask;
@@ -430,17 +497,45 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
             return 0u;
         };
-        // walk one list of the warp's: entries [lo, hi) of (b, c)'s R list,
-        // 32 a step, two steps in flight
+        // walk one list of the warp's: entries [lo, hi) of (b, c)'s R list in
+        // steps of CC_CH, first the filter bits of the lane's 32 entries
+        // (bit q: entry base + 32 q + lane), then the set for those that
+        // passed, whose a is read again.  Every lane of the warp calls this.
         auto walk = [&](uint32_t jb, uint32_t jc, uint32_t jst, uint32_t lo, uint32_t hi) {
-            for (uint32_t i0 = lo; i0 < hi; i0 += 64) {
-                const uint32_t i = i0 + lane, i2 = i + 32;
-                const uint32_t a = i < hi ? (uint32_t)__ldg(g.r.alist + jst + i) : 0u;
-                const uint32_t a2 = i2 < hi ? (uint32_t)__ldg(g.r.alist + jst + i2) : 0u;
-                const uint32_t m = i < hi ? count(jc, a) : 0u;
-                const uint32_t m2 = i2 < hi ? count(jc, a2) : 0u;
-                emit(a, jb, jc, m);
-                emit(a2, jb, jc, m2);
+            const uint32_t ch = chash(jc, g.seed);
+            for (uint32_t base = lo; base < hi; base += CC_CH) {
+                const int32_t *list = g.r.alist + jst + base + lane;
+                const uint32_t n = min(hi - base, CC_CH);
+                uint32_t hits = 0, s = 0;
+                for (; (s + 4u) * 32u <= n; s += 4u) {
+                    uint32_t a[4], h4 = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[q] = (uint32_t)__ldg(list + 32u * s + 32 * q);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) h4 |= fbit(filt, a[q], ch) << q;
+                    hits |= h4 << s;
+                }
+                if (32u * s < n) {
+                    uint32_t a[4], h4 = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        a[q] = 32u * (s + q) + lane < n ? (uint32_t)__ldg(list + 32u * s + 32 * q) : 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (32u * (s + q) + lane < n) h4 |= fbit(filt, a[q], ch) << q;
+                    hits |= h4 << s;
+                }
+                while (PASS == 0 ? hits != 0u : (bool)__any_sync(0xffffffffu, hits != 0u)) {
+                    uint32_t a = 0, m = 0;
+                    if (hits) {
+                        const uint32_t q = (uint32_t)__ffs((int)hits) - 1u;
+                        hits &= hits - 1u;
+                        a = (uint32_t)__ldg(list + 32u * q);
+                        m = count(jc, a, ch);
+                    }
+                    emit(a, jb, jc, m);
+                }
+                __syncwarp();
             }
         };
         // phase 1: warps take batches of 32 S tuples as they come free;
@@ -515,7 +610,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 uint32_t a = 0, m = 0;
                 if (wi < W) {
                     a = (uint32_t)__ldg(g.r.alist + ost + (wi - oex));
-                    m = count(oc, a);
+                    const uint32_t ch = chash(oc, g.seed);
+                    if (fbit(filt, a, ch)) m = count(oc, a, ch);
                 }
                 emit(a, ob, oc, m);
             }
@@ -583,7 +679,7 @@ uint32_t cyc_c_schunk(int64_t nS, int num_sms) {
 
 size_t cyc_c_rep_slots(int num_sms) { return (size_t)num_sms * CC_MAX_CTAS_PER_SM * CC_TSLOTS; }
 
-uint32_t cyc_c_tcap() { return CC_TCAP; }
+uint32_t cyc_c_tavg() { return CC_TAVG; }
 
 cudaError_t rgroup_build(const int32_t *Ra, const int32_t *Rb, int64_t nR, const RGroup &r, unsigned int *hll,
                          uint64_t reserve, unsigned int *bump, int32_t a_domain, DevStatus *status, int num_sms,
@@ -622,7 +718,7 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
     cudaError_t e;
     {
         ProfScope ps_("cyc_c_plan", st);
-        k_cc_plan<<<(z + 255) / 256, 256, 0, st>>>(g.offS, g.offT, z, g.schunk, items, big_slots);
+        k_cc_plan<<<1, CC_PLAN_T, 0, st>>>(g.offS, g.offT, z, g.schunk, items, (uint32_t *)g.order, big_slots);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(items + z, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
@@ -642,8 +738,8 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
                                                    (uint32_t *)g.bigcnt, (uint32_t *)g.big_neg, g.seed, g.st);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t smem = CC_TSLOTS * sizeof(unsigned long long) + CC_QCAP * sizeof(uint4) +
-                        (CC_QCAP + 1) * sizeof(uint32_t);
+    const size_t smem = CC_TSLOTS * sizeof(unsigned long long) + CC_FWORDS * sizeof(uint32_t) +
+                        CC_QCAP * sizeof(uint4) + (CC_QCAP + 1) * sizeof(uint32_t);
     if ((e = cudaFuncSetAttribute(k_cc_probe<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
         cudaSuccess)
         return e;

@@ -1,0 +1,71 @@
+"""The C-bucket plan's on-chip set and its filter at their edges: T chunks of
+6144 tuples, buckets that move to the L2 above 16384, R lists around the warp
+step of 1024 and the queue's 512, repeated pairs and the (-1, -1) pair behind
+the filter.  All results against the oracle, bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1905_13376_gb300 import binding
+
+from gpu_util import cu, sorted_rows
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    torch.cuda.set_device(0)
+    c = binding.Context(0)
+    yield c
+    c.close()
+
+
+def check(ctx, R, S, T, a_domain, shares):
+    want = oracle.cyclic(R, S, T, oracle.GROUP_BY_A, a_domain=a_domain)
+    got = ctx.join3_cyclic(cu(R), cu(S), cu(T), "group_by_a", shares=shares, a_domain=a_domain)
+    assert int(got["total"].item()) == want["total"]
+    assert np.array_equal(got["counts"].cpu().numpy(), want["counts"])
+    n = want["total"]
+    rows = oracle.cyclic(R, S, T, oracle.MATERIALIZE, capacity=n)["rows"]
+    got = ctx.join3_cyclic(cu(R), cu(S), cu(T), "rows", shares=shares, capacity=n)
+    assert int(got["n_rows"].item()) == n
+    assert np.array_equal(sorted_rows(got["rows"].cpu().numpy()), rows)
+    return n
+
+
+@pytest.mark.parametrize("nt", [6143, 6144, 6145, 12289, 16384, 16385])
+def test_chunk_edges(ctx, nt):
+    """One bucket holding nt T tuples: one, two and three on-chip chunks, and the
+    L2 set."""
+    g = np.random.default_rng(nt)
+    a_dom = 3000
+    T = (g.integers(0, 40, nt).astype(np.int32), g.integers(0, a_dom, nt).astype(np.int32))
+    R = (g.integers(0, a_dom, 5000).astype(np.int32), g.integers(0, 30, 5000).astype(np.int32))
+    S = (g.integers(0, 33, 300).astype(np.int32), g.integers(0, 44, 300).astype(np.int32))
+    assert check(ctx, R, S, T, a_dom, (1, 1, 1)) > 0
+
+
+@pytest.mark.parametrize("length", [1, 31, 32, 127, 128, 129, 511, 512, 1023, 1024, 1025, 2047, 3000])
+def test_list_lengths(ctx, length):
+    """Every b has a list of `length` a values: short, walked and queued lists,
+    full and partial steps; more lists than the queue holds."""
+    g = np.random.default_rng(length)
+    nb, a_dom = 20, 8192
+    R = (g.integers(0, a_dom, nb * length).astype(np.int32), np.repeat(np.arange(nb), length).astype(np.int32))
+    S = (g.integers(0, nb + 2, 900).astype(np.int32), g.integers(0, 50, 900).astype(np.int32))
+    T = (g.integers(0, 50, 6000).astype(np.int32), g.integers(0, a_dom, 6000).astype(np.int32))
+    check(ctx, R, S, T, a_dom, (1, 1, 3))
+
+
+def test_marker_pair_and_repeats(ctx):
+    """(-1, -1) pairs (the empty marker, counted apart) and repeated pairs pass
+    the filter like any other pair."""
+    R = (np.full(300, -1, np.int32), np.arange(300, dtype=np.int32) % 3)
+    S = (np.arange(600, dtype=np.int32) % 4, np.where(np.arange(600) % 2 == 0, -1, 7).astype(np.int32))
+    T = (np.where(np.arange(90) % 3 == 0, -1, 7).astype(np.int32), np.full(90, -1, np.int32))
+    want = oracle.cyclic(R, S, T, oracle.COUNT)["total"]
+    assert want > 0
+    for shares in ((1, 1, 1), (1, 1, 5), None):
+        assert int(ctx.join3_cyclic(cu(R), cu(S), cu(T), "count", shares=shares)["total"].item()) == want
