@@ -91,23 +91,15 @@ struct LinLayout {
     void *pscratch; size_t pscratch_bytes;
     void *pscratchR;   // single mode: R's own partition scratch (R is partitioned on the side stream)
     unsigned long long *rowcount, *base; void *sscratch;
-    WTable w; unsigned int *whll;   // one-bucket plan: S's weight table
+    OneBucket one;   // one-bucket plan
 };
 
 size_t lin_layout(Arena &A, const LinPlan &p, const mwj_rel &R, const mwj_rel &S,
                   const mwj_rel &T, int num_sms, LinLayout &L) {
     L = LinLayout{};
     if (p.l2) {   // nothing is partitioned: T's table and S's weight table
-        L.img = A.take<uint64_t>(single_table_slots(T.n));
-        L.meta = A.take<uint32_t>(kMetaWords);
-        L.hll = A.take<unsigned int>(hll_scratch_registers(num_sms));
-        const size_t ws = w_table_slots(S.n) + 2;
-        L.w.W = A.take<unsigned long long>(ws);
-        L.w.hi = A.take<uint32_t>(ws);
-        L.w.meta = A.take<uint32_t>(kMetaWords);
-        L.whll = A.take<unsigned int>(hll_scratch_registers(num_sms));
-        L.heavy = A.take<uint32_t>(kHeavyTableWords);
-        L.hw = A.take<unsigned long long>(kHeavySlots);
+        const mwj_rel rel[3] = {R, S, T};
+        one_bucket_layout(A, rel, 3, num_sms, L.one);
         return A.used;
     }
     const uint32_t extra = p.heavy ? 1u : 0u;   // the heavy-key bucket
@@ -399,6 +391,13 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
 
     const Seeds &sd = ctx->seeds;
     cudaError_t e;
+    if (p.l2) {
+        const mwj_rel rel[3] = {R, S, T};
+        e = one_bucket_run(L.one, rel, 3, sd, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
+                           (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
+                           ctx->dev.num_sms, st);
+        return e == cudaSuccess ? MWJ_OK : cuda_fail(ctx, e, "one-bucket plan");
+    }
     if ((e = cudaMemsetAsync(out->total, 0, sizeof(int64_t), st)) != cudaSuccess)
         return cuda_fail(ctx, e, "memset total");
     if (out->mode == MWJ_COUNT_GROUP_BY_A &&
@@ -422,50 +421,6 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
     // that each kernel's event pair times that kernel alone
     cudaStream_t side = ctx->prof.on ? st : ctx->side;
     cudaStream_t side2 = ctx->prof.on ? st : ctx->side2;
-    if (p.l2) {
-        // T's table on the side stream while S's weight table is sized and
-        // cleared here; then the S pass and the R pass.  T's C values and
-        // S's B values may get the direct-address layout (only these passes
-        // read the two tables).  When T's C column is S's B column (a
-        // self-join such as friends of friends of friends) one pass over it
-        // sizes both tables.
-        L.w.seed = sd.slot;
-        L.w.heavy = L.heavy;
-        const bool same_keys = T.x == S.x && T.n == S.n;
-        if (same_keys) {
-            e = w_table_size(S.x, S.n, L.w, L.whll, w_table_slots(S.n), ctx->dev.num_sms, st, L.meta,
-                             single_table_slots(T.n));
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "table sizes");
-        }
-        if ((e = cudaEventRecord(ctx->fork, st)) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(side, ctx->fork, 0)) != cudaSuccess)
-            return cuda_fail(ctx, e, "fork");
-        if (same_keys)
-            e = single_table_fill(T.x, T.n, sd.slot2, L.meta, L.img, ctx->status, ctx->dev.num_sms, side);
-        else
-            e = single_table_direct(T.x, T.n, sd.slot2, L.hll, L.meta, L.img, single_table_slots(T.n),
-                                    ctx->status, ctx->dev.num_sms, side, true);
-        const cudaError_t ej = cudaEventRecord(ctx->join, side);
-        if (ej != cudaSuccess) return cuda_fail(ctx, ej, "join");
-        join_guard.armed = true;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "T table");
-        if ((e = heavy_detect(R.y, R.n, S.x, S.n, kWHeavyBuckets, L.heavy, L.hw, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "heavy keys");
-        e = same_keys ? w_table_clear(L.w, ctx->dev.num_sms, st)
-                      : w_table_prepare(S.x, S.n, L.w, L.whll, w_table_slots(S.n), ctx->dev.num_sms, st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "S weight table");
-        e = cudaStreamWaitEvent(st, ctx->join, 0);
-        join_guard.armed = false;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "join");
-        const TImg t{L.img, nullptr, nullptr, nullptr, nullptr, L.meta, 0u, sd.C, sd.slot2};
-        e = w_table_build(S.x, S.y, S.n, t, L.w, ctx->status, ctx->dev.num_sms, st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "S pass");
-        const int mode = out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0;
-        e = w_table_probe(R.x, R.y, R.n, L.w, mode, out->a_domain, (unsigned long long *)out->group_counts,
-                          (unsigned long long *)out->total, ctx->status, ctx->dev.num_sms, st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "R pass");
-        return MWJ_OK;
-    }
     if (p.single) {
         if ((e = cudaEventRecord(ctx->fork, st)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(side, ctx->fork, 0)) != cudaSuccess)

@@ -14,8 +14,15 @@
 //     GROUP BY A     cnt[a] += sum over (b,c) in S of w_T(c)   for (a,b) in R
 // which is the definition of the chain's count summed level by level.  No
 // intermediate relation is materialised; every relation is read once.
+//
+// That is the plan of explicit shares.  Without shares the call takes the
+// one-bucket plan of linear_l2.cu, one level longer: the T pass builds w_T in
+// the same way as the S pass builds w, R and S are never partitioned.  F of the
+// 2^20-vertex power-law graph joined with itself four times: 1.59 ms
+// partitioned (scatter 0.48, probe 0.50, T weights 0.24), 0.50 ms in one bucket.
 #include "api_internal.h"
 #include "linear.h"
+#include "linear_l2.h"
 #include "tables.h"
 
 namespace mwj {
@@ -132,10 +139,13 @@ size_t j4_layout(Arena &A, uint32_t I, const mwj_rel &R, const mwj_rel &S, const
     return A.used;
 }
 
-mwj_status j4_shares(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T,
-                     const mwj_shares *shares, uint32_t *I, uint32_t *cap_log2) {
-    mwj_shares sh;
-    if (shares) sh = *shares; else plan_linear_default(ctx, R, S, T, &sh);
+// The one-bucket plan's tables, in the same workspace.
+size_t j4_one_layout(Arena &A, const mwj_rel (&rel)[4], int num_sms, OneBucket &L) {
+    one_bucket_layout(A, rel, 4, num_sms, L);
+    return A.used;
+}
+
+mwj_status j4_shares(mwj_ctx *ctx, const mwj_shares &sh, uint32_t *I, uint32_t *cap_log2) {
     if (sh.s[0] < 1 || (uint32_t)sh.s[0] > kMaxBuckets)
         return fail(ctx, MWJ_ERR_INVALID_ARG, "4-relation chain: s[0] must be in [1, %u]", kMaxBuckets);
     if (sh.s[1] != 1) return fail(ctx, MWJ_ERR_INVALID_ARG, "4-relation chain: s[1] must be 1");
@@ -158,10 +168,16 @@ extern "C" mwj_status mwj_join4_workspace_size(mwj_ctx *ctx, mwj_rel R, mwj_rel 
         return fail(ctx, MWJ_ERR_INVALID_ARG, "bad relation");
     if (mode != MWJ_COUNT && mode != MWJ_COUNT_GROUP_BY_A)
         return fail(ctx, MWJ_ERR_INVALID_ARG, "4-relation chain: COUNT or COUNT GROUP BY A only");
-    uint32_t I, cl;
-    mwj_status s = j4_shares(ctx, R, S, T, shares, &I, &cl);
-    if (s != MWJ_OK) return s;
     Arena A(nullptr, 0);
+    if (!shares) {
+        const mwj_rel rel[4] = {R, S, T, U};
+        OneBucket L;
+        *bytes = j4_one_layout(A, rel, ctx->dev.num_sms, L);
+        return MWJ_OK;
+    }
+    uint32_t I, cl;
+    mwj_status s = j4_shares(ctx, *shares, &I, &cl);
+    if (s != MWJ_OK) return s;
     J4Layout L;
     *bytes = j4_layout(A, I, R, S, T, U, ctx->dev.num_sms, L);
     return MWJ_OK;
@@ -178,9 +194,21 @@ extern "C" mwj_status mwj_join4_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
     if (s != MWJ_OK) return s;
     if (out->mode != MWJ_COUNT && out->mode != MWJ_COUNT_GROUP_BY_A)
         return fail(ctx, MWJ_ERR_INVALID_ARG, "4-relation chain: COUNT or COUNT GROUP BY A only");
-    uint32_t I, cap_log2;
-    if ((s = j4_shares(ctx, R, S, T, shares, &I, &cap_log2)) != MWJ_OK) return s;
     Arena A(workspace, ws_bytes);
+    if (!shares) {
+        const mwj_rel rel[4] = {R, S, T, U};
+        OneBucket L;
+        j4_one_layout(A, rel, ctx->dev.num_sms, L);
+        if (A.overflow || !workspace)
+            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
+        const cudaError_t eo =
+            one_bucket_run(L, rel, 4, ctx->seeds, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
+                           (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
+                           ctx->dev.num_sms, (cudaStream_t)stream);
+        return eo == cudaSuccess ? MWJ_OK : cuda_fail(ctx, eo, "chain of four, one bucket");
+    }
+    uint32_t I, cap_log2;
+    if ((s = j4_shares(ctx, *shares, &I, &cap_log2)) != MWJ_OK) return s;
     J4Layout L;
     j4_layout(A, I, R, S, T, U, ctx->dev.num_sms, L);
     if (A.overflow || !workspace)

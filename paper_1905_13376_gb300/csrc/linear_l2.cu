@@ -19,6 +19,8 @@
 // per distinct b, and runs of equal keys (edge lists sorted by source) are
 // summed inside each warp before they reach the L2; the R pass only reads
 // the table and adds each run of equal a once.
+#include <type_traits>
+
 #include "internal.h"
 #include "linear_l2.h"
 #include "skew.h"
@@ -55,53 +57,92 @@ __device__ __forceinline__ uint32_t load_pairs(const int32_t *__restrict__ X, co
     return m;
 }
 
-// deg_T(c) from the first probe (slot s, value v) of c in T's single table.
-__device__ __forceinline__ unsigned long long t_deg(const uint64_t *__restrict__ img, uint32_t tmask,
-                                                    uint32_t c, uint32_t s, unsigned long long v) {
-    for (uint32_t it = 0; it < tmask && v != kEmpty64 && (uint32_t)v != c; ++it) {
-        s = (s + 1) & tmask;
-        v = __ldg((const unsigned long long *)(img + s));
-    }
-    return (v == kEmpty64 || (uint32_t)v != c) ? 0ull : (v >> 32);
+// Hashed degrees: the pair of slots at which the search for key k starts.
+__device__ __forceinline__ uint32_t deg_home(uint32_t k, uint32_t seed, uint32_t mask) {
+    return slot_of(k, seed, mask) & ~1u;
 }
 
-// w(b) += x (x > 0).  The key is claimed with a CAS that also stores x's low
-// word; later adds go to the upper word, and the carry out of it (read back
-// from the add's old value) goes to hi[].
-__device__ __forceinline__ void w_add(const WTable &w, uint32_t mask, uint32_t b, unsigned long long x,
-                                      DevStatus *st) {
-    if (b == kEmptyKey) {
-        atomicAdd(w.W + mask + 1, x);
-        return;
+// deg(c) from its home pair (slot s, value v): the first slot holding c, or
+// none when a free slot comes first.
+__device__ __forceinline__ unsigned long long deg_get(const unsigned long long *__restrict__ slots, uint32_t mask,
+                                                      uint32_t c, uint32_t s, ulonglong2 v) {
+    for (uint32_t it = 0; it <= mask; it += 2) {
+        if ((uint32_t)v.x == c && v.x != kEmpty64) return v.x >> 32;
+        if ((uint32_t)v.y == c && v.y != kEmpty64) return v.y >> 32;
+        if (v.x == kEmpty64 || v.y == kEmpty64) break;
+        s = (s + 2) & mask;
+        v = __ldg((const ulonglong2 *)(slots + s));
     }
-    const unsigned long long lo = x & 0xFFFFFFFFull;
-    const uint32_t hx = (uint32_t)(x >> 32);
-    uint32_t s = slot_of(b, w.seed, mask);
-    for (uint32_t it = 0; it <= mask; ++it) {
-        unsigned long long v = __ldcg(w.W + s);
-        if (v == kEmpty64) {
-            const unsigned long long old = atomicCAS(w.W + s, kEmpty64, (lo << 32) | b);
-            if (old == kEmpty64) {
-                if (hx) {
-                    atomicAdd(w.hi + s, hx);
-                    atomicOr(w.meta + 2, 1u);
-                }
+    return 0ull;
+}
+
+// deg(c) += x from its home pair (possibly read before other threads claimed
+// slots of it: a claim is a CAS, a key once there stays).
+__device__ __forceinline__ void deg_add(unsigned long long *slots, uint32_t mask, uint32_t c, uint32_t s, ulonglong2 v,
+                                        uint32_t x, DevStatus *st) {
+    const unsigned long long fresh = ((unsigned long long)x << 32) | c;
+    for (uint32_t it = 0; it <= mask; it += 2) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            unsigned long long u = q ? v.y : v.x;
+            if (u == kEmpty64) {
+                u = atomicCAS(slots + s + q, kEmpty64, fresh);
+                if (u == kEmpty64) return;
+            }
+            if ((uint32_t)u == c) {
+                atomicAdd(slots + s + q, (unsigned long long)x << 32);
                 return;
             }
-            v = old;
         }
-        if ((uint32_t)v == b) {
-            const unsigned long long old = atomicAdd(w.W + s, lo << 32);
-            const uint32_t h = hx + (uint32_t)(((old >> 32) + lo) >> 32);
-            if (h) {
-                atomicAdd(w.hi + s, h);
-                atomicOr(w.meta + 2, 1u);
-            }
-            return;
-        }
-        s = (s + 1) & mask;
+        s = (s + 2) & mask;
+        v = __ldcg((const ulonglong2 *)(slots + s));
     }
-    set_status(st, MWJ_ERR_CHECK, 7);   // table full: the sizing step under-estimated
+    set_status(st, MWJ_ERR_CHECK, 3);   // table full: the sizing step under-estimated
+}
+
+// Hashed weights: the group of four keys at which the search for key k starts.
+__device__ __forceinline__ uint32_t w_home(uint32_t k, uint32_t seed, uint32_t mask) {
+    return slot_of(k, seed, mask) & ~3u;
+}
+
+// Slot of key k (not -1) from its home group (slot s, keys v); kEmptyKey when a
+// free slot comes first.
+__device__ __forceinline__ uint32_t w_find(const uint32_t *__restrict__ keys, uint32_t mask, uint32_t k, uint32_t s,
+                                           uint4 v) {
+    for (uint32_t it = 0; it <= mask; it += 4) {
+        if (v.x == k) return s;
+        if (v.y == k) return s + 1;
+        if (v.z == k) return s + 2;
+        if (v.w == k) return s + 3;
+        if (v.w == kEmptyKey) break;   // (a group fills in order: v.w free says that it is not full)
+        s = (s + 4) & mask;
+        v = __ldg((const uint4 *)(keys + s));
+    }
+    return kEmptyKey;
+}
+
+// Slot of key k (not -1), claimed if it is new, from its home group (possibly
+// read before other threads claimed slots of it); kEmptyKey: the table is full.
+__device__ __forceinline__ uint32_t w_claim(uint32_t *keys, uint32_t mask, uint32_t k, uint32_t s, uint4 v) {
+    for (uint32_t it = 0; it <= mask; it += 4) {
+        if (v.x == k) return s;
+        if (v.y == k) return s + 1;
+        if (v.z == k) return s + 2;
+        if (v.w == k) return s + 3;
+        if (v.w == kEmptyKey) {
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                uint32_t u = q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w;
+                if (u == kEmptyKey) {
+                    u = atomicCAS(keys + s + q, kEmptyKey, k);
+                    if (u == kEmptyKey || u == k) return s + q;
+                }
+            }
+        }
+        s = (s + 4) & mask;
+        v = __ldcg((const uint4 *)(keys + s));
+    }
+    return kEmptyKey;
 }
 
 // Direct-address weights (the sizing pass chose that layout for S's B
@@ -115,99 +156,147 @@ __device__ __forceinline__ void w_add_direct(unsigned long long *__restrict__ W,
         set_status(st, MWJ_ERR_CHECK, 9);   // a key outside the range the sizing pass saw
 }
 
-__global__ void k_w_clear(unsigned long long *__restrict__ W, uint32_t *__restrict__ hi,
-                          uint32_t *__restrict__ meta) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    if (meta[kMetaDense]) {
-        const uint32_t span = meta[kMetaSpan];
-        for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < span; s += stride) W[s] = 0ull;
-    } else {
-        const uint32_t slots = meta[0] + 1;   // a power of two >= 16
-        for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < slots / 2; s += stride) {
-            ((ulonglong2 *)W)[s] = make_ulonglong2(kEmpty64, kEmpty64);
-            ((uint2 *)hi)[s] = make_uint2(0u, 0u);
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            W[slots] = 0ull;
-            hi[slots] = 0u;
+// w(k[q]) for the lane's tuples q < m (0 for the others) from a weight table
+// in either layout; hashed: the key groups are loaded together, then the sums.
+template <bool WD>
+struct WLookup {
+    const WTable &w;
+    uint32_t mask, min, span;
+    __device__ explicit WLookup(const WTable &w_) : w(w_) {
+        mask = __ldg(w.meta);
+        min = WD ? __ldg(w.meta + kMetaMin) : 0u;
+        span = WD ? __ldg(w.meta + kMetaSpan) : 0u;
+    }
+    __device__ __forceinline__ void operator()(const int32_t (&k)[WQ], uint32_t m, unsigned long long (&x)[WQ]) const {
+        if constexpr (WD) {
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) {
+                const uint32_t i = (uint32_t)k[q] - min;
+                x[q] = ((uint32_t)q < m && i < span) ? __ldg(w.W + i) : 0ull;
+            }
+        } else {
+            uint32_t s[WQ];
+            uint4 v[WQ];
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) {
+                s[q] = w_home((uint32_t)k[q], w.seed, mask);
+                if ((uint32_t)q < m) v[q] = __ldg((const uint4 *)(w.keys + s[q]));
+            }
+#pragma unroll
+            for (int q = 0; q < WQ; ++q)
+                if ((uint32_t)q < m)
+                    s[q] = (uint32_t)k[q] == kEmptyKey ? mask + 1 : w_find(w.keys, mask, (uint32_t)k[q], s[q], v[q]);
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) x[q] = ((uint32_t)q < m && s[q] != kEmptyKey) ? __ldg(w.W + s[q]) : 0ull;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) meta[kMetaWide] = 0u;
+};
+
+// deg(k[q]) in the same way from a direct-address degree table.
+struct DegLookup {
+    const uint32_t *deg;
+    uint32_t min, span;
+    __device__ explicit DegLookup(const DegTable &t)
+        : deg((const uint32_t *)t.slots), min(__ldg(t.meta + kMetaMin)), span(__ldg(t.meta + kMetaSpan)) {}
+    __device__ __forceinline__ void operator()(const int32_t (&k)[WQ], uint32_t m, unsigned long long (&x)[WQ]) const {
+#pragma unroll
+        for (int q = 0; q < WQ; ++q) {
+            const uint32_t i = (uint32_t)k[q] - min;
+            x[q] = ((uint32_t)q < m && i < span) ? (unsigned long long)__ldg(deg + i) : 0ull;
+        }
+    }
+};
+
+// A CTA's sums of heavy keys in shared memory, 64 bits in two 32-bit words: a
+// 32-bit shared-memory add is one instruction, a 64-bit one a CAS loop, which
+// spins when a warp's lanes hold the same key -- and here they do.
+struct HeavySums {
+    uint32_t lo[kHeavySlots], hi[kHeavySlots];
+};
+__device__ __forceinline__ void heavy_add(HeavySums &h, int i, unsigned long long x) {
+    const uint32_t xl = (uint32_t)x;
+    uint32_t xh = (uint32_t)(x >> 32);
+    const uint32_t old = atomicAdd(&h.lo[i], xl);
+    xh += old + xl < xl ? 1u : 0u;
+    if (xh) atomicAdd(&h.hi[i], xh);
+}
+__device__ __forceinline__ unsigned long long heavy_sum(const HeavySums &h, uint32_t i) {
+    return ((unsigned long long)h.hi[i] << 32) | h.lo[i];
+}
+// The table of heavy keys and zero sums (every thread of the CTA calls this;
+// ends with a barrier when there are keys); null when there are none.
+__device__ __forceinline__ const uint32_t *heavy_begin(const uint32_t *heavy, uint32_t *buf, HeavySums &sums) {
+    const uint32_t *hs = heavy_to_smem(heavy, buf);
+    if (!hs) return nullptr;
+    for (uint32_t i = threadIdx.x; i < kHeavySlots; i += blockDim.x) sums.lo[i] = sums.hi[i] = 0u;
+    __syncthreads();
+    return hs;
 }
 
-// S pass.  Warp-uniform loop: a warp takes 128 consecutive tuples per round,
-// four per lane, and loads its next round before it works on this one.
-// Heavy keys (sampled, see heavy_detect) are summed per CTA in shared
-// memory and added to the table once per CTA, so that a key holding a large
-// share of S in no particular order does not funnel every warp's adds into
-// one L2 word.  TD / WD: T's table / S's weight table in the direct-address
-// layout (one load per T lookup, one fire-and-forget 64-bit add per run of
-// equal B values) rather than hashed.
-// One warp round of the S pass: lane l holds tuples (b[q], c[q]), q < m, of
-// 128 consecutive ones.  x = deg_T(c); heavy B keys go to the CTA's sums;
-// runs of equal b are summed in the warp and added to w(b) once.
-template <bool TD, bool WD>
+// The source of a weight pass: the degree table of the relation below, or
+// (chains of four) its weight table.
+struct Source {
+    DegTable t;
+    WTable w;
+};
+template <bool SW>
+using Lookup = typename std::conditional<SW, WLookup<true>, DegLookup>::type;
+template <bool SW>
+__device__ __forceinline__ bool source_dense(const Source &src) {
+    return __ldg((SW ? src.w.meta : src.t.meta) + kMetaDense) != 0u;
+}
+template <bool SW>
+__device__ __forceinline__ Lookup<SW> make_lookup(const Source &src) {
+    if constexpr (SW)
+        return WLookup<true>(src.w);
+    else
+        return DegLookup(src.t);
+}
+
+// S pass, both tables in the direct-address layout.  Warp-uniform loop: a warp
+// takes 128 consecutive tuples per round, four per lane, and loads its next
+// round before it works on this one.  Heavy keys (sampled, see skew.h) are
+// summed per CTA in shared memory and added to the table once per CTA, so
+// that a key holding a large share of S in no particular order does not funnel
+// every warp's adds into one L2 word.
+// SW: the source is a weight table (chains of four), not a degree table.
+// One warp round: lane l holds tuples (b[q], c[q]), q < m, of 128 consecutive
+// ones.  x = the source's value of c; heavy B keys go to the CTA's sums; runs
+// of equal b are summed in the warp and added to w(b) once (one
+// fire-and-forget 64-bit add).
+template <bool SW>
 struct SPass {
-    const TImg &t;
+    const Lookup<SW> look;
     const WTable &w;
     DevStatus *st;
     const uint32_t *hs;
-    unsigned long long *hacc;
-    uint32_t tmask, wmask, tmin, tspan, wmin, wspan;
+    HeavySums &hacc;
+    uint32_t wmin, wspan;
 
-    __device__ SPass(const TImg &t_, const WTable &w_, DevStatus *st_, const uint32_t *hs_,
-                     unsigned long long *hacc_)
-        : t(t_), w(w_), st(st_), hs(hs_), hacc(hacc_) {
-        tmask = __ldg(t.meta);
-        wmask = __ldg(w.meta);
-        tmin = TD ? __ldg(t.meta + kMetaMin) : 0u;
-        tspan = TD ? __ldg(t.meta + kMetaSpan) : 0u;
-        wmin = WD ? __ldg(w.meta + kMetaMin) : 0u;
-        wspan = WD ? __ldg(w.meta + kMetaSpan) : 0u;
+    __device__ SPass(const Source &src, const WTable &w_, DevStatus *st_, const uint32_t *hs_,
+                     HeavySums &hacc_)
+        : look(make_lookup<SW>(src)), w(w_), st(st_), hs(hs_), hacc(hacc_) {
+        wmin = __ldg(w.meta + kMetaMin);
+        wspan = __ldg(w.meta + kMetaSpan);
     }
 
     __device__ __forceinline__ void round(const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) {
         unsigned long long x[WQ];
-        if constexpr (TD) {
-            const uint32_t *tdeg = (const uint32_t *)t.img;
-#pragma unroll
-            for (int q = 0; q < WQ; ++q) {
-                const uint32_t k = (uint32_t)c[q] - tmin;
-                x[q] = ((uint32_t)q < m && k < tspan) ? (unsigned long long)__ldg(tdeg + k) : 0ull;
-            }
-        } else {
-            uint32_t ts[WQ];
-            unsigned long long tv[WQ];
-#pragma unroll
-            for (int q = 0; q < WQ; ++q) {
-                if ((uint32_t)q < m) {
-                    ts[q] = slot_of((uint32_t)c[q], t.seed_slot, tmask);
-                    tv[q] = __ldg((const unsigned long long *)(t.img + ts[q]));
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < WQ; ++q)
-                x[q] = ((uint32_t)q < m) ? t_deg(t.img, tmask, (uint32_t)c[q], ts[q], tv[q]) : 0ull;
-        }
+        look(c, m, x);
         if (hs) {
 #pragma unroll
             for (int q = 0; q < WQ; ++q) {
                 if (x[q] == 0) continue;
                 const int hsl = heavy_slot(hs, (uint32_t)b[q]);
                 if (hsl >= 0) {
-                    atomicAdd(&hacc[hsl], x[q]);
+                    heavy_add(hacc, hsl, x[q]);
                     x[q] = 0;
                 }
             }
         }
-        warp_runs(b, x, m, [&](int32_t key, unsigned long long sum) { add((uint32_t)key, sum); });
-    }
-
-    __device__ __forceinline__ void add(uint32_t b, unsigned long long x) {
-        if constexpr (WD)
-            w_add_direct(w.W, wmin, wspan, b, x, st);
-        else
-            w_add(w, wmask, b, x, st);
+        warp_runs(b, x, m, [&](int32_t key, unsigned long long sum) {
+            w_add_direct(w.W, wmin, wspan, (uint32_t)key, sum, st);
+        });
     }
 
     // the CTA's heavy-key sums into the table (every thread of the CTA calls this)
@@ -215,7 +304,7 @@ struct SPass {
         if (!hs) return;
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < kHeavySlots; i += nthreads)
-            if (hacc[i]) add(hs[i], hacc[i]);
+            if (heavy_sum(hacc, i)) w_add_direct(w.W, wmin, wspan, hs[i], heavy_sum(hacc, i), st);
     }
 };
 
@@ -250,65 +339,113 @@ __device__ __forceinline__ void rounds_plain(const int32_t *__restrict__ X, cons
     }
 }
 
-template <bool TD, bool WD>
-__device__ __forceinline__ void w_build_pass(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
-                                             uint32_t n, const TImg &t, const WTable &w, DevStatus *st,
-                                             const uint32_t *hs, unsigned long long *hacc) {
-    SPass<TD, WD> P(t, w, st, hs, hacc);
+// Two kernels share the S pass: the direct-address one (both tables in that
+// layout) and the general one; the call launches both and the one whose
+// layout the sizing passes did not choose returns at once.
+//
+// The general one: a tuple per lane, few registers, six CTAs per SM.  A hashed
+// add is a chain of dependent accesses (key group, perhaps a claim or the next
+// group, then the add) that the whole warp waits out; with four tuples per
+// lane a warp waited for four such chains, one after the other, and 80
+// registers left only three CTAs to fill the waits.  8.4 million id-keyed
+// tuples into 1.5 million keys: 0.235 ms with four, 0.154 ms with one.
+constexpr int GC = 6;
+template <bool SW>
+__global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
+                                                    uint32_t n, Source src, WTable w, DevStatus *st) {
+    const bool sd = source_dense<SW>(src), wd = __ldg(w.meta + kMetaDense) != 0u;
+    if (sd && wd) return;
+    __shared__ uint32_t hbuf[kHeavySlots];
+    __shared__ HeavySums hacc;
+    const uint32_t *hs = heavy_begin(w.heavy, hbuf, hacc);
+    const uint32_t *smeta = SW ? src.w.meta : src.t.meta;
+    const uint32_t smask = __ldg(smeta + kMetaMask), smin = sd ? __ldg(smeta + kMetaMin) : 0u,
+                   sspan = sd ? __ldg(smeta + kMetaSpan) : 0u;
+    const uint32_t wmask = __ldg(w.meta + kMetaMask), wmin = wd ? __ldg(w.meta + kMetaMin) : 0u,
+                   wspan = wd ? __ldg(w.meta + kMetaSpan) : 0u;
+    auto value = [&](uint32_t c) -> unsigned long long {
+        if (sd) {
+            const uint32_t i = c - smin;
+            if (i >= sspan) return 0ull;
+            return SW ? __ldg(src.w.W + i) : (unsigned long long)__ldg((const uint32_t *)src.t.slots + i);
+        }
+        if constexpr (SW) {
+            if (c == kEmptyKey) return __ldg(src.w.W + smask + 1);
+            const uint32_t s = w_home(c, src.w.seed, smask);
+            const uint32_t at = w_find(src.w.keys, smask, c, s, __ldg((const uint4 *)(src.w.keys + s)));
+            return at == kEmptyKey ? 0ull : __ldg(src.w.W + at);
+        } else {
+            const uint32_t s = deg_home(c, src.t.seed, smask);
+            return deg_get(src.t.slots, smask, c, s, __ldg((const ulonglong2 *)(src.t.slots + s)));
+        }
+    };
+    auto add = [&](uint32_t b, uint32_t s, uint4 v, unsigned long long x) {
+        if (wd) {
+            w_add_direct(w.W, wmin, wspan, b, x, st);
+            return;
+        }
+        const uint32_t at = b == kEmptyKey ? wmask + 1 : w_claim(w.keys, wmask, b, s, v);
+        if (at != kEmptyKey)
+            atomicAdd(w.W + at, x);
+        else
+            set_status(st, MWJ_ERR_CHECK, 7);   // table full: the sizing step under-estimated
+    };
+    const uint32_t T = gridDim.x * WT, lane = threadIdx.x & 31;
+    uint64_t i = (uint64_t)blockIdx.x * WT + threadIdx.x;
+    int32_t b = 0, c = 0;
+    if (i < n) {
+        b = __ldg(Sb + i);
+        c = __ldg(Sc + i);
+    }
+    for (; i - lane < n; i += T) {
+        int32_t nb = 0, nc = 0;
+        if (i + T < n) {
+            nb = __ldg(Sb + i + T);
+            nc = __ldg(Sc + i + T);
+        }
+        const bool has = i < n;
+        uint32_t s = 0;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (!wd) {   // the target's key group, with the source's slot
+            s = w_home((uint32_t)b, w.seed, wmask);
+            v = __ldcg((const uint4 *)(w.keys + s));
+        }
+        unsigned long long x = has ? value((uint32_t)c) : 0ull;
+        if (hs && x) {
+            const int hsl = heavy_slot(hs, (uint32_t)b);
+            if (hsl >= 0) {
+                heavy_add(hacc, hsl, x);
+                x = 0ull;
+            }
+        }
+        const unsigned long long sum = warp_run_sum1(b, x, has);
+        if (sum) add((uint32_t)b, s, v, sum);
+        b = nb;
+        c = nc;
+    }
+    if (!hs) return;
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < kHeavySlots; j += WT) {
+        const unsigned long long x = heavy_sum(hacc, j);
+        if (!x) continue;
+        const uint32_t s = wd ? 0u : w_home(hs[j], w.seed, wmask);
+        add(hs[j], s, wd ? make_uint4(0u, 0u, 0u, 0u) : __ldcg((const uint4 *)(w.keys + s)), x);
+    }
+}
+
+template <bool SW>
+__global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict__ Sb,
+                                                       const int32_t *__restrict__ Sc, uint32_t n, Source src,
+                                                       WTable w, DevStatus *st) {
+    if (!source_dense<SW>(src) || !__ldg(w.meta + kMetaDense)) return;
+    __shared__ uint32_t hbuf[kHeavySlots];
+    __shared__ HeavySums hacc;
+    const uint32_t *hs = heavy_begin(w.heavy, hbuf, hacc);
+    SPass<SW> P(src, w, st, hs, hacc);
     const uint32_t warp = (blockIdx.x * WT + threadIdx.x) >> 5, warps = (gridDim.x * WT) >> 5;
     rounds_plain(Sb, Sc, 0u, n, warp, warps,
                  [&](const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) { P.round(b, c, m); });
     P.flush_heavy(WT);
-}
-
-// Two kernels share the S pass: the direct-address one (both tables in that
-// layout, few registers) and the general one; the call launches both and the
-// one whose layout the sizing passes did not choose returns at once.
-__global__ void __launch_bounds__(WT) k_w_build(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
-                                                uint32_t n, TImg t, WTable w, DevStatus *st) {
-    const bool td = __ldg(t.meta + kMetaDense) != 0u, wd = __ldg(w.meta + kMetaDense) != 0u;
-    if (td && wd) return;
-    __shared__ uint32_t hbuf[kHeavySlots];
-    __shared__ unsigned long long hacc[kHeavySlots];
-    const uint32_t *hs = heavy_to_smem(w.heavy, hbuf);
-    if (hs) {
-        for (uint32_t i = threadIdx.x; i < kHeavySlots; i += WT) hacc[i] = 0ull;
-        __syncthreads();
-    }
-    if (td)
-        w_build_pass<true, false>(Sb, Sc, n, t, w, st, hs, hacc);
-    else if (wd)
-        w_build_pass<false, true>(Sb, Sc, n, t, w, st, hs, hacc);
-    else
-        w_build_pass<false, false>(Sb, Sc, n, t, w, st, hs, hacc);
-}
-
-__global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict__ Sb,
-                                                       const int32_t *__restrict__ Sc, uint32_t n, TImg t,
-                                                       WTable w, DevStatus *st) {
-    if (!__ldg(t.meta + kMetaDense) || !__ldg(w.meta + kMetaDense)) return;
-    __shared__ uint32_t hbuf[kHeavySlots];
-    __shared__ unsigned long long hacc[kHeavySlots];
-    const uint32_t *hs = heavy_to_smem(w.heavy, hbuf);
-    if (hs) {
-        for (uint32_t i = threadIdx.x; i < kHeavySlots; i += WT) hacc[i] = 0ull;
-        __syncthreads();
-    }
-    w_build_pass<true, true>(Sb, Sc, n, t, w, st, hs, hacc);
-}
-
-// w(b) from the first probe (slot s, value v); 0 when b is not in S.
-__device__ __forceinline__ unsigned long long w_get(const WTable &w, uint32_t mask, bool wide, uint32_t b,
-                                                    uint32_t s, unsigned long long v) {
-    if (b == kEmptyKey) return v;   // slot mask + 1: the plain sum of key -1
-    for (uint32_t it = 0; it < mask && v != kEmpty64 && (uint32_t)v != b; ++it) {
-        s = (s + 1) & mask;
-        v = __ldg(w.W + s);
-    }
-    if (v == kEmpty64 || (uint32_t)v != b) return 0ull;
-    unsigned long long r = v >> 32;
-    if (wide) r += (unsigned long long)__ldg(w.hi + s) << 32;
-    return r;
 }
 
 // R pass (MODE 0: COUNT, MODE 1: GROUP BY A); same loop as the S pass.
@@ -318,48 +455,20 @@ __device__ __forceinline__ unsigned long long w_get(const WTable &w, uint32_t ma
 // cnt[a].
 template <int MODE, bool WD>
 struct RPass {
-    const WTable &w;
+    const WLookup<WD> look;
     int32_t a_domain;
     unsigned long long *cnt;
     DevStatus *st;
-    uint32_t wmask, wmin, wspan;
-    bool wide;
     unsigned long long acc = 0;
 
-    __device__ RPass(const WTable &w_, int32_t a_domain_, unsigned long long *cnt_, DevStatus *st_)
-        : w(w_), a_domain(a_domain_), cnt(cnt_), st(st_) {
-        wmask = __ldg(w.meta);
-        wide = !WD && __ldg(w.meta + kMetaWide) != 0;
-        wmin = WD ? __ldg(w.meta + kMetaMin) : 0u;
-        wspan = WD ? __ldg(w.meta + kMetaSpan) : 0u;
-    }
+    __device__ RPass(const WTable &w, int32_t a_domain_, unsigned long long *cnt_, DevStatus *st_)
+        : look(w), a_domain(a_domain_), cnt(cnt_), st(st_) {}
 
     __device__ __forceinline__ void round(const int32_t (&a)[WQ], const int32_t (&b)[WQ], uint32_t m) {
         unsigned long long x[WQ];
-        if constexpr (WD) {
+        look(b, m, x);
 #pragma unroll
-            for (int q = 0; q < WQ; ++q) {
-                const uint32_t k = (uint32_t)b[q] - wmin;
-                x[q] = ((uint32_t)q < m && k < wspan) ? __ldg(w.W + k) : 0ull;
-                acc += x[q];
-            }
-        } else {
-            uint32_t ws[WQ];
-            unsigned long long wv[WQ];
-#pragma unroll
-            for (int q = 0; q < WQ; ++q) {
-                if ((uint32_t)q < m) {
-                    const uint32_t k = (uint32_t)b[q];
-                    ws[q] = (k == kEmptyKey) ? wmask + 1 : slot_of(k, w.seed, wmask);
-                    wv[q] = __ldg(w.W + ws[q]);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < WQ; ++q) {
-                x[q] = ((uint32_t)q < m) ? w_get(w, wmask, wide, (uint32_t)b[q], ws[q], wv[q]) : 0ull;
-                acc += x[q];
-            }
-        }
+        for (int q = 0; q < WQ; ++q) acc += x[q];
         if (MODE == 1) {
 #pragma unroll
             for (int q = 0; q < WQ; ++q)
@@ -406,13 +515,118 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
     w_probe_pass<MODE, true>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
 }
 
+// T pass: the degrees of the last relation's key column.
+//
+// Direct-address layout: a warp round is two blocks of 128 consecutive keys,
+// four per lane, both loaded, with the next round's loads issued, before they
+// are used.  deg[k] += i at the end of every run of equal keys k
+// and -= i at its start, i counted inside the block (32-bit adds whose results
+// are not needed, exact modulo 2^32): a lane needs only the key before its
+// own, no search for where a run ends, and a run inside one lane is one add.
+// Sorted keys cost two adds a run, random ones five adds for four keys.
+// Hashed slots: a key per lane, as in the general S pass.
+constexpr int DT = 512;
+__global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__ keys, uint32_t n, DegTable t,
+                                                     DevStatus *st) {
+    const uint32_t mask = t.meta[kMetaMask];
+    const bool dense = t.meta[kMetaDense] != 0u;
+    const uint32_t kmin = dense ? t.meta[kMetaMin] : 0u, span = dense ? t.meta[kMetaSpan] : 0u;
+    uint32_t *deg = (uint32_t *)t.slots;
+    const bool vec = ((uintptr_t)keys & 15) == 0;
+    const uint64_t pol = l2_evict_first();
+    constexpr int G = 2;   // blocks per warp round
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t warp = (blockIdx.x * DT + threadIdx.x) >> 5, warps = (gridDim.x * DT) >> 5;
+    const uint32_t blocks = (n + WCHUNK - 1) / WCHUNK;
+    auto load = [&](uint32_t blk, int32_t (&v)[WQ]) -> uint32_t {
+        const uint32_t i = blk * WCHUNK + lane * WQ;
+        if (blk >= blocks || i >= n) return 0u;
+        if (vec && i + WQ <= n) {
+            const int4 a = ld_stream((const int4 *)(keys + i), pol);
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+            return WQ;
+        }
+        const uint32_t m = min((uint32_t)WQ, n - i);
+#pragma unroll
+        for (int q = 0; q < WQ; ++q)
+            if ((uint32_t)q < m) v[q] = __ldg(keys + i + q);
+        return m;
+    };
+    if (!dense) {
+        const uint32_t T = gridDim.x * DT;
+        uint64_t i = (uint64_t)blockIdx.x * DT + threadIdx.x;
+        int32_t k = i < n ? __ldg(keys + i) : 0;
+        for (; i - lane < n; i += T) {
+            const int32_t nk = i + T < n ? __ldg(keys + i + T) : 0;
+            const uint32_t s = deg_home((uint32_t)k, t.seed, mask);
+            const ulonglong2 u = __ldcg((const ulonglong2 *)(t.slots + s));
+            const uint32_t len = (uint32_t)warp_run_sum1(k, 1ull, i < n);
+            if (len) deg_add(t.slots, mask, (uint32_t)k, s, u, len, st);
+            k = nk;
+        }
+        return;
+    }
+    auto add = [&](int32_t key, uint32_t x) {
+        const uint32_t k = (uint32_t)key - kmin;
+        if (k < span)
+            atomicAdd(deg + k, x);
+        else
+            set_status(st, MWJ_ERR_CHECK, 8);   // a key outside the range the sizing pass saw
+    };
+    auto block_dense = [&](const int32_t (&v)[WQ], uint32_t m, uint32_t valid) {
+        const int32_t prev = __shfl_up_sync(0xffffffffu, v[WQ - 1], 1);
+        if (m == 0) return;
+        int32_t cur = lane ? prev : v[0];
+        uint32_t starts = 0;   // bit q: a run starts at the lane's key q
+#pragma unroll
+        for (int q = 0; q < WQ; ++q)
+            starts |= (uint32_t)((uint32_t)q < m && v[q] != (q ? v[q - 1] : cur)) << q;
+        uint32_t x = 0;   // minus the position where cur's run starts, when it starts in this lane
+        while (starts) {
+            const uint32_t q = (uint32_t)__ffs((int)starts) - 1u;
+            starts &= starts - 1u;
+            const uint32_t i = lane * WQ + q;
+            add(cur, x + i);
+            cur = q < 2u ? (q ? v[1] : v[0]) : (q == 2u ? v[2] : v[3]);
+            x = 0u - i;
+        }
+        if (lane * WQ + m == valid) x += valid;   // the block ends here
+        if (x) add(cur, x);
+    };
+    const uint32_t rounds = (blocks + G - 1) / G;
+    int32_t v[G][WQ];
+    uint32_t m[G];
+    uint32_t r = warp;
+#pragma unroll
+    for (int g = 0; g < G; ++g) m[g] = load(r * G + g, v[g]);
+    while (r < rounds) {
+        const uint32_t nr = r + warps;
+        int32_t nv[G][WQ];
+        uint32_t nm[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) nm[g] = load(nr * G + g, nv[g]);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const uint32_t b0 = (r * G + g) * WCHUNK;
+            block_dense(v[g], m[g], b0 < n ? min(WCHUNK, n - b0) : 0u);
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            m[g] = nm[g];
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) v[g][q] = nv[g][q];
+        }
+        r = nr;
+    }
+}
+
 // CTAs of a grid-stride pass: every SM filled, no more warps than rounds.
 template <typename K>
-uint32_t pass_grid(K kernel, uint32_t n, int num_sms) {
+uint32_t pass_grid(K kernel, uint32_t n, int num_sms, uint32_t per_warp = WCHUNK) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, WT, 0) != cudaSuccess || per_sm < 1)
         per_sm = 1;
-    const uint64_t want = ((uint64_t)n + WCHUNK * (WT / 32) - 1) / (WCHUNK * (WT / 32));
+    const uint64_t want = ((uint64_t)n + per_warp * (WT / 32) - 1) / (per_warp * (WT / 32));
     const uint64_t full = (uint64_t)num_sms * (uint64_t)per_sm;
     return (uint32_t)(want < full ? (want ? want : 1) : full);
 }
@@ -421,64 +635,109 @@ uint32_t pass_grid(K kernel, uint32_t n, int num_sms) {
 
 size_t w_table_slots(int64_t nS) { return single_table_slots(nS); }
 
-cudaError_t w_table_size(const int32_t *Sb, int64_t nS, const WTable &w, unsigned int *hll,
-                         uint64_t reserve_slots, int num_sms, cudaStream_t st, uint32_t *tmeta,
-                         uint64_t treserve) {
-    return single_table_size(Sb, nS, w.seed, hll, w.meta, reserve_slots, num_sms, st, "w_hll", "w_size", true,
-                             tmeta, treserve);
-}
+namespace {
 
-cudaError_t w_table_clear(const WTable &w, int num_sms, cudaStream_t st) {
-    ProfScope ps_("w_clear", st);
-    k_w_clear<<<num_sms * 4, 512, 0, st>>>(w.W, w.hi, w.meta);
+cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, int num_sms, cudaStream_t st) {
+    if (T.n <= 0) return cudaSuccess;
+    const uint32_t n = (uint32_t)T.n;
+    const uint32_t groups = (n + WQ * DT - 1) / (WQ * DT), full = (uint32_t)num_sms * 3;
+    ProfScope ps_("t_insert", st);
+    k_deg_build<<<groups < full ? groups : full, DT, 0, st>>>(T.x, n, t, status);
     return cudaGetLastError();
 }
 
-cudaError_t w_table_prepare(const int32_t *Sb, int64_t nS, const WTable &w, unsigned int *hll,
-                            uint64_t reserve_slots, int num_sms, cudaStream_t st) {
-    cudaError_t e = w_table_size(Sb, nS, w, hll, reserve_slots, num_sms, st);
-    if (e != cudaSuccess) return e;
-    return w_table_clear(w, num_sms, st);
-}
-
-cudaError_t w_table_build(const int32_t *Sb, const int32_t *Sc, int64_t nS, const TImg &t,
-                          const WTable &w, DevStatus *status, int num_sms, cudaStream_t st) {
-    if (nS <= 0) return cudaSuccess;
-    const uint32_t n = (uint32_t)nS;
+cudaError_t w_table_build(const mwj_rel &S, const Source &src, bool weights, const WTable &w, DevStatus *status,
+                          int num_sms, cudaStream_t st) {
+    if (S.n <= 0) return cudaSuccess;
+    const uint32_t n = (uint32_t)S.n;
+    auto direct = weights ? k_w_build_direct<true> : k_w_build_direct<false>;
+    auto hashed = weights ? k_w_build<true> : k_w_build<false>;
     {
         ProfScope ps_("w_build", st);
-        k_w_build_direct<<<pass_grid(k_w_build_direct, n, num_sms), WT, 0, st>>>(Sb, Sc, n, t, w, status);
+        direct<<<pass_grid(direct, n, num_sms), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     }
     ProfScope ps_("w_build_hashed", st);
-    k_w_build<<<pass_grid(k_w_build, n, num_sms), WT, 0, st>>>(Sb, Sc, n, t, w, status);
+    hashed<<<pass_grid(hashed, n, num_sms, 32), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     return cudaGetLastError();
 }
 
-cudaError_t w_table_probe(const int32_t *Ra, const int32_t *Rb, int64_t nR, const WTable &w, int mode,
-                          int32_t a_domain, unsigned long long *cnt, unsigned long long *total,
-                          DevStatus *status, int num_sms, cudaStream_t st) {
-    if (nR <= 0) return cudaSuccess;
-    const uint32_t n = (uint32_t)nR;
-    if (mode == 1) {
-        {
-            ProfScope ps_("w_probe_groupby", st);
-            k_w_probe_direct<1><<<pass_grid(k_w_probe_direct<1>, n, num_sms), WT, 0, st>>>(
-                Ra, Rb, n, w, a_domain, cnt, total, status);
-        }
-        ProfScope ps_("w_probe_groupby_hashed", st);
-        k_w_probe<1><<<pass_grid(k_w_probe<1>, n, num_sms), WT, 0, st>>>(Ra, Rb, n, w, a_domain, cnt, total,
-                                                                         status);
-    } else {
-        {
-            ProfScope ps_("w_probe_count", st);
-            k_w_probe_direct<0><<<pass_grid(k_w_probe_direct<0>, n, num_sms), WT, 0, st>>>(
-                Ra, Rb, n, w, a_domain, cnt, total, status);
-        }
-        ProfScope ps_("w_probe_count_hashed", st);
-        k_w_probe<0><<<pass_grid(k_w_probe<0>, n, num_sms), WT, 0, st>>>(Ra, Rb, n, w, a_domain, cnt, total,
-                                                                         status);
+cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a_domain, unsigned long long *cnt,
+                          unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st) {
+    if (R.n <= 0) return cudaSuccess;
+    const uint32_t n = (uint32_t)R.n;
+    auto direct = mode == 1 ? k_w_probe_direct<1> : k_w_probe_direct<0>;
+    auto hashed = mode == 1 ? k_w_probe<1> : k_w_probe<0>;
+    {
+        ProfScope ps_(mode == 1 ? "w_probe_groupby" : "w_probe_count", st);
+        direct<<<pass_grid(direct, n, num_sms), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
     }
+    ProfScope ps_(mode == 1 ? "w_probe_groupby_hashed" : "w_probe_count_hashed", st);
+    hashed<<<pass_grid(hashed, n, num_sms), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+void one_bucket_layout(Arena &A, const mwj_rel *rel, int nrel, int num_sms, OneBucket &L) {
+    L = OneBucket{};
+    L.deg.slots = A.take<unsigned long long>(single_table_slots(rel[nrel - 1].n) + 2);
+    L.deg.meta = A.take<uint32_t>(kMetaWords);
+    for (int k = 0; k < nrel - 2; ++k) {
+        const size_t ws = w_table_slots(rel[nrel - 2 - k].n) + 2;
+        L.w[k].W = A.take<unsigned long long>(ws);
+        L.w[k].keys = A.take<uint32_t>(ws);
+        L.w[k].meta = A.take<uint32_t>(kMetaWords);
+        L.w[k].heavy = A.take<uint32_t>(kHeavyTableWords);
+    }
+    for (int k = 0; k < nrel - 1; ++k) L.hll[k] = A.take<unsigned int>(hll_scratch_registers(num_sms));
+}
+
+cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const Seeds &sd, int mode, int32_t a_domain,
+                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, int num_sms,
+                           cudaStream_t st) {
+    cudaError_t e;
+    const mwj_rel &last = rel[nrel - 1];
+    const uint32_t seeds[kChainMax - 2] = {nrel == 3 ? sd.slot : sd.slot ^ sd.D, sd.slot};
+    // the key columns (of every relation but R); a column that plays two
+    // parts (a self-join) is read once
+    SizeCol cols[kSizeCols];
+    uint32_t ncols = 0;
+    auto add = [&](const mwj_rel &r, uint32_t seed, uint32_t *meta, uint64_t reserve) {
+        for (uint32_t q = 0; q < ncols; ++q) {
+            if (cols[q].keys == r.x && cols[q].n == (uint32_t)r.n) {
+                cols[q].meta[cols[q].ntargets] = meta;
+                cols[q].reserve[cols[q].ntargets++] = reserve;
+                return;
+            }
+        }
+        cols[ncols] = SizeCol{r.x, (uint32_t)r.n, seed, L.hll[ncols], {meta}, {reserve}, 1u};
+        ++ncols;
+    };
+    HeavyCol heavy[kSizeCols];
+    ClearTable clear[kSizeCols];
+    L.deg.seed = sd.slot2;
+    add(last, L.deg.seed, L.deg.meta, single_table_slots(last.n));
+    clear[0] = ClearTable{L.deg.slots, nullptr, L.deg.meta};
+    for (int k = 0; k < nrel - 2; ++k) {
+        const mwj_rel &r = rel[nrel - 2 - k];
+        WTable &w = L.w[k];
+        w.seed = seeds[k];
+        add(r, w.seed, w.meta, w_table_slots(r.n));
+        heavy[k] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)w.heavy};
+        clear[k + 1] = ClearTable{w.W, w.keys, w.meta};
+    }
+    if ((e = size_columns(cols, ncols, heavy, (uint32_t)nrel - 2u, true, num_sms, st)) != cudaSuccess) return e;
+    if ((e = tables_clear(clear, (uint32_t)nrel - 1u, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull,
+                          total, num_sms, st)) != cudaSuccess)
+        return e;
+    if ((e = deg_build(last, L.deg, status, num_sms, st)) != cudaSuccess) return e;
+    Source src{};
+    src.t = L.deg;
+    for (int k = 0; k < nrel - 2; ++k) {
+        if ((e = w_table_build(rel[nrel - 2 - k], src, k > 0, L.w[k], status, num_sms, st)) != cudaSuccess) return e;
+        src.w = L.w[k];
+    }
+    return w_table_probe(rel[0], L.w[nrel - 3], mode, a_domain, cnt, total, status, num_sms, st);
 }
 
 }  // namespace mwj

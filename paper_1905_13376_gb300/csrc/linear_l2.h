@@ -1,56 +1,56 @@
-// linear_l2.h -- the linear 3-way join with one bucket on each side: S's
-// weight table w(b) = sum over (b, c) in S of deg_T(c), held in the L2.
+// linear_l2.h -- linear joins with one bucket on each side: the weight tables,
+// e.g. S's w(b) = sum over (b, c) in S of deg_T(c), held in the L2.
 #pragma once
 
+#include "internal.h"
 #include "tables.h"
 
 namespace mwj {
 
-// Open-addressing table of 2^k slots (k from a HyperLogLog estimate of S's
-// distinct B values), linear probing from slot_of(b, seed, mask).
-//   W[s]        (w(b) mod 2^32) << 32 | b, or kEmpty64 when free; key -1,
-//               which would make a full slot look free, lives in W[mask + 1]
-//               as a plain 64-bit sum
-//   hi[s]       w(b) >> 32 (touched only when some w(b) reaches 2^32)
-//   meta[0]     mask; meta[1] the distinct-key estimate; meta[2] set to 1
-//               when some hi[] entry is non-zero; meta[3..5] the
-//               direct-address layout (tables.h): when the sizing pass chose
-//               it, w(b) is the plain 64-bit word W[b - min] and hi[] is unused
-struct WTable {
-    unsigned long long *W;   // w_table_slots(nS) + 2 entries reserved
-    uint32_t *hi;            // w_table_slots(nS) + 2 entries reserved
-    uint32_t *meta;          // kMetaWords entries
+// Degrees of the chain's last relation, c -> deg(c).  meta (tables.h) says
+// which layout the sizing pass chose: the direct-address one (uint32 deg[c - min]),
+// or 2^k packed (deg << 32 | c) slots in pairs of 16 bytes: a key lives in the
+// first free slot at or after its home pair, so one 16-byte load nearly
+// always settles a lookup.  Key -1 is a key like any other (a count below
+// 2^31 keeps its slot different from kEmpty64).
+struct DegTable {
+    unsigned long long *slots;   // single_table_slots(n)
+    uint32_t *meta;              // kMetaWords entries
     uint32_t seed;
-    const uint32_t *heavy;   // heavy B keys of S (heavy_detect's table), or null
 };
 
-// Heavy keys of the S pass: a sampled share of at least 1 / (2 x this) of S
-// (heavy_detect's bucket-count argument).
+// Weights b -> w(b), exact modulo 2^64: the direct-address sums W[b - min], or
+// 2^k slots, keys and sums apart: keys[s] in groups of four (one 16-byte load),
+// W[s] the sum, added to with 64-bit adds whose results are not needed.  Key -1,
+// the mark of a free slot, has its sum in W[mask + 1].
+struct WTable {
+    unsigned long long *W;   // w_table_slots(n) + 2 entries reserved
+    uint32_t *keys;          // w_table_slots(n) entries reserved
+    uint32_t *meta;          // kMetaWords entries
+    uint32_t seed;
+    const uint32_t *heavy;   // heavy keys of the relation's key column (skew.h's table)
+};
+
+// Heavy keys of a weight pass: a sampled share of at least 1 / (2 x this).
 constexpr uint32_t kWHeavyBuckets = 128;
 
 // Slots to reserve for S of nS tuples (the table never grows past this).
 size_t w_table_slots(int64_t nS);
 
-// Size the table from S's B column (hll: hll_scratch_registers(num_sms) u32)
-// and clear it; or the two steps apart.
-cudaError_t w_table_prepare(const int32_t *Sb, int64_t nS, const WTable &w, unsigned int *hll,
-                            uint64_t reserve_slots, int num_sms, cudaStream_t st);
-// tmeta (optional): T's single table when its C column is S's B column,
-// sized from the same pass (at most treserve slots).
-cudaError_t w_table_size(const int32_t *Sb, int64_t nS, const WTable &w, unsigned int *hll,
-                         uint64_t reserve_slots, int num_sms, cudaStream_t st, uint32_t *tmeta = nullptr,
-                         uint64_t treserve = 0);
-cudaError_t w_table_clear(const WTable &w, int num_sms, cudaStream_t st);
-
-// S pass: w(b) += deg_T(c) for every (b, c) of S, T's single table t
-// (t.J == 0) already built.
-cudaError_t w_table_build(const int32_t *Sb, const int32_t *Sc, int64_t nS, const TImg &t,
-                          const WTable &w, DevStatus *status, int num_sms, cudaStream_t st);
-
-// R pass: total += w(b) for every (a, b) of R and, with mode 1 (GROUP BY A),
-// cnt[a] += w(b); a outside [0, a_domain) raises MWJ_ERR_DOMAIN.
-cudaError_t w_table_probe(const int32_t *Ra, const int32_t *Rb, int64_t nR, const WTable &w, int mode,
-                          int32_t a_domain, unsigned long long *cnt, unsigned long long *total,
-                          DevStatus *status, int num_sms, cudaStream_t st);
+// The one-bucket plan of a chain R(A,B) S(B,C) T(C,D) [U(D,E)]: the last
+// relation's degree table and one weight table per relation between it and R.
+constexpr int kChainMax = 4;
+struct OneBucket {
+    DegTable deg;                   // of the last relation
+    unsigned int *hll[kSizeCols];   // sizing scratch, one per key column
+    WTable w[kChainMax - 2];        // w[k]: weights of relation nrel - 2 - k (w[0] is looked up by w[1]'s pass)
+};
+// rel[0] = R ... rel[nrel - 1]: the last (nrel 3 or 4).
+void one_bucket_layout(Arena &A, const mwj_rel *rel, int nrel, int num_sms, OneBucket &L);
+// COUNT (mode 0: *total) or GROUP BY A (mode 1: cnt[0, a_domain) too); the
+// outputs are zeroed here.  a outside [0, a_domain) raises MWJ_ERR_DOMAIN.
+cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const Seeds &sd, int mode, int32_t a_domain,
+                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, int num_sms,
+                           cudaStream_t st);
 
 }  // namespace mwj

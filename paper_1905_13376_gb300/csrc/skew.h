@@ -40,6 +40,69 @@ __device__ __forceinline__ const uint32_t *heavy_to_smem(const uint32_t *heavy, 
     return buf;
 }
 
+// The heavy keys of one column from a strided sample of it, by one CTA of NT
+// threads (sm: its shared memory): those whose sampled share reaches
+// 1 / (2 buckets), and at least kHeavyMinCount sampled tuples.
+constexpr uint32_t kHeavySampled = 2048;     // sampled tuples
+constexpr uint32_t kHeavyCountSlots = 4096;  // count table, at most half full
+constexpr uint32_t kHeavyMinCount = 8;       // a heavy key is seen at least this often
+struct HeavySample {
+    uint32_t key[kHeavyCountSlots], cnt[kHeavyCountSlots], ht[kHeavySlots], nh;
+};
+
+template <int NT>
+__device__ __forceinline__ void heavy_sample_cta(const int32_t *__restrict__ col, uint32_t n, uint32_t buckets,
+                                                 uint32_t *__restrict__ heavy, HeavySample &sm) {
+    const uint32_t m = n < kHeavySampled ? n : kHeavySampled;
+    constexpr uint32_t PER = kHeavySampled / NT;
+    static_assert(PER * NT == kHeavySampled, "a whole number of samples per thread");
+    uint32_t ks[PER];
+#pragma unroll
+    for (uint32_t q = 0; q < PER; ++q) {
+        const uint32_t j = threadIdx.x + q * NT;
+        ks[q] = j < m ? (uint32_t)__ldg(col + (uint32_t)(((uint64_t)j * n) / m)) : kEmptyKey;
+    }
+    for (uint32_t i = threadIdx.x; i < kHeavyCountSlots; i += NT) {
+        sm.key[i] = kEmptyKey;
+        sm.cnt[i] = 0;
+    }
+    for (uint32_t i = threadIdx.x; i < kHeavySlots; i += NT) sm.ht[i] = kEmptyKey;
+    if (threadIdx.x == 0) sm.nh = 0;
+    __syncthreads();
+#pragma unroll
+    for (uint32_t q = 0; q < PER; ++q) {
+        const uint32_t k = ks[q];
+        if (k == kEmptyKey) continue;   // the table's empty marker is never heavy
+        uint32_t s = slot_of(k, kHeavySeed, kHeavyCountSlots - 1);
+        for (uint32_t it = 0; it < kHeavyCountSlots; ++it) {   // at most half full: ends early
+            uint32_t held = sm.key[s];
+            if (held == kEmptyKey) {
+                held = atomicCAS(&sm.key[s], kEmptyKey, k);
+                if (held == kEmptyKey) held = k;
+            }
+            if (held == k) {
+                atomicAdd(&sm.cnt[s], 1u);
+                break;
+            }
+            s = (s + 1) & (kHeavyCountSlots - 1);
+        }
+    }
+    __syncthreads();
+    const uint32_t t = max(kHeavyMinCount, m / (2u * buckets));
+    for (uint32_t i = threadIdx.x; i < kHeavyCountSlots; i += NT) {
+        const uint32_t k = sm.key[i];
+        if (k == kEmptyKey || sm.cnt[i] < t) continue;
+        if (atomicAdd(&sm.nh, 1u) >= kHeavyMax) continue;
+        // at most kHeavyMax = kHeavySlots / 2 keys: a free slot is always found
+        uint32_t s = slot_of(k, kHeavySeed, kHeavySlots - 1);
+        for (uint32_t it = 0; it < kHeavySlots && atomicCAS(&sm.ht[s], kEmptyKey, k) != kEmptyKey; ++it)
+            s = (s + 1) & (kHeavySlots - 1);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < kHeavySlots; i += NT) heavy[i] = sm.ht[i];
+    if (threadIdx.x == 0) heavy[kHeavySlots] = sm.nh < kHeavyMax ? sm.nh : kHeavyMax;
+}
+
 // Heavy keys of the join column B from samples of R's and S's B columns: a
 // key is heavy when its sampled share in either relation reaches half of an
 // average H(B) bucket (1 / (2 I)).  Also zeroes hw (kHeavySlots u64).

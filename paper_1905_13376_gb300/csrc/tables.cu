@@ -22,6 +22,7 @@
 #include <climits>
 
 #include "internal.h"
+#include "skew.h"
 #include "tables.h"
 #include "warp_runs.cuh"
 
@@ -34,6 +35,12 @@ constexpr uint32_t kAggSlots = 8192;          // shared-memory aggregation table
 // two at or above 4 x the estimate keeps the load between 1/8 and 1/4 (a
 // factor of 2 measured slower: longer probe runs in both insert and lookup).
 constexpr double kSingleTableFactor = 4.0;
+// Above 2^21 slots (16 MB) a factor of 2: two tables of 2 million distinct keys
+// at 4 x (64 MB each) spill out of the 129 MB L2 they share with the streams,
+// and every probe then moves DRAM sectors (8.4 million id-keyed tuples, one pass: 0.28
+// against 0.24 ms).
+constexpr double kSmallTableSlots = (double)(1u << 21);
+constexpr double kLargeTableFactor = 2.0;
 constexpr uint32_t kImgSmemSlots = 8192;      // 64 KB of packed slots (bucket images)
 
 // insert into a global region of arbitrary capacity (fastrange start), adding `add`
@@ -59,14 +66,13 @@ __device__ __forceinline__ uint32_t gagg_insert(unsigned long long *tbl, uint32_
     return 0;
 }
 
-// insert into the power-of-two single table
-__device__ __forceinline__ void single_insert(unsigned long long *tbl, uint32_t mask, uint32_t k,
-                                              uint32_t seed, unsigned long long add,
-                                              DevStatus *st) {
-    uint32_t s = slot_of(k, seed, mask);
+// insert into the power-of-two single table, from the first probe (slot s,
+// value v, possibly read before another thread claimed the slot)
+__device__ __forceinline__ void single_insert_from(unsigned long long *tbl, uint32_t mask, uint32_t k, uint32_t s,
+                                                   unsigned long long v, unsigned long long add,
+                                                   DevStatus *st) {
     const unsigned long long fresh = (add << 32) | (unsigned long long)k;
     for (uint32_t it = 0; it <= mask; ++it) {
-        unsigned long long v = tbl[s];
         if (v == kEmpty64) {
             unsigned long long old = atomicCAS(&tbl[s], kEmpty64, fresh);
             if (old == kEmpty64) return;
@@ -77,8 +83,15 @@ __device__ __forceinline__ void single_insert(unsigned long long *tbl, uint32_t 
             return;
         }
         s = (s + 1) & mask;
+        v = __ldcg(tbl + s);
     }
     set_status(st, MWJ_ERR_CHECK, 3);
+}
+
+__device__ __forceinline__ void single_insert(unsigned long long *tbl, uint32_t mask, uint32_t k,
+                                              uint32_t seed, unsigned long long add, DevStatus *st) {
+    const uint32_t s = slot_of(k, seed, mask);
+    single_insert_from(tbl, mask, k, s, __ldcg(tbl + s), add, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -166,14 +179,11 @@ __global__ void k_tsize(const uint32_t *__restrict__ ecount, uint32_t J, uint32_
     }
 }
 
-// Empty hashed slots, or zero degrees of the direct-address layout.
 __global__ void k_tclear(unsigned long long *__restrict__ tbl, const uint32_t *__restrict__ meta) {
-    const bool dense = meta[kMetaDense] != 0u;
-    const uint64_t words = dense ? ((uint64_t)meta[kMetaSpan] + 1) / 2 : (uint64_t)meta[0] + 1;
-    const unsigned long long fill = dense ? 0ull : kEmpty64;
+    const uint64_t words = (uint64_t)meta[0] + 1;
     for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < words;
          s += (uint64_t)gridDim.x * blockDim.x)
-        tbl[s] = fill;
+        tbl[s] = kEmpty64;
 }
 
 __global__ void __launch_bounds__(BT) k_tinsert(const uint32_t *__restrict__ ekey,
@@ -384,26 +394,168 @@ namespace {
 
 constexpr int HLL_BITS = 12;
 constexpr uint32_t HLL_M = 1u << HLL_BITS;
-constexpr int HLL_CTAS_PER_SM = 2;   // resident CTAs of the sizing pass (its registers allow two)
+constexpr int HLL_CTAS_PER_SM = 2;   // resident CTAs of the sizing passes (their registers allow two)
+constexpr int RANGE_CTAS_PER_SM = 4;
+constexpr uint32_t HLL_MB = 32;                  // registers merged per CTA
+constexpr uint32_t HLL_MCTAS = HLL_M / HLL_MB;   // merge CTAs
+// after the per-CTA registers: per merge CTA its part of the estimator's sum
+// (double) and of the empty-register count, then the finish counter
+constexpr size_t HLL_TAIL = 2 * HLL_MCTAS + HLL_MCTAS + 8;
+
+// a column's scratch: `rows` x HLL_M registers, the merge's tail, `range_rows` (min, max) pairs
+__device__ __forceinline__ unsigned int *size_tail(unsigned int *scratch, uint32_t rows) {
+    return scratch + (size_t)rows * HLL_M;
+}
+__device__ __forceinline__ int32_t *size_ranges(unsigned int *scratch, uint32_t rows) {
+    return (int32_t *)(size_tail(scratch, rows) + HLL_TAIL);
+}
+
+struct SizeArgs {
+    SizeCol c[kSizeCols];
+    HeavyCol h[kSizeCols];
+    uint32_t nheavy, rows, range_rows;
+    bool ranged;   // k_range has run: a compact column gets the direct-address layout
+};
+
+__device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t reserve) {
+    return lo <= hi && (uint64_t)((int64_t)hi - (int64_t)lo + 1) <= reserve;
+}
+
+// Key range of every column: `rows` CTAs per column, each leaving the
+// smallest and largest key it saw (INT32_MAX, INT32_MIN when it saw none).
+// A pure stream, four 16-byte loads per thread in flight: 131 MB in 0.027 ms,
+// where the HyperLogLog pass over the same column takes 0.037 ms (it hashes
+// every key) and its merge 0.014 ms more; a column whose range is compact
+// needs neither.  The first CTAs sample the heavy keys (skew.h) meanwhile.
+__global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
+    __shared__ HeavySample hsm;
+    if (blockIdx.x < g.nheavy) {
+        const HeavyCol &h = g.h[blockIdx.x];
+        heavy_sample_cta<BT>(h.keys, h.n, h.buckets, h.heavy, hsm);
+        return;
+    }
+    const uint32_t cta = (blockIdx.x - g.nheavy) % g.range_rows;
+    const SizeCol &c = g.c[(blockIdx.x - g.nheavy) / g.range_rows];
+    const int32_t *keys = c.keys;
+    const uint32_t n = c.n;
+    int32_t lo = INT32_MAX, hi = INT32_MIN;
+    auto see = [&](int32_t k) {
+        lo = min(lo, k);
+        hi = max(hi, k);
+    };
+    const uint32_t T = g.range_rows * BT, t = cta * BT + threadIdx.x;
+    // the elements before the first 16-byte boundary and after the last one
+    const uint32_t head = min(n, (uint32_t)(((16u - ((uintptr_t)keys & 15u)) & 15u) / 4u));
+    const uint32_t quads = (n - head) / 4u;
+    if (t < head) see(__ldg(keys + t));
+    if (t < n - head - 4u * quads) see(__ldg(keys + head + 4u * quads + t));
+    const int4 *v = (const int4 *)(keys + head);
+    const uint64_t pol = l2_evict_first();
+    // a thread whose keys already span more than every reservation stops: its
+    // part of the range settles the layout
+    uint64_t most = 0;
+    for (uint32_t q = 0; q < c.ntargets; ++q) most = c.reserve[q] > most ? c.reserve[q] : most;
+    const uint32_t wide = most > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)most;
+    uint32_t i = t;
+    for (; i < quads && quads - i > 3u * T; i += 4u * T) {
+        if (lo < hi && (uint32_t)hi - (uint32_t)lo >= wide) break;
+        int4 q[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) q[u] = ld_stream(v + i + u * T, pol);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            lo = min(lo, min(min(q[u].x, q[u].y), min(q[u].z, q[u].w)));
+            hi = max(hi, max(max(q[u].x, q[u].y), max(q[u].z, q[u].w)));
+        }
+    }
+    for (; i < quads; i += T) {
+        if (lo < hi && (uint32_t)hi - (uint32_t)lo >= wide) break;
+        const int4 q = ld_stream(v + i, pol);
+        see(q.x);
+        see(q.y);
+        see(q.z);
+        see(q.w);
+        if (quads - i <= T) break;   // (i + T may pass 2^32)
+    }
+    __shared__ int32_t slo[BT / 32], shi[BT / 32];
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        slo[threadIdx.x >> 5] = lo;
+        shi[threadIdx.x >> 5] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < BT / 32; ++w) {
+            lo = min(lo, slo[w]);
+            hi = max(hi, shi[w]);
+        }
+        int32_t *mm = size_ranges(c.scratch, g.rows);
+        mm[2 * cta] = lo;
+        mm[2 * cta + 1] = hi;
+    }
+}
 
 // HyperLogLog registers (Flajolet, Fusy, Gandouet, Meunier 2007): register
 // h >> (32 - HLL_BITS) keeps the largest rank (position of the first 1 bit)
 // of the remaining bits.  mix32 is a bijection of 32-bit keys, so distinct
 // keys have distinct hashes.
-// With mm != null the CTA also leaves the smallest and largest key it saw in
-// mm[2 b], mm[2 b + 1] (b = blockIdx.x; INT32_MAX, INT32_MIN when it saw none).
-__global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(const int32_t *__restrict__ keys, uint32_t n,
-                                            uint32_t seed, unsigned int *__restrict__ regs,
-                                            unsigned int *__restrict__ done, int32_t *__restrict__ mm) {
+//
+// Blocks (x, y): column y.  With `ranged` every CTA first merges the column's
+// key ranges: a table whose reserved slots hold the whole range gets the
+// direct-address layout (slot = key - min, no key stored), which is decided
+// from the range alone: the array is no larger than the hashed table's
+// reservation, clearing it costs at most 16 bytes per tuple, and only the
+// entries of keys that occur are touched again.  A column none of whose
+// tables is hashed ends there.
+__global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(SizeArgs g) {
     __shared__ unsigned int r[HLL_M];
-    __shared__ int32_t smin, smax;
-    if (done && blockIdx.x == 0 && threadIdx.x == 0) *done = 0;   // for k_hll_merge_size
-    for (uint32_t j = threadIdx.x; j < HLL_M; j += BT) r[j] = 0;
-    if (threadIdx.x == 0) {
-        smin = INT32_MAX;
-        smax = INT32_MIN;
+    const SizeCol &c = g.c[blockIdx.y];
+    const int32_t *keys = c.keys;
+    const uint32_t n = c.n, seed = c.seed;
+    unsigned int *regs = c.scratch;
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (first) size_tail(c.scratch, g.rows)[3 * HLL_MCTAS] = 0;   // k_hll_merge_size's finish counter
+    if (g.ranged) {
+        __shared__ int32_t slo, shi;
+        if (threadIdx.x == 0) {
+            slo = INT32_MAX;
+            shi = INT32_MIN;
+        }
+        __syncthreads();
+        int32_t lo = INT32_MAX, hi = INT32_MIN;
+        const int32_t *mm = size_ranges(c.scratch, g.rows);
+        for (uint32_t b = threadIdx.x; b < g.range_rows; b += BT) {
+            lo = min(lo, __ldcg(mm + 2 * b));
+            hi = max(hi, __ldcg(mm + 2 * b + 1));
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&slo, lo);
+            atomicMax(&shi, hi);
+        }
+        __syncthreads();
+        lo = slo;
+        hi = shi;
+        bool all = true;
+        for (uint32_t q = 0; q < c.ntargets; ++q) {
+            const bool dense = span_fits(lo, hi, c.reserve[q]);
+            all = all && dense;
+            if (first) {
+                c.meta[q][kMetaDense] = dense ? 1u : 0u;
+                if (dense) {
+                    c.meta[q][kMetaMask] = 15u;
+                    c.meta[q][kMetaMin] = (uint32_t)lo;
+                    c.meta[q][kMetaSpan] = (uint32_t)((int64_t)hi - (int64_t)lo + 1);
+                }
+            }
+        }
+        if (all) return;
+    } else if (first) {
+        for (uint32_t q = 0; q < c.ntargets; ++q) c.meta[q][kMetaDense] = 0u;
     }
-    int32_t kmin = INT32_MAX, kmax = INT32_MIN;
+    for (uint32_t j = threadIdx.x; j < HLL_M; j += BT) r[j] = 0;
     __syncthreads();
     const bool vec = ((uintptr_t)keys & 15) == 0;
     const uint64_t pol = l2_evict_first();
@@ -431,17 +583,15 @@ __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(const int32_t *__re
         return cnt;
     };
     int32_t v[16];
-    uint32_t c = blockIdx.x * BT + threadIdx.x;
-    uint32_t cnt = load(c, v);
-    for (; c < nst; c += T) {
+    uint32_t st = blockIdx.x * BT + threadIdx.x;
+    uint32_t cnt = load(st, v);
+    for (; st < nst; st += T) {
         int32_t nv[16];
-        const uint32_t ncnt = load(c + T, nv);
+        const uint32_t ncnt = load(st + T, nv);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
             if ((uint32_t)k >= cnt) break;
             if (k > 0 && v[k] == v[k - 1]) continue;   // nothing a repeat could change
-            kmin = min(kmin, v[k]);
-            kmax = max(kmax, v[k]);
             const uint32_t h = mix32((uint32_t)v[k] ^ seed);
             const uint32_t w = h << HLL_BITS;
             const uint32_t rank = (w == 0) ? (33u - HLL_BITS) : (uint32_t)__clz(w) + 1u;
@@ -452,23 +602,9 @@ __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(const int32_t *__re
         for (int k = 0; k < 16; ++k) v[k] = nv[k];
         cnt = ncnt;
     }
-    if (mm) {
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-            kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(&smin, kmin);
-            atomicMax(&smax, kmax);
-        }
-    }
     __syncthreads();
     // this CTA's registers; the size kernel takes the maximum over CTAs
     for (uint32_t j = threadIdx.x; j < HLL_M; j += BT) regs[(size_t)blockIdx.x * HLL_M + j] = r[j];
-    if (mm && threadIdx.x == 0) {
-        mm[2 * blockIdx.x] = smin;
-        mm[2 * blockIdx.x + 1] = smax;
-    }
 }
 
 // regs[0..HLL_M) = max over the rows of regs[ctas][HLL_M]
@@ -480,31 +616,24 @@ __global__ void k_hll_merge(unsigned int *__restrict__ regs, uint32_t ctas) {
     regs[j] = m;
 }
 
-constexpr uint32_t HLL_MB = 32;                  // registers merged per CTA
-constexpr uint32_t HLL_MCTAS = HLL_M / HLL_MB;   // merge CTAs
-// after the per-CTA registers: per merge CTA its part of the estimator's sum
-// (double) and of the empty-register count, then the finish counter
-constexpr size_t HLL_TAIL = 2 * HLL_MCTAS + HLL_MCTAS + 8;
-
-// Merge the per-CTA registers (maximum over `rows` rows) into row 0 and size
-// the table: CTA b merges registers [32 b, 32 b + 32) and leaves its part of
-// sum(2^-reg) and of the zero count; the last CTA to finish adds the parts
-// in a fixed order (so the estimate does not depend on the finishing order)
-// and writes meta: table of 2^k >= factor x estimate slots (at most
-// `reserve`).  With per-CTA key ranges kr (rows pairs, or null) the keys may
-// instead get the direct-address layout (slot = key - min, no key stored)
-// when their span max - min + 1 is at most the hashed table's slot count:
-// the keys then fill at least 1/(2 factor) of the span, the array is no
-// larger than the hashed table and a lookup is one load with no probing.
+// Merge a column's per-CTA registers (maximum over `rows` rows) into row 0
+// and size its hashed tables: CTA b merges registers [32 b, 32 b + 32) and
+// leaves its part of sum(2^-reg) and of the zero count; the last CTA to finish
+// adds the parts in a fixed order (so the estimate does not depend on the
+// finishing order) and writes meta: a table of 2^k >= factor x estimate slots,
+// at most the reservation.  Blocks (x, y): column y.
 constexpr int HLL_MW = 32;   // warps of a merge CTA, each over every HLL_MW-th row
 
-__global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(unsigned int *__restrict__ regs, uint32_t rows,
-                                                        unsigned int *__restrict__ tail, uint64_t reserve,
-                                                        double factor, uint32_t *__restrict__ meta,
-                                                        const int32_t *__restrict__ kr,
-                                                        uint32_t *__restrict__ meta2, uint64_t reserve2) {
+__global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(SizeArgs g) {
+    const SizeCol &c = g.c[blockIdx.y];
+    bool all = true;   // every table of the column is direct-address: nothing was counted
+    for (uint32_t q = 0; q < c.ntargets; ++q) all = all && __ldcg(c.meta[q] + kMetaDense) != 0u;
+    if (all) return;
     __shared__ unsigned int m[HLL_MW][HLL_MB];
     __shared__ bool last;
+    unsigned int *regs = c.scratch;
+    const uint32_t rows = g.rows;
+    unsigned int *tail = size_tail(c.scratch, rows);
     double *part_s = (double *)tail;
     unsigned int *part_z = tail + 2 * HLL_MCTAS;
     unsigned int *done = part_z + HLL_MCTAS;
@@ -541,87 +670,83 @@ __global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(unsigned int *__
         }
     }
     __syncthreads();
-    if (!last) return;
+    if (!last || w != 0) return;
     __threadfence();
     // the last CTA: the parts in a fixed order (lane l adds parts l, l + 32,
-    // ... in turn, then a fixed butterfly), and the key ranges with all threads
-    __shared__ int32_t rlo[HLL_MW], rhi[HLL_MW];
+    // ... in turn, then a fixed butterfly)
     double S = 0.0;
     unsigned int Z = 0;
-    if (w == 0) {
-        for (uint32_t b = lane; b < gridDim.x; b += 32) {
-            S += __ldcg(part_s + b);
-            Z += __ldcg(part_z + b);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            S += __shfl_xor_sync(0xffffffffu, S, o);
-            Z += __shfl_xor_sync(0xffffffffu, Z, o);
-        }
+    for (uint32_t b = lane; b < gridDim.x; b += 32) {
+        S += __ldcg(part_s + b);
+        Z += __ldcg(part_z + b);
     }
-    int32_t lo = INT32_MAX, hi = INT32_MIN;
-    if (kr) {
-        for (uint32_t b = threadIdx.x; b < rows; b += blockDim.x) {
-            lo = min(lo, __ldcg(kr + 2 * b));
-            hi = max(hi, __ldcg(kr + 2 * b + 1));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        }
-        if (lane == 0) {
-            rlo[w] = lo;
-            rhi[w] = hi;
-        }
-        __syncthreads();
-        for (uint32_t q = 0; q < blockDim.x / 32; ++q) {
-            lo = min(lo, rlo[q]);
-            hi = max(hi, rhi[q]);
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, o);
+        Z += __shfl_xor_sync(0xffffffffu, Z, o);
     }
-    if (threadIdx.x != 0) return;
+    if (lane != 0) return;
     const double mm = (double)HLL_M;
     double E = (0.7213 / (1.0 + 1.079 / mm)) * mm * mm / S;
     if (E <= 2.5 * mm && Z > 0) E = mm * log(mm / (double)Z);   // small-range correction
-    // meta2 (optional): a second table of the same keys, at most reserve2 slots
-    for (int t = 0; t < 2; ++t) {
-        uint32_t *mt = t ? meta2 : meta;
-        const uint64_t res = t ? reserve2 : reserve;
-        if (!mt) continue;
+    const double factor = kSingleTableFactor * E <= kSmallTableSlots ? kSingleTableFactor : kLargeTableFactor;
+    for (uint32_t t = 0; t < c.ntargets; ++t) {
+        uint32_t *mt = c.meta[t];
+        if (__ldcg(mt + kMetaDense)) continue;
+        const uint64_t res = c.reserve[t];
         uint64_t cap = 16;
         while ((double)cap < factor * E && cap < res) cap <<= 1;
         if (cap > res) cap = res;
-        mt[0] = (uint32_t)(cap - 1);
-        mt[1] = (uint32_t)E;
-        uint32_t dense = 0u;
-        if (kr) {
-            const int64_t span = (int64_t)hi - (int64_t)lo + 1;
-            if (lo <= hi && (uint64_t)span <= cap) {
-                dense = 1u;
-                mt[kMetaMin] = (uint32_t)lo;
-                mt[kMetaSpan] = (uint32_t)span;
-            }
-        }
-        mt[kMetaDense] = dense;
+        mt[kMetaMask] = (uint32_t)(cap - 1);
+        mt[kMetaEst] = (uint32_t)E;
     }
     *done = 0;
+}
+
+// Empty the tables that the sizing passes laid out (blocks (x, y): table y)
+// and zero the call's outputs (y = ntables).
+struct ClearArgs {
+    ClearTable t[kSizeCols];
+    uint32_t ntables;
+    unsigned long long *zero, *total;
+    uint64_t nzero;
+};
+
+__global__ void __launch_bounds__(BT) k_tables_clear(ClearArgs g) {
+    const uint64_t i0 = (uint64_t)blockIdx.x * BT + threadIdx.x, stride = (uint64_t)gridDim.x * BT;
+    if (blockIdx.y == g.ntables) {
+        for (uint64_t i = i0; i < g.nzero; i += stride) g.zero[i] = 0ull;
+        if (i0 == 0 && g.total) *g.total = 0ull;
+        return;
+    }
+    const ClearTable &t = g.t[blockIdx.y];
+    const bool dense = t.meta[kMetaDense] != 0u;
+    // arrays are 256-byte aligned and have two spare entries
+    if (t.keys == nullptr) {   // degrees: u32 entries, or packed hashed slots
+        const uint64_t words = dense ? (uint64_t)t.meta[kMetaSpan] / 2 + 1 : (uint64_t)t.meta[kMetaMask] + 1;
+        const unsigned long long fill = dense ? 0ull : kEmpty64;
+        for (uint64_t s = i0; s < (words + 1) / 2; s += stride) ((ulonglong2 *)t.tbl)[s] = make_ulonglong2(fill, fill);
+        return;
+    }
+    // weights: zero sums (hashed: of slot mask + 1, key -1, too), free keys
+    const uint64_t sums = dense ? (uint64_t)t.meta[kMetaSpan] : (uint64_t)t.meta[kMetaMask] + 2;
+    for (uint64_t s = i0; s < (sums + 1) / 2; s += stride) ((ulonglong2 *)t.tbl)[s] = make_ulonglong2(0ull, 0ull);
+    if (dense) return;
+    const uint4 free4 = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
+    for (uint64_t s = i0; s < ((uint64_t)t.meta[kMetaMask] + 1) / 4; s += stride) ((uint4 *)t.keys)[s] = free4;
 }
 
 // Insert T's C column.  A warp round is four blocks of 128 consecutive keys
 // (four per lane), all loaded, with the next round's loads issued, before
 // they are used; every run of equal keys in a block is measured once by
-// warp_run_lengths and added to its entry once:
-// hashed slots through single_insert, the direct-address layout as
-// deg[c - min] += run with a 32-bit add whose result is not needed.
-__global__ void __launch_bounds__(BT) k_tinsert_direct(const int32_t *__restrict__ keys, uint32_t n,
-                                                       uint32_t seed, unsigned long long *__restrict__ tbl,
-                                                       const uint32_t *__restrict__ meta, DevStatus *st) {
+// warp_run_lengths and added to its slot once, the first probes of a lane's
+// four keys issued together.
+__global__ void __launch_bounds__(BT, 2) k_tinsert_direct(const int32_t *__restrict__ keys, uint32_t n,
+                                                          uint32_t seed, unsigned long long *__restrict__ tbl,
+                                                          const uint32_t *__restrict__ meta, DevStatus *st) {
     const uint32_t mask = meta[0];
-    const bool dense = meta[kMetaDense] != 0u;
-    const uint32_t kmin = dense ? meta[kMetaMin] : 0u, span = dense ? meta[kMetaSpan] : 0u;
-    uint32_t *deg = (uint32_t *)tbl;
     const bool vec = ((uintptr_t)keys & 15) == 0;
     const uint64_t pol = l2_evict_first();
-    constexpr uint32_t CH = 32 * kRunQ;   // keys of one warp_runs block
+    constexpr uint32_t CH = 32 * kRunQ;   // keys of one block
     constexpr int G = 4;                  // blocks per warp round, loaded together
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * BT + threadIdx.x) >> 5, warps = (gridDim.x * BT) >> 5;
@@ -641,14 +766,21 @@ __global__ void __launch_bounds__(BT) k_tinsert_direct(const int32_t *__restrict
             if ((uint32_t)q < m) v[q] = __ldg(keys + i + q);
         return m;
     };
-    auto emit = [&](int32_t key, uint32_t run) {
-        const uint32_t k = (uint32_t)key;
-        if (!dense)
-            single_insert(tbl, mask, k, seed, (uint32_t)run, st);
-        else if (k - kmin < span)
-            atomicAdd(deg + (k - kmin), (uint32_t)run);
-        else
-            set_status(st, MWJ_ERR_CHECK, 8);   // a key outside the range the sizing pass saw
+    auto insert_block = [&](const int32_t (&v)[kRunQ], uint32_t m) {
+        uint32_t len[kRunQ] = {0u, 0u, 0u, 0u};
+        warp_run_lengths(v, m, [&](int q, int32_t, uint32_t l) { len[q] = l; });
+        uint32_t s[kRunQ];
+        unsigned long long x[kRunQ];
+#pragma unroll
+        for (int q = 0; q < kRunQ; ++q) {
+            if (len[q]) {
+                s[q] = slot_of((uint32_t)v[q], seed, mask);
+                x[q] = __ldcg(tbl + s[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kRunQ; ++q)
+            if (len[q]) single_insert_from(tbl, mask, (uint32_t)v[q], s[q], x[q], len[q], st);
     };
     int32_t v[G][kRunQ];
     uint32_t m[G];
@@ -662,7 +794,7 @@ __global__ void __launch_bounds__(BT) k_tinsert_direct(const int32_t *__restrict
 #pragma unroll
         for (int g = 0; g < G; ++g) nm[g] = load(nr * G + g, nv[g]);
 #pragma unroll
-        for (int g = 0; g < G; ++g) warp_run_lengths(v[g], m[g], emit);
+        for (int g = 0; g < G; ++g) insert_block(v[g], m[g]);
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             m[g] = nm[g];
@@ -675,48 +807,62 @@ __global__ void __launch_bounds__(BT) k_tinsert_direct(const int32_t *__restrict
 
 }  // namespace
 
-cudaError_t single_table_size(const int32_t *keys, int64_t n, uint32_t seed, unsigned int *hll_regs,
-                              uint32_t *meta, uint64_t reserve_slots, int num_sms, cudaStream_t st,
-                              const char *hll_name, const char *size_name, bool allow_dense,
-                              uint32_t *meta2, uint64_t reserve2) {
-    cudaError_t e;
-    const uint32_t nn = (uint32_t)n;
-    const uint32_t ctas = (uint32_t)num_sms * HLL_CTAS_PER_SM;
-    unsigned int *tail = hll_regs + (size_t)ctas * HLL_M;
-    unsigned int *done = tail + 3 * HLL_MCTAS;
-    int32_t *mm = (allow_dense && nn > 0) ? (int32_t *)(tail + HLL_TAIL) : nullptr;
-    uint32_t rows = ctas;
-    if (nn > 0) {
+cudaError_t size_columns(const SizeCol *cols, uint32_t ncols, const HeavyCol *heavy, uint32_t nheavy, bool allow_dense,
+                         int num_sms, cudaStream_t st, const char *hll_name, const char *size_name) {
+    SizeArgs g{};
+    for (uint32_t q = 0; q < ncols; ++q) g.c[q] = cols[q];
+    for (uint32_t q = 0; q < nheavy; ++q) g.h[q] = heavy[q];
+    g.nheavy = nheavy;
+    g.rows = (uint32_t)num_sms * HLL_CTAS_PER_SM;
+    // CTAs of a column's range pass: every one with four loads per thread
+    uint32_t most = 1;
+    for (uint32_t q = 0; q < ncols; ++q) most = cols[q].n > most ? cols[q].n : most;
+    const uint32_t want = (most + 16u * BT - 1) / (16u * BT), full = (uint32_t)num_sms * RANGE_CTAS_PER_SM;
+    g.range_rows = want < full ? want : full;
+    g.ranged = allow_dense;
+    if (allow_dense) {
+        ProfScope ps_("key_range", st);
+        k_range<<<nheavy + ncols * g.range_rows, BT, 0, st>>>(g);
+    }
+    {
         ProfScope ps_(hll_name, st);
-        k_hll<<<ctas, BT, 0, st>>>(keys, nn, seed, hll_regs, done, mm);
-    } else {
-        rows = 1;
-        if ((e = cudaMemsetAsync(hll_regs, 0, HLL_M * sizeof(unsigned int), st)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(done, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
+        k_hll<<<dim3(g.rows, ncols), BT, 0, st>>>(g);
     }
     ProfScope ps_(size_name, st);
-    k_hll_merge_size<<<HLL_MCTAS, HLL_MW * 32, 0, st>>>(hll_regs, rows, tail, reserve_slots, kSingleTableFactor,
-                                                         meta, mm, meta2, reserve2);
+    k_hll_merge_size<<<dim3(HLL_MCTAS, ncols), HLL_MW * 32, 0, st>>>(g);
     return cudaGetLastError();
+}
+
+cudaError_t tables_clear(const ClearTable *t, uint32_t n, unsigned long long *zero, uint64_t nzero,
+                         unsigned long long *total, int num_sms, cudaStream_t st) {
+    ClearArgs g{};
+    for (uint32_t q = 0; q < n; ++q) g.t[q] = t[q];
+    g.ntables = n;
+    g.zero = zero;
+    g.nzero = nzero;
+    g.total = total;
+    ProfScope ps_("tables_clear", st);
+    k_tables_clear<<<dim3(num_sms * 2, n + ((nzero || total) ? 1u : 0u)), BT, 0, st>>>(g);
+    return cudaGetLastError();
+}
+
+cudaError_t single_table_size(const int32_t *keys, int64_t n, uint32_t seed, unsigned int *hll_regs,
+                              uint32_t *meta, uint64_t reserve_slots, int num_sms, cudaStream_t st,
+                              const char *hll_name, const char *size_name, bool allow_dense) {
+    SizeCol c{keys, (uint32_t)n, seed, hll_regs, {meta}, {reserve_slots}, 1u};
+    return size_columns(&c, 1, nullptr, 0, allow_dense, num_sms, st, hll_name, size_name);
 }
 
 cudaError_t single_table_direct(const int32_t *keys, int64_t n, uint32_t seed, unsigned int *hll_regs,
                                 uint32_t *meta, uint64_t *tbl, uint64_t reserve_slots,
-                                DevStatus *status, int num_sms, cudaStream_t st, bool allow_dense) {
+                                DevStatus *status, int num_sms, cudaStream_t st) {
     cudaError_t e;
-    if ((e = single_table_size(keys, n, seed, hll_regs, meta, reserve_slots, num_sms, st, "t_hll", "t_size",
-                               allow_dense)) != cudaSuccess)
-        return e;
-    return single_table_fill(keys, n, seed, meta, tbl, status, num_sms, st);
-}
-
-cudaError_t single_table_fill(const int32_t *keys, int64_t n, uint32_t seed, const uint32_t *meta,
-                              uint64_t *tbl, DevStatus *status, int num_sms, cudaStream_t st) {
-    const uint32_t nn = (uint32_t)n;
+    if ((e = single_table_size(keys, n, seed, hll_regs, meta, reserve_slots, num_sms, st)) != cudaSuccess) return e;
     {
         ProfScope ps_("t_clear", st);
         k_tclear<<<num_sms * 4, 512, 0, st>>>((unsigned long long *)tbl, meta);
     }
+    const uint32_t nn = (uint32_t)n;
     if (nn > 0) {
         ProfScope ps_("t_insert", st);
         const uint32_t groups = (nn + 4 * kRunQ * BT - 1) / (4 * kRunQ * BT);
@@ -735,7 +881,10 @@ cudaError_t hll_regs(const int32_t *keys, int64_t n, uint32_t seed, unsigned int
         const uint32_t ctas = (uint32_t)num_sms * HLL_CTAS_PER_SM;
         {
             ProfScope ps_("sketch_hll", st);
-            k_hll<<<ctas, BT, 0, st>>>(keys, (uint32_t)n, seed, regs, nullptr, nullptr);
+            SizeArgs g{};
+            g.c[0] = SizeCol{keys, (uint32_t)n, seed, regs, {nullptr}, {0}, 0u};
+            g.rows = ctas;
+            k_hll<<<ctas, BT, 0, st>>>(g);
         }
         ProfScope ps_("sketch_hll_merge", st);
         k_hll_merge<<<(HLL_M + 255) / 256, 256, 0, st>>>(regs, ctas);
@@ -747,7 +896,8 @@ cudaError_t hll_regs(const int32_t *keys, int64_t n, uint32_t seed, unsigned int
 
 size_t hll_scratch_registers(int num_sms) {
     const size_t ctas = (size_t)num_sms * HLL_CTAS_PER_SM;
-    return ctas * HLL_M + HLL_TAIL + 2 * ctas;   // registers, sizing tail, per-CTA key ranges
+    // registers, sizing tail, per-CTA key ranges
+    return ctas * HLL_M + HLL_TAIL + 2 * (size_t)num_sms * RANGE_CTAS_PER_SM;
 }
 
 }  // namespace mwj

@@ -57,6 +57,38 @@ __device__ __forceinline__ void warp_runs(const int32_t (&k)[kRunQ], const unsig
     // starts the chain); lanes of one run that continue it add their sum
     unsigned long long v = has ? run : 0ull;   // single: the lane's only run
     bool head = !(cont && single);
+    unsigned long long prev = 0;   // chain through lane - 1
+    if (__any_sync(0xffffffffu, cont)) {   // (keys in no order: no run crosses a lane)
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long pv = __shfl_up_sync(0xffffffffu, v, o);
+            const int ph = __shfl_up_sync(0xffffffffu, (int)head, o);
+            if (lane >= (uint32_t)o && !head) {
+                v += pv;
+                head = ph != 0;
+            }
+        }
+        prev = __shfl_up_sync(0xffffffffu, v, 1);
+    }
+    const int next_cont = __shfl_down_sync(0xffffffffu, (int)cont, 1);
+    if (!has) return;
+    if (!single) {   // the first run ends inside this lane
+        const unsigned long long s = cont ? prev + sf : sf;
+        if (s) emit(kf, s);
+    }
+    if ((lane == 31 || !next_cont) && v) emit(kl, v);   // the chain ends here
+}
+
+// The same for one key per lane: the sum of the run that ends at this lane, 0
+// where none ends.
+__device__ __forceinline__ unsigned long long warp_run_sum1(int32_t k, unsigned long long x, bool has) {
+    const uint32_t lane = threadIdx.x & 31;
+    const int32_t pk = __shfl_up_sync(0xffffffffu, k, 1);
+    const bool cont = has && lane > 0 && pk == k;   // (valid lanes are a prefix)
+    const unsigned conts = __ballot_sync(0xffffffffu, cont);
+    if (conts == 0u) return has ? x : 0ull;
+    unsigned long long v = has ? x : 0ull;
+    bool head = !cont;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long pv = __shfl_up_sync(0xffffffffu, v, o);
@@ -66,14 +98,7 @@ __device__ __forceinline__ void warp_runs(const int32_t (&k)[kRunQ], const unsig
             head = ph != 0;
         }
     }
-    const unsigned long long prev = __shfl_up_sync(0xffffffffu, v, 1);   // chain through lane - 1
-    const int next_cont = __shfl_down_sync(0xffffffffu, (int)cont, 1);
-    if (!has) return;
-    if (!single) {   // the first run ends inside this lane
-        const unsigned long long s = cont ? prev + sf : sf;
-        if (s) emit(kf, s);
-    }
-    if ((lane == 31 || !next_cont) && v) emit(kl, v);   // the chain ends here
+    return (conts >> 1 >> lane) & 1u ? 0ull : v;   // the next lane continues the run
 }
 
 }  // namespace mwj
@@ -87,8 +112,8 @@ namespace mwj {
 // the next start or at the first invalid position.  Each lane finds the ends
 // of its own runs from its four start flags, and the end of its last run
 // from the first later lane that holds a start or an invalid position (one
-// ballot, one shuffle).  emit(key, length) is called once per run by the lane
-// where it starts.  Runs that continue into the next block are emitted in
+// ballot, one shuffle).  emit(q, key, length) is called once per run by the lane
+// where it starts (position q of the lane).  Runs that continue into the next block are emitted in
 // parts.  Every lane of the warp calls this.
 template <typename F>
 __device__ __forceinline__ void warp_run_lengths(const int32_t (&k)[kRunQ], uint32_t m, F &&emit) {
@@ -112,7 +137,7 @@ __device__ __forceinline__ void warp_run_lengths(const int32_t (&k)[kRunQ], uint
         if (!((start >> q) & 1u)) continue;
         const uint32_t rest = endm & ~((2u << q) - 1u);   // ends after position q in this lane
         const uint32_t end = rest ? 4u * lane + (uint32_t)(__ffs(rest) - 1) : block_end;
-        emit(k[q], end - (4u * lane + (uint32_t)q));
+        emit(q, k[q], end - (4u * lane + (uint32_t)q));
     }
 }
 

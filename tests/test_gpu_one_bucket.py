@@ -1,0 +1,107 @@
+"""The one-bucket plan's tables where their layouts change: direct-address
+arrays with gaps and at the largest range they are given to, hashed pairs and
+groups of four, key -1, runs and random order, ragged sizes and unaligned
+columns, chains of three and of four.  Bit-exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1905_13376_gb300 import binding
+
+from gpu_util import cu
+
+pytestmark = pytest.mark.gpu
+
+LAYOUTS = {
+    "compact": lambda k: k,
+    "gaps": lambda k: 7 * k - 1000,                                  # a direct-address range, mostly unused
+    "hashed": lambda k: (k * 2654435761 + 12345) % (1 << 32) - (1 << 31),
+    "extremes": lambda k: np.where(k % 3 == 0, -1, np.where(k % 3 == 1, -(1 << 31) + k, (1 << 31) - 1 - k)),
+}
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch.cuda.set_device(0)
+    c = binding.Context(0)
+    yield c
+    c.close()
+
+
+def rel(g, n, xdom, ydom, fx, fy, sort=False):
+    x, y = g.integers(0, xdom, n), g.integers(0, ydom, n)
+    if sort:
+        x = np.sort(x)
+    return fx(x).astype(np.int32), fy(y).astype(np.int32)
+
+
+def unaligned(r):
+    """The same columns four bytes off a 16-byte boundary."""
+    out = []
+    for c in r:
+        t = torch.empty(len(c) + 1, dtype=torch.int32, device="cuda")
+        t[1:] = torch.from_numpy(np.ascontiguousarray(c)).cuda()
+        out.append(t[1:])
+    return tuple(out)
+
+
+def same(got, want):
+    assert int(got["total"].item()) == want["total"]
+    if "counts" in got:
+        assert np.array_equal(got["counts"].cpu().numpy(), want["counts"])
+
+
+@pytest.mark.parametrize("layout", list(LAYOUTS))
+@pytest.mark.parametrize("n", [1, 3, 127, 129, 4097, 70001])
+def test_chains(ctx, layout, n):
+    g = np.random.default_rng(n + 7 * len(layout))
+    f = LAYOUTS[layout]
+    ident = lambda k: k
+    dom, adom = max(2, n // 5), 50
+    R = rel(g, n, adom, dom, ident, f)
+    S = rel(g, max(1, n - 1), dom, dom, f, f, sort=n % 2 == 0)
+    T = rel(g, n + 2, dom, dom, f, f, sort=n % 4 == 1)
+    U = rel(g, n, dom, 9, f, ident)
+    want = oracle.linear(R, S, T, oracle.GROUP_BY_A, a_domain=adom)
+    for take in (cu, unaligned):
+        d = [take(x) for x in (R, S, T, U)]
+        same(ctx.join3_linear(*d[:3], "group_by_a", a_domain=adom), want)
+        same(ctx.join3_linear(*d[:3], "count"), want)
+        same(ctx.join4_linear(*d, "group_by_a", a_domain=adom), oracle.linear4(R, S, T, U, oracle.GROUP_BY_A,
+                                                                                a_domain=adom))
+
+
+@pytest.mark.parametrize("span", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1])
+def test_largest_direct_range(ctx, span):
+    """2^16 tuples reserve 2^17 slots: a key range of exactly that many values is
+    the largest direct-address one."""
+    g = np.random.default_rng(span)
+    n = 1 << 16
+    k = g.integers(0, span, n)
+    k[:2] = (0, span - 1)
+    k = (k - 77).astype(np.int32)
+    R = (g.integers(0, 64, n).astype(np.int32), g.permutation(k))
+    S = (k, g.permutation(k))
+    T = (g.permutation(k), np.zeros(n, np.int32))
+    want = oracle.linear(R, S, T, oracle.GROUP_BY_A, a_domain=64)
+    same(ctx.join3_linear(cu(R), cu(S), cu(T), "group_by_a", a_domain=64), want)
+
+
+@pytest.mark.parametrize("layout", ["compact", "hashed", "extremes"])
+def test_heavy_keys_and_wide_weights(ctx, layout):
+    """A few keys hold most of S in no order (heavy sums) and weights pass 2^32,
+    in chains of three and four."""
+    g = np.random.default_rng(5)
+    f = LAYOUTS[layout]
+    n = 30000
+    b = np.where(g.random(n) < 0.6, g.integers(0, 3, n), g.integers(0, 500, n))
+    S = (f(b).astype(np.int32), f(np.zeros(n, np.int64)).astype(np.int32))
+    T = (f(np.where(g.random(200000) < 0.9, 0, 5)).astype(np.int32), f(np.zeros(200000, np.int64)).astype(np.int32))
+    R = (g.integers(0, 20, 900).astype(np.int32), f(g.integers(0, 500, 900)).astype(np.int32))
+    want = oracle.linear(R, S, T, oracle.GROUP_BY_A, a_domain=20)
+    assert want["total"] > 1 << 33
+    same(ctx.join3_linear(cu(R), cu(S), cu(T), "group_by_a", a_domain=20), want)
+    U = (f(np.zeros(5000, np.int64)).astype(np.int32), np.zeros(5000, np.int32))
+    want = oracle.linear4(R, S, T, U, oracle.GROUP_BY_A, a_domain=20)
+    same(ctx.join4_linear(cu(R), cu(S), cu(T), cu(U), "group_by_a", a_domain=20), want)
