@@ -15,12 +15,20 @@
 //     w(b)   = OR of skT(c) over S_i's (b, c)                (on chip, per bucket)
 //     sk(a) |= w(b) for every (a, b) of R_i                  (global, per bucket)
 //
-// R and S are partitioned by H(B) as in Algorithm 1; bucket i's on-chip table
-// holds S_i's B values with their 64-byte sketches (the "~100 bytes per
-// tuple" of the paper's footnote).  Four lanes handle one tuple, four
-// bitmaps (16 bytes) per lane.  The estimate of |D(a)| is (M / PHI) * 2^(mean R_j),
+// By default nothing is partitioned (the one-bucket plan of linear_l2.cu with
+// sketches for weights): T's and S's sketches are rows of 64 bytes (the "~100
+// bytes per tuple" of the paper's footnote) in two arrays indexed by the key,
+// and the S and the R pass each gather one row per tuple.  On this GPU a
+// gathered 64-byte row costs little more than a gathered word (238 against
+// 289 G/s, L2-resident: the L1's tag rate bounds both), so the passes run at
+// the speed of the counting ones.  With explicit shares, and for relations
+// whose rows would not be reserved (kFmOneMax), R and S are partitioned by
+// H(B) as in Algorithm 1; bucket i's on-chip table holds S_i's B values with
+// their sketches.  F of the 2^20-vertex graph: 3.8 ms partitioned, 1.0 ms in
+// one bucket.  Four lanes handle one tuple, four bitmaps (16 bytes) per lane.  The estimate of |D(a)| is (M / PHI) * 2^(mean R_j),
 // R_j the lowest 0 bit of bitmap j, PHI = 0.77351.
 #include "api_internal.h"
+#include "group_table.cuh"
 #include "tables.h"
 
 namespace mwj {
@@ -260,16 +268,328 @@ __global__ void __launch_bounds__(FT) k_fm_probe(FmArgs g) {
     }
 }
 
-__global__ void k_fm_estimate(const uint32_t *__restrict__ sk, int32_t a_domain, float *__restrict__ est) {
-    for (uint32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < (uint32_t)a_domain; a += gridDim.x * blockDim.x) {
-        uint32_t tot = 0;
-#pragma unroll
-        for (uint32_t j = 0; j < FM_M; ++j) {   // index of the lowest 0 bit (32 when none)
-            const uint32_t word = __ldg(sk + (size_t)a * FM_M + j);
-            tot += word == 0xFFFFFFFFu ? 32u : (uint32_t)__ffs((int)~word) - 1u;
-        }
-        est[a] = (float)((FM_M / FM_PHI) * exp2((double)tot / FM_M));
+// The estimates.  A sketch's sum of lowest zeros is at most 16 x 32, and a
+// double exp2 costs more than reading the sketch (0.051 ms for 2^20 of them,
+// 0.033 ms this way): every CTA tabulates the estimate of each sum first.  Four
+// lanes per sketch, 16 bytes each.
+constexpr uint32_t kFmSums = 32 * FM_M + 1;
+__global__ void __launch_bounds__(FT) k_fm_estimate(const uint32_t *__restrict__ sk, int32_t a_domain,
+                                                    float *__restrict__ est) {
+    __shared__ float of_sum[kFmSums];
+    for (uint32_t t = threadIdx.x; t < kFmSums; t += FT) of_sum[t] = (float)((FM_M / FM_PHI) * exp2((double)t / FM_M));
+    __syncthreads();
+    const uint64_t words = (uint64_t)a_domain * 4;   // 16-byte quarters
+    const uint64_t stride = (uint64_t)gridDim.x * FT;
+    for (uint64_t i = (uint64_t)blockIdx.x * FT + threadIdx.x; i - (threadIdx.x & 31) < words; i += stride) {
+        const uint4 v = i < words ? __ldg((const uint4 *)sk + i) : make_uint4(0u, 0u, 0u, 0u);
+        auto low = [](uint32_t w) {   // index of the lowest 0 bit (32 when none)
+            return w == 0xFFFFFFFFu ? 32u : (uint32_t)__ffs((int)~w) - 1u;
+        };
+        uint32_t tot = low(v.x) + low(v.y) + low(v.z) + low(v.w);
+        tot += __shfl_xor_sync(0xffffffffu, tot, 1);
+        tot += __shfl_xor_sync(0xffffffffu, tot, 2);
+        if (i < words && (i & 3) == 0) est[i >> 2] = of_sum[tot];
     }
+}
+
+// ---------------------------------------------------------------------------
+// one bucket: rows of sketches indexed by key
+// ---------------------------------------------------------------------------
+
+// A relation's rows: direct-address (row k - min), or the index that a table of
+// its distinct keys gives (group_table.cuh; key -1, which marks free slots, has
+// the last row).  Direct-address when the key range is at most the number of
+// tuples, so that either way n + 1 rows are enough.
+struct FmRows {
+    uint32_t *keys, *idx;   // hashed: slots and their row indices
+    uint32_t *meta;
+    uint32_t *rows;         // (n + 1) x FM_M
+    unsigned int *count;    // rows given out
+    uint32_t seed, n;
+};
+
+struct FmOne {
+    FmRows t, s;
+};
+
+// the row of a key; the layout's words are read once per thread.  DENSE: known
+// to be direct-address.
+template <bool DENSE>
+struct FmIndex {
+    const FmRows &r;
+    bool dense;
+    uint32_t min, span, mask;
+    __device__ explicit FmIndex(const FmRows &r_) : r(r_) {
+        dense = DENSE || __ldg(r.meta + kMetaDense) != 0u;
+        min = dense ? __ldg(r.meta + kMetaMin) : 0u;
+        span = dense ? __ldg(r.meta + kMetaSpan) : 0u;
+        mask = DENSE ? 0u : __ldg(r.meta + kMetaMask);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t k) const {
+        if (DENSE || dense) return k - min < span ? k - min : kNoIndex;
+        if (k == kEmptyKey) return r.n;
+        const uint32_t s = w_home(k, r.seed, mask);
+        const uint32_t at = w_find(r.keys, mask, k, s, __ldg((const uint4 *)(r.keys + s)));
+        return at == kEmptyKey ? kNoIndex : __ldg(r.idx + at);
+    }
+};
+
+// y 0 / 1: T's / S's rows (direct-address) or free keys and key -1's row
+// (hashed); y 2: the output sketches.
+__global__ void __launch_bounds__(FT) k_fm_clear(FmOne g, uint32_t *__restrict__ out, uint64_t out_rows) {
+    const uint64_t i0 = (uint64_t)blockIdx.x * FT + threadIdx.x, stride = (uint64_t)gridDim.x * FT;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.y == 2) {
+        for (uint64_t i = i0; i < 4 * out_rows; i += stride) ((uint4 *)out)[i] = zero;
+        return;
+    }
+    const FmRows &r = blockIdx.y ? g.s : g.t;
+    if (i0 == 0) *r.count = 0u;
+    if (__ldg(r.meta + kMetaDense)) {
+        const uint64_t rows = __ldg(r.meta + kMetaSpan);
+        for (uint64_t i = i0; i < 4 * rows; i += stride) ((uint4 *)r.rows)[i] = zero;
+        return;
+    }
+    const uint4 free4 = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
+    for (uint64_t i = i0; i < ((uint64_t)__ldg(r.meta + kMetaMask) + 1) / 4; i += stride) ((uint4 *)r.keys)[i] = free4;
+    if (i0 < 4) ((uint4 *)(r.rows + (size_t)r.n * FM_M))[i0] = zero;
+}
+
+// Hashed: the distinct keys of a column (y 0: T's C, y 1: S's B).
+__global__ void __launch_bounds__(256) k_fm_keys(FmOne g, const int32_t *__restrict__ tc,
+                                                 const int32_t *__restrict__ sb, DevStatus *st) {
+    const FmRows &r = blockIdx.y ? g.s : g.t;
+    if (__ldg(r.meta + kMetaDense)) return;
+    const int32_t *col = blockIdx.y ? sb : tc;
+    const uint32_t mask = __ldg(r.meta + kMetaMask), lane = threadIdx.x & 31;
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i - lane < r.n; i += (uint64_t)gridDim.x * 256) {
+        const uint32_t k = i < r.n ? (uint32_t)__ldg(col + i) : kEmptyKey;
+        const uint32_t prev = __shfl_up_sync(0xffffffffu, k, 1);
+        if (k == kEmptyKey || (lane > 0 && prev == k)) continue;   // (a run needs its key once)
+        const uint32_t s = w_home(k, r.seed, mask);
+        if (w_claim(r.keys, mask, k, s, __ldcg((const uint4 *)(r.keys + s))) == kEmptyKey)
+            set_status(st, MWJ_ERR_CHECK, 10);   // table full: the sizing step under-estimated
+    }
+}
+
+// Hashed: a row for every key, zeroed by the thread that gives it out.
+__global__ void __launch_bounds__(256) k_fm_rows(FmOne g) {
+    const FmRows &r = blockIdx.y ? g.s : g.t;
+    if (__ldg(r.meta + kMetaDense)) return;
+    const uint64_t slots = (uint64_t)__ldg(r.meta + kMetaMask) + 1;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint64_t s = (uint64_t)blockIdx.x * 256 + threadIdx.x; s - lane < slots; s += (uint64_t)gridDim.x * 256) {
+        const bool occ = s < slots && r.keys[s] != kEmptyKey;
+        const unsigned m = __ballot_sync(0xffffffffu, occ);
+        unsigned base = 0;
+        if (lane == 0 && m) base = atomicAdd(r.count, (unsigned)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        const uint32_t row = base + __popc(m & ((1u << lane) - 1u));
+        if (!occ || row >= r.n) continue;   // (distinct keys: at most n)
+        r.idx[s] = row;
+        uint4 *dst = (uint4 *)(r.rows + (size_t)row * FM_M);
+        for (int q = 0; q < 4; ++q) dst[q] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+// T pass: the bit of d in c's row, a tuple per lane, one 32-bit OR each (their
+// results are not needed; the tuples of one c share two sectors).
+__global__ void __launch_bounds__(256) k_fm_tbits(const int32_t *__restrict__ tc, const int32_t *__restrict__ td,
+                                                  uint32_t n, FmRows r) {
+    const uint32_t T = gridDim.x * 256;
+    const FmIndex<false> index(r);
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += T) {
+        const uint32_t row = index((uint32_t)__ldg(tc + i));
+        uint32_t j, bit;
+        fm_bit(__ldg(td + i), &j, &bit);
+        if (row != kNoIndex) atomicOr(r.rows + (size_t)row * FM_M + j, 1u << bit);   // (every c of T has a row)
+    }
+}
+
+// S and R pass: row(x) |= row(y) over the relation's tuples (x, y).  A group of
+// four lanes takes FM_K consecutive tuples, gathers their rows four at a time
+// (16 bytes per lane) and ORs a run of equal x in registers; at the run's end
+// only the bits that the target row lacks cost an atomic.  OUT: the target is
+// the output, indexed by a in [0, a_domain).
+// The next four tuples are loaded while the rows of these are on their way,
+// and a run's target row is read when the run ends and compared when the next
+// one does (or the group's tuples end): without the two the group waited out
+// three memory latencies per four tuples (0.53 ms a pass on F, 0.37 ms with
+// them and the layout's words in registers).
+// DENSE: all rows of the pass direct-address; the call launches both kernels
+// and the one whose layout the sizing pass did not choose returns at once.
+// What bounds it now: 64 bytes per tuple from a 64 MB array that the L2 keeps
+// only in part (59 % hits: 0.8 GB of row sectors come from DRAM in a pass).
+constexpr uint32_t FM_K = 32;
+template <bool OUT, bool DENSE>
+__global__ void __launch_bounds__(256, 4) k_fm_pass(const int32_t *__restrict__ X, const int32_t *__restrict__ Y,
+                                                    uint32_t n, FmRows src, FmRows dst,
+                                                                uint32_t *__restrict__ out, int32_t a_domain,
+                                                                DevStatus *st) {
+    if ((__ldg(src.meta + kMetaDense) && (OUT || __ldg(dst.meta + kMetaDense))) != DENSE) return;
+    const uint32_t l4 = threadIdx.x & 3;
+    const uint64_t groups = (uint64_t)gridDim.x * 64;
+    const FmIndex<DENSE> from(src), to(dst);
+    // lane l4 of a group holds tuple i + l4; the others read it by shuffle
+    const unsigned group = 0xFu << (threadIdx.x & 28);
+    auto load = [&](uint32_t i, uint32_t e, int32_t &x, int32_t &y) {
+        x = i + l4 < e ? __ldg(X + i + l4) : 0;
+        y = i + l4 < e ? __ldg(Y + i + l4) : 0;
+    };
+    // the run that ended last: its target (null: none), its OR, the target's
+    // bits as read then
+    uint32_t *pend = nullptr;
+    uint4 pv = make_uint4(0u, 0u, 0u, 0u), pc = pv;
+    auto settle = [&]() {
+        if (!pend) return;
+        if (pv.x & ~pc.x) atomicOr(pend, pv.x);
+        if (pv.y & ~pc.y) atomicOr(pend + 1, pv.y);
+        if (pv.z & ~pc.z) atomicOr(pend + 2, pv.z);
+        if (pv.w & ~pc.w) atomicOr(pend + 3, pv.w);
+        pend = nullptr;
+    };
+    auto flush = [&](int32_t x, const uint4 &v) {
+        settle();
+        if (!(v.x | v.y | v.z | v.w)) return;
+        if (OUT) {
+            if ((uint32_t)x >= (uint32_t)a_domain) return;   // reported below
+            pend = out + (size_t)(uint32_t)x * FM_M + 4 * l4;
+        } else {
+            const uint32_t row = to((uint32_t)x);
+            if (row == kNoIndex) return;   // (every b of S has a row)
+            pend = dst.rows + (size_t)row * FM_M + 4 * l4;
+        }
+        pv = v;
+        pc = __ldcg((const uint4 *)pend);
+    };
+    for (uint64_t i0 = ((uint64_t)blockIdx.x * 64 + (threadIdx.x >> 2)) * FM_K; i0 < n; i0 += groups * FM_K) {
+        const uint32_t e = (uint32_t)(i0 + FM_K < n ? i0 + FM_K : n);
+        uint4 acc = make_uint4(0u, 0u, 0u, 0u);
+        int32_t x, y;
+        load((uint32_t)i0, e, x, y);
+        int32_t cur = __shfl_sync(group, x, 0, 4);
+        for (uint32_t i = (uint32_t)i0; i < e; i += 4) {
+            const uint32_t m = min(4u, e - i);
+            if (OUT && l4 < m && (uint32_t)x >= (uint32_t)a_domain) set_status(st, MWJ_ERR_DOMAIN, x);
+            uint4 v[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t row = from((uint32_t)__shfl_sync(group, y, q, 4));
+                v[q] = make_uint4(0u, 0u, 0u, 0u);
+                if (q < m && row != kNoIndex) v[q] = __ldg((const uint4 *)(src.rows + (size_t)row * FM_M) + l4);
+            }
+            int32_t nx, ny;
+            load(i + 4, e, nx, ny);
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const int32_t xq = __shfl_sync(group, x, q, 4);
+                if (q >= m) break;
+                if (xq != cur) {
+                    flush(cur, acc);
+                    acc = make_uint4(0u, 0u, 0u, 0u);
+                    cur = xq;
+                }
+                acc.x |= v[q].x;
+                acc.y |= v[q].y;
+                acc.z |= v[q].z;
+                acc.w |= v[q].w;
+            }
+            x = nx;
+            y = ny;
+        }
+        flush(cur, acc);
+    }
+    settle();
+}
+
+// Tuples of S and T up to which their rows are reserved: 64 bytes each, so at
+// most 17 GB a relation; larger relations are partitioned.
+constexpr int64_t kFmOneMax = 1ll << 28;
+bool fm_one(const mwj_rel &S, const mwj_rel &T, const mwj_shares *sh) {
+    return !sh && S.n <= kFmOneMax && T.n <= kFmOneMax;
+}
+
+struct FmOneLayout {
+    FmOne one;
+    unsigned int *hll[2];
+};
+
+size_t fm_one_layout(Arena &A, const mwj_rel &S, const mwj_rel &T, int num_sms, const Seeds &sd, FmOneLayout &L) {
+    auto take = [&](const mwj_rel &r, uint32_t seed) {
+        FmRows f{};
+        f.keys = A.take<uint32_t>(single_table_slots(r.n));
+        f.idx = A.take<uint32_t>(single_table_slots(r.n));
+        f.meta = A.take<uint32_t>(kMetaWords);
+        f.rows = A.take<uint32_t>((size_t)(r.n + 1) * FM_M);
+        f.count = A.take<unsigned int>(4);
+        f.seed = seed;
+        f.n = (uint32_t)r.n;
+        return f;
+    };
+    L.one.t = take(T, sd.slot2);
+    L.one.s = take(S, sd.slot);
+    for (int k = 0; k < 2; ++k) L.hll[k] = A.take<unsigned int>(hll_scratch_registers(num_sms));
+    return A.used;
+}
+
+unsigned fm_grid(uint64_t n, uint64_t per_cta, int num_sms, int ctas_per_sm) {
+    const uint64_t want = (n + per_cta - 1) / per_cta, full = (uint64_t)num_sms * ctas_per_sm;
+    return (unsigned)(want < full ? (want ? want : 1) : full);
+}
+
+cudaError_t fm_one_run(const FmOneLayout &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int32_t a_domain,
+                       uint32_t *sketches, DevStatus *status, int sms, cudaStream_t st) {
+    const FmOne &g = L.one;
+    SizeCol cols[kSizeCols];
+    uint32_t ncols = 1;
+    cols[0] = SizeCol{T.x, (uint32_t)T.n, g.t.seed, L.hll[0], {g.t.meta}, {single_table_slots(T.n)}, {(uint64_t)T.n}, 1u};
+    if (S.x == T.x && S.n == T.n) {   // a self-join: one pass sizes both
+        cols[0].meta[1] = g.s.meta;
+        cols[0].reserve[1] = cols[0].reserve[0];
+        cols[0].range[1] = cols[0].range[0];
+        cols[0].ntargets = 2;
+    } else {
+        cols[1] = SizeCol{S.x, (uint32_t)S.n, g.s.seed, L.hll[1], {g.s.meta}, {single_table_slots(S.n)}, {(uint64_t)S.n}, 1u};
+        ncols = 2;
+    }
+    cudaError_t e;
+    if ((e = size_columns(cols, ncols, nullptr, 0, true, sms, st)) != cudaSuccess) return e;
+    const uint64_t most = (uint64_t)(T.n > S.n ? T.n : S.n);
+    {
+        ProfScope ps_("fm_clear", st);
+        k_fm_clear<<<dim3(sms * 2, 3), FT, 0, st>>>(g, sketches, (uint64_t)a_domain);
+    }
+    {
+        ProfScope ps_("fm_keys", st);
+        k_fm_keys<<<dim3(fm_grid(most, 256, sms, 8), 2), 256, 0, st>>>(g, T.x, S.x, status);
+    }
+    {
+        ProfScope ps_("fm_rows", st);
+        k_fm_rows<<<dim3(fm_grid(4 * most, 256, sms, 8), 2), 256, 0, st>>>(g);
+    }
+    if (T.n > 0) {
+        ProfScope ps_("fm_tbits", st);
+        k_fm_tbits<<<fm_grid(T.n, 256, sms, 8), 256, 0, st>>>(T.x, T.y, (uint32_t)T.n, g.t);
+    }
+    if (S.n > 0) {
+        const unsigned grid = fm_grid(S.n, 64 * FM_K, sms, 8);
+        {
+            ProfScope ps_("fm_spass", st);
+            k_fm_pass<false, true><<<grid, 256, 0, st>>>(S.x, S.y, (uint32_t)S.n, g.t, g.s, nullptr, 0, status);
+        }
+        ProfScope ps_("fm_spass_hashed", st);
+        k_fm_pass<false, false><<<grid, 256, 0, st>>>(S.x, S.y, (uint32_t)S.n, g.t, g.s, nullptr, 0, status);
+    }
+    if (R.n > 0) {
+        const unsigned grid = fm_grid(R.n, 64 * FM_K, sms, 8);
+        {
+            ProfScope ps_("fm_rpass", st);
+            k_fm_pass<true, true><<<grid, 256, 0, st>>>(R.x, R.y, (uint32_t)R.n, g.s, g.s, sketches, a_domain, status);
+        }
+        ProfScope ps_("fm_rpass_hashed", st);
+        k_fm_pass<true, false><<<grid, 256, 0, st>>>(R.x, R.y, (uint32_t)R.n, g.s, g.s, sketches, a_domain, status);
+    }
+    return cudaGetLastError();
 }
 
 struct FmLayout {
@@ -329,10 +649,15 @@ extern "C" mwj_status mwj_fm_workspace_size(mwj_ctx *ctx, mwj_rel R, mwj_rel S, 
                                             const mwj_shares *shares, size_t *bytes) {
     if (!ctx || !bytes) return MWJ_ERR_INVALID_ARG;
     if (!rel_ok(R) || !rel_ok(S) || !rel_ok(T)) return fail(ctx, MWJ_ERR_INVALID_ARG, "bad relation");
+    Arena A(nullptr, 0);
+    if (fm_one(S, T, shares)) {
+        FmOneLayout L;
+        *bytes = fm_one_layout(A, S, T, ctx->dev.num_sms, ctx->seeds, L);
+        return MWJ_OK;
+    }
     uint32_t I;
     mwj_status s = fm_buckets(ctx, S, shares, &I);
     if (s != MWJ_OK) return s;
-    Arena A(nullptr, 0);
     FmLayout L;
     *bytes = fm_layout(A, I, R, S, T, ctx->dev.num_sms, L);
     return MWJ_OK;
@@ -344,19 +669,35 @@ extern "C" mwj_status mwj_fm_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel 
     if (!ctx || !sketches || a_domain <= 0 || ((uintptr_t)sketches & 15)) return MWJ_ERR_INVALID_ARG;
     ApiScope api_scope(&ctx->prof);
     if (!rel_ok(R) || !rel_ok(S) || !rel_ok(T)) return fail(ctx, MWJ_ERR_INVALID_ARG, "bad relation");
+    cudaStream_t st = (cudaStream_t)stream;
+    const Seeds &sd = ctx->seeds;
+    const int sms = ctx->dev.num_sms;
+    cudaError_t e;
+    Arena A(workspace, ws_bytes);
+    auto estimate = [&]() -> mwj_status {
+        if (!estimates) return MWJ_OK;
+        ProfScope ps_("fm_estimate", st);
+        k_fm_estimate<<<fm_grid((uint64_t)a_domain * 4, FT, sms, 2), FT, 0, st>>>(sketches, a_domain, estimates);
+        const cudaError_t ee = cudaGetLastError();
+        return ee == cudaSuccess ? MWJ_OK : cuda_fail(ctx, ee, "fm estimate");
+    };
+    if (fm_one(S, T, shares)) {
+        FmOneLayout L;
+        fm_one_layout(A, S, T, sms, sd, L);
+        if (A.overflow || !workspace)
+            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
+        if ((e = fm_one_run(L, R, S, T, a_domain, sketches, ctx->status, sms, st)) != cudaSuccess)
+            return cuda_fail(ctx, e, "fm one bucket");
+        return estimate();
+    }
     uint32_t I;
     mwj_status s = fm_buckets(ctx, S, shares, &I);
     if (s != MWJ_OK) return s;
-    Arena A(workspace, ws_bytes);
     FmLayout L;
     fm_layout(A, I, R, S, T, ctx->dev.num_sms, L);
     if (A.overflow || !workspace)
         return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
 
-    cudaStream_t st = (cudaStream_t)stream;
-    const Seeds &sd = ctx->seeds;
-    const int sms = ctx->dev.num_sms;
-    cudaError_t e;
     if ((e = cudaMemsetAsync(sketches, 0, sizeof(uint32_t) * FM_M * (size_t)a_domain, st)) != cudaSuccess)
         return cuda_fail(ctx, e, "memset sketches");
     if ((e = cudaMemsetAsync(L.tcount, 0, sizeof(unsigned int), st)) != cudaSuccess)
@@ -412,10 +753,5 @@ extern "C" mwj_status mwj_fm_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel 
         k_fm_probe<<<I, FT, smem, st>>>(g);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "fm probe");
-    if (estimates) {
-        ProfScope ps_("fm_estimate", st);
-        k_fm_estimate<<<sms * 4, 256, 0, st>>>(sketches, a_domain, estimates);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "fm estimate");
-    }
-    return MWJ_OK;
+    return estimate();
 }

@@ -21,6 +21,7 @@
 // the table and adds each run of equal a once.
 #include <type_traits>
 
+#include "group_table.cuh"
 #include "internal.h"
 #include "linear_l2.h"
 #include "skew.h"
@@ -98,51 +99,6 @@ __device__ __forceinline__ void deg_add(unsigned long long *slots, uint32_t mask
         v = __ldcg((const ulonglong2 *)(slots + s));
     }
     set_status(st, MWJ_ERR_CHECK, 3);   // table full: the sizing step under-estimated
-}
-
-// Hashed weights: the group of four keys at which the search for key k starts.
-__device__ __forceinline__ uint32_t w_home(uint32_t k, uint32_t seed, uint32_t mask) {
-    return slot_of(k, seed, mask) & ~3u;
-}
-
-// Slot of key k (not -1) from its home group (slot s, keys v); kEmptyKey when a
-// free slot comes first.
-__device__ __forceinline__ uint32_t w_find(const uint32_t *__restrict__ keys, uint32_t mask, uint32_t k, uint32_t s,
-                                           uint4 v) {
-    for (uint32_t it = 0; it <= mask; it += 4) {
-        if (v.x == k) return s;
-        if (v.y == k) return s + 1;
-        if (v.z == k) return s + 2;
-        if (v.w == k) return s + 3;
-        if (v.w == kEmptyKey) break;   // (a group fills in order: v.w free says that it is not full)
-        s = (s + 4) & mask;
-        v = __ldg((const uint4 *)(keys + s));
-    }
-    return kEmptyKey;
-}
-
-// Slot of key k (not -1), claimed if it is new, from its home group (possibly
-// read before other threads claimed slots of it); kEmptyKey: the table is full.
-__device__ __forceinline__ uint32_t w_claim(uint32_t *keys, uint32_t mask, uint32_t k, uint32_t s, uint4 v) {
-    for (uint32_t it = 0; it <= mask; it += 4) {
-        if (v.x == k) return s;
-        if (v.y == k) return s + 1;
-        if (v.z == k) return s + 2;
-        if (v.w == k) return s + 3;
-        if (v.w == kEmptyKey) {
-#pragma unroll
-            for (uint32_t q = 0; q < 4; ++q) {
-                uint32_t u = q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w;
-                if (u == kEmptyKey) {
-                    u = atomicCAS(keys + s + q, kEmptyKey, k);
-                    if (u == kEmptyKey || u == k) return s + q;
-                }
-            }
-        }
-        s = (s + 4) & mask;
-        v = __ldcg((const uint4 *)(keys + s));
-    }
-    return kEmptyKey;
 }
 
 // Direct-address weights (the sizing pass chose that layout for S's B
@@ -706,11 +662,12 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
         for (uint32_t q = 0; q < ncols; ++q) {
             if (cols[q].keys == r.x && cols[q].n == (uint32_t)r.n) {
                 cols[q].meta[cols[q].ntargets] = meta;
-                cols[q].reserve[cols[q].ntargets++] = reserve;
+                cols[q].reserve[cols[q].ntargets] = reserve;
+                cols[q].range[cols[q].ntargets++] = reserve;
                 return;
             }
         }
-        cols[ncols] = SizeCol{r.x, (uint32_t)r.n, seed, L.hll[ncols], {meta}, {reserve}, 1u};
+        cols[ncols] = SizeCol{r.x, (uint32_t)r.n, seed, L.hll[ncols], {meta}, {reserve}, {reserve}, 1u};
         ++ncols;
     };
     HeavyCol heavy[kSizeCols];

@@ -417,8 +417,8 @@ struct SizeArgs {
     bool ranged;   // k_range has run: a compact column gets the direct-address layout
 };
 
-__device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t reserve) {
-    return lo <= hi && (uint64_t)((int64_t)hi - (int64_t)lo + 1) <= reserve;
+__device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t most) {
+    return lo <= hi && (uint64_t)((int64_t)hi - (int64_t)lo + 1) <= most;
 }
 
 // Key range of every column: `rows` CTAs per column, each leaving the
@@ -451,10 +451,10 @@ __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
     if (t < n - head - 4u * quads) see(__ldg(keys + head + 4u * quads + t));
     const int4 *v = (const int4 *)(keys + head);
     const uint64_t pol = l2_evict_first();
-    // a thread whose keys already span more than every reservation stops: its
+    // a thread whose keys already span more than every direct-address table stops: its
     // part of the range settles the layout
     uint64_t most = 0;
-    for (uint32_t q = 0; q < c.ntargets; ++q) most = c.reserve[q] > most ? c.reserve[q] : most;
+    for (uint32_t q = 0; q < c.ntargets; ++q) most = c.range[q] > most ? c.range[q] : most;
     const uint32_t wide = most > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)most;
     uint32_t i = t;
     for (; i < quads && quads - i > 3u * T; i += 4u * T) {
@@ -502,8 +502,8 @@ __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
 // keys have distinct hashes.
 //
 // Blocks (x, y): column y.  With `ranged` every CTA first merges the column's
-// key ranges: a table whose reserved slots hold the whole range gets the
-// direct-address layout (slot = key - min, no key stored), which is decided
+// key ranges: a table whose direct-address entries (range[q]) hold the whole
+// range gets that layout (slot = key - min, no key stored), which is decided
 // from the range alone: the array is no larger than the hashed table's
 // reservation, clearing it costs at most 16 bytes per tuple, and only the
 // entries of keys that occur are touched again.  A column none of whose
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(SizeArgs g) {
         hi = shi;
         bool all = true;
         for (uint32_t q = 0; q < c.ntargets; ++q) {
-            const bool dense = span_fits(lo, hi, c.reserve[q]);
+            const bool dense = span_fits(lo, hi, c.range[q]);
             all = all && dense;
             if (first) {
                 c.meta[q][kMetaDense] = dense ? 1u : 0u;
@@ -849,7 +849,7 @@ cudaError_t tables_clear(const ClearTable *t, uint32_t n, unsigned long long *ze
 cudaError_t single_table_size(const int32_t *keys, int64_t n, uint32_t seed, unsigned int *hll_regs,
                               uint32_t *meta, uint64_t reserve_slots, int num_sms, cudaStream_t st,
                               const char *hll_name, const char *size_name, bool allow_dense) {
-    SizeCol c{keys, (uint32_t)n, seed, hll_regs, {meta}, {reserve_slots}, 1u};
+    SizeCol c{keys, (uint32_t)n, seed, hll_regs, {meta}, {reserve_slots}, {reserve_slots}, 1u};
     return size_columns(&c, 1, nullptr, 0, allow_dense, num_sms, st, hll_name, size_name);
 }
 
@@ -882,7 +882,7 @@ cudaError_t hll_regs(const int32_t *keys, int64_t n, uint32_t seed, unsigned int
         {
             ProfScope ps_("sketch_hll", st);
             SizeArgs g{};
-            g.c[0] = SizeCol{keys, (uint32_t)n, seed, regs, {nullptr}, {0}, 0u};
+            g.c[0] = SizeCol{keys, (uint32_t)n, seed, regs, {nullptr}, {0}, {0}, 0u};
             g.rows = ctas;
             k_hll<<<ctas, BT, 0, st>>>(g);
         }

@@ -86,14 +86,15 @@ cudaError_t single_table_size(const int32_t *keys, int64_t n, uint32_t seed, uns
                               bool allow_dense = false);
 
 // Several key columns sized in the same launches, a column for up to
-// kSizeCols tables of its keys (meta[q], at most reserve[q] slots each).
+// kSizeCols tables of its keys (meta[q], at most reserve[q] hashed slots and
+// range[q] direct-address entries each).
 constexpr uint32_t kSizeCols = 3;
 struct SizeCol {
     const int32_t *keys;
     uint32_t n, seed;
     unsigned int *scratch;   // hll_scratch_registers(num_sms) u32 of its own
     uint32_t *meta[kSizeCols];
-    uint64_t reserve[kSizeCols];
+    uint64_t reserve[kSizeCols], range[kSizeCols];
     uint32_t ntargets;
 };
 // A column whose heavy keys (sampled share at least 1 / (2 x buckets)) are
