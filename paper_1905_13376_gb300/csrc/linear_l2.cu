@@ -19,6 +19,11 @@
 // per distinct b, and runs of equal keys (edge lists sorted by source) are
 // summed inside each warp before they reach the L2; the R pass only reads
 // the table and adds each run of equal a once.
+//
+// A star join is the same three passes with the weight table laid out for R's
+// B values instead of S's (star_bucket_run): R is the small relation, so its
+// column is the cheap one to size, and S tuples whose b is not R's are
+// skipped.
 #include <type_traits>
 
 #include "group_table.cuh"
@@ -104,11 +109,14 @@ __device__ __forceinline__ void deg_add(unsigned long long *slots, uint32_t mask
 // Direct-address weights (the sizing pass chose that layout for S's B
 // values): w(b) is the plain 64-bit word W[b - min], added to with 64-bit
 // atomics whose results are not needed (exact modulo 2^64, no carry word).
+// FILTER: a key outside the table's range is no error but a tuple that joins
+// nothing (star joins, whose table holds R's keys).
+template <bool FILTER>
 __device__ __forceinline__ void w_add_direct(unsigned long long *__restrict__ W, uint32_t wmin, uint32_t wspan,
                                              uint32_t b, unsigned long long x, DevStatus *st) {
     if (b - wmin < wspan)
         atomicAdd(W + (b - wmin), x);
-    else
+    else if (!FILTER)
         set_status(st, MWJ_ERR_CHECK, 9);   // a key outside the range the sizing pass saw
 }
 
@@ -220,7 +228,7 @@ __device__ __forceinline__ Lookup<SW> make_lookup(const Source &src) {
 // ones.  x = the source's value of c; heavy B keys go to the CTA's sums; runs
 // of equal b are summed in the warp and added to w(b) once (one
 // fire-and-forget 64-bit add).
-template <bool SW>
+template <bool SW, bool FILTER>
 struct SPass {
     const Lookup<SW> look;
     const WTable &w;
@@ -251,7 +259,7 @@ struct SPass {
             }
         }
         warp_runs(b, x, m, [&](int32_t key, unsigned long long sum) {
-            w_add_direct(w.W, wmin, wspan, (uint32_t)key, sum, st);
+            w_add_direct<FILTER>(w.W, wmin, wspan, (uint32_t)key, sum, st);
         });
     }
 
@@ -260,7 +268,7 @@ struct SPass {
         if (!hs) return;
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < kHeavySlots; i += nthreads)
-            if (heavy_sum(hacc, i)) w_add_direct(w.W, wmin, wspan, hs[i], heavy_sum(hacc, i), st);
+            if (heavy_sum(hacc, i)) w_add_direct<FILTER>(w.W, wmin, wspan, hs[i], heavy_sum(hacc, i), st);
     }
 };
 
@@ -305,8 +313,9 @@ __device__ __forceinline__ void rounds_plain(const int32_t *__restrict__ X, cons
 // lane a warp waited for four such chains, one after the other, and 80
 // registers left only three CTAs to fill the waits.  8.4 million id-keyed
 // tuples into 1.5 million keys: 0.235 ms with four, 0.154 ms with one.
+// FILTER: the table's keys are there already (k_w_keys); others are skipped.
 constexpr int GC = 6;
-template <bool SW>
+template <bool SW, bool FILTER>
 __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
                                                     uint32_t n, Source src, WTable w, DevStatus *st) {
     const bool sd = source_dense<SW>(src), wd = __ldg(w.meta + kMetaDense) != 0u;
@@ -337,13 +346,15 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
     };
     auto add = [&](uint32_t b, uint32_t s, uint4 v, unsigned long long x) {
         if (wd) {
-            w_add_direct(w.W, wmin, wspan, b, x, st);
+            w_add_direct<FILTER>(w.W, wmin, wspan, b, x, st);
             return;
         }
-        const uint32_t at = b == kEmptyKey ? wmask + 1 : w_claim(w.keys, wmask, b, s, v);
+        const uint32_t at = b == kEmptyKey ? wmask + 1
+                            : FILTER       ? w_find(w.keys, wmask, b, s, v)
+                                           : w_claim(w.keys, wmask, b, s, v);
         if (at != kEmptyKey)
             atomicAdd(w.W + at, x);
-        else
+        else if (!FILTER)
             set_status(st, MWJ_ERR_CHECK, 7);   // table full: the sizing step under-estimated
     };
     const uint32_t T = gridDim.x * WT, lane = threadIdx.x & 31;
@@ -389,7 +400,7 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
     }
 }
 
-template <bool SW>
+template <bool SW, bool FILTER>
 __global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict__ Sb,
                                                        const int32_t *__restrict__ Sc, uint32_t n, Source src,
                                                        WTable w, DevStatus *st) {
@@ -397,11 +408,25 @@ __global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict
     __shared__ uint32_t hbuf[kHeavySlots];
     __shared__ HeavySums hacc;
     const uint32_t *hs = heavy_begin(w.heavy, hbuf, hacc);
-    SPass<SW> P(src, w, st, hs, hacc);
+    SPass<SW, FILTER> P(src, w, st, hs, hacc);
     const uint32_t warp = (blockIdx.x * WT + threadIdx.x) >> 5, warps = (gridDim.x * WT) >> 5;
     rounds_plain(Sb, Sc, 0u, n, warp, warps,
                  [&](const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) { P.round(b, c, m); });
     P.flush_heavy(WT);
+}
+
+// Star joins, hashed layout: R's keys into the weight table, so that the S pass
+// keeps only the tuples that meet one.
+__global__ void __launch_bounds__(WT) k_w_keys(const int32_t *__restrict__ Rb, uint32_t n, WTable w, DevStatus *st) {
+    if (__ldg(w.meta + kMetaDense)) return;
+    const uint32_t mask = __ldg(w.meta + kMetaMask);
+    for (uint64_t i = (uint64_t)blockIdx.x * WT + threadIdx.x; i < n; i += gridDim.x * WT) {
+        const uint32_t k = (uint32_t)__ldg(Rb + i);
+        if (k == kEmptyKey) continue;   // its sum has a place of its own
+        const uint32_t s = w_home(k, w.seed, mask);
+        if (w_claim(w.keys, mask, k, s, __ldcg((const uint4 *)(w.keys + s))) == kEmptyKey)
+            set_status(st, MWJ_ERR_CHECK, 11);   // table full: the sizing step under-estimated
+    }
 }
 
 // R pass (MODE 0: COUNT, MODE 1: GROUP BY A); same loop as the S pass.
@@ -477,9 +502,8 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
 // four per lane, both loaded, with the next round's loads issued, before they
 // are used.  deg[k] += i at the end of every run of equal keys k
 // and -= i at its start, i counted inside the block (32-bit adds whose results
-// are not needed, exact modulo 2^32): a lane needs only the key before its
+// are not needed, exact modulo 2^32): a lane needs only the keys beside its
 // own, no search for where a run ends, and a run inside one lane is one add.
-// Sorted keys cost two adds a run, random ones five adds for four keys.
 // Hashed slots: a key per lane, as in the general S pass.
 constexpr int DT = 512;
 __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__ keys, uint32_t n, DegTable t,
@@ -531,22 +555,23 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
     };
     auto block_dense = [&](const int32_t (&v)[WQ], uint32_t m, uint32_t valid) {
         const int32_t prev = __shfl_up_sync(0xffffffffu, v[WQ - 1], 1);
+        const int32_t next = __shfl_down_sync(0xffffffffu, v[0], 1);
         if (m == 0) return;
-        int32_t cur = lane ? prev : v[0];
-        uint32_t starts = 0;   // bit q: a run starts at the lane's key q
+        const uint32_t i0 = lane * WQ;
+        uint32_t starts = 0;   // bit q: a run starts at the lane's key q > 0
 #pragma unroll
-        for (int q = 0; q < WQ; ++q)
-            starts |= (uint32_t)((uint32_t)q < m && v[q] != (q ? v[q - 1] : cur)) << q;
-        uint32_t x = 0;   // minus the position where cur's run starts, when it starts in this lane
+        for (int q = 1; q < WQ; ++q) starts |= (uint32_t)((uint32_t)q < m && v[q] != v[q - 1]) << q;
+        int32_t cur = v[0];
+        // minus the position where cur's run starts, when it starts in this lane
+        uint32_t x = lane == 0 || v[0] != prev ? 0u - i0 : 0u;
         while (starts) {
             const uint32_t q = (uint32_t)__ffs((int)starts) - 1u;
             starts &= starts - 1u;
-            const uint32_t i = lane * WQ + q;
-            add(cur, x + i);
-            cur = q < 2u ? (q ? v[1] : v[0]) : (q == 2u ? v[2] : v[3]);
-            x = 0u - i;
+            add(cur, x + i0 + q);
+            cur = q == 1u ? v[1] : (q == 2u ? v[2] : v[3]);
+            x = 0u - (i0 + q);
         }
-        if (lane * WQ + m == valid) x += valid;   // the block ends here
+        if (i0 + m == valid || cur != next) x += i0 + m;   // the run ends with this lane
         if (x) add(cur, x);
     };
     const uint32_t rounds = (blocks + G - 1) / G;
@@ -602,17 +627,23 @@ cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, in
     return cudaGetLastError();
 }
 
-cudaError_t w_table_build(const mwj_rel &S, const Source &src, bool weights, const WTable &w, DevStatus *status,
+enum Pass { PASS_DEGREES, PASS_WEIGHTS, PASS_STAR };   // what a weight pass looks up, or a star's S pass
+
+cudaError_t w_table_build(const mwj_rel &S, const Source &src, Pass pass, const WTable &w, DevStatus *status,
                           int num_sms, cudaStream_t st) {
     if (S.n <= 0) return cudaSuccess;
     const uint32_t n = (uint32_t)S.n;
-    auto direct = weights ? k_w_build_direct<true> : k_w_build_direct<false>;
-    auto hashed = weights ? k_w_build<true> : k_w_build<false>;
+    auto direct = pass == PASS_STAR      ? k_w_build_direct<false, true>
+                  : pass == PASS_WEIGHTS ? k_w_build_direct<true, false>
+                                         : k_w_build_direct<false, false>;
+    auto hashed = pass == PASS_STAR      ? k_w_build<false, true>
+                  : pass == PASS_WEIGHTS ? k_w_build<true, false>
+                                         : k_w_build<false, false>;
     {
-        ProfScope ps_("w_build", st);
+        ProfScope ps_(pass == PASS_STAR ? "star_probe" : "w_build", st);
         direct<<<pass_grid(direct, n, num_sms), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     }
-    ProfScope ps_("w_build_hashed", st);
+    ProfScope ps_(pass == PASS_STAR ? "star_probe_hashed" : "w_build_hashed", st);
     hashed<<<pass_grid(hashed, n, num_sms, 32), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     return cudaGetLastError();
 }
@@ -691,10 +722,42 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     Source src{};
     src.t = L.deg;
     for (int k = 0; k < nrel - 2; ++k) {
-        if ((e = w_table_build(rel[nrel - 2 - k], src, k > 0, L.w[k], status, num_sms, st)) != cudaSuccess) return e;
+        if ((e = w_table_build(rel[nrel - 2 - k], src, k > 0 ? PASS_WEIGHTS : PASS_DEGREES, L.w[k], status, num_sms, st)) != cudaSuccess) return e;
         src.w = L.w[k];
     }
     return w_table_probe(rel[0], L.w[nrel - 3], mode, a_domain, cnt, total, status, num_sms, st);
+}
+
+void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &T, int num_sms, OneBucket &L) {
+    const mwj_rel rel[3] = {R, R, T};   // the weights are R's, not S's
+    one_bucket_layout(A, rel, 3, num_sms, L);
+}
+
+cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd, int mode,
+                            int32_t a_domain, unsigned long long *cnt, unsigned long long *total, DevStatus *status,
+                            int num_sms, cudaStream_t st) {
+    cudaError_t e;
+    L.deg.seed = sd.slot2;
+    L.w[0].seed = sd.slot;
+    const uint64_t tr = single_table_slots(T.n), rr = w_table_slots(R.n);
+    const SizeCol cols[2] = {SizeCol{T.x, (uint32_t)T.n, sd.slot2, L.hll[0], {L.deg.meta}, {tr}, {tr}, 1u},
+                             SizeCol{R.y, (uint32_t)R.n, sd.slot, L.hll[1], {L.w[0].meta}, {rr}, {rr}, 1u}};
+    const HeavyCol heavy{S.x, (uint32_t)S.n, kWHeavyBuckets, (uint32_t *)L.w[0].heavy};
+    const ClearTable clear[2] = {ClearTable{L.deg.slots, nullptr, L.deg.meta},
+                                 ClearTable{L.w[0].W, L.w[0].keys, L.w[0].meta}};
+    if ((e = size_columns(cols, 2, &heavy, 1, true, num_sms, st)) != cudaSuccess) return e;
+    if ((e = tables_clear(clear, 2, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull, total, num_sms,
+                          st)) != cudaSuccess)
+        return e;
+    if ((e = deg_build(T, L.deg, status, num_sms, st)) != cudaSuccess) return e;
+    if (R.n > 0) {
+        ProfScope ps_("star_keys", st);
+        k_w_keys<<<pass_grid(k_w_keys, (uint32_t)R.n, num_sms, 32), WT, 0, st>>>(R.y, (uint32_t)R.n, L.w[0], status);
+    }
+    Source src{};
+    src.t = L.deg;
+    if ((e = w_table_build(S, src, PASS_STAR, L.w[0], status, num_sms, st)) != cudaSuccess) return e;
+    return w_table_probe(R, L.w[0], mode, a_domain, cnt, total, status, num_sms, st);
 }
 
 }  // namespace mwj

@@ -6,22 +6,26 @@
 // The paper maps each (h(b), g(c)) pair of hash values to one memory unit,
 // loads R and T into the units first and then routes every S tuple to the
 // unit of its pair.  On this GPU the on-chip memory that every SM can reach
-// is the L2 (with the L1 in front of it).  For the two aggregates R and T
-// each become one table of their keys' degrees (b -> deg_R(b), c ->
-// deg_T(c)), sized from a HyperLogLog estimate of the distinct keys and
-// filled without partitioning; for row output R is grouped by h(B) and T by
-// g(C) into bucket tables that also hold the lists b -> [a] and c -> [d].
-// Either way the tables stay resident in the L2, and every CTA streams its
-// own contiguous stretch of S straight from the input columns, looking each
-// tuple up in both tables:
+// is the L2 (with the L1 in front of it).  The two aggregates are passes of
+// the one-bucket plan (linear_l2.cu, star_bucket_run): T's degrees, then
 //
-//   COUNT(*)             total += deg_R(b) * deg_T(c)            per S tuple
-//   COUNT(*) GROUP BY A  w[b] += deg_T(c)  per S tuple, then
-//                        cnt[a] += w[b]    per (a, b) of R       (flush)
-//   rows                 (a,b,c,d) for a in R[b], d in T[c]      (two passes)
+//   w[b] += deg_T(c)                    per S tuple whose b is R's
+//   cnt[a] += w[b], total += w[b]       per (a, b) of R
 //
-// S is never partitioned and never re-read (twice in total for rows).
+// with both tables direct-address arrays when the dimension keys are compact.
+// Row output groups R by h(B) and T by g(C) into bucket tables that also hold
+// the lists b -> [a] and c -> [d]; every CTA streams its own contiguous
+// stretch of S straight from the input columns, looking each tuple up in both:
+// (a,b,c,d) for a in R[b], d in T[c], in two passes.
+//
+// S is never partitioned; it is read once (twice for rows).
+//
+// 2^26 fact tuples sorted by B, dimensions of 2^20 unique keys, GROUP BY A: the
+// aggregates as two hashed lookups per tuple (8-byte slots, 32 MB a table) took
+// 0.56 ms, 0.455 of it that pass; 0.34 ms now, 0.275 of it the S pass, at one
+// L1 tag per tuple (0.96 -> 0.64 ms with S in random order).
 #include "api_internal.h"
+#include "linear_l2.h"
 #include "tables.h"
 
 namespace mwj {
@@ -85,50 +89,6 @@ __device__ __forceinline__ void img_find_batch(const TImg &t, const int32_t (&k)
     }
 }
 
-// Lookups of a batch in the two single tables (packed deg << 32 | key,
-// mask + 1 slots, home slot slot_of): R's slot (-1 when absent) and degree of
-// every b, T's degree of every c.  All 2 * SB first probes are in flight
-// before any is resolved.
-struct Single {
-    const unsigned long long *tbl;
-    uint32_t mask, seed;
-};
-
-__device__ __forceinline__ uint32_t single_resolve(const Single &t, uint32_t k, uint32_t &s,
-                                                   unsigned long long x) {
-    for (uint32_t it = 0; it < t.mask && x != kEmpty64 && (uint32_t)x != k; ++it) {
-        s = (s + 1) & t.mask;
-        x = __ldg(t.tbl + s);
-    }
-    return (x == kEmpty64 || (uint32_t)x != k) ? 0u : (uint32_t)(x >> 32);
-}
-
-__device__ __forceinline__ void single_find2(const Single &r, const Single &t, const int32_t (&b)[SB],
-                                             const int32_t (&c)[SB], const bool (&use)[SB],
-                                             long long (&rs)[SB], uint32_t (&dR)[SB],
-                                             uint32_t (&dT)[SB]) {
-    uint32_t sr[SB], stt[SB];
-    unsigned long long vr[SB], vt[SB];
-#pragma unroll
-    for (int q = 0; q < SB; ++q) {
-        if (use[q]) {
-            sr[q] = slot_of((uint32_t)b[q], r.seed, r.mask);
-            stt[q] = slot_of((uint32_t)c[q], t.seed, t.mask);
-            vr[q] = __ldg(r.tbl + sr[q]);
-            vt[q] = __ldg(t.tbl + stt[q]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < SB; ++q) {
-        rs[q] = -1;
-        dR[q] = dT[q] = 0;
-        if (!use[q]) continue;
-        dR[q] = single_resolve(r, (uint32_t)b[q], sr[q], vr[q]);
-        if (dR[q]) rs[q] = sr[q];
-        dT[q] = single_resolve(t, (uint32_t)c[q], stt[q], vt[q]);
-    }
-}
-
 // The S tuples [c.begin, c.end) of this CTA in batches of SB per thread
 // (16-byte loads of both columns where aligned); f(b, c, n) per batch.
 template <typename F>
@@ -171,102 +131,30 @@ __device__ __forceinline__ void star_stream(const int32_t *__restrict__ sx, cons
 struct StarArgs {
     const int32_t *sx, *sy;     // S columns (b, c), unpartitioned
     uint32_t nS, chunk;
-    const unsigned long long *tr, *tt;   // aggregates: R's b table, T's c table
-    const uint32_t *metaR, *metaT;       // their masks (meta[0])
-    uint32_t seedR, seedT;
-    TImg r, t;                  // row output: R's b images (payload a), T's c images (payload d)
-    unsigned long long *w;      // GROUP BY A: per slot of R's table
-    unsigned long long *total;
-    unsigned long long *rowcount;   // row output pass 1: per CTA
+    TImg r, t;                  // R's b images (payload a), T's c images (payload d)
+    unsigned long long *rowcount;   // pass 1: per CTA
     DevStatus *st;
 };
 
-// MODE 0: COUNT; 1: GROUP BY A (w per R image slot); 2: per-CTA row counts.
-template <int MODE>
-__global__ void __launch_bounds__(ST, kStarCtasPerSm) k_star_agg(StarArgs g) {
+// Row output, pass 1: the rows of every CTA's stretch of S.
+__global__ void __launch_bounds__(ST, kStarCtasPerSm) k_star_count(StarArgs g) {
     __shared__ unsigned long long red[32];
     const StarChunk c = star_chunk(g.nS, g.chunk);
     const bool vec = (((uintptr_t)g.sx | (uintptr_t)g.sy) & 15) == 0;
     unsigned long long acc = 0;
-    const Single sr{g.tr, MODE == 2 ? 0u : __ldg(g.metaR), g.seedR};
-    const Single stt{g.tt, MODE == 2 ? 0u : __ldg(g.metaT), g.seedT};
     star_stream(g.sx, g.sy, c, vec, [&](const int32_t (&b)[SB], const int32_t (&cc)[SB], uint32_t n) {
         bool use[SB];
 #pragma unroll
         for (int q = 0; q < SB; ++q) use[q] = q < (int)n;
-        long long rs[SB];
+        long long rs[SB], ts[SB];
         uint32_t dR[SB], dT[SB];
-        if (MODE == 2) {
-            long long ts[SB];
-            img_find_batch(g.r, b, use, rs, dR);
-            img_find_batch(g.t, cc, use, ts, dT);
-        } else {
-            single_find2(sr, stt, b, cc, use, rs, dR, dT);
-        }
+        img_find_batch(g.r, b, use, rs, dR);
+        img_find_batch(g.t, cc, use, ts, dT);
 #pragma unroll
         for (int q = 0; q < SB; ++q) acc += (unsigned long long)dR[q] * dT[q];
-        if (MODE == 1) {
-            // w[slot of b] += deg_T(c), runs of equal b merged
-            long long cur = -1;
-            unsigned long long run = 0;
-#pragma unroll
-            for (int q = 0; q < SB; ++q) {
-                if (rs[q] < 0 || !dT[q]) continue;
-                if (rs[q] == cur) {
-                    run += dT[q];
-                } else {
-                    if (cur >= 0) atomicAdd(g.w + cur, run);
-                    cur = rs[q];
-                    run = dT[q];
-                }
-            }
-            if (cur >= 0) atomicAdd(g.w + cur, run);
-        }
     });
     const unsigned long long tot = block_sum_u64(acc, red);
-    if (threadIdx.x == 0) {
-        if (MODE == 2) g.rowcount[blockIdx.x] = tot;
-        else if (tot) atomicAdd(g.total, tot);
-    }
-}
-
-// GROUP BY A flush: cnt[a] += w[slot of b] for every (a, b) of R, read from
-// its input columns; a outside [0, a_domain) is reported and skipped.
-__global__ void __launch_bounds__(ST) k_star_flush(const int32_t *__restrict__ ra,
-                                                   const int32_t *__restrict__ rb, uint32_t nR,
-                                                   const unsigned long long *__restrict__ tr,
-                                                   const uint32_t *__restrict__ metaR, uint32_t seedR,
-                                                   const unsigned long long *__restrict__ w,
-                                                   int32_t a_domain, unsigned long long *__restrict__ cnt,
-                                                   DevStatus *st) {
-    const Single r{tr, __ldg(metaR), seedR};
-    for (uint32_t i0 = (blockIdx.x * ST + threadIdx.x) * SB; i0 < nR; i0 += gridDim.x * ST * SB) {
-        int32_t b[SB], a[SB];
-        bool use[SB];
-        uint32_t s[SB];
-        unsigned long long v[SB];
-#pragma unroll
-        for (int q = 0; q < SB; ++q) {
-            use[q] = i0 + q < nR;
-            a[q] = use[q] ? __ldg(ra + i0 + q) : 0;
-            b[q] = use[q] ? __ldg(rb + i0 + q) : 0;
-            if (use[q]) {
-                s[q] = slot_of((uint32_t)b[q], r.seed, r.mask);
-                v[q] = __ldg(r.tbl + s[q]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < SB; ++q) {
-            if (!use[q]) continue;
-            if ((uint32_t)a[q] >= (uint32_t)a_domain) {
-                set_status(st, MWJ_ERR_DOMAIN, a[q]);
-                continue;
-            }
-            if (!single_resolve(r, (uint32_t)b[q], s[q], v[q])) continue;   // cannot happen: b is in R
-            const unsigned long long x = __ldg(w + s[q]);
-            if (x) atomicAdd(cnt + a[q], x);
-        }
-    }
+    if (threadIdx.x == 0) g.rowcount[blockIdx.x] = tot;
 }
 
 // Row output, pass 2: the same chunks as pass 1; lane l of a warp takes one S
@@ -328,16 +216,13 @@ struct StarPlan {
 };
 
 struct StarLayout {
-    uint64_t *tblR, *tblT;          // aggregates: single tables
-    uint32_t *metaR, *metaT;
-    unsigned int *hll, *hllT;       // separate scratch: the two tables are built concurrently
+    OneBucket one;                  // aggregates
     uint2 *Rp, *Tp;
     uint32_t *offR, *offT;
     uint64_t *imgR, *imgT;
     uint32_t *capR, *capT;
     uint32_t *startR, *startT;
     int32_t *alist, *dlist;
-    unsigned long long *w;
     unsigned long long *rowcount, *base;
     void *sscratch;
     void *pscratch;
@@ -377,27 +262,11 @@ mwj_status star_plan(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, const mwj
 
 size_t star_layout(Arena &A, const StarPlan &p, const mwj_rel &R, const mwj_rel &T, int num_sms,
                    StarLayout &L) {
+    L = StarLayout{};
     if (!p.rows) {
-        L.tblR = A.take<uint64_t>(single_table_slots(R.n));
-        L.metaR = A.take<uint32_t>(4);
-        L.tblT = A.take<uint64_t>(single_table_slots(T.n));
-        L.metaT = A.take<uint32_t>(4);
-        L.hll = A.take<unsigned int>(hll_scratch_registers(num_sms));
-        L.hllT = A.take<unsigned int>(hll_scratch_registers(num_sms));
-        L.w = p.group ? A.take<unsigned long long>(single_table_slots(R.n)) : nullptr;
-        L.Rp = L.Tp = nullptr;
-        L.offR = L.offT = L.capR = L.capT = L.startR = L.startT = nullptr;
-        L.imgR = L.imgT = nullptr;
-        L.alist = L.dlist = nullptr;
-        L.rowcount = L.base = nullptr;
-        L.sscratch = L.pscratch = nullptr;
-        L.pscratch_bytes = 0;
+        star_bucket_layout(A, R, T, num_sms, L.one);
         return A.used;
     }
-    L.tblR = L.tblT = nullptr;
-    L.metaR = L.metaT = nullptr;
-    L.hll = L.hllT = nullptr;
-    L.w = nullptr;
     L.Rp = A.take<uint2>(R.n + 2);
     L.offR = A.take<uint32_t>(p.JR + 1);
     L.Tp = A.take<uint2>(T.n + 2);
@@ -465,124 +334,61 @@ extern "C" mwj_status mwj_join3_star(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel
     const Seeds &sd = ctx->seeds;
     const int sms = ctx->dev.num_sms;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(out->total, 0, sizeof(int64_t), st)) != cudaSuccess)
-        return cuda_fail(ctx, e, "memset total");
-    if (p.group &&
-        (e = cudaMemsetAsync(out->group_counts, 0, sizeof(int64_t) * (size_t)out->a_domain, st)) !=
-            cudaSuccess)
-        return cuda_fail(ctx, e, "memset group_counts");
-    // the caller's stream waits for the side stream on every return after
-    // the fork, so no work of this call outlives it
-    struct JoinGuard {
-        cudaStream_t st;
-        cudaEvent_t ev;
-        bool armed;
-        ~JoinGuard() {
-            if (armed) cudaStreamWaitEvent(st, ev, 0);
-        }
-    } join_guard{st, ctx->join, false};
     if (!p.rows) {
-        // the aggregates: one degree table per dimension relation, T's on the
-        // side stream while R's is built here
-        // (with per-kernel profiling on, on the caller's stream: see the linear join)
-        cudaStream_t side = ctx->prof.on ? st : ctx->side;
-        if ((e = cudaEventRecord(ctx->fork, st)) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(side, ctx->fork, 0)) != cudaSuccess)
-            return cuda_fail(ctx, e, "fork");
-        e = single_table_direct(T.x, T.n, sd.slot2, L.hllT, L.metaT, L.tblT, single_table_slots(T.n),
-                                ctx->status, sms, side);
-        const cudaError_t ej = cudaEventRecord(ctx->join, side);
-        if (ej != cudaSuccess) return cuda_fail(ctx, ej, "join");
-        join_guard.armed = true;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "T table");
-        if ((e = single_table_direct(R.y, R.n, sd.slot, L.hll, L.metaR, L.tblR, single_table_slots(R.n),
-                                     ctx->status, sms, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "R table");
-        if ((e = cudaStreamWaitEvent(st, ctx->join, 0)) != cudaSuccess) return cuda_fail(ctx, e, "join");
-        join_guard.armed = false;
-        if (p.group &&
-            (e = cudaMemsetAsync(L.w, 0, sizeof(unsigned long long) * single_table_slots(R.n), st)) !=
-                cudaSuccess)
-            return cuda_fail(ctx, e, "memset w");
-    } else {
-        // row output: R as (b, a) pairs by h(B), T as (c, d) pairs by g(C),
-        // each bucket a table of its keys' degrees and lists
-        PartSpec pr{0, sd.B, p.JR, -1, 0, 1};
-        pr.st = ctx->status;
-        if ((e = part_run(R.y, R.x, R.n, pr, PAY_PAIR, L.Rp, L.offR, L.pscratch, L.pscratch_bytes, sms,
-                          st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "partition R");
-        PartSpec pt{0, sd.C, p.JT, -1, 0, 1};
-        pt.st = ctx->status;
-        if ((e = part_run(T.x, T.y, T.n, pt, PAY_PAIR, L.Tp, L.offT, L.pscratch, L.pscratch_bytes, sms,
-                          st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "partition T");
-        if ((e = tables_build(nullptr, L.Rp, L.offR, p.JR, sd.slot, L.imgR, L.capR, L.startR, L.alist,
-                              ctx->status, sms, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "R tables");
-        if ((e = tables_build(nullptr, L.Tp, L.offT, p.JT, sd.slot2, L.imgT, L.capT, L.startT, L.dlist,
-                              ctx->status, sms, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "T tables");
+        e = star_bucket_run(L.one, R, S, T, sd, p.group ? 1 : 0, out->a_domain, (unsigned long long *)out->group_counts,
+                            (unsigned long long *)out->total, ctx->status, sms, st);
+        return e == cudaSuccess ? MWJ_OK : cuda_fail(ctx, e, "star aggregates");
     }
+    // row output: R as (b, a) pairs by h(B), T as (c, d) pairs by g(C),
+    // each bucket a table of its keys' degrees and lists
+    PartSpec pr{0, sd.B, p.JR, -1, 0, 1};
+    pr.st = ctx->status;
+    if ((e = part_run(R.y, R.x, R.n, pr, PAY_PAIR, L.Rp, L.offR, L.pscratch, L.pscratch_bytes, sms,
+                      st)) != cudaSuccess)
+        return cuda_fail(ctx, e, "partition R");
+    PartSpec pt{0, sd.C, p.JT, -1, 0, 1};
+    pt.st = ctx->status;
+    if ((e = part_run(T.x, T.y, T.n, pt, PAY_PAIR, L.Tp, L.offT, L.pscratch, L.pscratch_bytes, sms,
+                      st)) != cudaSuccess)
+        return cuda_fail(ctx, e, "partition T");
+    if ((e = tables_build(nullptr, L.Rp, L.offR, p.JR, sd.slot, L.imgR, L.capR, L.startR, L.alist,
+                          ctx->status, sms, st)) != cudaSuccess)
+        return cuda_fail(ctx, e, "R tables");
+    if ((e = tables_build(nullptr, L.Tp, L.offT, p.JT, sd.slot2, L.imgT, L.capT, L.startT, L.dlist,
+                          ctx->status, sms, st)) != cudaSuccess)
+        return cuda_fail(ctx, e, "T tables");
 
     StarArgs g{};
     g.sx = S.x;
     g.sy = S.y;
     g.nS = (uint32_t)S.n;
     g.chunk = p.chunk;
-    g.tr = (const unsigned long long *)L.tblR;
-    g.tt = (const unsigned long long *)L.tblT;
-    g.metaR = L.metaR;
-    g.metaT = L.metaT;
-    g.seedR = sd.slot;
-    g.seedT = sd.slot2;
     g.r = TImg{L.imgR, L.offR, L.capR, L.startR, L.alist, nullptr, p.JR, sd.B, sd.slot};
     g.t = TImg{L.imgT, L.offT, L.capT, L.startT, L.dlist, nullptr, p.JT, sd.C, sd.slot2};
-    g.w = L.w;
-    g.total = (unsigned long long *)out->total;
     g.rowcount = L.rowcount;
     g.st = ctx->status;
     if (S.n > 0) {
-        if (p.rows) {
-            ProfScope ps_("star_rowcount", st);
-            k_star_agg<2><<<p.G, ST, 0, st>>>(g);
-        } else if (p.group) {
-            ProfScope ps_("star_probe_groupby", st);
-            k_star_agg<1><<<p.G, ST, 0, st>>>(g);
-        } else {
-            ProfScope ps_("star_probe_count", st);
-            k_star_agg<0><<<p.G, ST, 0, st>>>(g);
-        }
+        ProfScope ps_("star_rowcount", st);
+        k_star_count<<<p.G, ST, 0, st>>>(g);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "star probe");
     }
-    if (p.group && R.n > 0) {
-        const uint64_t want = ((uint64_t)R.n + (uint64_t)ST * SB - 1) / ((uint64_t)ST * SB);
-        const unsigned grid = (unsigned)(want < (uint64_t)sms * 4 ? want : (uint64_t)sms * 4);
-        ProfScope ps_("star_flush", st);
-        k_star_flush<<<grid, ST, 0, st>>>(R.x, R.y, (uint32_t)R.n, g.tr, L.metaR, sd.slot, L.w,
-                                           out->a_domain, (unsigned long long *)out->group_counts,
+    if (S.n == 0 && (e = cudaMemsetAsync(L.rowcount, 0, sizeof(unsigned long long) * p.G, st)) != cudaSuccess)
+        return cuda_fail(ctx, e, "memset row counts");
+    e = scan_excl_u64((const uint64_t *)L.rowcount, (uint64_t *)L.base, p.G, true, L.sscratch, st);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "row scan");
+    {
+        ProfScope ps_("rows_check", st);
+        k_star_rows_check<<<1, 1, 0, st>>>(L.base, p.G, out->capacity, (long long *)out->n_rows,
                                            ctx->status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "star flush");
     }
-    if (p.rows) {
-        if (S.n == 0 && (e = cudaMemsetAsync(L.rowcount, 0, sizeof(unsigned long long) * p.G, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "memset row counts");
-        e = scan_excl_u64((const uint64_t *)L.rowcount, (uint64_t *)L.base, p.G, true, L.sscratch, st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "row scan");
-        {
-            ProfScope ps_("rows_check", st);
-            k_star_rows_check<<<1, 1, 0, st>>>(L.base, p.G, out->capacity, (long long *)out->n_rows,
-                                               ctx->status);
-        }
-        if (S.n > 0) {
-            ProfScope ps_("star_rows", st);
-            k_star_rows<<<p.G, ST, 0, st>>>(g, L.base, (int4 *)out->rows, out->capacity);
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "star rows");
-        // total = number of rows
-        if ((e = cudaMemcpyAsync(out->total, L.base + p.G, sizeof(int64_t), cudaMemcpyDeviceToDevice, st)) !=
-            cudaSuccess)
-            return cuda_fail(ctx, e, "total");
+    if (S.n > 0) {
+        ProfScope ps_("star_rows", st);
+        k_star_rows<<<p.G, ST, 0, st>>>(g, L.base, (int4 *)out->rows, out->capacity);
     }
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "star rows");
+    // total = number of rows
+    if ((e = cudaMemcpyAsync(out->total, L.base + p.G, sizeof(int64_t), cudaMemcpyDeviceToDevice, st)) !=
+        cudaSuccess)
+        return cuda_fail(ctx, e, "total");
     return MWJ_OK;
 }

@@ -105,3 +105,23 @@ def test_heavy_keys_and_wide_weights(ctx, layout):
     U = (f(np.zeros(5000, np.int64)).astype(np.int32), np.zeros(5000, np.int32))
     want = oracle.linear4(R, S, T, U, oracle.GROUP_BY_A, a_domain=20)
     same(ctx.join4_linear(cu(R), cu(S), cu(T), cu(U), "group_by_a", a_domain=20), want)
+
+
+@pytest.mark.parametrize("lr", list(LAYOUTS))
+@pytest.mark.parametrize("lt", list(LAYOUTS))
+@pytest.mark.parametrize("n", [1, 130, 30001])
+def test_star_keeps_only_r_keys(ctx, lr, lt, n):
+    """Star joins lay the weights out for R's keys: S tuples inside and outside
+    R's range, heavy ones among them, in every layout of both dimensions."""
+    g = np.random.default_rng(n)
+    fr, ft = LAYOUTS[lr], LAYOUTS[lt]
+    dim = max(1, n // 30)
+    R = (g.integers(0, 25, dim).astype(np.int32), fr(np.arange(dim) * 2).astype(np.int32))
+    T = (ft(g.integers(0, 2 * dim, 2 * dim)).astype(np.int32), g.integers(0, 9, 2 * dim).astype(np.int32))
+    b = np.where(g.random(n) < 0.4, 4 * dim, g.integers(0, 5 * dim, n))
+    S = (fr(np.sort(b) if n % 2 else b).astype(np.int32), ft(g.integers(0, 3 * dim, n)).astype(np.int32))
+    want = oracle.linear(R, S, T, oracle.GROUP_BY_A, a_domain=25)
+    for take in (cu, unaligned):
+        d = [take(x) for x in (R, S, T)]
+        same(ctx.join3_star(*d, "group_by_a", a_domain=25), want)
+        same(ctx.join3_star(*d, "count"), want)
