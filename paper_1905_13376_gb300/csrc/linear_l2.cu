@@ -505,9 +505,22 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
 // are not needed, exact modulo 2^32): a lane needs only the keys beside its
 // own, no search for where a run ends, and a run inside one lane is one add.
 // Hashed slots: a key per lane, as in the general S pass.
+// The first nheavy CTAs sample the heavy keys of the weight passes instead (the
+// medium plan, which has no range pass to do it in).
 constexpr int DT = 512;
+struct HeavyArgs {
+    HeavyCol h[kChainMax - 2];
+    uint32_t n;
+};
 __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__ keys, uint32_t n, DegTable t,
-                                                     DevStatus *st) {
+                                                     HeavyArgs heavy, DevStatus *st) {
+    __shared__ HeavySample<1024> hsm;
+    if (blockIdx.x < heavy.n) {
+        const HeavyCol &h = heavy.h[blockIdx.x];
+        heavy_sample_cta<DT, 1024>(h.keys, h.n, h.buckets, h.heavy, hsm);
+        return;
+    }
+    const uint32_t cta = blockIdx.x - heavy.n, ctas = gridDim.x - heavy.n;
     const uint32_t mask = t.meta[kMetaMask];
     const bool dense = t.meta[kMetaDense] != 0u;
     const uint32_t kmin = dense ? t.meta[kMetaMin] : 0u, span = dense ? t.meta[kMetaSpan] : 0u;
@@ -516,7 +529,7 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
     const uint64_t pol = l2_evict_first();
     constexpr int G = 2;   // blocks per warp round
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warp = (blockIdx.x * DT + threadIdx.x) >> 5, warps = (gridDim.x * DT) >> 5;
+    const uint32_t warp = (cta * DT + threadIdx.x) >> 5, warps = (ctas * DT) >> 5;
     const uint32_t blocks = (n + WCHUNK - 1) / WCHUNK;
     auto load = [&](uint32_t blk, int32_t (&v)[WQ]) -> uint32_t {
         const uint32_t i = blk * WCHUNK + lane * WQ;
@@ -533,8 +546,8 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
         return m;
     };
     if (!dense) {
-        const uint32_t T = gridDim.x * DT;
-        uint64_t i = (uint64_t)blockIdx.x * DT + threadIdx.x;
+        const uint32_t T = ctas * DT;
+        uint64_t i = (uint64_t)cta * DT + threadIdx.x;
         int32_t k = i < n ? __ldg(keys + i) : 0;
         for (; i - lane < n; i += T) {
             const int32_t nk = i + T < n ? __ldg(keys + i + T) : 0;
@@ -601,16 +614,291 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
     }
 }
 
-// CTAs of a grid-stride pass: every SM filled, no more warps than rounds.
-template <typename K>
-uint32_t pass_grid(K kernel, uint32_t n, int num_sms, uint32_t per_warp = WCHUNK) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, WT, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
+// ---------------------------------------------------------------------------
+// small chains
+// ---------------------------------------------------------------------------
+//
+// A call on a few thousand tuples spends its time between kernels: nine
+// launches of 2 to 4 us each, most of them sizing and choosing layouts.  Two
+// ways around that, both on hashed tables of two slots per tuple, which need
+// neither:
+//
+//  * up to kSmallMax tuples per relation the whole call is one launch: one
+//    thread-block cluster does the passes in turn, with the cluster's hardware
+//    barrier between them (no flags in memory, no co-residency to ask for
+//    beyond the cluster itself).  A cluster is at most 16 SMs.
+//  * up to kMediumMax: four launches, one that empties the tables and says how
+//    large they are, then the general passes on the whole GPU.
+//
+// Device time of a call with uniform keys, GROUP BY A (2^20 groups), and in
+// brackets of calls queued back to back by the binding, us:
+//
+//   tuples per relation   nine launches   four launches   one cluster
+//   2^10                  28 (53)         12 (36)         20 (27)
+//   2^14                  30 (51)         14 (36)         22 (27)
+//   2^16                  30 (53)         16 (37)         40 (42)
+//   2^18                  35 (57)         22 (37)         102 (106)
+//   2^19                  42 (64)         32 (42)
+//   2^20                  55 (77)         56 (66)
+//
+// (id keys, nine against four launches: 66 against 37 at 2^18, 109 against 75 at
+// 2^20; Zipf 1.5: 36 against 29, 48 against 53.)
+constexpr int CT = 1024;              // threads per CTA
+constexpr int kSmallCtas = 16;        // CTAs of the largest cluster
+constexpr int64_t kSmallMax = 1 << 14;      // tuples per relation
+constexpr int64_t kMediumMax = 1 << 19;
+constexpr int64_t kMediumHeavy = 1 << 16;   // relations above it have their heavy keys sampled
+constexpr int64_t kSmallGroups = 1 << 21;   // groups zeroed by the cluster
+
+struct SmallArgs {
+    mwj_rel rel[kChainMax];
+    int nrel, mode;
+    DegTable deg;
+    WTable w[kChainMax - 2];
+    uint32_t dmask, wmask[kChainMax - 2];
+    int32_t a_domain;
+    unsigned long long *cnt, *total;
+    DevStatus *st;
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Tables written in this kernel are read through the L2 (ld.cg).
+__device__ __forceinline__ unsigned long long small_deg(const DegTable &t, uint32_t mask, uint32_t c, uint32_t s,
+                                                        ulonglong2 v) {
+    for (uint32_t it = 0; it <= mask; it += 2) {
+        if ((uint32_t)v.x == c && v.x != kEmpty64) return v.x >> 32;
+        if ((uint32_t)v.y == c && v.y != kEmpty64) return v.y >> 32;
+        if (v.x == kEmpty64 || v.y == kEmpty64) break;
+        s = (s + 2) & mask;
+        v = __ldcg((const ulonglong2 *)(t.slots + s));
+    }
+    return 0ull;
+}
+
+__device__ __forceinline__ unsigned long long small_w(const WTable &w, uint32_t mask, uint32_t k, uint32_t s, uint4 v) {
+    if (k == kEmptyKey) return __ldcg(w.W + mask + 1);
+    for (uint32_t it = 0; it <= mask; it += 4) {
+        const uint32_t at = v.x == k ? 0u : v.y == k ? 1u : v.z == k ? 2u : v.w == k ? 3u : 4u;
+        if (at < 4u) return __ldcg(w.W + s + at);
+        if (v.w == kEmptyKey) break;
+        s = (s + 4) & mask;
+        v = __ldcg((const uint4 *)(w.keys + s));
+    }
+    return 0ull;
+}
+
+// Empty tables and zero outputs (thread t of T).
+__device__ __forceinline__ void small_clear(const SmallArgs &g, uint32_t t, uint32_t T) {
+    for (uint32_t s = t; s <= g.dmask / 2; s += T) ((ulonglong2 *)g.deg.slots)[s] = make_ulonglong2(kEmpty64, kEmpty64);
+    for (int k = 0; k < g.nrel - 2; ++k) {
+        const uint32_t m = g.wmask[k];
+        for (uint32_t s = t; s <= m / 4; s += T)
+            ((uint4 *)g.w[k].keys)[s] = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
+        for (uint32_t s = t; s <= m / 2; s += T) ((ulonglong2 *)g.w[k].W)[s] = make_ulonglong2(0ull, 0ull);
+        if (t == 0) g.w[k].W[m + 1] = 0ull;
+    }
+    if (g.mode == 1)
+        for (uint32_t a = t; a < (uint32_t)g.a_domain; a += T) g.cnt[a] = 0ull;
+    if (t == 0) *g.total = 0ull;
+}
+
+__global__ void __launch_bounds__(WT) k_chain_clear(SmallArgs g) {
+    const uint32_t t = blockIdx.x * WT + threadIdx.x;
+    small_clear(g, t, gridDim.x * WT);
+    if (t == 0) {
+        g.deg.meta[kMetaMask] = g.dmask;
+        g.deg.meta[kMetaDense] = 0u;
+        for (int k = 0; k < g.nrel - 2; ++k) {
+            g.w[k].meta[kMetaMask] = g.wmask[k];
+            g.w[k].meta[kMetaDense] = 0u;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(CT) k_chain_small(SmallArgs g) {
+    constexpr int U = 4;   // tuples per thread in flight
+    __shared__ unsigned long long red[32];
+    const uint32_t T = gridDim.x * CT, t = blockIdx.x * CT + threadIdx.x, lane = threadIdx.x & 31;
+    small_clear(g, t, T);
+    cluster_barrier();
+    {   // degrees of the last relation
+        const mwj_rel r = g.rel[g.nrel - 1];
+        const uint32_t n = (uint32_t)r.n, mask = g.dmask;
+        for (uint32_t i = t; i - lane < n; i += U * T) {
+            int32_t k[U];
+            uint32_t s[U], len[U];
+            ulonglong2 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) k[u] = i + u * T < n ? __ldg(r.x + i + u * T) : 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                s[u] = deg_home((uint32_t)k[u], g.deg.seed, mask);
+                if (i + u * T < n) v[u] = __ldcg((const ulonglong2 *)(g.deg.slots + s[u]));
+                len[u] = (uint32_t)warp_run_sum1(k[u], 1ull, i + u * T < n);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (len[u]) deg_add(g.deg.slots, mask, (uint32_t)k[u], s[u], v[u], len[u], g.st);
+        }
+    }
+    cluster_barrier();
+    for (int p = 0; p < g.nrel - 2; ++p) {   // weights, from the bottom up
+        const mwj_rel r = g.rel[g.nrel - 2 - p];
+        const WTable &w = g.w[p];
+        const uint32_t n = (uint32_t)r.n, mask = g.wmask[p];
+        for (uint32_t i = t; i - lane < n; i += U * T) {
+            int32_t b[U], c[U];
+            uint32_t s[U];
+            uint4 v[U];
+            unsigned long long x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool has = i + u * T < n;
+                b[u] = has ? __ldg(r.x + i + u * T) : 0;
+                c[u] = has ? __ldg(r.y + i + u * T) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                s[u] = w_home((uint32_t)b[u], w.seed, mask);
+                if (i + u * T < n) v[u] = __ldcg((const uint4 *)(w.keys + s[u]));
+            }
+            if (p == 0) {
+                uint32_t ds[U];
+                ulonglong2 dv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    ds[u] = deg_home((uint32_t)c[u], g.deg.seed, g.dmask);
+                    if (i + u * T < n) dv[u] = __ldcg((const ulonglong2 *)(g.deg.slots + ds[u]));
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    x[u] = i + u * T < n ? small_deg(g.deg, g.dmask, (uint32_t)c[u], ds[u], dv[u]) : 0ull;
+            } else {
+                const WTable &src = g.w[p - 1];
+                const uint32_t sm = g.wmask[p - 1];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t q = w_home((uint32_t)c[u], src.seed, sm);
+                    x[u] = i + u * T < n
+                               ? small_w(src, sm, (uint32_t)c[u], q, __ldcg((const uint4 *)(src.keys + q)))
+                               : 0ull;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned long long sum = warp_run_sum1(b[u], x[u], i + u * T < n);
+                if (!sum) continue;
+                const uint32_t k = (uint32_t)b[u];
+                const uint32_t at = k == kEmptyKey ? mask + 1 : w_claim(w.keys, mask, k, s[u], v[u]);
+                if (at != kEmptyKey)
+                    atomicAdd(w.W + at, sum);
+                else
+                    set_status(g.st, MWJ_ERR_CHECK, 7);   // cannot happen: two slots per tuple
+            }
+        }
+        cluster_barrier();
+    }
+    // R
+    const mwj_rel r = g.rel[0];
+    const WTable &w = g.w[g.nrel - 3];
+    const uint32_t n = (uint32_t)r.n, mask = g.wmask[g.nrel - 3];
+    unsigned long long acc = 0;
+    for (uint32_t i = t; i - lane < n; i += U * T) {
+        int32_t a[U], b[U];
+        uint32_t s[U];
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool has = i + u * T < n;
+            a[u] = has && g.mode == 1 ? __ldg(r.x + i + u * T) : 0;
+            b[u] = has ? __ldg(r.y + i + u * T) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            s[u] = w_home((uint32_t)b[u], w.seed, mask);
+            if (i + u * T < n) v[u] = __ldcg((const uint4 *)(w.keys + s[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool has = i + u * T < n;
+            const unsigned long long x = has ? small_w(w, mask, (uint32_t)b[u], s[u], v[u]) : 0ull;
+            acc += x;
+            if (g.mode == 1) {
+                const unsigned long long sum = warp_run_sum1(a[u], x, has);
+                if (has && (uint32_t)a[u] >= (uint32_t)g.a_domain)
+                    set_status(g.st, MWJ_ERR_DOMAIN, a[u]);
+                else if (sum)
+                    atomicAdd(g.cnt + a[u], sum);
+            }
+        }
+    }
+    acc = block_sum_u64(acc, red);
+    if (threadIdx.x == 0 && acc) atomicAdd(g.total, acc);
+}
+
+bool chain_within(const mwj_rel *rel, int nrel, int64_t most) {
+    for (int k = 0; k < nrel; ++k)
+        if (rel[k].n > most) return false;
+    return true;
+}
+bool chain_is_small(const mwj_rel *rel, int nrel, int mode, int32_t a_domain) {
+    return chain_within(rel, nrel, kSmallMax) && (mode != 1 || a_domain <= kSmallGroups);
+}
+
+// Tables as one_bucket_layout laid them out (at least two slots per tuple).
+SmallArgs small_args(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32_t a_domain,
+                     unsigned long long *cnt, unsigned long long *total, DevStatus *status) {
+    SmallArgs g{};
+    for (int k = 0; k < nrel; ++k) g.rel[k] = rel[k];
+    g.nrel = nrel;
+    g.mode = mode;
+    g.deg = L.deg;
+    g.dmask = (uint32_t)single_table_slots(rel[nrel - 1].n) - 1u;
+    for (int k = 0; k < nrel - 2; ++k) {
+        g.w[k] = L.w[k];
+        g.wmask[k] = (uint32_t)w_table_slots(rel[nrel - 2 - k].n) - 1u;
+    }
+    g.a_domain = a_domain;
+    g.cnt = cnt;
+    g.total = total;
+    g.st = status;
+    return g;
+}
+
+cudaError_t chain_small(const SmallArgs &g, cudaStream_t st) {
+    int64_t most = 1;
+    for (int k = 0; k < g.nrel; ++k) most = g.rel[k].n > most ? g.rel[k].n : most;
+    // a CTA per 1024 tuples (and per 16K groups to zero), a power of two up to a cluster's 16
+    const int64_t want = (most + CT - 1) / CT, wantg = g.mode == 1 ? ((int64_t)g.a_domain + 16383) / 16384 : 1;
+    int ctas = 1;
+    while (ctas < kSmallCtas && (ctas < want || ctas < wantg)) ctas <<= 1;
+    cudaError_t e = cudaFuncSetAttribute(k_chain_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(ctas);
+    c.blockDim = dim3(CT);
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    ProfScope ps_("chain_small", st);
+    return cudaLaunchKernelEx(&c, k_chain_small, g);
+}
+
+// CTAs of a grid-stride pass: per_sm of them on every SM (what the registers
+// leave room for), no more warps than rounds of per_warp tuples.
+uint32_t pass_grid(uint32_t n, int num_sms, uint32_t per_sm, uint32_t per_warp) {
     const uint64_t want = ((uint64_t)n + per_warp * (WT / 32) - 1) / (per_warp * (WT / 32));
-    const uint64_t full = (uint64_t)num_sms * (uint64_t)per_sm;
+    const uint64_t full = (uint64_t)num_sms * per_sm;
     return (uint32_t)(want < full ? (want ? want : 1) : full);
 }
+constexpr uint32_t kDirectCtas = 5, kProbeCtas = 5, kHashedProbeCtas = 4;
 
 }  // namespace
 
@@ -618,19 +906,22 @@ size_t w_table_slots(int64_t nS) { return single_table_slots(nS); }
 
 namespace {
 
-cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, int num_sms, cudaStream_t st) {
-    if (T.n <= 0) return cudaSuccess;
+cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, int num_sms, cudaStream_t st,
+                      const HeavyArgs &heavy = HeavyArgs{}) {
     const uint32_t n = (uint32_t)T.n;
+    if (n + heavy.n == 0) return cudaSuccess;
     const uint32_t groups = (n + WQ * DT - 1) / (WQ * DT), full = (uint32_t)num_sms * 3;
     ProfScope ps_("t_insert", st);
-    k_deg_build<<<groups < full ? groups : full, DT, 0, st>>>(T.x, n, t, status);
+    k_deg_build<<<heavy.n + (groups < full ? (groups ? groups : 1u) : full), DT, 0, st>>>(T.x, n, t, heavy, status);
     return cudaGetLastError();
 }
 
 enum Pass { PASS_DEGREES, PASS_WEIGHTS, PASS_STAR };   // what a weight pass looks up, or a star's S pass
 
+// hashed_only: the tables are known to be hashed (the other kernel of the pass
+// is not launched)
 cudaError_t w_table_build(const mwj_rel &S, const Source &src, Pass pass, const WTable &w, DevStatus *status,
-                          int num_sms, cudaStream_t st) {
+                          int num_sms, cudaStream_t st, bool hashed_only = false) {
     if (S.n <= 0) return cudaSuccess;
     const uint32_t n = (uint32_t)S.n;
     auto direct = pass == PASS_STAR      ? k_w_build_direct<false, true>
@@ -639,28 +930,67 @@ cudaError_t w_table_build(const mwj_rel &S, const Source &src, Pass pass, const 
     auto hashed = pass == PASS_STAR      ? k_w_build<false, true>
                   : pass == PASS_WEIGHTS ? k_w_build<true, false>
                                          : k_w_build<false, false>;
-    {
+    if (!hashed_only) {
         ProfScope ps_(pass == PASS_STAR ? "star_probe" : "w_build", st);
-        direct<<<pass_grid(direct, n, num_sms), WT, 0, st>>>(S.x, S.y, n, src, w, status);
+        direct<<<pass_grid(n, num_sms, kDirectCtas, WCHUNK), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     }
     ProfScope ps_(pass == PASS_STAR ? "star_probe_hashed" : "w_build_hashed", st);
-    hashed<<<pass_grid(hashed, n, num_sms, 32), WT, 0, st>>>(S.x, S.y, n, src, w, status);
+    hashed<<<pass_grid(n, num_sms, GC, 32), WT, 0, st>>>(S.x, S.y, n, src, w, status);
     return cudaGetLastError();
 }
 
 cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a_domain, unsigned long long *cnt,
-                          unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st) {
+                          unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st,
+                          bool hashed_only = false) {
     if (R.n <= 0) return cudaSuccess;
     const uint32_t n = (uint32_t)R.n;
     auto direct = mode == 1 ? k_w_probe_direct<1> : k_w_probe_direct<0>;
     auto hashed = mode == 1 ? k_w_probe<1> : k_w_probe<0>;
-    {
+    if (!hashed_only) {
         ProfScope ps_(mode == 1 ? "w_probe_groupby" : "w_probe_count", st);
-        direct<<<pass_grid(direct, n, num_sms), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
+        direct<<<pass_grid(n, num_sms, mode == 1 ? kProbeCtas : kProbeCtas + 1, WCHUNK), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
     }
     ProfScope ps_(mode == 1 ? "w_probe_groupby_hashed" : "w_probe_count_hashed", st);
-    hashed<<<pass_grid(hashed, n, num_sms), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
+    hashed<<<pass_grid(n, num_sms, mode == 1 ? kHashedProbeCtas : kHashedProbeCtas + 1, WCHUNK), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+namespace {
+
+// The small plans; false when the call is larger.
+bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32_t a_domain, unsigned long long *cnt,
+               unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st, cudaError_t *e) {
+    if (!chain_within(rel, nrel, kMediumMax)) return false;
+    SmallArgs g = small_args(L, rel, nrel, mode, a_domain, cnt, total, status);
+    if (chain_is_small(rel, nrel, mode, a_domain)) {
+        *e = chain_small(g, st);
+        return true;
+    }
+    {
+        ProfScope ps_("chain_clear", st);
+        k_chain_clear<<<num_sms * 2, WT, 0, st>>>(g);
+    }
+    HeavyArgs heavy{};
+    for (int k = 0; k < nrel - 2; ++k) {
+        const mwj_rel &r = rel[nrel - 2 - k];
+        if (r.n > kMediumHeavy)
+            heavy.h[heavy.n++] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)L.w[k].heavy};
+    }
+    if ((*e = deg_build(rel[nrel - 1], L.deg, status, num_sms, st, heavy)) != cudaSuccess) return true;
+    Source src{};
+    src.t = L.deg;
+    for (int k = 0; k < nrel - 2; ++k) {
+        WTable w = L.w[k];
+        if (rel[nrel - 2 - k].n <= kMediumHeavy) w.heavy = nullptr;
+        if ((*e = w_table_build(rel[nrel - 2 - k], src, k > 0 ? PASS_WEIGHTS : PASS_DEGREES, w, status, num_sms, st,
+                                true)) != cudaSuccess)
+            return true;
+        src.w = w;
+    }
+    *e = w_table_probe(rel[0], L.w[nrel - 3], mode, a_domain, cnt, total, status, num_sms, st, true);
+    return true;
 }
 
 }  // namespace
@@ -714,6 +1044,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
         heavy[k] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)w.heavy};
         clear[k + 1] = ClearTable{w.W, w.keys, w.meta};
     }
+    if (small_run(L, rel, nrel, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
     if ((e = size_columns(cols, ncols, heavy, (uint32_t)nrel - 2u, true, num_sms, st)) != cudaSuccess) return e;
     if ((e = tables_clear(clear, (uint32_t)nrel - 1u, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull,
                           total, num_sms, st)) != cudaSuccess)
@@ -728,8 +1059,9 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     return w_table_probe(rel[0], L.w[nrel - 3], mode, a_domain, cnt, total, status, num_sms, st);
 }
 
-void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &T, int num_sms, OneBucket &L) {
-    const mwj_rel rel[3] = {R, R, T};   // the weights are R's, not S's
+void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, OneBucket &L) {
+    // the weights are R's, not S's, except in a small call (a chain like any other)
+    const mwj_rel rel[3] = {R, S.n <= kMediumMax && S.n > R.n ? S : R, T};
     one_bucket_layout(A, rel, 3, num_sms, L);
 }
 
@@ -739,6 +1071,8 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     cudaError_t e;
     L.deg.seed = sd.slot2;
     L.w[0].seed = sd.slot;
+    const mwj_rel rel[3] = {R, S, T};
+    if (small_run(L, rel, 3, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
     const uint64_t tr = single_table_slots(T.n), rr = w_table_slots(R.n);
     const SizeCol cols[2] = {SizeCol{T.x, (uint32_t)T.n, sd.slot2, L.hll[0], {L.deg.meta}, {tr}, {tr}, 1u},
                              SizeCol{R.y, (uint32_t)R.n, sd.slot, L.hll[1], {L.w[0].meta}, {rr}, {rr}, 1u}};
@@ -752,7 +1086,7 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     if ((e = deg_build(T, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     if (R.n > 0) {
         ProfScope ps_("star_keys", st);
-        k_w_keys<<<pass_grid(k_w_keys, (uint32_t)R.n, num_sms, 32), WT, 0, st>>>(R.y, (uint32_t)R.n, L.w[0], status);
+        k_w_keys<<<pass_grid((uint32_t)R.n, num_sms, 8, 32), WT, 0, st>>>(R.y, (uint32_t)R.n, L.w[0], status);
     }
     Source src{};
     src.t = L.deg;

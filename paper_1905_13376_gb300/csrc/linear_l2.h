@@ -53,7 +53,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
                            unsigned long long *cnt, unsigned long long *total, DevStatus *status, int num_sms,
                            cudaStream_t st);
 // The same for a star join (small R and T, large S): w[0] holds R's keys.
-void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &T, int num_sms, OneBucket &L);
+void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, OneBucket &L);
 cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd, int mode,
                             int32_t a_domain, unsigned long long *cnt, unsigned long long *total, DevStatus *status,
                             int num_sms, cudaStream_t st);

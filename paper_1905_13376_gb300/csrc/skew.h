@@ -40,22 +40,23 @@ __device__ __forceinline__ const uint32_t *heavy_to_smem(const uint32_t *heavy, 
     return buf;
 }
 
-// The heavy keys of one column from a strided sample of it, by one CTA of NT
-// threads (sm: its shared memory): those whose sampled share reaches
-// 1 / (2 buckets), and at least kHeavyMinCount sampled tuples.
-constexpr uint32_t kHeavySampled = 2048;     // sampled tuples
-constexpr uint32_t kHeavyCountSlots = 4096;  // count table, at most half full
-constexpr uint32_t kHeavyMinCount = 8;       // a heavy key is seen at least this often
+// The heavy keys of one column from a strided sample of SAMPLED of its tuples,
+// by one CTA of NT threads (sm: its shared memory): those whose sampled share
+// reaches 1 / (2 buckets), and at least kHeavyMinCount sampled tuples.
+constexpr uint32_t kHeavyMinCount = 8;
+template <uint32_t SAMPLED>
 struct HeavySample {
-    uint32_t key[kHeavyCountSlots], cnt[kHeavyCountSlots], ht[kHeavySlots], nh;
+    static constexpr uint32_t slots = 2 * SAMPLED;   // count table, at most half full
+    uint32_t key[slots], cnt[slots], ht[kHeavySlots], nh;
 };
 
-template <int NT>
+template <int NT, uint32_t SAMPLED>
 __device__ __forceinline__ void heavy_sample_cta(const int32_t *__restrict__ col, uint32_t n, uint32_t buckets,
-                                                 uint32_t *__restrict__ heavy, HeavySample &sm) {
-    const uint32_t m = n < kHeavySampled ? n : kHeavySampled;
-    constexpr uint32_t PER = kHeavySampled / NT;
-    static_assert(PER * NT == kHeavySampled, "a whole number of samples per thread");
+                                                 uint32_t *__restrict__ heavy, HeavySample<SAMPLED> &sm) {
+    constexpr uint32_t kHeavyCountSlots = HeavySample<SAMPLED>::slots;
+    const uint32_t m = n < SAMPLED ? n : SAMPLED;
+    constexpr uint32_t PER = SAMPLED / NT;
+    static_assert(PER * NT == SAMPLED, "a whole number of samples per thread");
     uint32_t ks[PER];
 #pragma unroll
     for (uint32_t q = 0; q < PER; ++q) {

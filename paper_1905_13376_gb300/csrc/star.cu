@@ -260,11 +260,11 @@ mwj_status star_plan(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, const mwj
     return MWJ_OK;
 }
 
-size_t star_layout(Arena &A, const StarPlan &p, const mwj_rel &R, const mwj_rel &T, int num_sms,
+size_t star_layout(Arena &A, const StarPlan &p, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms,
                    StarLayout &L) {
     L = StarLayout{};
     if (!p.rows) {
-        star_bucket_layout(A, R, T, num_sms, L.one);
+        star_bucket_layout(A, R, S, T, num_sms, L.one);
         return A.used;
     }
     L.Rp = A.take<uint2>(R.n + 2);
@@ -306,7 +306,7 @@ mwj_status star_workspace(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, cons
     if (s != MWJ_OK) return s;
     Arena A(nullptr, 0);
     StarLayout L;
-    *bytes = star_layout(A, p, R, T, ctx->dev.num_sms, L);
+    *bytes = star_layout(A, p, R, S, T, ctx->dev.num_sms, L);
     return MWJ_OK;
 }
 
@@ -326,7 +326,7 @@ extern "C" mwj_status mwj_join3_star(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel
     if ((s = star_plan(ctx, R, S, T, shares, out->mode, &p)) != MWJ_OK) return s;
     Arena A(workspace, ws_bytes);
     StarLayout L;
-    star_layout(A, p, R, T, ctx->dev.num_sms, L);
+    star_layout(A, p, R, S, T, ctx->dev.num_sms, L);
     if (A.overflow || !workspace)
         return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
 

@@ -428,10 +428,10 @@ __device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t most)
 // every key) and its merge 0.014 ms more; a column whose range is compact
 // needs neither.  The first CTAs sample the heavy keys (skew.h) meanwhile.
 __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
-    __shared__ HeavySample hsm;
+    __shared__ HeavySample<2048> hsm;
     if (blockIdx.x < g.nheavy) {
         const HeavyCol &h = g.h[blockIdx.x];
-        heavy_sample_cta<BT>(h.keys, h.n, h.buckets, h.heavy, hsm);
+        heavy_sample_cta<BT, 2048>(h.keys, h.n, h.buckets, h.heavy, hsm);
         return;
     }
     const uint32_t cta = (blockIdx.x - g.nheavy) % g.range_rows;
