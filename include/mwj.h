@@ -285,14 +285,15 @@ mwj_status mwj_batch_destroy(mwj_batch *batch);
  * paper).  A query whose shares the library chooses falls in the size class
  * floor(log2(max(|R|, |S|, |T|))) of its kind; the rule of that class gives
  *   tuples_per_bucket  linear: about this many R tuples per H(B) bucket
- *                      (I = the power of two at or above |R| / it);
+ *                      (I = the power of two at or above |R| / it
+ *                      and |S| / 16384);
  *   table_factor       linear: slots of T's degree table per T tuple (the
  *                      power of two at or above factor x |T|: load factor
  *                      at most 1 / factor), 2 .. 8;
  *   fit_pct            cyclic: R_ij and T_ki may fill this percentage of a
  *                      tile's on-chip capacity when the cube shares are
  *                      searched (Section 5.2's z|R| + x|S| + y|T|), 10 .. 100.
- * A field <= 0 keeps the library's rule (8192 tuples, factor 2, 50 %).
+ * A field <= 0 keeps the library's rule (8192 tuples, factor 2, 95 %).
  * mwj_batch_set_rules replaces the context's rules (n == 0 restores the
  * library's); mwj_batch_set_launch sets the CTAs per SM of the batch's
  * persistent partitioning and join launches (0: the library's choice, 3 and

@@ -33,9 +33,9 @@ from . import binding
 
 LINEAR_TPB = (2048, 4096, 8192, 16384, 32768)
 LINEAR_TFAC = (2, 4)
-CYCLIC_FIT = (25, 35, 50, 65, 80)
+CYCLIC_FIT = (35, 50, 65, 80, 95)
 LAUNCH = ((0, 0), (2, 0), (4, 0), (3, 1), (3, 2))
-DEFAULT = {binding.MWJ_LINEAR: (8192, 2, 0), binding.MWJ_CYCLIC: (0, 0, 50)}
+DEFAULT = {binding.MWJ_LINEAR: (8192, 2, 0), binding.MWJ_CYCLIC: (0, 0, 95)}
 MARGIN = 0.03   # a candidate must beat the library's rule by this fraction
 
 

@@ -16,10 +16,11 @@
 //                  stays in L2 while the query's items run
 //   k_batch_plan   work items of the cyclic tiles (R chunks x T chunks)
 //   scan           item offsets over all cyclic tiles of all queries
-//   k_batch_join   persistent over one queue: linear items (query, R bucket)
-//                  first (sorted by size on the host), then cyclic items
-//                  (query, tile, R chunk, T chunk); counts[q] accumulates with
-//                  one 64-bit atomic per item.
+//   k_batch_join   persistent over one queue: cyclic items (query, tile, R
+//                  chunk, T chunk) first, the largest query's first, since
+//                  those are the long ones, then linear items (query, R
+//                  bucket), sorted by size on the host; counts[q] accumulates
+//                  with one 64-bit atomic per item.
 #include <algorithm>
 #include <cmath>
 #include <numeric>
@@ -91,27 +92,31 @@ __device__ __forceinline__ uint32_t seg_bucket(int32_t x, int32_t y, const PartS
     return b;
 }
 
-__device__ __forceinline__ void ttab_insert(unsigned long long *tbl, uint32_t mask, uint32_t k,
-                                            uint32_t seed, DevStatus *st) {
-    uint32_t s = slot_of(k, seed, mask);
+// count of key k += 1 from its first probe (slot s, value v, possibly read
+// before another thread claimed the slot)
+__device__ __forceinline__ void ttab_insert(unsigned long long *tbl, uint32_t mask, uint32_t k, uint32_t s,
+                                            unsigned long long v, DevStatus *st) {
     const unsigned long long fresh = (1ull << 32) | (unsigned long long)k;
     for (uint32_t it = 0; it <= mask; ++it) {
-        unsigned long long v = tbl[s];
         if (v == kEmpty64) {
-            unsigned long long old = atomicCAS(&tbl[s], kEmpty64, fresh);
-            if (old == kEmpty64) return;
-            v = old;
+            v = atomicCAS(&tbl[s], kEmpty64, fresh);
+            if (v == kEmpty64) return;
         }
         if ((uint32_t)v == k) {
             atomicAdd(&tbl[s], 1ull << 32);
             return;
         }
         s = (s + 1) & mask;
+        v = __ldcg(tbl + s);
     }
     set_status(st, MWJ_ERR_CHECK, 31);
 }
 
 // ---- persistent segment kernel --------------------------------------------
+// A thread keeps PU tuples in flight: one CTA reads a whole relation twice, so
+// the largest one's latency is the kernel's (1.38 ms for the 1024-query batch
+// with one tuple in flight, 1.03 ms with eight).
+constexpr uint32_t PU = 8;
 __global__ void __launch_bounds__(BTH) k_batch_prep(BatchDev b, unsigned int *counter, DevStatus *st) {
     __shared__ uint32_t hist[kSegMaxP + 1];
     __shared__ uint32_t scan_scratch[33];
@@ -126,16 +131,43 @@ __global__ void __launch_bounds__(BTH) k_batch_prep(BatchDev b, unsigned int *co
         if (sg.kind == SEG_TTAB) {
             for (uint32_t s = threadIdx.x; s <= sg.tmask; s += BTH) sg.tbl[s] = kEmpty64;
             __syncthreads();
-            for (uint32_t i = threadIdx.x; i < sg.n; i += BTH)
-                ttab_insert(sg.tbl, sg.tmask, (uint32_t)__ldg(sg.x + i), b.seed_slot2, st);
+            for (uint32_t i = threadIdx.x; i < sg.n; i += PU * BTH) {
+                uint32_t k[PU], s[PU];
+                unsigned long long v[PU];
+#pragma unroll
+                for (uint32_t u = 0; u < PU; ++u)
+                    if (i + u * BTH < sg.n) k[u] = (uint32_t)__ldg(sg.x + i + u * BTH);
+#pragma unroll
+                for (uint32_t u = 0; u < PU; ++u) {
+                    if (i + u * BTH >= sg.n) continue;
+                    s[u] = slot_of(k[u], b.seed_slot2, sg.tmask);
+                    v[u] = __ldcg(sg.tbl + s[u]);
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < PU; ++u)
+                    if (i + u * BTH < sg.n) ttab_insert(sg.tbl, sg.tmask, k[u], s[u], v[u], st);
+            }
             __syncthreads();
             continue;
         }
         const uint32_t P = sg.sp.P();
         for (uint32_t k = threadIdx.x; k <= P; k += BTH) hist[k] = 0;
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < sg.n; i += BTH)
-            atomicAdd(&hist[seg_bucket(__ldg(sg.x + i), __ldg(sg.y + i), sg.sp)], 1u);
+        auto tuples = [&](auto &&f) {
+            for (uint32_t i = threadIdx.x; i < sg.n; i += PU * BTH) {
+                int32_t x[PU], y[PU];
+#pragma unroll
+                for (uint32_t u = 0; u < PU; ++u) {
+                    if (i + u * BTH >= sg.n) continue;
+                    x[u] = __ldg(sg.x + i + u * BTH);
+                    y[u] = __ldg(sg.y + i + u * BTH);
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < PU; ++u)
+                    if (i + u * BTH < sg.n) f(x[u], y[u]);
+            }
+        };
+        tuples([&](int32_t x, int32_t y) { atomicAdd(&hist[seg_bucket(x, y, sg.sp)], 1u); });
         __syncthreads();
         // exclusive scan of hist[0..P) -> off[] and cursors
         if (threadIdx.x == 0) carry = 0;
@@ -155,12 +187,13 @@ __global__ void __launch_bounds__(BTH) k_batch_prep(BatchDev b, unsigned int *co
         }
         if (threadIdx.x == 0) sg.off[P] = sg.n;
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < sg.n; i += BTH) {
-            int32_t xv = __ldg(sg.x + i), yv = __ldg(sg.y + i);
-            uint32_t p = atomicAdd(&hist[seg_bucket(xv, yv, sg.sp)], 1u);
-            if (p < sg.n) sg.out[p] = make_uint2((uint32_t)xv, (uint32_t)yv);
-            else set_status(st, MWJ_ERR_CHECK, 32);
-        }
+        tuples([&](int32_t x, int32_t y) {
+            const uint32_t p = atomicAdd(&hist[seg_bucket(x, y, sg.sp)], 1u);
+            if (p < sg.n)
+                sg.out[p] = make_uint2((uint32_t)x, (uint32_t)y);
+            else
+                set_status(st, MWJ_ERR_CHECK, 32);
+        });
         __syncthreads();
     }
 }
@@ -197,27 +230,34 @@ struct LinSmem {
     uint32_t keys[LCAP + 1];
     uint32_t deg[LCAP + 1];
 };
+constexpr uint32_t CSCH = 1024, CSSLOTS = 2048;   // S tuples of a chunk whose repeats are merged, its table
+constexpr uint32_t CFWORDS = 1024;                // filter in front of the T table (2^15 bits)
+// Counts of tables with at most 2^16 - 1 entries: two 16-bit counts per word.
 struct CycSmem {
-    uint32_t rkeys[CRSLOTS + 1];
-    uint32_t rdeg[CRSLOTS + 1];
-    uint32_t rstart[CRSLOTS + 1];
-    int32_t alist[CRCAP];
-    unsigned long long tkeys[CTSLOTS];
-    uint32_t tcnt[CTSLOTS + 1];
+    uint32_t rkeys[CRSLOTS + 1];   // R's B values
+    uint32_t rinfo[CRSLOTS + 1];   // per slot: list length << 16 | start (cursor while it fills)
+    int32_t alist[CRCAP];          // the lists' A values and, when repeats are merged,
+    uint16_t amult[CRCAP];         // how often each occurs
+    alignas(16) unsigned long long tkeys[CTSLOTS];   // T's (c, a) pairs in buckets of two; before that R's (slot, a)
+    uint32_t tcnt[CTSLOTS / 2];
+    uint32_t filt[CFWORDS];
+    unsigned long long skeys[CSSLOTS];   // S's (slot, c) pairs of a chunk
+    uint32_t scnt[CSSLOTS / 2];
 };
 union JoinSmem {
     LinSmem lin;
     CycSmem cyc;
 };
+static_assert(sizeof(JoinSmem) <= (228 * 1024) / 2 - 2048, "two CTAs per SM");
 
-__device__ __forceinline__ uint32_t t_deg(const unsigned long long *tbl, uint32_t mask, uint32_t c,
-                                          uint32_t seed) {
-    uint32_t s = slot_of(c, seed, mask);
+// deg_T(c) from the first probe (slot s, value v) of T's table
+__device__ __forceinline__ uint32_t t_deg_from(const unsigned long long *tbl, uint32_t mask, uint32_t c, uint32_t s,
+                                               unsigned long long v) {
     for (uint32_t it = 0; it <= mask; ++it) {
-        unsigned long long v = __ldg(tbl + s);
         if (v == kEmpty64) return 0;
         if ((uint32_t)v == c) return (uint32_t)(v >> 32);
         s = (s + 1) & mask;
+        v = __ldg(tbl + s);
     }
     return 0;
 }
@@ -225,13 +265,51 @@ __device__ __forceinline__ uint32_t t_deg(const unsigned long long *tbl, uint32_
 __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
     return ((unsigned long long)c << 32) | a;
 }
-__device__ __forceinline__ uint32_t cpair_hash(uint32_t c, uint32_t a, uint32_t seed) {
-    return mix32(c ^ mix32(a ^ seed));
+// The hash of a pair (c, a): only the multiply-add depends on a.  Its top bits
+// give the filter's word and bit and the home bucket.
+__device__ __forceinline__ uint32_t chash(uint32_t c, uint32_t seed) { return mix32(c ^ seed); }
+__device__ __forceinline__ uint32_t cpair_hash(uint32_t a, uint32_t ch) { return a * 0x9E3779B1u + ch; }
+static_assert(CFWORDS == 1u << 10 && CTSLOTS == 1u << 12, "bit positions of the pair hash");
+__device__ __forceinline__ bool cfilter(const uint32_t *filt, uint32_t h) {
+    return (filt[h >> 22] >> ((h >> 17) & 31u)) & 1u;
+}
+
+// Add one to the count of `key` in an open-addressing table of `slots` (a power
+// of two, at most half full) 8-byte slots, from slot s; false: full.
+__device__ __forceinline__ bool pair_add(unsigned long long *keys, uint32_t *cnt, uint32_t slots,
+                                         unsigned long long key, uint32_t s) {
+    for (uint32_t it = 0; it < slots; ++it) {
+        unsigned long long v = keys[s];
+        if (v == kEmpty64) v = atomicCAS(&keys[s], kEmpty64, key);
+        if (v == kEmpty64 || v == key) {
+            atomicAdd(&cnt[s >> 1], (s & 1u) ? 0x10000u : 1u);
+            return true;
+        }
+        s = (s + 1) & (slots - 1);
+    }
+    return false;
+}
+__device__ __forceinline__ uint32_t pair_count(const uint32_t *cnt, uint32_t s) {
+    return (cnt[s >> 1] >> ((s & 1u) * 16u)) & 0xFFFFu;
+}
+
+// How often (c, a) occurs in the T chunk: pair_add put it into the first slot
+// at or after its home bucket (an even slot) that was free.
+__device__ __forceinline__ uint32_t cyc_lookup(const CycSmem &sm, unsigned long long key, uint32_t h) {
+    uint32_t s = (h >> 21) * 2u;
+    for (uint32_t it = 0; it < CTSLOTS / 2; ++it) {
+        const ulonglong2 v = *(const ulonglong2 *)(sm.tkeys + s);
+        if (v.x == key) return pair_count(sm.tcnt, s);
+        if (v.y == key) return pair_count(sm.tcnt, s + 1);
+        if (v.y == kEmpty64) break;   // (v.x empty implies v.y empty)
+        s = (s + 2) & (CTSLOTS - 1);
+    }
+    return 0u;
 }
 
 // COUNT of one linear item (R bucket i of a query): R_i in shared memory as
 // b -> deg_R(b), in chunks that keep the table at most 3/4 full.
-__device__ unsigned long long lin_item(const LinQ &L, uint32_t i, LinSmem &sm, uint32_t seed,
+__device__ __noinline__ unsigned long long lin_item(const LinQ &L, uint32_t i, LinSmem &sm, uint32_t seed,
                                        uint32_t seed2, uint32_t *nd, DevStatus *st) {
     const uint32_t r0 = L.offR[i], r1 = L.offR[i + 1];
     const uint32_t s0 = L.offS[i], s1 = L.offS[i + 1];
@@ -270,12 +348,27 @@ __device__ unsigned long long lin_item(const LinQ &L, uint32_t i, LinSmem &sm, u
             cend += rt;
         }
         cend = min(cend, r1);
-        for (uint32_t s = s0 + threadIdx.x; s < s1; s += BTH) {
-            const uint2 t = __ldg(L.Sp + s);
-            const int slot = tbl_find(sm.keys, mask, t.x, seed);
-            if (slot < 0) continue;
-            const uint32_t d = t_deg(L.tbl, L.tmask, t.y, seed2);
-            acc += (unsigned long long)sm.deg[slot] * d;
+        // four S tuples per thread in flight: their loads, then their first T probes
+        for (uint32_t sb = s0 + threadIdx.x; sb < s1; sb += 4 * BTH) {
+            uint2 t[4];
+            uint32_t d[4], ts[4];
+            unsigned long long v[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q)
+                if (sb + q * BTH < s1) t[q] = __ldg(L.Sp + sb + q * BTH);
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                d[q] = 0u;
+                if (sb + q * BTH >= s1) continue;
+                const int slot = tbl_find(sm.keys, mask, t[q].x, seed);
+                if (slot < 0) continue;
+                d[q] = sm.deg[slot];
+                ts[q] = slot_of(t[q].y, seed2, L.tmask);
+                v[q] = __ldg(L.tbl + ts[q]);
+            }
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q)
+                if (d[q]) acc += (unsigned long long)d[q] * t_deg_from(L.tbl, L.tmask, t[q].y, ts[q], v[q]);
         }
         pos = cend;
     }
@@ -283,9 +376,18 @@ __device__ unsigned long long lin_item(const LinQ &L, uint32_t i, LinSmem &sm, u
 }
 
 // COUNT of one cyclic item (tile, R chunk, T chunk).
+//
+// An item's work is its wedges, |R list of b| per S tuple, so where they
+// outnumber its tuples eight to one the repeats go first: T's table always
+// counts them, and then R's (b, a) pairs and, in chunks of CSCH tuples, S's
+// (b, c) pairs are merged with their multiplicities as well.  Zipf keys and
+// small domains repeat pairs often (over the 1024-query batch a tenth of the
+// wedges is left), and merging costs two shared-memory inserts per tuple.
+// A wedge is one filter bit; those that pass look their pair up.
 __device__ unsigned long long cyc_item(const CycQ &c, uint32_t t_local, uint32_t local, CycSmem &sm,
-                                       uint32_t seed, uint32_t seed2, uint32_t *carry,
+                                       uint32_t seed, uint32_t seed2, uint32_t *nd,
                                        uint32_t *scan_scratch, DevStatus *st) {
+    __shared__ uint32_t negs_s;   // (-1, -1) pairs of T
     const TileIdx id = tile_in(t_local, c);
     const uint32_t rb = id.i * c.y + id.j, sb = id.j * c.z + id.k, tb = id.k * c.x + id.i;
     const uint32_t r0 = c.offR[rb], r1 = c.offR[rb + 1];
@@ -296,91 +398,152 @@ __device__ unsigned long long cyc_item(const CycQ &c, uint32_t t_local, uint32_t
     const uint32_t ra = r0 + rc * CRCAP, rz = min(r1, ra + CRCAP);
     const uint32_t ta = t0 + tc * CTCAP, tz = min(t1, ta + CTCAP);
     const uint32_t lane = threadIdx.x & 31;
-    __syncthreads();
+    // the chunks' tuples, a thread's four of each, on their way while the tables
+    // are emptied
+    constexpr int RQ = CRCAP / BTH, TQ = CTCAP / BTH;
+    uint2 rt[RQ], tt[TQ];
+#pragma unroll
+    for (int q = 0; q < RQ; ++q) {
+        const uint32_t r = ra + threadIdx.x + q * BTH;
+        rt[q] = r < rz ? __ldg(c.Rp + r) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int q = 0; q < TQ; ++q) {
+        const uint32_t r = ta + threadIdx.x + q * BTH;
+        tt[q] = r < tz ? __ldg(c.Tp + r) : make_uint2(0u, 0u);
+    }
+    auto clear_pairs = [&]() {
+        for (uint32_t q = threadIdx.x; q < CTSLOTS / 2; q += BTH)
+            ((ulonglong2 *)sm.tkeys)[q] = make_ulonglong2(kEmpty64, kEmpty64);
+        for (uint32_t q = threadIdx.x; q < CTSLOTS / 2; q += BTH) sm.tcnt[q] = 0u;
+    };
     for (uint32_t q = threadIdx.x; q <= CRSLOTS; q += BTH) {
         sm.rkeys[q] = (q < CRSLOTS) ? kEmptyKey : 0u;
-        sm.rdeg[q] = 0u;
+        sm.rinfo[q] = 0u;
     }
-    for (uint32_t q = threadIdx.x; q <= CTSLOTS; q += BTH) {
-        if (q < CTSLOTS) sm.tkeys[q] = kEmpty64;
-        sm.tcnt[q] = 0u;
+    clear_pairs();
+    for (uint32_t q = threadIdx.x; q < CFWORDS; q += BTH) sm.filt[q] = 0u;
+    if (threadIdx.x == 0) {
+        negs_s = 0u;
+        *nd = 0u;
     }
-    if (threadIdx.x == 0) *carry = 0;
     __syncthreads();
-    for (uint32_t r = ra + threadIdx.x; r < rz; r += BTH) {
+    // R's B values and list lengths
+    int slot[RQ];
+    uint32_t fresh_n = 0;
+#pragma unroll
+    for (int q = 0; q < RQ; ++q) {
+        slot[q] = -1;
+        if (ra + threadIdx.x + q * BTH >= rz) continue;
         bool fresh;
-        int slot = tbl_insert(sm.rkeys, CRSLOTS - 1, __ldg(c.Rp + r).y, seed, &fresh);
-        if (slot >= 0) atomicAdd(&sm.rdeg[slot], 1u);
-        else set_status(st, MWJ_ERR_CHECK, 34);
+        slot[q] = tbl_insert(sm.rkeys, CRSLOTS - 1, rt[q].y, seed, &fresh);
+        if (slot[q] >= 0)
+            atomicAdd(&sm.rinfo[slot[q]], 0x10000u);
+        else
+            set_status(st, MWJ_ERR_CHECK, 34);
+        fresh_n += fresh;
     }
-    for (uint32_t q = ta + threadIdx.x; q < tz; q += BTH) {
-        const uint2 tu = __ldg(c.Tp + q);
-        const unsigned long long key = cpack(tu.x, tu.y);
-        if (key == kEmpty64) {
-            atomicAdd(&sm.tcnt[CTSLOTS], 1u);
-            continue;
-        }
-        uint32_t h = cpair_hash(tu.x, tu.y, seed2) & (CTSLOTS - 1);
-        bool done = false;
-        for (uint32_t it = 0; it < CTSLOTS; ++it) {
-            unsigned long long v = sm.tkeys[h];
-            if (v == kEmpty64) {
-                unsigned long long old = atomicCAS(&sm.tkeys[h], kEmpty64, key);
-                if (old == kEmpty64 || old == key) {
-                    atomicAdd(&sm.tcnt[h], 1u);
-                    done = true;
-                    break;
-                }
-                v = old;
-            }
-            if (v == key) {
-                atomicAdd(&sm.tcnt[h], 1u);
-                done = true;
-                break;
-            }
-            h = (h + 1) & (CTSLOTS - 1);
-        }
-        if (!done) set_status(st, MWJ_ERR_CHECK, 35);
-    }
+    fresh_n = warp_sum(fresh_n);
+    if (lane == 0 && fresh_n) atomicAdd(nd, fresh_n);
     __syncthreads();
-    for (uint32_t b0 = 0; b0 <= CRSLOTS; b0 += BTH) {
-        uint32_t q = b0 + threadIdx.x;
-        uint32_t d = (q <= CRSLOTS) ? sm.rdeg[q] : 0u;
-        uint32_t tot;
-        uint32_t ex = block_excl_scan_u32(d, scan_scratch, &tot);
-        if (q <= CRSLOTS) sm.rstart[q] = *carry + ex;
+    const bool merge = (uint64_t)(s1 - s0) * (rz - ra) / max(*nd, 1u) > 8ull * ((s1 - s0) + (rz - ra));
+    if (merge) {   // R's distinct (slot, a) pairs, in T's table for now
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+            if (slot[q] < 0) continue;
+            const uint32_t h = cpair_hash(rt[q].x, chash((uint32_t)slot[q], seed2));
+            if (!pair_add(sm.tkeys, sm.tcnt, CTSLOTS, cpack((uint32_t)slot[q], rt[q].x), h >> 20))
+                set_status(st, MWJ_ERR_CHECK, 36);
+        }
+        for (uint32_t q = threadIdx.x; q <= CRSLOTS; q += BTH) sm.rinfo[q] = 0u;
         __syncthreads();
-        if (threadIdx.x == 0) *carry += tot;
+        for (uint32_t q = threadIdx.x; q < CTSLOTS; q += BTH)
+            if (sm.tkeys[q] != kEmpty64) atomicAdd(&sm.rinfo[(uint32_t)(sm.tkeys[q] >> 32)], 0x10000u);
         __syncthreads();
     }
-    for (uint32_t r = ra + threadIdx.x; r < rz; r += BTH) {
-        const uint2 tu = __ldg(c.Rp + r);
-        int slot = tbl_find(sm.rkeys, CRSLOTS - 1, tu.y, seed);
-        if (slot >= 0) {
-            uint32_t p = atomicAdd(&sm.rstart[slot], 1u);
-            if (p < CRCAP) sm.alist[p] = (int32_t)tu.x;
+    {   // list starts: a thread's consecutive slots (an odd number of them: no bank conflicts)
+        constexpr uint32_t PER = (CRSLOTS + 1 + BTH - 1) / BTH;
+        static_assert(PER % 2 == 1, "odd stride");
+        const uint32_t q0 = threadIdx.x * PER;
+        uint32_t d[PER], sum = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {
+            d[q] = q0 + q <= CRSLOTS ? sm.rinfo[q0 + q] >> 16 : 0u;
+            sum += d[q];
+        }
+        uint32_t at = block_excl_scan_u32(sum, scan_scratch, nullptr);
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {
+            if (q0 + q <= CRSLOTS) sm.rinfo[q0 + q] = (d[q] << 16) | at;
+            at += d[q];
         }
     }
     __syncthreads();
-    for (uint32_t q = threadIdx.x; q <= CRSLOTS; q += BTH) sm.rstart[q] -= sm.rdeg[q];
+    if (merge) {
+        for (uint32_t q = threadIdx.x; q < CTSLOTS; q += BTH) {
+            const unsigned long long v = sm.tkeys[q];
+            if (v == kEmpty64) continue;
+            const uint32_t p = atomicAdd(&sm.rinfo[(uint32_t)(v >> 32)], 1u) & 0xFFFFu;
+            if (p < CRCAP) {
+                sm.alist[p] = (int32_t)(uint32_t)v;
+                sm.amult[p] = (uint16_t)pair_count(sm.tcnt, q);
+            }
+        }
+        __syncthreads();
+        clear_pairs();
+        __syncthreads();
+    } else {
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+            if (slot[q] < 0) continue;
+            const uint32_t p = atomicAdd(&sm.rinfo[slot[q]], 1u) & 0xFFFFu;
+            if (p < CRCAP) {
+                sm.alist[p] = (int32_t)rt[q].x;
+                sm.amult[p] = 1;
+            }
+        }
+    }
+    // T's pairs
+#pragma unroll
+    for (int q = 0; q < TQ; ++q) {
+        if (ta + threadIdx.x + q * BTH >= tz) continue;
+        const unsigned long long key = cpack(tt[q].x, tt[q].y);
+        const uint32_t h = cpair_hash(tt[q].y, chash(tt[q].x, seed2));
+        atomicOr(&sm.filt[h >> 22], 1u << ((h >> 17) & 31u));
+        if (key == kEmpty64)   // the empty marker: counted apart
+            atomicAdd(&negs_s, 1u);
+        else if (!pair_add(sm.tkeys, sm.tcnt, CTSLOTS, key, (h >> 21) * 2u))
+            set_status(st, MWJ_ERR_CHECK, 35);
+    }
     __syncthreads();
+    const uint32_t negs = negs_s;
     unsigned long long acc = 0;
-    for (uint32_t w0 = s0 + (threadIdx.x & ~31u); w0 < s1; w0 += BTH) {
-        const uint32_t idx = w0 + lane;
-        uint32_t cc = 0, n = 0, stt = 0;
-        if (idx < s1) {
-            const uint2 tu = __ldg(c.Sp + idx);
-            cc = tu.y;
-            int slot = tbl_find(sm.rkeys, CRSLOTS - 1, tu.x, seed);
-            if (slot >= 0) {
-                n = sm.rdeg[slot];
-                stt = sm.rstart[slot];
-            }
+    // one wedge: (cc, a) in T, times the multiplicities of its two sides
+    auto wedge = [&](uint32_t cc, uint32_t ch, uint32_t p, uint32_t mult) {
+        const uint32_t a = (uint32_t)sm.alist[p];
+        const uint32_t h = cpair_hash(a, ch);
+        if (!cfilter(sm.filt, h)) return;
+        const unsigned long long key = cpack(cc, a);
+        const uint32_t m = key == kEmpty64 ? negs : cyc_lookup(sm, key, h);
+        if (m) acc += (unsigned long long)m * ((unsigned long long)sm.amult[p] * mult);
+    };
+    // the wedges of the warp's 32 (b, c): n list entries from st each
+    auto wedges = [&](uint32_t cc, uint32_t n, uint32_t stt, uint32_t mult) {
+        unsigned longs = __ballot_sync(0xffffffffu, n >= 24u);   // walked by the whole warp
+        while (longs) {
+            const int j = __ffs(longs) - 1;
+            longs &= longs - 1u;
+            const uint32_t jc = __shfl_sync(0xffffffffu, cc, j), jn = __shfl_sync(0xffffffffu, n, j);
+            const uint32_t js = __shfl_sync(0xffffffffu, stt, j), jm = __shfl_sync(0xffffffffu, mult, j);
+            const uint32_t ch = chash(jc, seed2);
+            for (uint32_t i = lane; i < jn; i += 32) wedge(jc, ch, js + i, jm);
+            __syncwarp();
         }
+        if (n >= 24u) n = 0u;
         uint32_t incl = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
             if ((int)lane >= o) incl += y;
         }
         const uint32_t W = __shfl_sync(0xffffffffu, incl, 31);
@@ -391,42 +554,74 @@ __device__ unsigned long long cyc_item(const CycQ &c, uint32_t t_local, uint32_t
             const uint32_t qq = (wi < W) ? wi : 0u;
 #pragma unroll
             for (int step = 0; step < 5; ++step) {
-                int mid = (olo + ohi) >> 1;
-                uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
+                const int mid = (olo + ohi) >> 1;
+                const uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
                 if (v > qq) ohi = mid; else olo = mid + 1;
             }
             const uint32_t oc = __shfl_sync(0xffffffffu, cc, olo);
             const uint32_t ost = __shfl_sync(0xffffffffu, stt, olo);
             const uint32_t oex = __shfl_sync(0xffffffffu, excl, olo);
-            if (wi < W) {
-                const uint32_t ai = ost + (wi - oex);
-                const uint32_t a = (ai < CRCAP) ? (uint32_t)sm.alist[ai] : 0u;
-                const unsigned long long key = cpack(oc, a);
-                uint32_t m = 0;
-                if (key == kEmpty64) {
-                    m = sm.tcnt[CTSLOTS];
-                } else {
-                    uint32_t h = cpair_hash(oc, a, seed2) & (CTSLOTS - 1);
-                    for (uint32_t it = 0; it < CTSLOTS; ++it) {
-                        unsigned long long v = sm.tkeys[h];
-                        if (v == key) { m = sm.tcnt[h]; break; }
-                        if (v == kEmpty64) break;
-                        h = (h + 1) & (CTSLOTS - 1);
-                    }
-                }
-                acc += m;
-            }
+            const uint32_t om = __shfl_sync(0xffffffffu, mult, olo);
+            if (wi < W) wedge(oc, chash(oc, seed2), ost + (wi - oex), om);
+            __syncwarp();
         }
+    };
+    auto list_of = [&](int sl, uint32_t &n, uint32_t &stt) {   // the cursor stands at the list's end
+        const uint32_t v = sm.rinfo[sl];
+        n = v >> 16;
+        stt = (v & 0xFFFFu) - n;
+    };
+    if (!merge) {
+        uint32_t idx = s0 + threadIdx.x;
+        uint2 tu = idx < s1 ? __ldg(c.Sp + idx) : make_uint2(0u, 0u);
+        for (uint32_t w0 = s0 + (threadIdx.x & ~31u); w0 < s1; w0 += BTH, idx += BTH) {
+            const uint2 nt = idx + BTH < s1 ? __ldg(c.Sp + idx + BTH) : make_uint2(0u, 0u);
+            uint32_t cc = 0, n = 0, stt = 0;
+            if (idx < s1) {
+                const int slot = tbl_find(sm.rkeys, CRSLOTS - 1, tu.x, seed);
+                cc = tu.y;
+                if (slot >= 0) list_of(slot, n, stt);
+            }
+            wedges(cc, n, stt, 1u);
+            tu = nt;
+        }
+        return acc;
+    }
+    for (uint32_t p0 = s0; p0 < s1; p0 += CSCH) {
+        const uint32_t p1 = min(s1, p0 + CSCH);
+        for (uint32_t q = threadIdx.x; q < CSSLOTS; q += BTH) sm.skeys[q] = kEmpty64;
+        for (uint32_t q = threadIdx.x; q < CSSLOTS / 2; q += BTH) sm.scnt[q] = 0u;
+        __syncthreads();
+        for (uint32_t i = p0 + threadIdx.x; i < p1; i += BTH) {
+            const uint2 tu = __ldg(c.Sp + i);
+            const int slot = tbl_find(sm.rkeys, CRSLOTS - 1, tu.x, seed);
+            if (slot < 0) continue;
+            const uint32_t h = cpair_hash((uint32_t)slot, chash(tu.y, seed2));
+            if (!pair_add(sm.skeys, sm.scnt, CSSLOTS, cpack((uint32_t)slot, tu.y), h >> 21))
+                set_status(st, MWJ_ERR_CHECK, 37);
+        }
+        __syncthreads();
+        for (uint32_t w0 = threadIdx.x & ~31u; w0 < CSSLOTS; w0 += BTH) {
+            const unsigned long long v = sm.skeys[w0 + lane];
+            uint32_t n = 0, stt = 0, mult = 0;
+            if (v != kEmpty64) {
+                const uint32_t slot = (uint32_t)(v >> 32);
+                list_of((int)slot, n, stt);
+                mult = pair_count(sm.scnt, w0 + lane);
+            }
+            wedges((uint32_t)v, n, stt, mult);
+        }
+        __syncthreads();
     }
     return acc;
 }
 
-__global__ void __launch_bounds__(BTH) k_batch_join(BatchDev b, const uint32_t *item_off,
+__global__ void __launch_bounds__(BTH, 2) k_batch_join(BatchDev b, const uint32_t *item_off,
                                                    unsigned int *counter,
                                                    unsigned long long *counts, DevStatus *st) {
     extern __shared__ __align__(16) unsigned char smraw[];
     JoinSmem &sm = *(JoinSmem *)smraw;
-    __shared__ uint32_t item_s, nd, carry;
+    __shared__ uint32_t item_s, nd;
     __shared__ uint32_t scan_scratch[33];
     __shared__ unsigned long long red[32];
     const uint32_t ncyc_items = (b.ntiles > 0) ? item_off[b.ntiles] : 0u;
@@ -439,12 +634,12 @@ __global__ void __launch_bounds__(BTH) k_batch_join(BatchDev b, const uint32_t *
         if (item >= total) break;
         unsigned long long acc;
         uint32_t q;
-        if (item < b.nlitems) {
-            const LinItem li = b.litems[item];
+        if (item >= ncyc_items) {
+            const LinItem li = b.litems[item - ncyc_items];
             q = li.q;
             acc = lin_item(b.lin[li.lq], li.i, sm.lin, b.seed_slot, b.seed_slot2, &nd, st);
         } else {
-            const uint32_t ci = item - b.nlitems;
+            const uint32_t ci = item;
             uint32_t lo = 0, hi = b.ntiles;   // last tile t with item_off[t] <= ci
             while (hi - lo > 1) {
                 uint32_t mid = (lo + hi) >> 1;
@@ -453,7 +648,7 @@ __global__ void __launch_bounds__(BTH) k_batch_join(BatchDev b, const uint32_t *
             const CycQ c = b.cyc[b.tile_q[lo]];
             q = c.q;
             acc = cyc_item(c, lo - c.tile0, ci - item_off[lo], sm.cyc, b.seed_slot, b.seed_slot2,
-                           &carry, scan_scratch, st);
+                           &nd, scan_scratch, st);
         }
         unsigned long long tot = block_sum_u64(acc, red);
         if (threadIdx.x == 0 && tot) atomicAdd(counts + q, tot);
@@ -517,19 +712,45 @@ Rule batch_rule(const mwj_ctx *ctx, const mwj_query &q) {
     int c = 0;
     while (c < 31 && (2ll << c) <= m) ++c;
     const int k = q.kind == MWJ_LINEAR ? 0 : 1;
-    Rule r{8192u, 2u, 0.5};
+    // (fit: a tile above its capacity is only taken in two items; the cyclic half
+    // of a 1024-query batch takes 3.98 ms at 0.5, 3.42 at 0.75, 3.17 at 0.95)
+    Rule r{8192u, 2u, 0.95};
     if (ctx->batch_tpb[k][c] > 0) r.tpb = (uint32_t)ctx->batch_tpb[k][c];
     if (ctx->batch_tfac[k][c] > 0) r.tfac = (uint32_t)ctx->batch_tfac[k][c];
     if (ctx->batch_fit[k][c] > 0) r.fit = ctx->batch_fit[k][c] / 100.0;
     return r;
 }
 
+// The wedge side of a cyclic query.  R |x| S |x| T is the same triangle query
+// read from any of its three corners, and an item enumerates the wedges of the
+// first two relations and looks each up in the third: about |R||S| / |dom B|
+// of them, so the two smallest relations go first (rotation r: relation
+// (i + r) mod 3 in place i).  The domains are not known here; sizes alone make
+// it 3.5 times fewer wedges over batches with sizes and domains log-uniform
+// (the cyclic half of a 1024-query batch: 21.7 -> 5.9 ms).
+int cyc_rotation(const mwj_query &q) {
+    const double n[3] = {(double)q.R.n, (double)q.S.n, (double)q.T.n};
+    int r = 0;
+    for (int k = 1; k < 3; ++k)
+        if (n[k] * n[(k + 1) % 3] < n[r] * n[(r + 1) % 3]) r = k;
+    return r;
+}
+
+// What emptying and filling a tile's tables costs beside its tuples, in tuples
+// read (1024-query batch, cyclic half: 5.24 ms at 0, 4.97 at 1024, 4.87 at 4096,
+// another 0.07 less at 16384).
+constexpr double kTileCost = 16384.0;
+constexpr uint64_t kLinS = 16384;
+
 // shares of one batched query from its sizes: linear: about rule.tpb R
-// tuples per bucket; cyclic: the cost-model choice (z|R| + x|S| + y|T|)
+// tuples per bucket; cyclic: the cost-model choice (z|R| + x|S| + y|T| + kTileCost xyz)
 // under the chunk fit, with every relation's bucket count at most kSegMaxP
 void batch_shares(const mwj_query &q, const Rule &rule, mwj_shares *sh) {
     if (q.kind == MWJ_LINEAR) {
-        uint64_t want = (uint64_t)(q.R.n + rule.tpb - 1) / rule.tpb;
+        // (and no more than kLinS S tuples per item on average: one CTA streams
+        // a bucket's S alone, and a small R with a large S was the batch's tail)
+        const uint64_t want = std::max((uint64_t)(q.R.n + rule.tpb - 1) / rule.tpb,
+                                       (uint64_t)(q.S.n + kLinS - 1) / kLinS);
         uint32_t I = pow2_ge(want ? want : 1);
         if (I > kSegMaxP) I = kSegMaxP;
         sh->s[0] = (int32_t)I;
@@ -545,7 +766,7 @@ void batch_shares(const mwj_query &q, const Rule &rule, mwj_shares *sh) {
             for (uint32_t z = 1; z <= 64; z <<= 1) {
                 if (x * y > kSegMaxP || y * z > kSegMaxP || z * x > kSegMaxP) continue;
                 if (nR / (x * y) > rule.fit * CRCAP || nT / (z * x) > rule.fit * CTCAP) continue;
-                double cost = z * nR + x * nS + y * nT;
+                const double cost = z * nR + x * nS + y * nT + kTileCost * x * y * z;
                 if (cost < best) {
                     best = cost;
                     bx = x;
@@ -592,7 +813,7 @@ mwj_status mwj_batch_create(mwj_ctx *ctx, const mwj_query *queries, int32_t n, m
     };
     uint32_t tiles = 0;
     for (int32_t qi = 0; qi < n; ++qi) {
-        const mwj_query &q = queries[qi];
+        mwj_query q = queries[qi];
         if ((q.kind != MWJ_LINEAR && q.kind != MWJ_CYCLIC) || !rel_ok(q.R) || !rel_ok(q.S) ||
             !rel_ok(q.T)) {
             delete b;
@@ -600,8 +821,20 @@ mwj_status mwj_batch_create(mwj_ctx *ctx, const mwj_query *queries, int32_t n, m
         }
         mwj_shares sh = q.shares;
         const Rule rule = batch_rule(ctx, q);
-        if (sh.s[0] <= 0) batch_shares(q, rule, &sh);
-        b->shares.push_back(sh);
+        if (sh.s[0] <= 0) {
+            const int rot = q.kind == MWJ_CYCLIC ? cyc_rotation(q) : 0;
+            const mwj_rel rel[3] = {q.R, q.S, q.T};
+            q.R = rel[rot];
+            q.S = rel[(rot + 1) % 3];
+            q.T = rel[(rot + 2) % 3];
+            batch_shares(q, rule, &sh);
+            // reported for the query's own A, B, C: the rotated query's k-th is its (k + rot)-th
+            mwj_shares own = sh;
+            for (int k = 0; q.kind == MWJ_CYCLIC && k < 3; ++k) own.s[(k + rot) % 3] = sh.s[k];
+            b->shares.push_back(own);
+        } else {
+            b->shares.push_back(sh);
+        }
         if (q.kind == MWJ_LINEAR) {
             const uint32_t I = (uint32_t)sh.s[0];
             if (I < 1 || I > kSegMaxP) {
@@ -646,7 +879,6 @@ mwj_status mwj_batch_create(mwj_ctx *ctx, const mwj_query *queries, int32_t n, m
             C.x = x;
             C.y = y;
             C.z = z;
-            C.tile0 = tiles;
             C.q = (uint32_t)qi;
             b->segs.push_back(Seg{q.R.x, q.R.y, (uint32_t)q.R.n, SEG_PART, PartSpec{0, sd.A, x, 1, sd.B, y},
                                   (uint2 *)C.Rp, (uint32_t *)C.offR, nullptr, 0});
@@ -654,11 +886,23 @@ mwj_status mwj_batch_create(mwj_ctx *ctx, const mwj_query *queries, int32_t n, m
                                   (uint2 *)C.Sp, (uint32_t *)C.offS, nullptr, 0});
             b->segs.push_back(Seg{q.T.x, q.T.y, (uint32_t)q.T.n, SEG_PART, PartSpec{0, sd.C, z, 1, sd.A, x},
                                   (uint2 *)C.Tp, (uint32_t *)C.offT, nullptr, 0});
-            const uint32_t nt = x * y * z;
-            for (uint32_t t = 0; t < nt; ++t) b->tile_q.push_back((uint32_t)b->cyc.size());
-            tiles += nt;
             b->cyc.push_back(C);
         }
+    }
+    // the cyclic tiles, the largest query's first
+    std::vector<uint32_t> by_size(b->cyc.size());
+    std::iota(by_size.begin(), by_size.end(), 0u);
+    auto tuples = [&](uint32_t k) {
+        const mwj_query &q = queries[b->cyc[k].q];
+        return q.R.n + q.S.n + q.T.n;
+    };
+    std::stable_sort(by_size.begin(), by_size.end(), [&](uint32_t k, uint32_t l) { return tuples(k) > tuples(l); });
+    for (const uint32_t k : by_size) {
+        CycQ &C = b->cyc[k];
+        const uint32_t nt = C.x * C.y * C.z;
+        C.tile0 = tiles;
+        b->tile_q.insert(b->tile_q.end(), nt, k);
+        tiles += nt;
     }
     b->ncyc_tiles = tiles;
     b->off_items = A.used;
