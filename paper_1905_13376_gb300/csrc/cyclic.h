@@ -69,6 +69,10 @@ size_t cyc_c_rep_slots(int num_sms);
 cudaError_t rgroup_build(const int32_t *Ra, const int32_t *Rb, int64_t nR, const RGroup &r, unsigned int *hll,
                          uint64_t reserve, unsigned int *bump, int32_t a_domain, DevStatus *status, int num_sms,
                          cudaStream_t st);
+// S's tuples (b, c) with the end whose list in r is shorter first: u, v of nS
+// entries each.  Self-joins only (R's lists are T's), and not for row output.
+cudaError_t cyc_c_orient(const int32_t *Sb, const int32_t *Sc, int64_t nS, const RGroup &r, int32_t *u, int32_t *v,
+                         int num_sms, cudaStream_t st);
 // items: z + 1 u32; big_slots: z u64 (scanned into g.big_off, z + 2 u64,
 // with scan_tmp64b); g.bigset: 4 |T| + 16 u64 slots, g.bigcnt as many u32;
 // g.big_neg: z u32;

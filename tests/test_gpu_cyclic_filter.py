@@ -35,7 +35,7 @@ def check(ctx, R, S, T, a_domain, shares):
     return n
 
 
-@pytest.mark.parametrize("nt", [6143, 6144, 6145, 12289, 16384, 16385])
+@pytest.mark.parametrize("nt", [6143, 6144, 6145, 7167, 7168, 7169, 12289, 16384, 16385])
 def test_chunk_edges(ctx, nt):
     """One bucket holding nt T tuples: one, two and three on-chip chunks, and the
     L2 set."""
@@ -69,3 +69,33 @@ def test_marker_pair_and_repeats(ctx):
     assert want > 0
     for shares in ((1, 1, 1), (1, 1, 5), None):
         assert int(ctx.join3_cyclic(cu(R), cu(S), cu(T), "count", shares=shares)["total"].item()) == want
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_self_join_takes_the_shorter_list(ctx, seed):
+    """T holds R's pairs with the columns exchanged (the same device columns):
+    S's tuples are turned to their shorter list.  R a bag with repeats, S another
+    relation or the same one, keys inside and outside R, -1 among them."""
+    import torch
+    g = np.random.default_rng(seed)
+    dom = (40, 300, 2000, 90)[seed]
+    n = (3000, 9000, 9000, 20000)[seed]
+    a = g.integers(0, dom, n).astype(np.int32)
+    b = np.minimum(g.integers(0, dom, n), g.integers(0, dom, n)).astype(np.int32)
+    if seed == 3:
+        b[g.random(n) < 0.1] = -1
+    S = (g.integers(-1, dom + 5, 2500).astype(np.int32), g.integers(-1, dom + 5, 2500).astype(np.int32))
+    x, y = cu((a, b))
+    for own, dev in ((S, cu(S)), ((b, a), (y, x))):
+        if len(own[0]) > 10000:
+            continue   # (the oracle's walk)
+        want = oracle.cyclic((a, b), own, (b, a), oracle.GROUP_BY_A, a_domain=dom)
+        for shares in (None, (1, 1, 7), (2, 2, 2)):
+            got = ctx.join3_cyclic((x, y), dev, (y, x), "group_by_a", shares=shares, a_domain=dom)
+            assert int(got["total"].item()) == want["total"]
+            assert np.array_equal(got["counts"].cpu().numpy(), want["counts"])
+        n_rows = want["total"]
+        if n_rows < 3_000_000:
+            rows = oracle.cyclic((a, b), own, (b, a), oracle.MATERIALIZE, capacity=n_rows)["rows"]
+            got = ctx.join3_cyclic((x, y), dev, (y, x), "rows", capacity=n_rows)
+            assert np.array_equal(sorted_rows(got["rows"].cpu().numpy()), rows)
