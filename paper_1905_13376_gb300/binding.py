@@ -177,10 +177,12 @@ def __getattr__(name):
 def _rel(pair):
     import torch
     x, y = pair
-    assert x.dtype == torch.int32 and y.dtype == torch.int32, "relations are int32 column pairs"
+    i32 = torch.int32
+    assert x.dtype is i32 and y.dtype is i32, "relations are int32 column pairs"
     assert x.is_cuda and y.is_cuda and x.is_contiguous() and y.is_contiguous()
-    assert x.numel() == y.numel()
-    return mwj_rel(x.data_ptr(), y.data_ptr(), x.numel())
+    n = x.numel()
+    assert n == y.numel()
+    return mwj_rel(x.data_ptr(), y.data_ptr(), n)
 
 
 def _shares(s):
@@ -291,8 +293,9 @@ class Context:
 
     def _stream(self, stream):
         import torch
-        s = stream if stream is not None else torch.cuda.current_stream(self.device)
-        return ctypes.c_void_p(s.cuda_stream)
+        if stream is None:   # the current stream's handle without building a Stream object (2 us)
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(self.device.index))
+        return ctypes.c_void_p(stream.cuda_stream)
 
     def _outputs(self, mode, a_domain, capacity, arity, reuse=None):
         import torch
@@ -336,16 +339,18 @@ class Context:
             mode = MODES[mode]
         o, res = self._outputs(mode, a_domain, capacity, arity, out)
         with_shares = kind_ws in (MWJ_LINEAR, MWJ_CYCLIC, MWJ_STAR)
-        nb = self.workspace_size(kind_ws, R, S, T, shares if with_shares else None, mode)
-        ws = self.workspace(nb)
-        args = (self.h,) + tuple(extra) + (_rel(R), _rel(S), _rel(T))
+        r, s, t, hs = _rel(R), _rel(S), _rel(T), self._stream(stream)
+        sh = _shares(shares) if with_shares else None
+        nb = ctypes.c_size_t()
+        self._check(self.lib.mwj_workspace_size(self.h, kind_ws, r, s, t, sh, mode, ctypes.byref(nb)))
+        ws = self.workspace(nb.value)
+        args = (self.h,) + tuple(extra) + (r, s, t)
         if with_shares:
-            args = args + (_shares(shares),)
-        st = fn(*args, ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
-                self._stream(stream))
+            args = args + (sh,)
+        st = fn(*args, ctypes.byref(o), ws.data_ptr(), ws.numel(), hs)
         self._check(st)
         if sync:
-            self._check(self.lib.mwj_stream_status(self.h, self._stream(stream)))
+            self._check(self.lib.mwj_stream_status(self.h, hs))
             if mode == MWJ_MATERIALIZE:
                 n = int(res["n_rows"].item())
                 res["rows"] = res["rows"][:n]
@@ -378,11 +383,10 @@ class Context:
             mode = MODES[mode]
         o, res = self._outputs(mode, a_domain, 0, 4)
         nb = ctypes.c_size_t(0)
-        self._check(self.lib.mwj_join4_workspace_size(self.h, _rel(R), _rel(S), _rel(T), _rel(U),
-                                                      _shares(shares), int(mode), ctypes.byref(nb)))
+        rels, sh = (_rel(R), _rel(S), _rel(T), _rel(U)), _shares(shares)
+        self._check(self.lib.mwj_join4_workspace_size(self.h, *rels, sh, int(mode), ctypes.byref(nb)))
         ws = self.workspace(nb.value)
-        self._check(self.lib.mwj_join4_linear(self.h, _rel(R), _rel(S), _rel(T), _rel(U), _shares(shares),
-                                              ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+        self._check(self.lib.mwj_join4_linear(self.h, *rels, sh, ctypes.byref(o), ws.data_ptr(), ws.numel(),
                                               self._stream(stream)))
         if sync:
             self._check(self.lib.mwj_stream_status(self.h, self._stream(stream)))
@@ -397,13 +401,12 @@ class Context:
         sk = torch.empty((int(a_domain), 16), dtype=torch.int32, device=self.device)
         est = torch.empty(int(a_domain), dtype=torch.float32, device=self.device) if estimates else None
         nb = ctypes.c_size_t(0)
-        self._check(self.lib.mwj_fm_workspace_size(self.h, _rel(R), _rel(S), _rel(T), _shares(shares),
-                                                   ctypes.byref(nb)))
+        rels, sh = (_rel(R), _rel(S), _rel(T)), _shares(shares)
+        self._check(self.lib.mwj_fm_workspace_size(self.h, *rels, sh, ctypes.byref(nb)))
         ws = self.workspace(nb.value)
-        self._check(self.lib.mwj_fm_linear(self.h, _rel(R), _rel(S), _rel(T), _shares(shares), int(a_domain),
-                                           ctypes.c_void_p(sk.data_ptr()),
-                                           ctypes.c_void_p(est.data_ptr()) if est is not None else None,
-                                           ctypes.c_void_p(ws.data_ptr()), ws.numel(), self._stream(stream)))
+        self._check(self.lib.mwj_fm_linear(self.h, *rels, sh, int(a_domain), sk.data_ptr(),
+                                           est.data_ptr() if est is not None else None,
+                                           ws.data_ptr(), ws.numel(), self._stream(stream)))
         if sync:
             self._check(self.lib.mwj_stream_status(self.h, self._stream(stream)))
         return {"sketches": sk, "estimates": est}

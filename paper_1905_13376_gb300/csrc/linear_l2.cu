@@ -875,8 +875,10 @@ cudaError_t chain_small(const SmallArgs &g, cudaStream_t st) {
     const int64_t want = (most + CT - 1) / CT, wantg = g.mode == 1 ? ((int64_t)g.a_domain + 16383) / 16384 : 1;
     int ctas = 1;
     while (ctas < kSmallCtas && (ctas < want || ctas < wantg)) ctas <<= 1;
-    cudaError_t e = cudaFuncSetAttribute(k_chain_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+    if (ctas > 8) {   // more than the portable cluster size
+        const cudaError_t e = cudaFuncSetAttribute(k_chain_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(ctas);
     c.blockDim = dim3(CT);
