@@ -7,6 +7,7 @@
 #include "api_internal.h"
 #include "linear.h"
 #include "linear_l2.h"
+#include "linear_rows.h"
 #include "tables.h"
 #include "skew.h"
 
@@ -343,6 +344,13 @@ mwj_status mwj_workspace_size(mwj_ctx *ctx, int kind, mwj_rel R, mwj_rel S, mwj_
     if (mode < MWJ_COUNT || mode > MWJ_MATERIALIZE) return fail(ctx, MWJ_ERR_INVALID_ARG, "bad mode");
     mwj_shares sh;
     if (kind == MWJ_LINEAR) {
+        if (!shares && mode == MWJ_MATERIALIZE) {
+            Arena A(nullptr, 0);
+            LinRowsLayout L;
+            lin_rows_layout(A, R, S, T, ctx->dev.num_sms, L);
+            *bytes = A.used;
+            return MWJ_OK;
+        }
         if (shares) sh = *shares; else linear_default_shares(ctx, R, S, T, mode, &sh);
         LinPlan p;
         mwj_status s = lin_check_shares(ctx, &sh, &p.I, &p.J);
@@ -373,6 +381,17 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
     mwj_status s = check_out(ctx, out, 4);
     if (s != MWJ_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
+    if (!shares && out->mode == MWJ_MATERIALIZE) {   // rows: lists of R and T, S streamed past them
+        Arena A(workspace, ws_bytes);
+        LinRowsLayout L;
+        lin_rows_layout(A, R, S, T, ctx->dev.num_sms, L);
+        if (A.overflow || !workspace)
+            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
+        const cudaError_t er =
+            lin_rows_run(L, R, S, T, ctx->seeds, (int4 *)out->rows, out->capacity, (long long *)out->n_rows,
+                         (unsigned long long *)out->total, ctx->status, ctx->dev.num_sms, st);
+        return er == cudaSuccess ? MWJ_OK : cuda_fail(ctx, er, "linear rows");
+    }
     mwj_shares sh;
     if (shares) sh = *shares; else linear_default_shares(ctx, R, S, T, out->mode, &sh);
     LinPlan p;

@@ -21,6 +21,7 @@
 // that its wedges are checked once.  Results do not depend on z.
 #include "api_internal.h"
 #include "cyclic.h"
+#include "rgroup.cuh"
 #include "tables.h"
 
 namespace mwj {
@@ -112,20 +113,6 @@ __device__ __forceinline__ uint32_t cset_count(const unsigned long long *tk, uns
         bk = (bk + 1) & (CC_NB - 1);
     }
     return 0u;
-}
-
-// Entries of R's grouping: the direct-address layout (key b at b - min) or
-// the hashed key table's slot (slot mask + 1 holds key -1).
-__device__ __forceinline__ uint32_t rg_entries(const uint32_t *meta) {
-    return meta[kMetaDense] ? meta[kMetaSpan] : meta[kMetaMask] + 2u;
-}
-
-__device__ __forceinline__ int rg_find(const RGroup &r, const uint32_t *meta, uint32_t b) {
-    if (meta[kMetaDense]) {
-        const uint32_t k = b - meta[kMetaMin];
-        return k < meta[kMetaSpan] ? (int)k : -1;
-    }
-    return tbl_find(r.keys, meta[kMetaMask], b, r.seed);
 }
 
 __global__ void k_rg_clear(RGroup r) {
