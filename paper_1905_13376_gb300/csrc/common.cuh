@@ -261,6 +261,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, uint3
     return false;
 }
 
+// First statement of kernels launched with launch_after (internal.h).
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

@@ -273,8 +273,9 @@ struct SPass {
 };
 
 // Tuples [lo, hi) of a column pair in warp rounds of 128 (warp `warp` of
-// `warps` takes rounds warp, warp + warps, ...), each round's loads issued
-// before the previous round is used; round(x, y, m) per round.
+// `warps` takes a consecutive stretch of them: 1 % faster on the sorted friends
+// graph and star than every warps-th one), each round's loads issued before
+// the previous round is used; round(x, y, m) per round.
 template <typename F>
 __device__ __forceinline__ void rounds_plain(const int32_t *__restrict__ X, const int32_t *__restrict__ Y,
                                              uint32_t lo, uint32_t hi, uint32_t warp, uint32_t warps, F &&round) {
@@ -282,13 +283,14 @@ __device__ __forceinline__ void rounds_plain(const int32_t *__restrict__ X, cons
     const bool vec = (((uintptr_t)X | (uintptr_t)Y) & 15) == 0 && (lo & 3u) == 0;
     const uint64_t pol = l2_evict_first();
     const uint32_t n = hi;
-    const uint32_t rounds = (hi - lo + WCHUNK - 1) / WCHUNK;
+    const uint32_t all = (hi - lo + WCHUNK - 1) / WCHUNK, per = (all + warps - 1) / warps;
+    const uint32_t rounds = min(all, (warp + 1) * per);
     int32_t x[WQ], y[WQ];
     uint32_t m = 0;
-    uint32_t r = warp;
+    uint32_t r = warp * per;
     if (r < rounds) m = load_pairs(X, Y, n, lo + r * WCHUNK + lane * WQ, vec, pol, x, y);
     while (r < rounds) {
-        const uint32_t nr = r + warps;
+        const uint32_t nr = r + 1;
         int32_t nx[WQ], ny[WQ];
         uint32_t nm = 0;
         if (nr < rounds) nm = load_pairs(X, Y, n, lo + nr * WCHUNK + lane * WQ, vec, pol, nx, ny);
@@ -318,6 +320,7 @@ constexpr int GC = 6;
 template <bool SW, bool FILTER>
 __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
                                                     uint32_t n, Source src, WTable w, DevStatus *st) {
+    after_previous();
     const bool sd = source_dense<SW>(src), wd = __ldg(w.meta + kMetaDense) != 0u;
     if (sd && wd) return;
     __shared__ uint32_t hbuf[kHeavySlots];
@@ -404,6 +407,7 @@ template <bool SW, bool FILTER>
 __global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict__ Sb,
                                                        const int32_t *__restrict__ Sc, uint32_t n, Source src,
                                                        WTable w, DevStatus *st) {
+    after_previous();
     if (!source_dense<SW>(src) || !__ldg(w.meta + kMetaDense)) return;
     __shared__ uint32_t hbuf[kHeavySlots];
     __shared__ HeavySums hacc;
@@ -418,6 +422,7 @@ __global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict
 // Star joins, hashed layout: R's keys into the weight table, so that the S pass
 // keeps only the tuples that meet one.
 __global__ void __launch_bounds__(WT) k_w_keys(const int32_t *__restrict__ Rb, uint32_t n, WTable w, DevStatus *st) {
+    after_previous();
     if (__ldg(w.meta + kMetaDense)) return;
     const uint32_t mask = __ldg(w.meta + kMetaMask);
     for (uint64_t i = (uint64_t)blockIdx.x * WT + threadIdx.x; i < n; i += gridDim.x * WT) {
@@ -481,6 +486,7 @@ __global__ void __launch_bounds__(WT) k_w_probe(const int32_t *__restrict__ Ra, 
                                                 uint32_t n, WTable w, int32_t a_domain,
                                                 unsigned long long *__restrict__ cnt,
                                                 unsigned long long *__restrict__ total, DevStatus *st) {
+    after_previous();
     if (__ldg(w.meta + kMetaDense)) return;
     __shared__ unsigned long long red[32];
     w_probe_pass<MODE, false>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
@@ -491,6 +497,7 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
                                                        const int32_t *__restrict__ Rb, uint32_t n, WTable w,
                                                        int32_t a_domain, unsigned long long *__restrict__ cnt,
                                                        unsigned long long *__restrict__ total, DevStatus *st) {
+    after_previous();
     if (!__ldg(w.meta + kMetaDense)) return;
     __shared__ unsigned long long red[32];
     w_probe_pass<MODE, true>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
@@ -514,6 +521,7 @@ struct HeavyArgs {
 };
 __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__ keys, uint32_t n, DegTable t,
                                                      HeavyArgs heavy, DevStatus *st) {
+    after_previous();
     __shared__ HeavySample<1024> hsm;
     if (blockIdx.x < heavy.n) {
         const HeavyCol &h = heavy.h[blockIdx.x];
@@ -706,6 +714,7 @@ __device__ __forceinline__ void small_clear(const SmallArgs &g, uint32_t t, uint
 }
 
 __global__ void __launch_bounds__(WT) k_chain_clear(SmallArgs g) {
+    after_previous();
     const uint32_t t = blockIdx.x * WT + threadIdx.x;
     small_clear(g, t, gridDim.x * WT);
     if (t == 0) {
@@ -914,8 +923,8 @@ cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, in
     if (n + heavy.n == 0) return cudaSuccess;
     const uint32_t groups = (n + WQ * DT - 1) / (WQ * DT), full = (uint32_t)num_sms * 3;
     ProfScope ps_("t_insert", st);
-    k_deg_build<<<heavy.n + (groups < full ? (groups ? groups : 1u) : full), DT, 0, st>>>(T.x, n, t, heavy, status);
-    return cudaGetLastError();
+    return launch_after(k_deg_build, heavy.n + (groups < full ? (groups ? groups : 1u) : full), DT, st, T.x, n, t, heavy,
+                        status);
 }
 
 enum Pass { PASS_DEGREES, PASS_WEIGHTS, PASS_STAR };   // what a weight pass looks up, or a star's S pass
@@ -934,11 +943,12 @@ cudaError_t w_table_build(const mwj_rel &S, const Source &src, Pass pass, const 
                                          : k_w_build<false, false>;
     if (!hashed_only) {
         ProfScope ps_(pass == PASS_STAR ? "star_probe" : "w_build", st);
-        direct<<<pass_grid(n, num_sms, kDirectCtas, WCHUNK), WT, 0, st>>>(S.x, S.y, n, src, w, status);
+        const cudaError_t e = launch_after(direct, pass_grid(n, num_sms, kDirectCtas, WCHUNK), WT, st, S.x, S.y, n, src, w,
+                                           status);
+        if (e != cudaSuccess) return e;
     }
     ProfScope ps_(pass == PASS_STAR ? "star_probe_hashed" : "w_build_hashed", st);
-    hashed<<<pass_grid(n, num_sms, GC, 32), WT, 0, st>>>(S.x, S.y, n, src, w, status);
-    return cudaGetLastError();
+    return launch_after(hashed, pass_grid(n, num_sms, GC, 32), WT, st, S.x, S.y, n, src, w, status);
 }
 
 cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a_domain, unsigned long long *cnt,
@@ -950,11 +960,13 @@ cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a
     auto hashed = mode == 1 ? k_w_probe<1> : k_w_probe<0>;
     if (!hashed_only) {
         ProfScope ps_(mode == 1 ? "w_probe_groupby" : "w_probe_count", st);
-        direct<<<pass_grid(n, num_sms, mode == 1 ? kProbeCtas : kProbeCtas + 1, WCHUNK), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
+        const cudaError_t e = launch_after(direct, pass_grid(n, num_sms, mode == 1 ? kProbeCtas : kProbeCtas + 1, WCHUNK), WT,
+                                           st, R.x, R.y, n, w, a_domain, cnt, total, status);
+        if (e != cudaSuccess) return e;
     }
     ProfScope ps_(mode == 1 ? "w_probe_groupby_hashed" : "w_probe_count_hashed", st);
-    hashed<<<pass_grid(n, num_sms, mode == 1 ? kHashedProbeCtas : kHashedProbeCtas + 1, WCHUNK), WT, 0, st>>>(R.x, R.y, n, w, a_domain, cnt, total, status);
-    return cudaGetLastError();
+    return launch_after(hashed, pass_grid(n, num_sms, mode == 1 ? kHashedProbeCtas : kHashedProbeCtas + 1, WCHUNK), WT, st,
+                        R.x, R.y, n, w, a_domain, cnt, total, status);
 }
 
 }  // namespace
@@ -972,7 +984,7 @@ bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32
     }
     {
         ProfScope ps_("chain_clear", st);
-        k_chain_clear<<<num_sms * 2, WT, 0, st>>>(g);
+        if ((*e = launch_after(k_chain_clear, num_sms * 2, WT, st, g)) != cudaSuccess) return true;
     }
     HeavyArgs heavy{};
     for (int k = 0; k < nrel - 2; ++k) {
@@ -1088,7 +1100,9 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     if ((e = deg_build(T, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     if (R.n > 0) {
         ProfScope ps_("star_keys", st);
-        k_w_keys<<<pass_grid((uint32_t)R.n, num_sms, 8, 32), WT, 0, st>>>(R.y, (uint32_t)R.n, L.w[0], status);
+        if ((e = launch_after(k_w_keys, pass_grid((uint32_t)R.n, num_sms, 8, 32), WT, st, R.y, (uint32_t)R.n, L.w[0],
+                              status)) != cudaSuccess)
+            return e;
     }
     Source src{};
     src.t = L.deg;

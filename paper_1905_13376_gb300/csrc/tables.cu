@@ -428,6 +428,7 @@ __device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t most)
 // every key) and its merge 0.014 ms more; a column whose range is compact
 // needs neither.  The first CTAs sample the heavy keys (skew.h) meanwhile.
 __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
+    after_previous();
     __shared__ HeavySample<2048> hsm;
     if (blockIdx.x < g.nheavy) {
         const HeavyCol &h = g.h[blockIdx.x];
@@ -509,6 +510,7 @@ __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
 // entries of keys that occur are touched again.  A column none of whose
 // tables is hashed ends there.
 __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(SizeArgs g) {
+    after_previous();
     __shared__ unsigned int r[HLL_M];
     const SizeCol &c = g.c[blockIdx.y];
     const int32_t *keys = c.keys;
@@ -625,6 +627,7 @@ __global__ void k_hll_merge(unsigned int *__restrict__ regs, uint32_t ctas) {
 constexpr int HLL_MW = 32;   // warps of a merge CTA, each over every HLL_MW-th row
 
 __global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(SizeArgs g) {
+    after_previous();
     const SizeCol &c = g.c[blockIdx.y];
     bool all = true;   // every table of the column is direct-address: nothing was counted
     for (uint32_t q = 0; q < c.ntargets; ++q) all = all && __ldcg(c.meta[q] + kMetaDense) != 0u;
@@ -712,6 +715,7 @@ struct ClearArgs {
 };
 
 __global__ void __launch_bounds__(BT) k_tables_clear(ClearArgs g) {
+    after_previous();
     const uint64_t i0 = (uint64_t)blockIdx.x * BT + threadIdx.x, stride = (uint64_t)gridDim.x * BT;
     if (blockIdx.y == g.ntables) {
         for (uint64_t i = i0; i < g.nzero; i += stride) g.zero[i] = 0ull;
@@ -822,15 +826,16 @@ cudaError_t size_columns(const SizeCol *cols, uint32_t ncols, const HeavyCol *he
     g.ranged = allow_dense;
     if (allow_dense) {
         ProfScope ps_("key_range", st);
-        k_range<<<nheavy + ncols * g.range_rows, BT, 0, st>>>(g);
+        const cudaError_t e = launch_after(k_range, nheavy + ncols * g.range_rows, BT, st, g);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps_(hll_name, st);
-        k_hll<<<dim3(g.rows, ncols), BT, 0, st>>>(g);
+        const cudaError_t e = launch_after(k_hll, dim3(g.rows, ncols), BT, st, g);
+        if (e != cudaSuccess) return e;
     }
     ProfScope ps_(size_name, st);
-    k_hll_merge_size<<<dim3(HLL_MCTAS, ncols), HLL_MW * 32, 0, st>>>(g);
-    return cudaGetLastError();
+    return launch_after(k_hll_merge_size, dim3(HLL_MCTAS, ncols), HLL_MW * 32, st, g);
 }
 
 cudaError_t tables_clear(const ClearTable *t, uint32_t n, unsigned long long *zero, uint64_t nzero,
@@ -842,8 +847,7 @@ cudaError_t tables_clear(const ClearTable *t, uint32_t n, unsigned long long *ze
     g.nzero = nzero;
     g.total = total;
     ProfScope ps_("tables_clear", st);
-    k_tables_clear<<<dim3(num_sms * 2, n + ((nzero || total) ? 1u : 0u)), BT, 0, st>>>(g);
-    return cudaGetLastError();
+    return launch_after(k_tables_clear, dim3(num_sms * 2, n + ((nzero || total) ? 1u : 0u)), BT, st, g);
 }
 
 cudaError_t single_table_size(const int32_t *keys, int64_t n, uint32_t seed, unsigned int *hll_regs,
