@@ -115,7 +115,9 @@ __device__ __forceinline__ uint32_t cset_count(const unsigned long long *tk, uns
     return 0u;
 }
 
-__global__ void k_rg_clear(RGroup r) {
+__global__ void k_rg_clear(RGroup r, unsigned int *__restrict__ bump) {
+    after_previous();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *bump = 0u;
     const uint32_t *meta = r.meta;
     const uint32_t n = rg_entries(meta);
     const bool hashed = meta[kMetaDense] == 0u;
@@ -130,6 +132,7 @@ __global__ void k_rg_clear(RGroup r) {
 // with a_domain > 0 every a must lie in [0, a_domain).
 __global__ void __launch_bounds__(RG_T) k_rg_count(const int32_t *__restrict__ Ra, const int32_t *__restrict__ Rb,
                                                    uint32_t n, RGroup r, int32_t a_domain, DevStatus *st) {
+    after_previous();
     const uint32_t *meta = r.meta;
     const bool dense = meta[kMetaDense] != 0u;
     const uint32_t kmin = meta[kMetaMin], span = meta[kMetaSpan], mask = meta[kMetaMask];
@@ -155,6 +158,7 @@ __global__ void __launch_bounds__(RG_T) k_rg_count(const int32_t *__restrict__ R
 // lists are contiguous per key, in no particular key order); the scatter
 // advances end[i] to the list's end.
 __global__ void __launch_bounds__(RG_T) k_rg_offsets(RGroup r, unsigned int *__restrict__ bump) {
+    after_previous();
     __shared__ uint32_t scratch[33];
     __shared__ uint32_t base;
     const uint32_t n = rg_entries(r.meta);
@@ -173,6 +177,7 @@ __global__ void __launch_bounds__(RG_T) k_rg_offsets(RGroup r, unsigned int *__r
 __global__ void __launch_bounds__(RG_T) k_rg_scatter(const int32_t *__restrict__ Ra,
                                                      const int32_t *__restrict__ Rb, uint32_t n, RGroup r,
                                                      uint32_t nR, DevStatus *st) {
+    after_previous();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int idx = rg_find(r, r.meta, (uint32_t)__ldg(Rb + i));
         if (idx < 0) {
@@ -199,6 +204,7 @@ __global__ void __launch_bounds__(RG_T) k_rg_scatter(const int32_t *__restrict__
 __global__ void __launch_bounds__(RG_T) k_cc_orient(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
                                                     uint32_t n, RGroup r, int32_t *__restrict__ u,
                                                     int32_t *__restrict__ v) {
+    after_previous();
     constexpr uint32_t Q = 4;
     const uint32_t T = gridDim.x * RG_T;
     auto length = [&](uint32_t k) -> uint32_t {
@@ -256,6 +262,7 @@ __global__ void __launch_bounds__(CC_PLAN_T) k_cc_plan(const uint32_t *__restric
                                                        uint32_t schunk, uint32_t *__restrict__ items,
                                                        uint32_t *__restrict__ order,
                                                        unsigned long long *__restrict__ big_slots) {
+    after_previous();
     __shared__ uint32_t cursor[4];
     if (threadIdx.x < 4) cursor[threadIdx.x] = 0u;
     __syncthreads();
@@ -300,6 +307,7 @@ __global__ void __launch_bounds__(CC_PLAN_T) k_cc_plan(const uint32_t *__restric
 // scan's last entry).
 __global__ void k_cc_bigclear(unsigned long long *__restrict__ gs, uint32_t *__restrict__ gc,
                               const unsigned long long *__restrict__ big_off, uint32_t z) {
+    after_previous();
     const unsigned long long total = big_off[z];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -324,6 +332,7 @@ __global__ void k_cc_bigbuild(const uint2 *__restrict__ Tp, const uint32_t *__re
                               const unsigned long long *__restrict__ big_off, unsigned long long *__restrict__ gs,
                               uint32_t *__restrict__ gc, uint32_t *__restrict__ big_neg, uint32_t seed,
                               DevStatus *st) {
+    after_previous();
     __shared__ uint32_t negs;
     for (uint32_t k = blockIdx.x; k < z; k += gridDim.x) {
         const unsigned long long base = big_off[k], slots = big_off[k + 1] - base;
@@ -371,6 +380,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                                                       int32_t *__restrict__ rows, long long capacity,
                                                       unsigned long long *__restrict__ rep_set,
                                                       uint32_t *__restrict__ rep_cnt) {
+    after_previous();
     extern __shared__ __align__(16) unsigned char smraw[];
     unsigned long long *tk = (unsigned long long *)smraw;                      // CC_TSLOTS
     uint32_t *filt = (uint32_t *)(tk + CC_TSLOTS);                              // CC_FWORDS
@@ -689,6 +699,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
 
 __global__ void k_cc_rows_check(const unsigned long long *base, uint32_t z, long long capacity, long long *n_rows,
                                 DevStatus *st) {
+    after_previous();
     const unsigned long long tot = base[z];
     *n_rows = (long long)tot;
     if (tot > (unsigned long long)capacity) set_status(st, MWJ_ERR_CAPACITY, (long long)tot);
@@ -715,33 +726,30 @@ cudaError_t rgroup_build(const int32_t *Ra, const int32_t *Rb, int64_t nR, const
     cudaError_t e = single_table_size(Rb, nR, r.seed, hll, (uint32_t *)r.meta, reserve, num_sms, st, "rg_hll",
                                       "rg_size", true);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bump, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
     const uint32_t n = (uint32_t)nR;
     const unsigned grid = (unsigned)num_sms * 4;
     {
         ProfScope ps_("rg_clear", st);
-        k_rg_clear<<<grid, RG_T, 0, st>>>(r);
+        if ((e = launch_after(k_rg_clear, grid, RG_T, st, r, bump)) != cudaSuccess) return e;
     }
-    if (n == 0) return cudaGetLastError();
+    if (n == 0) return cudaSuccess;
     {
         ProfScope ps_("rg_count", st);
-        k_rg_count<<<grid, RG_T, 0, st>>>(Ra, Rb, n, r, a_domain, status);
+        if ((e = launch_after(k_rg_count, grid, RG_T, st, Ra, Rb, n, r, a_domain, status)) != cudaSuccess) return e;
     }
     {
         ProfScope ps_("rg_offsets", st);
-        k_rg_offsets<<<grid, RG_T, 0, st>>>(r, bump);
+        if ((e = launch_after(k_rg_offsets, grid, RG_T, st, r, bump)) != cudaSuccess) return e;
     }
     ProfScope ps_("rg_scatter", st);
-    k_rg_scatter<<<grid, RG_T, 0, st>>>(Ra, Rb, n, r, n, status);
-    return cudaGetLastError();
+    return launch_after(k_rg_scatter, grid, RG_T, st, Ra, Rb, n, r, n, status);
 }
 
 cudaError_t cyc_c_orient(const int32_t *Sb, const int32_t *Sc, int64_t nS, const RGroup &r, int32_t *u, int32_t *v,
                          int num_sms, cudaStream_t st) {
     if (nS <= 0) return cudaSuccess;
     ProfScope ps_("cyc_c_orient", st);
-    k_cc_orient<<<num_sms * 4, RG_T, 0, st>>>(Sb, Sc, (uint32_t)nS, r, u, v);
-    return cudaGetLastError();
+    return launch_after(k_cc_orient, num_sms * 4, RG_T, st, Sb, Sc, (uint32_t)nS, r, u, v);
 }
 
 cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsigned int *counter,
@@ -754,7 +762,8 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
     cudaError_t e;
     {
         ProfScope ps_("cyc_c_plan", st);
-        k_cc_plan<<<1, CC_PLAN_T, 0, st>>>(g.offS, g.offT, z, g.schunk, items, (uint32_t *)g.order, big_slots);
+        e = launch_after(k_cc_plan, 1, CC_PLAN_T, st, g.offS, g.offT, z, g.schunk, items, (uint32_t *)g.order, big_slots);
+        if (e != cudaSuccess) return e;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(items + z, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
@@ -765,13 +774,15 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
         return e;
     {
         ProfScope ps_("cyc_c_bigclear", st);
-        k_cc_bigclear<<<num_sms * 4, 512, 0, st>>>((unsigned long long *)g.bigset, (uint32_t *)g.bigcnt,
-                                                   g.big_off, z);
+        e = launch_after(k_cc_bigclear, num_sms * 4, 512, st, (unsigned long long *)g.bigset, (uint32_t *)g.bigcnt,
+                         g.big_off, z);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps_("cyc_c_bigbuild", st);
-        k_cc_bigbuild<<<num_sms * 2, 512, 0, st>>>(g.Tp, g.offT, z, g.big_off, (unsigned long long *)g.bigset,
-                                                   (uint32_t *)g.bigcnt, (uint32_t *)g.big_neg, g.seed, g.st);
+        e = launch_after(k_cc_bigbuild, num_sms * 2, 512, st, g.Tp, g.offT, z, g.big_off,
+                         (unsigned long long *)g.bigset, (uint32_t *)g.bigcnt, (uint32_t *)g.big_neg, g.seed, g.st);
+        if (e != cudaSuccess) return e;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const size_t smem = CC_TSLOTS * sizeof(unsigned long long) + CC_FWORDS * sizeof(uint32_t) +
@@ -793,8 +804,9 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
         return e;
     {
         ProfScope ps_("cyc_c_probe", st);
-        k_cc_probe<0><<<grid, CC_T, smem, st>>>(g, items, counter, with_rows ? bucket_rows : nullptr, nullptr, 0,
-                                                rep_set, rep_cnt);
+        e = launch_after_smem(k_cc_probe<0>, grid, CC_T, smem, st, g, items, counter, with_rows ? bucket_rows : nullptr,
+                              (int32_t *)nullptr, 0ll, rep_set, rep_cnt);
+        if (e != cudaSuccess) return e;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (!with_rows) return cudaSuccess;
@@ -803,12 +815,12 @@ cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsign
         return e;
     {
         ProfScope ps_("rows_check", st);
-        k_cc_rows_check<<<1, 1, 0, st>>>(bucket_base, z, capacity, n_rows, g.st);
+        if ((e = launch_after(k_cc_rows_check, 1, 1, st, bucket_base, z, capacity, n_rows, g.st)) != cudaSuccess) return e;
     }
     if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
     ProfScope ps_("cyc_c_rows", st);
-    k_cc_probe<1><<<grid, CC_T, smem, st>>>(g, items, counter, bucket_base, rows, capacity, rep_set, rep_cnt);
-    return cudaGetLastError();
+    return launch_after_smem(k_cc_probe<1>, grid, CC_T, smem, st, g, items, counter, bucket_base, rows, capacity, rep_set,
+                             rep_cnt);
 }
 
 }  // namespace mwj

@@ -275,6 +275,7 @@ __global__ void __launch_bounds__(FT) k_fm_probe(FmArgs g) {
 constexpr uint32_t kFmSums = 32 * FM_M + 1;
 __global__ void __launch_bounds__(FT) k_fm_estimate(const uint32_t *__restrict__ sk, int32_t a_domain,
                                                     float *__restrict__ est) {
+    after_previous();
     __shared__ float of_sum[kFmSums];
     for (uint32_t t = threadIdx.x; t < kFmSums; t += FT) of_sum[t] = (float)((FM_M / FM_PHI) * exp2((double)t / FM_M));
     __syncthreads();
@@ -337,6 +338,7 @@ struct FmIndex {
 // y 0 / 1: T's / S's rows (direct-address) or free keys and key -1's row
 // (hashed); y 2: the output sketches.
 __global__ void __launch_bounds__(FT) k_fm_clear(FmOne g, uint32_t *__restrict__ out, uint64_t out_rows) {
+    after_previous();
     const uint64_t i0 = (uint64_t)blockIdx.x * FT + threadIdx.x, stride = (uint64_t)gridDim.x * FT;
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
     if (blockIdx.y == 2) {
@@ -358,6 +360,7 @@ __global__ void __launch_bounds__(FT) k_fm_clear(FmOne g, uint32_t *__restrict__
 // Hashed: the distinct keys of a column (y 0: T's C, y 1: S's B).
 __global__ void __launch_bounds__(256) k_fm_keys(FmOne g, const int32_t *__restrict__ tc,
                                                  const int32_t *__restrict__ sb, DevStatus *st) {
+    after_previous();
     const FmRows &r = blockIdx.y ? g.s : g.t;
     if (__ldg(r.meta + kMetaDense)) return;
     const int32_t *col = blockIdx.y ? sb : tc;
@@ -374,6 +377,7 @@ __global__ void __launch_bounds__(256) k_fm_keys(FmOne g, const int32_t *__restr
 
 // Hashed: a row for every key, zeroed by the thread that gives it out.
 __global__ void __launch_bounds__(256) k_fm_rows(FmOne g) {
+    after_previous();
     const FmRows &r = blockIdx.y ? g.s : g.t;
     if (__ldg(r.meta + kMetaDense)) return;
     const uint64_t slots = (uint64_t)__ldg(r.meta + kMetaMask) + 1;
@@ -396,6 +400,7 @@ __global__ void __launch_bounds__(256) k_fm_rows(FmOne g) {
 // results are not needed; the tuples of one c share two sectors).
 __global__ void __launch_bounds__(256) k_fm_tbits(const int32_t *__restrict__ tc, const int32_t *__restrict__ td,
                                                   uint32_t n, FmRows r) {
+    after_previous();
     const uint32_t T = gridDim.x * 256;
     const FmIndex<false> index(r);
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += T) {
@@ -426,6 +431,7 @@ __global__ void __launch_bounds__(256, 4) k_fm_pass(const int32_t *__restrict__ 
                                                     uint32_t n, FmRows src, FmRows dst,
                                                                 uint32_t *__restrict__ out, int32_t a_domain,
                                                                 DevStatus *st) {
+    after_previous();
     if ((__ldg(src.meta + kMetaDense) && (OUT || __ldg(dst.meta + kMetaDense))) != DENSE) return;
     const uint32_t l4 = threadIdx.x & 3;
     const uint64_t groups = (uint64_t)gridDim.x * 64;
@@ -557,37 +563,47 @@ cudaError_t fm_one_run(const FmOneLayout &L, const mwj_rel &R, const mwj_rel &S,
     const uint64_t most = (uint64_t)(T.n > S.n ? T.n : S.n);
     {
         ProfScope ps_("fm_clear", st);
-        k_fm_clear<<<dim3(sms * 2, 3), FT, 0, st>>>(g, sketches, (uint64_t)a_domain);
+        if ((e = launch_after(k_fm_clear, dim3(sms * 2, 3), FT, st, g, sketches, (uint64_t)a_domain)) != cudaSuccess) return e;
     }
     {
         ProfScope ps_("fm_keys", st);
-        k_fm_keys<<<dim3(fm_grid(most, 256, sms, 8), 2), 256, 0, st>>>(g, T.x, S.x, status);
+        e = launch_after(k_fm_keys, dim3(fm_grid(most, 256, sms, 8), 2), 256, st, g, T.x, S.x, status);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps_("fm_rows", st);
-        k_fm_rows<<<dim3(fm_grid(4 * most, 256, sms, 8), 2), 256, 0, st>>>(g);
+        if ((e = launch_after(k_fm_rows, dim3(fm_grid(4 * most, 256, sms, 8), 2), 256, st, g)) != cudaSuccess) return e;
     }
     if (T.n > 0) {
         ProfScope ps_("fm_tbits", st);
-        k_fm_tbits<<<fm_grid(T.n, 256, sms, 8), 256, 0, st>>>(T.x, T.y, (uint32_t)T.n, g.t);
+        e = launch_after(k_fm_tbits, fm_grid(T.n, 256, sms, 8), 256, st, T.x, T.y, (uint32_t)T.n, g.t);
+        if (e != cudaSuccess) return e;
     }
     if (S.n > 0) {
         const unsigned grid = fm_grid(S.n, 64 * FM_K, sms, 8);
         {
             ProfScope ps_("fm_spass", st);
-            k_fm_pass<false, true><<<grid, 256, 0, st>>>(S.x, S.y, (uint32_t)S.n, g.t, g.s, nullptr, 0, status);
+            e = launch_after(k_fm_pass<false, true>, grid, 256, st, S.x, S.y, (uint32_t)S.n, g.t, g.s,
+                             (uint32_t *)nullptr, 0, status);
+            if (e != cudaSuccess) return e;
         }
         ProfScope ps_("fm_spass_hashed", st);
-        k_fm_pass<false, false><<<grid, 256, 0, st>>>(S.x, S.y, (uint32_t)S.n, g.t, g.s, nullptr, 0, status);
+        e = launch_after(k_fm_pass<false, false>, grid, 256, st, S.x, S.y, (uint32_t)S.n, g.t, g.s,
+                         (uint32_t *)nullptr, 0, status);
+        if (e != cudaSuccess) return e;
     }
     if (R.n > 0) {
         const unsigned grid = fm_grid(R.n, 64 * FM_K, sms, 8);
         {
             ProfScope ps_("fm_rpass", st);
-            k_fm_pass<true, true><<<grid, 256, 0, st>>>(R.x, R.y, (uint32_t)R.n, g.s, g.s, sketches, a_domain, status);
+            e = launch_after(k_fm_pass<true, true>, grid, 256, st, R.x, R.y, (uint32_t)R.n, g.s, g.s,
+                             sketches, a_domain, status);
+            if (e != cudaSuccess) return e;
         }
         ProfScope ps_("fm_rpass_hashed", st);
-        k_fm_pass<true, false><<<grid, 256, 0, st>>>(R.x, R.y, (uint32_t)R.n, g.s, g.s, sketches, a_domain, status);
+        e = launch_after(k_fm_pass<true, false>, grid, 256, st, R.x, R.y, (uint32_t)R.n, g.s, g.s,
+                         sketches, a_domain, status);
+        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }
@@ -677,8 +693,8 @@ extern "C" mwj_status mwj_fm_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel 
     auto estimate = [&]() -> mwj_status {
         if (!estimates) return MWJ_OK;
         ProfScope ps_("fm_estimate", st);
-        k_fm_estimate<<<fm_grid((uint64_t)a_domain * 4, FT, sms, 2), FT, 0, st>>>(sketches, a_domain, estimates);
-        const cudaError_t ee = cudaGetLastError();
+        const cudaError_t ee =
+            launch_after(k_fm_estimate, fm_grid((uint64_t)a_domain * 4, FT, sms, 2), FT, st, sketches, a_domain, estimates);
         return ee == cudaSuccess ? MWJ_OK : cuda_fail(ctx, ee, "fm estimate");
     };
     if (fm_one(S, T, shares)) {

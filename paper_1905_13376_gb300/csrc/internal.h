@@ -103,10 +103,12 @@ namespace mwj {
 // griddepcontrol.launch_dependents, costs what the waiting CTAs take from the
 // running ones: friends 364 us, a chain of four launches at 2^18 21 -> 28 us.)
 template <typename... P, typename... A>
-inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const A &...args) {
+inline cudaError_t launch_after_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                     const A &...args) {
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = block;
+    c.dynamicSmemBytes = smem;
     c.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -114,6 +116,10 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cud
     c.attrs = at;
     c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const A &...args) {
+    return launch_after_smem(kernel, grid, block, 0, st, args...);
 }
 
 struct Profiler;

@@ -47,6 +47,7 @@ __device__ __forceinline__ Lists lists_of(const LinRowsArgs &g, int32_t b, int32
 }
 
 __global__ void __launch_bounds__(LT) k_lrows_count(LinRowsArgs g, unsigned long long *__restrict__ chunk_rows) {
+    after_previous();
     __shared__ unsigned long long red[32];
     const uint32_t i0 = blockIdx.x * LCHUNK + threadIdx.x;
     int32_t b[LQ], c[LQ];
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(LT) k_lrows_count(LinRowsArgs g, unsigned long
 // total = n_rows = all rows; more than the capacity is an error and nothing is written.
 __global__ void k_lrows_check(const unsigned long long *base, uint32_t chunks, long long capacity, long long *n_rows,
                               unsigned long long *total, uint32_t *big_n, DevStatus *st) {
+    after_previous();
     const unsigned long long tot = base[chunks];
     *n_rows = (long long)tot;
     *total = tot;
@@ -89,6 +91,7 @@ __global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, const unsigne
                                                     uint32_t chunks, uint32_t *__restrict__ big_n,
                                                     uint32_t *__restrict__ big_i,
                                                     unsigned long long *__restrict__ big_p) {
+    after_previous();
     if (base[chunks] > (unsigned long long)g.capacity) return;   // the check recorded it
     __shared__ unsigned long long cursor;
     if (threadIdx.x == 0) cursor = base[blockIdx.x];
@@ -150,6 +153,7 @@ __global__ void __launch_bounds__(LT) k_lrows_big(LinRowsArgs g, const unsigned 
                                                   uint32_t chunks, const uint32_t *__restrict__ big_n,
                                                   const uint32_t *__restrict__ big_i,
                                                   const unsigned long long *__restrict__ big_p) {
+    after_previous();
     if (base[chunks] > (unsigned long long)g.capacity) return;
     const uint32_t n = *big_n;
     const unsigned long long T = (unsigned long long)gridDim.x * LT;
@@ -219,25 +223,26 @@ cudaError_t lin_rows_run(LinRowsLayout &L, const mwj_rel &R, const mwj_rel &S, c
     uint32_t *big_n = L.bump + 2;
     if (chunks) {
         ProfScope ps_("lin_rows_count", st);
-        k_lrows_count<<<chunks, LT, 0, st>>>(g, L.chunk_rows);
+        if ((e = launch_after(k_lrows_count, chunks, LT, st, g, L.chunk_rows)) != cudaSuccess) return e;
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = scan_excl_u64((const uint64_t *)L.chunk_rows, (uint64_t *)L.base, chunks, true, L.sscratch, st)) !=
         cudaSuccess)
         return e;
     {
         ProfScope ps_("rows_check", st);
-        k_lrows_check<<<1, 1, 0, st>>>(L.base, chunks, capacity, n_rows, total, big_n, status);
+        e = launch_after(k_lrows_check, 1, 1, st, L.base, chunks, capacity, n_rows, total, big_n, status);
+        if (e != cudaSuccess) return e;
     }
     if (chunks) {
         {
             ProfScope ps_("lin_rows", st);
-            k_lrows_write<<<chunks, LT, 0, st>>>(g, L.base, chunks, big_n, L.big_i, L.big_p);
+            if ((e = launch_after(k_lrows_write, chunks, LT, st, g, L.base, chunks, big_n, L.big_i, L.big_p)) != cudaSuccess)
+                return e;
         }
         ProfScope ps_("lin_rows_big", st);
-        k_lrows_big<<<num_sms * 4, LT, 0, st>>>(g, L.base, chunks, big_n, L.big_i, L.big_p);
+        return launch_after(k_lrows_big, num_sms * 4, LT, st, g, L.base, chunks, big_n, L.big_i, L.big_p);
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace mwj

@@ -13,6 +13,7 @@ constexpr int SC_TILE = SC_THREADS * SC_ITEMS;
 
 template <typename T>
 __global__ void k_tile_sums(const T *in, size_t n, T *sums) {
+    after_previous();
     size_t base = (size_t)blockIdx.x * SC_TILE;
     T s = 0;
     for (int k = 0; k < SC_ITEMS; ++k) {
@@ -27,6 +28,7 @@ __global__ void k_tile_sums(const T *in, size_t n, T *sums) {
 // One CTA: exclusive scan of the tile totals, in place.
 template <typename T>
 __global__ void k_scan_sums(T *sums, size_t m) {
+    after_previous();
     __shared__ unsigned long long carry_s;
     if (threadIdx.x == 0) carry_s = 0;
     __syncthreads();
@@ -64,6 +66,7 @@ __global__ void k_scan_sums(T *sums, size_t m) {
 
 template <typename T>
 __global__ void k_tile_scan(const T *in, T *out, size_t n, const T *sums, bool with_total) {
+    after_previous();
     size_t base = (size_t)blockIdx.x * SC_TILE + (size_t)threadIdx.x * SC_ITEMS;
     T v[SC_ITEMS];
     T local = 0;
@@ -116,17 +119,18 @@ cudaError_t scan_impl(const T *in, T *out, size_t n, bool with_total, void *scra
     T *sums = (T *)scratch;
     {
         ProfScope ps_("scan_tile_sums", st);
-        k_tile_sums<T><<<(unsigned)tiles, SC_THREADS, 0, st>>>(in, n, sums);
+        const cudaError_t e = launch_after(k_tile_sums<T>, (unsigned)tiles, SC_THREADS, st, in, n, sums);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps_("scan_sums", st);
-        k_scan_sums<T><<<1, SC_THREADS, 0, st>>>(sums, tiles);
+        const cudaError_t e = launch_after(k_scan_sums<T>, 1, SC_THREADS, st, sums, tiles);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps_("scan_tiles", st);
-        k_tile_scan<T><<<(unsigned)tiles, SC_THREADS, 0, st>>>(in, out, n, sums, with_total);
+        return launch_after(k_tile_scan<T>, (unsigned)tiles, SC_THREADS, st, in, out, n, sums, with_total);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace
