@@ -32,7 +32,8 @@ struct CycCLayout {
     RGroup r;
     uint32_t *rmeta;
     unsigned int *hll, *bump;
-    int32_t *su, *sv;   // self-joins: S's tuples, shorter list first
+    int32_t *su, *sv;   // self-joins: S's tuples, shorter list first,
+    int32_t *sm, *smp;  // and for rows which ones were turned, as they come and partitioned
     uint2 *Sp, *Tp;
     uint32_t *offS, *offT;
     uint32_t *items, *order;
@@ -50,10 +51,9 @@ struct CycCLayout {
 };
 
 // T holds R's pairs with the columns exchanged (triangle counting over one edge
-// list): R's lists and sets are T's.  Rows need to know b from c and take the
-// tuples as they come.
-bool cyc_self(const mwj_rel &R, const mwj_rel &T, bool rows) {
-    return !rows && R.n == T.n && R.n > 0 && R.x == T.y && R.y == T.x;
+// list): R's lists and sets are T's.
+bool cyc_self(const mwj_rel &R, const mwj_rel &T) {
+    return R.n == T.n && R.n > 0 && R.x == T.y && R.y == T.x;
 }
 
 size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, bool rows,
@@ -67,9 +67,11 @@ size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, co
     L.r.deg = A.take<uint32_t>(reserve + 2);
     L.r.end = A.take<uint32_t>(reserve + 2);
     L.r.alist = A.take<int32_t>(R.n + 4);
-    const bool self = cyc_self(R, T, rows);
+    const bool self = cyc_self(R, T);
     L.su = self ? A.take<int32_t>(S.n + 4) : nullptr;
     L.sv = self ? A.take<int32_t>(S.n + 4) : nullptr;
+    L.sm = self && rows ? A.take<int32_t>(S.n + 4) : nullptr;
+    L.smp = self && rows ? A.take<int32_t>(S.n + 4) : nullptr;
     L.Sp = A.take<uint2>(S.n + 2);
     L.offS = A.take<uint32_t>(z + 1);
     L.Tp = A.take<uint2>(T.n + 2);
@@ -269,15 +271,15 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
         e = rgroup_build(R.x, R.y, R.n, LC.r, LC.hll, single_table_slots(R.n), LC.bump,
                          out->mode == MWJ_COUNT_GROUP_BY_A ? out->a_domain : 0, ctx->status, ctx->dev.num_sms, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group R by B");
-        const bool self = cyc_self(R, T, rows);
+        const bool self = cyc_self(R, T);
         if (self) {
-            e = cyc_c_orient(S.x, S.y, S.n, LC.r, LC.su, LC.sv, ctx->dev.num_sms, st);
+            e = cyc_c_orient(S.x, S.y, S.n, LC.r, LC.su, LC.sv, LC.sm, ctx->dev.num_sms, st);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "orient S");
         }
         PartSpec ps{1, sd.C, p.z, -1, 0, 1};
         ps.st = ctx->status;
-        e = part_run(self ? LC.su : S.x, self ? LC.sv : S.y, S.n, ps, PAY_PAIR, LC.Sp, LC.offS, LC.pscratch, LC.pscratch_bytes,
-                     ctx->dev.num_sms, st);
+        e = part_run(self ? LC.su : S.x, self ? LC.sv : S.y, S.n, ps, PAY_PAIR, LC.Sp, LC.offS, LC.pscratch,
+                     LC.pscratch_bytes, ctx->dev.num_sms, st, LC.sm, LC.smp);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "partition S");
         PartSpec pt{0, sd.C, p.z, -1, 0, 1};
         pt.st = ctx->status;
@@ -289,6 +291,7 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
         g.Sp = LC.Sp; g.offS = LC.offS; g.Tp = LC.Tp; g.offT = LC.offT;
         g.z = p.z;
         g.order = LC.order;
+        g.turned = LC.smp;
         g.schunk = cyc_c_schunk(S.n, ctx->dev.num_sms);
         g.big_off = LC.big_off;
         g.bigset = LC.bigset;

@@ -38,6 +38,7 @@ struct CycCArgs {
     RGroup r;
     const uint2 *Sp;            // S grouped by F(c): (b, c)
     const uint32_t *offS;       // z + 1
+    const int32_t *turned;      // row output of a self-join: S's tuples that are (c, b), or null
     const uint2 *Tp;            // T grouped by F(c): (c, a)
     const uint32_t *offT;       // z + 1
     uint32_t z;
@@ -70,9 +71,10 @@ cudaError_t rgroup_build(const int32_t *Ra, const int32_t *Rb, int64_t nR, const
                          uint64_t reserve, unsigned int *bump, int32_t a_domain, DevStatus *status, int num_sms,
                          cudaStream_t st);
 // S's tuples (b, c) with the end whose list in r is shorter first: u, v of nS
-// entries each.  Self-joins only (R's lists are T's), and not for row output.
+// entries each; turned (row output, or null): 1 for those that are (c, b) now.
+// Self-joins only (R's lists are T's).
 cudaError_t cyc_c_orient(const int32_t *Sb, const int32_t *Sc, int64_t nS, const RGroup &r, int32_t *u, int32_t *v,
-                         int num_sms, cudaStream_t st);
+                         int32_t *turned, int num_sms, cudaStream_t st);
 // items: z + 1 u32; big_slots: z u64 (scanned into g.big_off, z + 2 u64,
 // with scan_tmp64b); g.bigset: 4 |T| + 16 u64 slots, g.bigcnt as many u32;
 // g.big_neg: z u32;

@@ -37,6 +37,7 @@ constexpr int RG_T = 512;                // threads of the grouping kernels
 constexpr uint32_t CC_QCAP = 768;        // long R lists queued per work item
 constexpr uint32_t CC_CH = 1024;         // wedges of a list per warp step (32 per lane, one mask word)
 constexpr uint32_t kQueueMin = 512;      // lists this long go to the item's queue
+constexpr uint32_t kTurned = 0x80000000u;   // row output: mark of a turned tuple, in its list's start
 constexpr uint32_t CC_SCHUNK_MIN = 32;   // S tuples of a bucket's work item, at least (a warp's batch)
 
 __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
@@ -200,10 +201,12 @@ __global__ void __launch_bounds__(RG_T) k_rg_scatter(const int32_t *__restrict__
 // sum of min(|R[b]|, |T[c]|) wedges instead of sum of |R[b]| (0.42 of them on the
 // power-law graphs).  Two list lengths per tuple, read in one pass over S
 // (0.34 ms for 6.7e7 tuples); the probe goes from 38 to 25 ms on the
-// 2^22-vertex graph, the call from 45 to 31.
+// 2^22-vertex graph, the call from 45 to 31.  Row output carries a mark of the
+// turned tuples: 7.6e6 triangles of a 2^20-edge graph, both passes, 7.3 to 6.4 ms
+// with the sort of the rows.
 __global__ void __launch_bounds__(RG_T) k_cc_orient(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
                                                     uint32_t n, RGroup r, int32_t *__restrict__ u,
-                                                    int32_t *__restrict__ v) {
+                                                    int32_t *__restrict__ v, int32_t *__restrict__ turned) {
     after_previous();
     constexpr uint32_t Q = 4;
     const uint32_t T = gridDim.x * RG_T;
@@ -230,6 +233,7 @@ __global__ void __launch_bounds__(RG_T) k_cc_orient(const int32_t *__restrict__ 
             const bool turn = lc[q] < lb[q];
             u[i + q * T] = turn ? c[q] : b[q];
             v[i + q * T] = turn ? b[q] : c[q];
+            if (turned) turned[i + q * T] = turn;
         }
     }
 }
@@ -491,7 +495,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         // PASS 1 writes the rows, reserving the warp's positions at once.
         // Every lane of the warp calls this.
         unsigned long long acc = 0;
-        auto emit = [&](uint32_t a, uint32_t b, uint32_t c, uint32_t m) {
+        auto emit = [&](uint32_t a, uint32_t b, uint32_t c, uint32_t m, bool turned) {
             if (PASS == 0) {
                 acc += m;
                 if (g.cnt && m && a < (uint32_t)g.a_domain) atomicAdd(g.cnt + a, (unsigned long long)m);
@@ -513,8 +517,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 if (p < (unsigned long long)capacity) {
                     int32_t *row = rows + 3 * p;
                     row[0] = (int32_t)a;
-                    row[1] = (int32_t)b;
-                    row[2] = (int32_t)c;
+                    row[1] = (int32_t)(turned ? c : b);
+                    row[2] = (int32_t)(turned ? b : c);
                 } else {
                     set_status(g.st, MWJ_ERR_CHECK, 25);
                 }
@@ -542,7 +546,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         auto walk = [&](uint32_t jb, uint32_t jc, uint32_t jst, uint32_t lo, uint32_t hi) {
             const uint32_t ch = chash(jc, g.seed);
             for (uint32_t base = lo; base < hi; base += CC_CH) {
-                const int32_t *list = g.r.alist + jst + base + lane;
+                const int32_t *list = g.r.alist + (PASS == 1 ? jst & ~kTurned : jst) + base + lane;
                 const uint32_t n = min(hi - base, CC_CH);
                 uint32_t hits = 0, s = 0;
                 for (; (s + 4u) * 32u <= n; s += 4u) {
@@ -571,7 +575,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                         a = (uint32_t)__ldg(list + 32u * q);
                         m = count(jc, a, ch);
                     }
-                    emit(a, jb, jc, m);
+                    emit(a, jb, jc, m, PASS == 1 && (jst & kTurned));
                 }
                 __syncwarp();
             }
@@ -597,6 +601,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 if (e >= 0) {
                     n = __ldg(g.r.deg + e);
                     st = __ldg(g.r.end + e) - n;
+                    if (PASS == 1 && g.turned && __ldg(g.turned + idx)) st |= kTurned;
                 }
             }
             bool spill = false;
@@ -647,11 +652,11 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 const uint32_t oex = __shfl_sync(0xffffffffu, excl, olo);
                 uint32_t a = 0, m = 0;
                 if (wi < W) {
-                    a = (uint32_t)__ldg(g.r.alist + ost + (wi - oex));
+                    a = (uint32_t)__ldg(g.r.alist + (PASS == 1 ? ost & ~kTurned : ost) + (wi - oex));
                     const uint32_t ch = chash(oc, g.seed);
                     if (fbit(filt, a, ch)) m = count(oc, a, ch);
                 }
-                emit(a, ob, oc, m);
+                emit(a, ob, oc, m, PASS == 1 && (ost & kTurned));
             }
         }
         __syncthreads();
@@ -746,10 +751,10 @@ cudaError_t rgroup_build(const int32_t *Ra, const int32_t *Rb, int64_t nR, const
 }
 
 cudaError_t cyc_c_orient(const int32_t *Sb, const int32_t *Sc, int64_t nS, const RGroup &r, int32_t *u, int32_t *v,
-                         int num_sms, cudaStream_t st) {
+                         int32_t *turned, int num_sms, cudaStream_t st) {
     if (nS <= 0) return cudaSuccess;
     ProfScope ps_("cyc_c_orient", st);
-    return launch_after(k_cc_orient, num_sms * 4, RG_T, st, Sb, Sc, (uint32_t)nS, r, u, v);
+    return launch_after(k_cc_orient, num_sms * 4, RG_T, st, Sb, Sc, (uint32_t)nS, r, u, v, turned);
 }
 
 cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsigned int *counter,
