@@ -17,7 +17,7 @@
 //               and then writes each bucket's run with consecutive threads on
 //               consecutive addresses, so the scattered output is written in
 //               full sectors; for more than 4096 buckets the tile sort is
-//               skipped and tuples go straight to their cursor.
+//               skipped and tuples go straight to their bucket's cursor.
 //
 // The order of tuples inside a bucket is not specified (atomics decide it);
 // consumers never depend on it.
@@ -498,49 +498,70 @@ __global__ void __launch_bounds__(PT, 2) k_part_scatter_wc(
     }
 }
 
-// K3 (P > 4096): direct scatter through shared-memory cursors.
-template <int PAY>
+// K3 (P > 4096): direct scatter.  A tile's tuples are too few per bucket to be
+// sorted into runs, so every tuple goes straight to its bucket; what counts is
+// that the sectors the tuples land in fill up while they are in the L2.  The
+// CTAs share one cursor per bucket (the scanned count of CTA 0, the bucket's
+// start): a tile counts its buckets in shared memory, the first tuple of each
+// takes the run with one atomic, and P open sectors are written to at a time.
+// With a cursor per bucket and CTA, P x CTAs sectors were open, more than the L2
+// holds, and 6.7e7 pairs into 1e4 buckets took 1.9 ms; now 1.1.
+// z, outz: a third carried column, for pairs (the cascade's second cyclic join
+// partitions I(a,b,c) by (c,a) and carries b), any P.
+template <int PAY, bool Z>
 __global__ void __launch_bounds__(PT) k_part_scatter_direct(
     const int32_t *__restrict__ x, const int32_t *__restrict__ y, uint32_t n, PartSpec sp,
-    uint32_t tiles_per_cta, const uint32_t *__restrict__ scanned,
-    typename PayT<PAY>::T *__restrict__ out) {
+    uint32_t tiles_per_cta, uint32_t *__restrict__ scanned, typename PayT<PAY>::T *__restrict__ out,
+    const int32_t *__restrict__ z, int32_t *__restrict__ outz) {
     __shared__ uint32_t hbuf[kHeavySlots];
     const uint32_t *hs = heavy_to_smem(sp.heavy, hbuf);
-    extern __shared__ uint32_t cur[];
+    extern __shared__ uint32_t cnt[];
     const uint32_t P = sp.P();
     const uint32_t G = gridDim.x;
-    for (uint32_t b = threadIdx.x; b < P; b += PT) cur[b] = scanned[(size_t)b * G + blockIdx.x];
+    for (uint32_t b = threadIdx.x; b < P; b += PT) cnt[b] = 0;
     __syncthreads();
-    Chunk c = cta_chunk(n, tiles_per_cta);
-    for (uint32_t i = c.begin + threadIdx.x; i < c.end; i += PT) {
-        int32_t xv = __ldg(x + i), yv = __ldg(y + i);
-        if (sp.dom && (uint32_t)xv >= sp.dom && sp.st) set_status(sp.st, MWJ_ERR_DOMAIN, xv);
-        uint32_t b = bucket_tuple(xv, yv, sp, hs);
-        uint32_t p = atomicAdd(&cur[b], 1u);
-        out[p] = make_pay<PAY>(xv, yv);
-    }
-}
-
-// K3 with a third carried column z (pairs + z, direct scatter): the cascade's
-// second cyclic join partitions I(a,b,c) by (c,a) and carries b.
-__global__ void __launch_bounds__(PT) k_part_scatter_z(
-    const int32_t *__restrict__ x, const int32_t *__restrict__ y, const int32_t *__restrict__ z,
-    uint32_t n, PartSpec sp, uint32_t tiles_per_cta, const uint32_t *__restrict__ scanned,
-    uint2 *__restrict__ out, int32_t *__restrict__ outz) {
-    __shared__ uint32_t hbuf[kHeavySlots];
-    const uint32_t *hs = heavy_to_smem(sp.heavy, hbuf);
-    extern __shared__ uint32_t cur[];
-    const uint32_t P = sp.P();
-    const uint32_t G = gridDim.x;
-    for (uint32_t b = threadIdx.x; b < P; b += PT) cur[b] = scanned[(size_t)b * G + blockIdx.x];
-    __syncthreads();
-    Chunk c = cta_chunk(n, tiles_per_cta);
-    for (uint32_t i = c.begin + threadIdx.x; i < c.end; i += PT) {
-        int32_t xv = __ldg(x + i), yv = __ldg(y + i);
-        uint32_t b = bucket_tuple(xv, yv, sp, hs);
-        uint32_t p = atomicAdd(&cur[b], 1u);
-        out[p] = make_uint2((uint32_t)xv, (uint32_t)yv);
-        outz[p] = __ldg(z + i);
+    const Chunk c = cta_chunk(n, tiles_per_cta);
+    for (uint32_t t0 = c.begin; t0 < c.end; t0 += TILE) {
+        int32_t xs[IPT], ys[IPT];
+        uint32_t bk[IPT], rk[IPT];
+#pragma unroll
+        for (int j = 0; j < IPT; ++j) {
+            const uint32_t i = t0 + j * PT + threadIdx.x;
+            xs[j] = i < c.end ? __ldg(x + i) : 0;
+            ys[j] = i < c.end ? __ldg(y + i) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < IPT; ++j) {
+            bk[j] = rk[j] = 0u;
+            if (t0 + j * PT + threadIdx.x >= c.end) continue;
+            if (!Z && sp.dom && (uint32_t)xs[j] >= sp.dom && sp.st) set_status(sp.st, MWJ_ERR_DOMAIN, xs[j]);
+            bk[j] = bucket_tuple(xs[j], ys[j], sp, hs);
+            rk[j] = atomicAdd(&cnt[bk[j]], 1u);
+        }
+        __syncthreads();
+        uint32_t base[IPT];
+#pragma unroll
+        for (int j = 0; j < IPT; ++j) {
+            const bool first = rk[j] == 0u && t0 + j * PT + threadIdx.x < c.end;
+            base[j] = first ? atomicAdd(&scanned[(size_t)bk[j] * G], cnt[bk[j]]) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < IPT; ++j)
+            if (rk[j] == 0u && t0 + j * PT + threadIdx.x < c.end) cnt[bk[j]] = base[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < IPT; ++j) {
+            const uint32_t i = t0 + j * PT + threadIdx.x;
+            if (i >= c.end) continue;
+            const uint32_t p = cnt[bk[j]] + rk[j];
+            out[p] = make_pay<PAY>(xs[j], ys[j]);
+            if (Z) outz[p] = __ldg(z + i);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < IPT; ++j)
+            if (rk[j] == 0u && t0 + j * PT + threadIdx.x < c.end) cnt[bk[j]] = 0;
+        __syncthreads();
     }
 }
 
@@ -566,7 +587,7 @@ size_t hist_smem(uint32_t P, bool warp_private) {
 
 template <int PAY>
 cudaError_t scatter_launch(const int32_t *x, const int32_t *y, uint32_t n, const PartSpec &sp,
-                           Geometry g, const uint32_t *scanned, void *out, cudaStream_t st) {
+                           Geometry g, uint32_t *scanned, void *out, cudaStream_t st) {
     using T = typename PayT<PAY>::T;
     const uint32_t P = sp.P();
     if (P <= kWcMaxP) {
@@ -588,12 +609,12 @@ cudaError_t scatter_launch(const int32_t *x, const int32_t *y, uint32_t n, const
         kern<<<g.G, PT, smem, st>>>(x, y, n, sp, g.tiles_per_cta, scanned, (T *)out);
     } else {
         size_t smem = P * sizeof(uint32_t);
-        auto kern = k_part_scatter_direct<PAY>;
+        auto kern = k_part_scatter_direct<PAY, false>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
         ProfScope ps_("part_scatter_direct", st);
-        kern<<<g.G, PT, smem, st>>>(x, y, n, sp, g.tiles_per_cta, scanned, (T *)out);
+        kern<<<g.G, PT, smem, st>>>(x, y, n, sp, g.tiles_per_cta, scanned, (T *)out, nullptr, nullptr);
     }
     return cudaGetLastError();
 }
@@ -633,8 +654,8 @@ cudaError_t part_run(const int32_t *x, const int32_t *y, int64_t n64, const Part
                              : P * sizeof(uint32_t);
         const void *kern = staged ? (pair ? (const void *)k_part_scatter_staged<PAY_PAIR>
                                           : (const void *)k_part_scatter_staged<PAY_X>)
-                                  : (pair ? (const void *)k_part_scatter_direct<PAY_PAIR>
-                                          : (const void *)k_part_scatter_direct<PAY_X>);
+                                  : (pair ? (const void *)k_part_scatter_direct<PAY_PAIR, false>
+                                          : (const void *)k_part_scatter_direct<PAY_X, false>);
         if (P <= kWcMaxP && !z) {
             smem = pair ? wc_smem<PAY_PAIR>(P) : wc_smem<PAY_X>(P);
             kern = pair ? (const void *)k_part_scatter_wc<PAY_PAIR> : (const void *)k_part_scatter_wc<PAY_X>;
@@ -669,11 +690,11 @@ cudaError_t part_run(const int32_t *x, const int32_t *y, int64_t n64, const Part
     if (!need_x) x = y;
     if (z) {
         size_t smem = P * sizeof(uint32_t);
-        e = cudaFuncSetAttribute(k_part_scatter_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        auto kern = k_part_scatter_direct<PAY_PAIR, true>;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         ProfScope ps_("part_scatter_z", st);
-        k_part_scatter_z<<<g.G, PT, smem, st>>>(x, y, z, n, sp, g.tiles_per_cta, counts, (uint2 *)out,
-                                                outz);
+        kern<<<g.G, PT, smem, st>>>(x, y, n, sp, g.tiles_per_cta, counts, (uint2 *)out, z, outz);
         return cudaGetLastError();
     }
     switch (payload) {
