@@ -51,12 +51,13 @@ struct CycCLayout {
 };
 
 // T holds R's pairs with the columns exchanged (triangle counting over one edge
-// list): R's lists and sets are T's.
+// list): R's lists and sets are T's.  Taken where the workspace has room for the
+// turned tuples: one sized for other buffers of the same lengths serves too.
 bool cyc_self(const mwj_rel &R, const mwj_rel &T) {
     return R.n == T.n && R.n > 0 && R.x == T.y && R.y == T.x;
 }
 
-size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, bool rows,
+size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, bool self, bool rows,
                     int num_sms, CycCLayout &L) {
     const size_t reserve = single_table_slots(R.n);
     L.rmeta = A.take<uint32_t>(kMetaWords);
@@ -67,7 +68,6 @@ size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, co
     L.r.deg = A.take<uint32_t>(reserve + 2);
     L.r.end = A.take<uint32_t>(reserve + 2);
     L.r.alist = A.take<int32_t>(R.n + 4);
-    const bool self = cyc_self(R, T);
     L.su = self ? A.take<int32_t>(S.n + 4) : nullptr;
     L.sv = self ? A.take<int32_t>(S.n + 4) : nullptr;
     L.sm = self && rows ? A.take<int32_t>(S.n + 4) : nullptr;
@@ -220,7 +220,7 @@ mwj_status cyc_workspace(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, const
     Arena A(nullptr, 0);
     if (p.cbuckets()) {
         CycCLayout L;
-        *bytes = cyc_c_layout(A, p.z, R, S, T, mode == MWJ_MATERIALIZE, ctx->dev.num_sms, L);
+        *bytes = cyc_c_layout(A, p.z, R, S, T, cyc_self(R, T), mode == MWJ_MATERIALIZE, ctx->dev.num_sms, L);
         return MWJ_OK;
     }
     CycLayout L;
@@ -249,10 +249,17 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
     Arena A(workspace, ws_bytes);
     CycLayout L;
     CycCLayout LC;
-    if (p.cbuckets())
-        cyc_c_layout(A, p.z, R, S, T, rows, ctx->dev.num_sms, LC);
-    else
+    bool self = cyc_self(R, T);
+    if (p.cbuckets()) {
+        cyc_c_layout(A, p.z, R, S, T, self, rows, ctx->dev.num_sms, LC);
+        if (A.overflow && self) {
+            self = false;
+            A = Arena(workspace, ws_bytes);
+            cyc_c_layout(A, p.z, R, S, T, self, rows, ctx->dev.num_sms, LC);
+        }
+    } else {
         cyc_layout(A, p, R, S, T, rows, ctx->dev.num_sms, L);
+    }
     if (A.overflow || !workspace)
         return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
 
@@ -271,7 +278,6 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
         e = rgroup_build(R.x, R.y, R.n, LC.r, LC.hll, single_table_slots(R.n), LC.bump,
                          out->mode == MWJ_COUNT_GROUP_BY_A ? out->a_domain : 0, ctx->status, ctx->dev.num_sms, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group R by B");
-        const bool self = cyc_self(R, T);
         if (self) {
             e = cyc_c_orient(S.x, S.y, S.n, LC.r, LC.su, LC.sv, LC.sm, ctx->dev.num_sms, st);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "orient S");

@@ -99,3 +99,29 @@ def test_self_join_takes_the_shorter_list(ctx, seed):
             rows = oracle.cyclic((a, b), own, (b, a), oracle.MATERIALIZE, capacity=n_rows)["rows"]
             got = ctx.join3_cyclic((x, y), dev, (y, x), "rows", capacity=n_rows)
             assert np.array_equal(sorted_rows(got["rows"].cpu().numpy()), rows)
+
+
+@pytest.mark.parametrize("mode", ["count", "rows"])
+def test_self_join_in_a_workspace_of_other_buffers(ctx, mode):
+    """A workspace sized for equal relations in buffers of their own has no room
+    for the turned tuples; the self-join takes it all the same."""
+    import ctypes
+    import torch
+    g = np.random.default_rng(5)
+    a, b = (g.integers(0, 3000, 40_000).astype(np.int32) for _ in range(2))
+    x, y = cu((a, b))
+    m = binding.MODES[mode]
+    nb = ctx.workspace_size(binding.MWJ_CYCLIC, (x, y), (x, y), (y.clone(), x.clone()), mode=m)
+    assert nb < ctx.workspace_size(binding.MWJ_CYCLIC, (x, y), (x, y), (y, x), mode=m)
+    want = oracle.cyclic((a, b), (a, b), (b, a), oracle.MATERIALIZE, capacity=200_000)
+    o, res = ctx._outputs(m, None, 200_000, 3)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    hs = torch.cuda.current_stream().cuda_stream
+    rel = binding._rel
+    ctx._check(ctx.lib.mwj_join3_cyclic(ctx.h, rel((x, y)), rel((x, y)), rel((y, x)), None, ctypes.byref(o),
+                                        ws.data_ptr(), nb, hs))
+    ctx._check(ctx.lib.mwj_stream_status(ctx.h, hs))
+    assert int(res["total"].item()) == want["total"]
+    if mode == "rows":
+        n = int(res["n_rows"].item())
+        assert np.array_equal(sorted_rows(res["rows"][:n].cpu().numpy()), want["rows"][:n])
