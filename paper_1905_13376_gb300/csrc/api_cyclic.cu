@@ -44,8 +44,6 @@ struct CycCLayout {
     unsigned long long *rep_set;   // the probe CTAs' regions for chunks that repeat (c, a) pairs
     uint32_t *rep_cnt;
     void *scan_tmp64b;
-    unsigned long long *bucket_rows, *bucket_base;
-    void *scan_tmp64;
     void *pscratch;
     size_t pscratch_bytes;
 };
@@ -88,14 +86,6 @@ size_t cyc_c_layout(Arena &A, uint32_t z, const mwj_rel &R, const mwj_rel &S, co
     L.rep_cnt = A.take<uint32_t>(cyc_c_rep_slots(num_sms));
     L.big_neg = A.take<uint32_t>(z + 1);
     L.scan_tmp64b = A.take<char>(scan_scratch_bytes(z + 1));
-    if (rows) {
-        L.bucket_rows = A.take<unsigned long long>(z + 1);
-        L.bucket_base = A.take<unsigned long long>(z + 2);
-        L.scan_tmp64 = A.take<char>(scan_scratch_bytes(z + 1));
-    } else {
-        L.bucket_rows = L.bucket_base = nullptr;
-        L.scan_tmp64 = nullptr;
-    }
     size_t ps = part_scratch_bytes(S.n, z, num_sms);
     const size_t ps2 = part_scratch_bytes(T.n, z, num_sms);
     if (ps2 > ps) ps = ps2;
@@ -308,8 +298,8 @@ extern "C" mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
         g.cnt = out->mode == MWJ_COUNT_GROUP_BY_A ? (unsigned long long *)out->group_counts : nullptr;
         g.total = (unsigned long long *)out->total;
         g.st = ctx->status;
-        e = cyc_c_run(g, LC.items, LC.scan_tmp, LC.counter, LC.big_slots, LC.scan_tmp64b, LC.bucket_rows,
-                      LC.bucket_base, LC.scan_tmp64, rows ? out->rows : nullptr, rows ? out->capacity : 0,
+        e = cyc_c_run(g, LC.items, LC.scan_tmp, LC.counter, LC.big_slots, LC.scan_tmp64b,
+                      rows ? out->rows : nullptr, rows ? out->capacity : 0,
                       rows ? (long long *)out->n_rows : nullptr, LC.rep_set, LC.rep_cnt, ctx->dev.num_sms, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cyclic probe");
         return MWJ_OK;

@@ -78,11 +78,9 @@ cudaError_t cyc_c_orient(const int32_t *Sb, const int32_t *Sc, int64_t nS, const
 // items: z + 1 u32; big_slots: z u64 (scanned into g.big_off, z + 2 u64,
 // with scan_tmp64b); g.bigset: 4 |T| + 16 u64 slots, g.bigcnt as many u32;
 // g.big_neg: z u32;
-// bucket_rows: z + 1 u64, bucket_base: z + 2 u64 (row output); rep_set,
-// rep_cnt: cyc_c_rep_slots(num_sms) u64 and u32.
+// rep_set, rep_cnt: cyc_c_rep_slots(num_sms) u64 and u32; n_rows: row output, or null.
 cudaError_t cyc_c_run(const CycCArgs &g, uint32_t *items, void *scan_tmp, unsigned int *counter,
-                      unsigned long long *big_slots, void *scan_tmp64b, unsigned long long *bucket_rows,
-                      unsigned long long *bucket_base, void *scan_tmp64, int32_t *rows, long long capacity,
+                      unsigned long long *big_slots, void *scan_tmp64b, int32_t *rows, long long capacity,
                       long long *n_rows, unsigned long long *rep_set, uint32_t *rep_cnt, int num_sms,
                       cudaStream_t st);
 

@@ -125,3 +125,21 @@ def test_self_join_in_a_workspace_of_other_buffers(ctx, mode):
     if mode == "rows":
         n = int(res["n_rows"].item())
         assert np.array_equal(sorted_rows(res["rows"][:n].cpu().numpy()), want["rows"][:n])
+
+
+@pytest.mark.parametrize("copies", [1, 31, 33, 400])
+def test_rows_staged_and_not(ctx, copies):
+    """Row output at the staging's edges: pairs of T repeated below and above the
+    32 rows that a warp stages, and a capacity that all but one row fits."""
+    g = np.random.default_rng(copies)
+    a, b, c = (g.integers(0, 200, 900).astype(np.int32) for _ in range(3))
+    T = (np.repeat(c[:100], copies), np.repeat(a[:100], copies))
+    R, S = (a, b), (b, c)
+    want = oracle.cyclic(R, S, T, oracle.COUNT)["total"]
+    rows = oracle.cyclic(R, S, T, oracle.MATERIALIZE, capacity=want)["rows"]
+    got = ctx.join3_cyclic(cu(R), cu(S), cu(T), "rows", shares=(1, 1, 4), capacity=want)
+    assert int(got["n_rows"].item()) == want and int(got["total"].item()) == want
+    assert np.array_equal(sorted_rows(got["rows"].cpu().numpy()), rows)
+    with pytest.raises(binding.MwjError) as ei:
+        ctx.join3_cyclic(cu(R), cu(S), cu(T), "rows", shares=(1, 1, 4), capacity=want - 1)
+    assert ei.value.status == binding.MWJ_ERR_CAPACITY and str(want) in str(ei.value)
