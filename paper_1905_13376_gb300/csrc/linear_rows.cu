@@ -2,12 +2,15 @@
 // bucket on each side.
 //
 // R is grouped by B (b -> [a]) and T by C (c -> [d]) in global memory, both read
-// through the L2 by every SM (rgroup_build), and S is streamed past them twice
+// through the L2 by every SM (rgroup_build), and S is streamed past them once
 // without being partitioned: an S tuple (b, c) makes |R[b]| |T[c]| rows.
 //
-//   pass 1  rows of every chunk of S            -> scan: where a chunk's rows start
-//   pass 2  the rows; tuples that make more than kBigRows are set aside
-//   pass 3  the rows of those, one tuple at a time by the whole GPU
+//   pass 1  the rows of every chunk of S, at the place that one atomic on the
+//           number of rows reserves for the chunk; tuples that make more than
+//           kBigRows are set aside
+//   pass 2  the rows of those, one tuple at a time by the whole GPU
+//
+// Rows past the capacity are counted only.
 //
 // A warp lays the rows of its 32 tuples side by side and writes 32 consecutive
 // ones per step, so that the output, most of the traffic, is written in whole
@@ -15,7 +18,8 @@
 //
 // 2^21 R, 2^22 S and 2^20 T tuples, 2^23 rows: the partitioned plan (R and S by
 // H(B), T's bucket images with lists, rows per bucket) took 0.77 ms in 25
-// launches, this one 0.34 ms in 21.  The lists cost about as much as the
+// launches, this one 0.29 ms in 17 (0.34 with a pass of its own that counts every
+// chunk's rows and a scan that places them).  The lists cost about as much as the
 // partitions did, but S is not moved and a row is not looked for in a
 // shared-memory table.
 #include "api_internal.h"
@@ -46,56 +50,17 @@ __device__ __forceinline__ Lists lists_of(const LinRowsArgs &g, int32_t b, int32
     return l;
 }
 
-__global__ void __launch_bounds__(LT) k_lrows_count(LinRowsArgs g, unsigned long long *__restrict__ chunk_rows) {
-    after_previous();
-    __shared__ unsigned long long red[32];
-    const uint32_t i0 = blockIdx.x * LCHUNK + threadIdx.x;
-    int32_t b[LQ], c[LQ];
-#pragma unroll
-    for (uint32_t q = 0; q < LQ; ++q) {
-        const uint32_t i = i0 + q * LT;
-        b[q] = i < g.n ? __ldg(g.sb + i) : 0;
-        c[q] = i < g.n ? __ldg(g.sc + i) : 0;
-    }
-    unsigned long long acc = 0;
-#pragma unroll
-    for (uint32_t q = 0; q < LQ; ++q) {
-        if (i0 + q * LT >= g.n) continue;
-        const Lists l = lists_of(g, b[q], c[q]);
-        acc += (unsigned long long)l.nr * l.nt;
-    }
-    acc = block_sum_u64(acc, red);
-    if (threadIdx.x == 0) chunk_rows[blockIdx.x] = acc;
-}
-
-// total = n_rows = all rows; more than the capacity is an error and nothing is written.
-__global__ void k_lrows_check(const unsigned long long *base, uint32_t chunks, long long capacity, long long *n_rows,
-                              unsigned long long *total, uint32_t *big_n, DevStatus *st) {
-    after_previous();
-    const unsigned long long tot = base[chunks];
-    *n_rows = (long long)tot;
-    *total = tot;
-    *big_n = 0u;
-    if (tot > (unsigned long long)capacity) set_status(st, MWJ_ERR_CAPACITY, (long long)tot);
-}
-
 __device__ __forceinline__ void put_row(const LinRowsArgs &g, unsigned long long p, int32_t a, int32_t b, int32_t c,
                                         int32_t d) {
-    if (p < (unsigned long long)g.capacity)
-        g.rows[p] = make_int4(a, b, c, d);
-    else   // the two passes disagree: record it, write nothing
-        set_status(g.st, MWJ_ERR_CHECK, (long long)p);
+    if (p < (unsigned long long)g.capacity) g.rows[p] = make_int4(a, b, c, d);
 }
 
-__global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, const unsigned long long *__restrict__ base,
-                                                    uint32_t chunks, uint32_t *__restrict__ big_n,
-                                                    uint32_t *__restrict__ big_i,
+__global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, unsigned long long *__restrict__ n_rows,
+                                                    uint32_t *__restrict__ big_n, uint32_t *__restrict__ big_i,
                                                     unsigned long long *__restrict__ big_p) {
     after_previous();
-    if (base[chunks] > (unsigned long long)g.capacity) return;   // the check recorded it
     __shared__ unsigned long long cursor;
-    if (threadIdx.x == 0) cursor = base[blockIdx.x];
-    __syncthreads();
+    __shared__ unsigned long long red[32];
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t i0 = blockIdx.x * LCHUNK + threadIdx.x;
     int32_t b[LQ], c[LQ];
@@ -108,6 +73,12 @@ __global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, const unsigne
     }
 #pragma unroll
     for (uint32_t q = 0; q < LQ; ++q) l[q] = i0 + q * LT < g.n ? lists_of(g, b[q], c[q]) : Lists{0u, 0u, 0u, 0u};
+    unsigned long long all = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < LQ; ++q) all += (unsigned long long)l[q].nr * l[q].nt;
+    all = block_sum_u64(all, red);
+    if (threadIdx.x == 0 && all) cursor = atomicAdd(n_rows, all);
+    __syncthreads();
 #pragma unroll
     for (uint32_t q = 0; q < LQ; ++q) {
         // the warp's rows: the small tuples' first, in lane order, then the big ones'
@@ -128,7 +99,7 @@ __global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, const unsigne
             big_i[at] = i0 + q * LT;
             big_p[at] = atomicAdd(&cursor, k);
         }
-        for (uint32_t w0 = 0; w0 < W; w0 += 32) {
+        for (uint32_t w0 = 0; w0 < W && p0 + w0 < (unsigned long long)g.capacity; w0 += 32) {
             const uint32_t w = w0 + lane;
             int lo = 0, hi = 31;   // the tuple of row w: the first whose inclusive count exceeds it
             const uint32_t wq = w < W ? w : 0u;
@@ -149,12 +120,10 @@ __global__ void __launch_bounds__(LT) k_lrows_write(LinRowsArgs g, const unsigne
     }
 }
 
-__global__ void __launch_bounds__(LT) k_lrows_big(LinRowsArgs g, const unsigned long long *__restrict__ base,
-                                                  uint32_t chunks, const uint32_t *__restrict__ big_n,
+__global__ void __launch_bounds__(LT) k_lrows_big(LinRowsArgs g, const uint32_t *__restrict__ big_n,
                                                   const uint32_t *__restrict__ big_i,
                                                   const unsigned long long *__restrict__ big_p) {
     after_previous();
-    if (base[chunks] > (unsigned long long)g.capacity) return;
     const uint32_t n = *big_n;
     const unsigned long long T = (unsigned long long)gridDim.x * LT;
     for (uint32_t e = 0; e < n; ++e) {
@@ -162,12 +131,21 @@ __global__ void __launch_bounds__(LT) k_lrows_big(LinRowsArgs g, const unsigned 
         const unsigned long long p = big_p[e];
         const int32_t b = __ldg(g.sb + i), c = __ldg(g.sc + i);
         const Lists l = lists_of(g, b, c);
-        const unsigned long long k = (unsigned long long)l.nr * l.nt;
+        const unsigned long long room = p < (unsigned long long)g.capacity ? (unsigned long long)g.capacity - p : 0ull;
+        const unsigned long long k = min((unsigned long long)l.nr * l.nt, room);
         for (unsigned long long r = (unsigned long long)blockIdx.x * LT + threadIdx.x; r < k; r += T) {
             const unsigned long long ia = r / l.nt;
             put_row(g, p + r, __ldg(g.r.alist + l.r0 + ia), b, c, __ldg(g.t.alist + l.t0 + (r - ia * l.nt)));
         }
     }
+}
+
+// total = n_rows; more rows than the capacity is an error.
+__global__ void k_lrows_check(const unsigned long long *n_rows, unsigned long long capacity, unsigned long long *total,
+                              DevStatus *st) {
+    after_previous();
+    *total = *n_rows;
+    if (*n_rows > capacity) set_status(st, MWJ_ERR_CAPACITY, (long long)*n_rows);
 }
 
 uint32_t lrows_chunks(int64_t nS) { return (uint32_t)((nS + LCHUNK - 1) / LCHUNK); }
@@ -190,10 +168,6 @@ void lin_rows_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel
     L.t = group(T, &L.tmeta);
     L.hll = A.take<unsigned int>(hll_scratch_registers(num_sms));
     L.bump = A.take<unsigned int>(4);
-    const uint32_t chunks = lrows_chunks(S.n);
-    L.chunk_rows = A.take<unsigned long long>(chunks + 1);
-    L.base = A.take<unsigned long long>(chunks + 2);
-    L.sscratch = A.take<char>(scan_scratch_bytes(chunks + 1));
     L.big_i = A.take<uint32_t>(S.n + 1);
     L.big_p = A.take<unsigned long long>(S.n + 1);
 }
@@ -204,6 +178,9 @@ cudaError_t lin_rows_run(LinRowsLayout &L, const mwj_rel &R, const mwj_rel &S, c
     cudaError_t e;
     L.r.seed = sd.slot;
     L.t.seed = sd.slot2;
+    uint32_t *big_n = L.bump + 2;
+    if ((e = cudaMemsetAsync(n_rows, 0, sizeof(*n_rows), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(big_n, 0, sizeof(*big_n), st)) != cudaSuccess) return e;
     if ((e = rgroup_build(R.x, R.y, R.n, L.r, L.hll, single_table_slots(R.n), L.bump, 0, status, num_sms, st)) !=
         cudaSuccess)
         return e;
@@ -220,29 +197,18 @@ cudaError_t lin_rows_run(LinRowsLayout &L, const mwj_rel &R, const mwj_rel &S, c
     g.capacity = capacity;
     g.st = status;
     const uint32_t chunks = lrows_chunks(S.n);
-    uint32_t *big_n = L.bump + 2;
-    if (chunks) {
-        ProfScope ps_("lin_rows_count", st);
-        if ((e = launch_after(k_lrows_count, chunks, LT, st, g, L.chunk_rows)) != cudaSuccess) return e;
-    }
-    if ((e = scan_excl_u64((const uint64_t *)L.chunk_rows, (uint64_t *)L.base, chunks, true, L.sscratch, st)) !=
-        cudaSuccess)
-        return e;
-    {
-        ProfScope ps_("rows_check", st);
-        e = launch_after(k_lrows_check, 1, 1, st, L.base, chunks, capacity, n_rows, total, big_n, status);
-        if (e != cudaSuccess) return e;
-    }
     if (chunks) {
         {
             ProfScope ps_("lin_rows", st);
-            if ((e = launch_after(k_lrows_write, chunks, LT, st, g, L.base, chunks, big_n, L.big_i, L.big_p)) != cudaSuccess)
-                return e;
+            e = launch_after(k_lrows_write, chunks, LT, st, g, (unsigned long long *)n_rows, big_n, L.big_i, L.big_p);
+            if (e != cudaSuccess) return e;
         }
         ProfScope ps_("lin_rows_big", st);
-        return launch_after(k_lrows_big, num_sms * 4, LT, st, g, L.base, chunks, big_n, L.big_i, L.big_p);
+        if ((e = launch_after(k_lrows_big, num_sms * 4, LT, st, g, big_n, L.big_i, L.big_p)) != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    ProfScope ps_("rows_check", st);
+    return launch_after(k_lrows_check, 1, 1, st, (unsigned long long *)n_rows, (unsigned long long)capacity, total,
+                        status);
 }
 
 }  // namespace mwj

@@ -19,13 +19,11 @@ struct LinRowsLayout {
     RGroup r, t;
     uint32_t *rmeta, *tmeta;
     unsigned int *hll, *bump;
-    unsigned long long *chunk_rows, *base;
-    void *sscratch;
     uint32_t *big_i;               // S tuples with many rows, and where they go
     unsigned long long *big_p;
 };
 void lin_rows_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, LinRowsLayout &L);
-// rows (a, b, c, d) into rows[0, n_rows) when n_rows <= capacity; *total = n_rows.
+// rows (a, b, c, d) into rows[0, min(n_rows, capacity)); *total = n_rows; more rows than the capacity is an error.
 cudaError_t lin_rows_run(LinRowsLayout &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd,
                          int4 *rows, long long capacity, long long *n_rows, unsigned long long *total,
                          DevStatus *status, int num_sms, cudaStream_t st);

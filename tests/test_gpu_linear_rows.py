@@ -76,3 +76,28 @@ def test_empty_and_capacity(ctx):
         ctx.join3_linear(cu(R), cu(S), cu(T), "rows", capacity=n - 1)
     assert e.value.status == binding.MWJ_ERR_CAPACITY
     check(ctx, R, S, T)
+
+
+@pytest.mark.parametrize("nr,nt,short", [(3, 5, 1), (4097, 1, 1), (4097, 1, 4000), (300, 900, 500_000)])
+def test_rows_past_the_capacity(ctx, nr, nt, short):
+    """They are counted and not written, also in the middle of a tuple with many rows."""
+    import ctypes
+    import torch
+    R = (np.arange(nr, dtype=np.int32), np.full(nr, 7, np.int32))
+    T = (np.full(nt, 3, np.int32), np.arange(nt, dtype=np.int32))
+    S = (np.full(2, 7, np.int32), np.full(2, 3, np.int32))
+    n = 2 * nr * nt
+    dR, dS, dT = cu(R), cu(S), cu(T)
+    m = binding.MODES["rows"]
+    o, res = ctx._outputs(m, None, n, 4)
+    res["rows"].fill_(-7)
+    o.capacity = n - short
+    ws = ctx.workspace(ctx.workspace_size(binding.MWJ_LINEAR, dR, dS, dT, mode=m))
+    hs = torch.cuda.current_stream().cuda_stream
+    rel = binding._rel
+    ctx._check(ctx.lib.mwj_join3_linear(ctx.h, rel(dR), rel(dS), rel(dT), None, ctypes.byref(o), ws.data_ptr(),
+                                        ws.numel(), hs))
+    with pytest.raises(binding.MwjError) as e:
+        ctx._check(ctx.lib.mwj_stream_status(ctx.h, hs))
+    assert e.value.status == binding.MWJ_ERR_CAPACITY and int(res["n_rows"].item()) == n
+    assert int((res["rows"][n - short:] != -7).sum().item()) == 0
