@@ -55,17 +55,18 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
 // workspace with a multiplicity per slot and looked up there like a big
 // bucket's set.
 //
-// Nearly every wedge is open (about 1 in 90 closes on the 2^22-vertex power-law
-// graph), so the set is not looked up per wedge: a filter of 2^18 bits, one
-// bit per (c, a) pair, answers first.  The bit of a wedge is a multiply-add of
-// its a (the hash of c is computed once per list), one 4-byte shared-memory
-// load and a shift, with no probe chain whose longest lane the whole warp
-// waits for; the set is looked up for the 1 to 2 % that pass (2048 pairs
-// leave 0.8 % of the open wedges standing, 6144 pairs 2.3 %).  On the
-// 2^22-vertex graph (2.79e10 wedges, one GB300) the probe took 122 ms when it
-// looked every wedge up in the set and takes 38 ms: 26 ms for the filter's
-// side (issue slots and the 3.5 shared-memory wavefronts of a divergent load)
-// and 12 ms for the lookups of what passes.
+// Nearly every wedge is open (about 1 in 40 of the shorter lists' closes on the
+// 2^22-vertex power-law graph), so the set is not looked up per wedge: a filter
+// of 2^18 bits, two bits of one word per (c, a) pair, answers first.  The bits
+// of a wedge are a multiply-add of its a (the hash of c is computed once per
+// list), one 4-byte shared-memory load and two shifts, with no probe chain
+// whose longest lane the whole warp waits for; the set is looked up for what
+// passes (2048 pairs leave 0.1 % of the open wedges standing, 6144 pairs 0.5 %;
+// with one bit per pair 0.8 and 2.3 %).  On the 2^22-vertex graph (2.79e10
+// wedges, one GB300) the probe took 122 ms when it looked every wedge up in the
+// set, 38 with one bit, 24.4 from the shorter lists, and 21.2 with 16-byte
+// loads and the second bit.  Issue slots bound it (70 % taken), and the 3.5
+// shared-memory wavefronts of a divergent load.
 constexpr uint32_t CC_NB = CC_TSLOTS / 2;
 constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); one region each
 // two probe CTAs per SM: each keeps below half of the SM's 228 KB of shared
@@ -73,8 +74,10 @@ constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); on
 static_assert(CC_TSLOTS * 8 + CC_FWORDS * 4 + CC_QCAP * 16 + (CC_QCAP + 1) * 4 + 1024 <= 228 * 1024 / 2 - 1024,
               "the probe's shared memory must leave room for two CTAs per SM");
 
-// The filter bit of (c, a): word h >> 19, bit (h >> 14) & 31 of
-// h = a * K + chash(c), so that only the multiply-add depends on a.
+// The filter bits of (c, a): word h >> 19, bits (h >> 14) & 31 and h & 31 from
+// the top, of h = a * K + chash(c), so that only the multiply-add depends on a.
+// (h & 31 says no more than a's low five bits, and takes no shift: 21.2 ms, with
+// (h >> 9) & 31 21.6.)
 constexpr uint32_t CC_FMUL = 0x9E3779B1u;
 static_assert(CC_FWORDS == 1u << 13, "the filter's word index is the top 13 bits");
 __device__ __forceinline__ uint32_t chash(uint32_t c, uint32_t seed) { return mix32(c ^ seed); }
@@ -84,9 +87,14 @@ __device__ __forceinline__ uint32_t chash_a(uint32_t a, uint32_t ch) { return a 
 static_assert(CC_NB == 1u << 12, "the home bucket is the top 12 bits");
 __device__ __forceinline__ uint32_t cbucket(uint32_t h) { return h >> 20; }
 
-__device__ __forceinline__ uint32_t fbit(const uint32_t *filt, uint32_t a, uint32_t ch) {
+__device__ __forceinline__ void fset(uint32_t *filt, uint32_t h) {
+    atomicOr(filt + (h >> 19), (0x80000000u >> ((h >> 14) & 31u)) | (0x80000000u >> (h & 31u)));
+}
+// on top of a word: whether both are set (shifts take their amount modulo 32)
+__device__ __forceinline__ uint32_t ftop(const uint32_t *filt, uint32_t a, uint32_t ch) {
     const uint32_t h = chash_a(a, ch);
-    return (filt[h >> 19] >> ((h >> 14) & 31u)) & 1u;
+    const uint32_t w = filt[h >> 19];
+    return __funnelshift_l(0u, w, h >> 14) & __funnelshift_l(0u, w, h);
 }
 
 // 1: the pair took a free slot; 2: it was there already; 0: the set is full.
@@ -204,8 +212,8 @@ __global__ void __launch_bounds__(RG_T) k_rg_scatter(const int32_t *__restrict__
 // power-law graphs).  Two list lengths per tuple, read in one pass over S
 // (0.34 ms for 6.7e7 tuples); the probe goes from 38 to 25 ms on the
 // 2^22-vertex graph, the call from 45 to 31.  Row output carries a mark of the
-// turned tuples: 7.6e6 triangles of a 2^20-edge graph, both passes, 7.3 to 6.4 ms
-// with the sort of the rows.
+// turned tuples: 7.6e6 triangles of a 2^20-vertex graph, with the sort of the
+// rows, 7.3 to 6.4 ms (when every wedge was still enumerated twice).
 __global__ void __launch_bounds__(RG_T) k_cc_orient(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
                                                     uint32_t n, RGroup r, int32_t *__restrict__ u,
                                                     int32_t *__restrict__ v, int32_t *__restrict__ turned) {
@@ -466,7 +474,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             const uint2 tu = __ldg(g.Tp + q);   // (c, a)
             const unsigned long long key = cpack(tu.x, tu.y);
             const uint32_t h = chash_a(tu.y, chash(tu.x, g.seed));
-            atomicOr(filt + (h >> 19), 1u << ((h >> 14) & 31u));
+            fset(filt, h);
             if (key == kEmpty64) {               // (-1, -1) is the empty marker: counted apart
                 atomicAdd(&tneg, 1u);
                 continue;
@@ -566,40 +574,48 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
             return 0u;
         };
-        // walk one list of the warp's: entries [lo, hi) of (b, c)'s R list in
-        // steps of CC_CH, first the filter bits of the lane's 32 entries
-        // (bit q: entry base + 32 q + lane), then the set for those that
-        // passed, whose a is read again.  Every lane of the warp calls this.
+        // walk one list of the warp's: entries [lo, hi) from alist[jst & ~3] on,
+        // those before jst left out, lo a multiple of CC_CH.  In steps of CC_CH
+        // entries: first the filter bits, 16 bytes of the list per lane and load
+        // (a lane's 32 bits in the order of its entries, the first one on top),
+        // then the set for those that passed, whose a is read again.  Every lane
+        // of the warp calls this.  (4 bytes per lane and load: 24.4 ms for the
+        // probe of the 2^22-vertex graph, 22.9 this way; reading four of the
+        // passed a's at once instead: 31.5.)
         auto walk = [&](uint32_t jb, uint32_t jc, uint32_t jst, uint32_t lo, uint32_t hi) {
             const uint32_t ch = chash(jc, g.seed);
+            const uint32_t start = ROWS ? jst & ~kTurned : jst;
+            const int32_t *list = g.r.alist + (start & ~3u);
+            const uint32_t skip = start & 3u;
             for (uint32_t base = lo; base < hi; base += CC_CH) {
-                const int32_t *list = g.r.alist + (ROWS ? jst & ~kTurned : jst) + base + lane;
+                const int32_t *at = list + base + 4u * lane;
                 const uint32_t n = min(hi - base, CC_CH);
-                uint32_t hits = 0, s = 0;
-                for (; (s + 4u) * 32u <= n; s += 4u) {
-                    uint32_t a[4], h4 = 0;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) a[q] = (uint32_t)__ldg(list + 32u * s + 32 * q);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) h4 |= fbit(filt, a[q], ch) << q;
-                    hits |= h4 << s;
+                uint32_t hits = 0;
+                auto four = [&](const int4 &v) {
+                    hits = __funnelshift_l(ftop(filt, (uint32_t)v.x, ch), hits, 1);
+                    hits = __funnelshift_l(ftop(filt, (uint32_t)v.y, ch), hits, 1);
+                    hits = __funnelshift_l(ftop(filt, (uint32_t)v.z, ch), hits, 1);
+                    hits = __funnelshift_l(ftop(filt, (uint32_t)v.w, ch), hits, 1);
+                };
+                uint32_t done = 0;
+                for (; done + 256u <= n; done += 256u) {
+                    const int4 v0 = __ldg((const int4 *)(at + done)), v1 = __ldg((const int4 *)(at + done + 128u));
+                    four(v0);
+                    four(v1);
                 }
-                if (32u * s < n) {
-                    uint32_t a[4], h4 = 0;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        a[q] = 32u * (s + q) + lane < n ? (uint32_t)__ldg(list + 32u * s + 32 * q) : 0u;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (32u * (s + q) + lane < n) h4 |= fbit(filt, a[q], ch) << q;
-                    hits |= h4 << s;
+                for (; done < n; done += 128u) {   // (the list's room ends 4 entries after it)
+                    const uint32_t e = done + 4u * lane;
+                    four(e < n ? __ldg((const int4 *)(at + done)) : make_int4(0, 0, 0, 0));
+                    if (e + 4u > n) hits &= e < n ? 0xffffffffu << (e + 4u - n) : ~15u;
                 }
+                hits <<= 32u - done / 32u;   // (done / 32 bits so far)
+                if (base == 0u && lane == 0) hits &= 0xffffffffu >> skip;
                 while (!ROWS ? hits != 0u : (bool)__any_sync(0xffffffffu, hits != 0u)) {
                     uint32_t a = 0, m = 0;
                     if (hits) {
-                        const uint32_t q = (uint32_t)__ffs((int)hits) - 1u;
-                        hits &= hits - 1u;
-                        a = (uint32_t)__ldg(list + 32u * q);
+                        const uint32_t e = (uint32_t)__clz((int)hits);
+                        hits &= ~(0x80000000u >> e);
+                        a = (uint32_t)__ldg(at + (e >> 2) * 128u + (e & 3u));
                         m = count(jc, a, ch);
                     }
                     emit(a, jb, jc, m, ROWS && (jst & kTurned));
@@ -644,7 +660,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 const int j = __ffs(sm_) - 1;
                 sm_ &= sm_ - 1u;
                 walk(__shfl_sync(0xffffffffu, b, j), __shfl_sync(0xffffffffu, c, j),
-                     __shfl_sync(0xffffffffu, st, j), 0u, __shfl_sync(0xffffffffu, n, j));
+                     __shfl_sync(0xffffffffu, st, j), 0u,
+                     __shfl_sync(0xffffffffu, n + (st & 3u), j));
             }
             // lists of 32 .. kQueueMin - 1 entries: the warp walks each one
             unsigned mid_ = __ballot_sync(0xffffffffu, n >= 32u && n < kQueueMin);
@@ -652,7 +669,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 const int j = __ffs(mid_) - 1;
                 mid_ &= mid_ - 1u;
                 walk(__shfl_sync(0xffffffffu, b, j), __shfl_sync(0xffffffffu, c, j),
-                     __shfl_sync(0xffffffffu, st, j), 0u, __shfl_sync(0xffffffffu, n, j));
+                     __shfl_sync(0xffffffffu, st, j), 0u,
+                     __shfl_sync(0xffffffffu, n + (st & 3u), j));
             }
             const uint32_t ns = n < 32u ? n : 0u;
             uint32_t incl = ns;
@@ -681,7 +699,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 if (wi < W) {
                     a = (uint32_t)__ldg(g.r.alist + (ROWS ? ost & ~kTurned : ost) + (wi - oex));
                     const uint32_t ch = chash(oc, g.seed);
-                    if (fbit(filt, a, ch)) m = count(oc, a, ch);
+                    if ((int32_t)ftop(filt, a, ch) < 0) m = count(oc, a, ch);
                 }
                 emit(a, ob, oc, m, ROWS && (ost & kTurned));
             }
@@ -692,7 +710,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         const uint32_t nq = min(qn, QCAP);
         for (uint32_t q0 = 0; q0 <= nq; q0 += CC_T) {
             const uint32_t q = q0 + threadIdx.x;
-            const uint32_t d = q < nq ? (queue[q].w + CC_CH - 1) / CC_CH : 0u;
+            const uint32_t d = q < nq ? ((queue[q].z & 3u) + queue[q].w + CC_CH - 1) / CC_CH : 0u;
             uint32_t tot;
             const uint32_t ex = block_excl_scan_u32(d, scan_scratch, &tot);
             if (q <= nq) cpre[q] = carry + ex;
@@ -713,7 +731,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
             const uint4 L = queue[lo];
             const uint32_t first = (ci - cpre[lo]) * CC_CH;
-            walk(L.x, L.y, L.z, first, min(first + CC_CH, L.w));
+            walk(L.x, L.y, L.z, first, min(first + CC_CH, (L.z & 3u) + L.w));
         }
         acc_all += acc;
         __syncthreads();

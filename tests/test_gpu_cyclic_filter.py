@@ -143,3 +143,21 @@ def test_rows_staged_and_not(ctx, copies):
     with pytest.raises(binding.MwjError) as ei:
         ctx.join3_cyclic(cu(R), cu(S), cu(T), "rows", shares=(1, 1, 4), capacity=want - 1)
     assert ei.value.status == binding.MWJ_ERR_CAPACITY and str(want) in str(ei.value)
+
+
+def test_list_lengths_and_alignments(ctx):
+    """Lists of every length around the warp's 32, the 128 and 256 entries of its
+    loads and the 1024 of a step, one after the other, so that they start at all
+    places of a 16-byte load; every a of a list's first and last entries closes."""
+    g = np.random.default_rng(17)
+    lens = np.r_[29:38, 124:134, 253:260, 508:516, 1020:1030, 2045:2051]
+    b = np.repeat(np.arange(len(lens)), lens).astype(np.int32)
+    a = np.concatenate([g.permutation(5000)[:n] for n in lens]).astype(np.int32)
+    first = np.cumsum(lens) - lens
+    ends = np.r_[first, first + 1, first + 2, first + 3, first + lens - 1, first + lens - 2, first + lens - 4]
+    c = g.integers(0, 6, 300).astype(np.int32)
+    S = (g.integers(0, len(lens) + 2, 300).astype(np.int32), c)
+    T = (g.integers(0, 6, 2400).astype(np.int32), np.r_[a[ends], g.integers(0, 5000, 2400 - len(ends))].astype(np.int32))
+    assert check(ctx, (a, b), S, T, 5000, (1, 1, 3)) > 0
+    T = (np.repeat(np.arange(6, dtype=np.int32), len(ends)), np.tile(a[ends], 6))
+    assert check(ctx, (a, b), S, T, 5000, (1, 1, 3)) >= 7 * 290
