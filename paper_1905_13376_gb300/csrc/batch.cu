@@ -266,12 +266,18 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
     return ((unsigned long long)c << 32) | a;
 }
 // The hash of a pair (c, a): only the multiply-add depends on a.  Its top bits
-// give the filter's word and bit and the home bucket.
+// give the filter's word and one bit and the home bucket, its low five another
+// bit of that word (with one bit per pair the 1024-query batch's join took 3.07
+// ms, with two 3.00).
 __device__ __forceinline__ uint32_t chash(uint32_t c, uint32_t seed) { return mix32(c ^ seed); }
 __device__ __forceinline__ uint32_t cpair_hash(uint32_t a, uint32_t ch) { return a * 0x9E3779B1u + ch; }
 static_assert(CFWORDS == 1u << 10 && CTSLOTS == 1u << 12, "bit positions of the pair hash");
-__device__ __forceinline__ bool cfilter(const uint32_t *filt, uint32_t h) {
-    return (filt[h >> 22] >> ((h >> 17) & 31u)) & 1u;
+__device__ __forceinline__ void cfilter_set(uint32_t *filt, uint32_t h) {
+    atomicOr(&filt[h >> 22], (0x80000000u >> ((h >> 17) & 31u)) | (0x80000000u >> (h & 31u)));
+}
+__device__ __forceinline__ bool cfilter(const uint32_t *filt, uint32_t h) {   // both bits (shifts are modulo 32)
+    const uint32_t w = filt[h >> 22];
+    return (int32_t)(__funnelshift_l(0u, w, h >> 17) & __funnelshift_l(0u, w, h)) < 0;
 }
 
 // Add one to the count of `key` in an open-addressing table of `slots` (a power
@@ -509,7 +515,7 @@ __device__ unsigned long long cyc_item(const CycQ &c, uint32_t t_local, uint32_t
         if (ta + threadIdx.x + q * BTH >= tz) continue;
         const unsigned long long key = cpack(tt[q].x, tt[q].y);
         const uint32_t h = cpair_hash(tt[q].y, chash(tt[q].x, seed2));
-        atomicOr(&sm.filt[h >> 22], 1u << ((h >> 17) & 31u));
+        cfilter_set(sm.filt, h);
         if (key == kEmpty64)   // the empty marker: counted apart
             atomicAdd(&negs_s, 1u);
         else if (!pair_add(sm.tkeys, sm.tcnt, CTSLOTS, key, (h >> 21) * 2u))
