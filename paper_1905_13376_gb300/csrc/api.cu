@@ -180,8 +180,8 @@ mwj_status plan_linear_default(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S,
 
 // Default shares of mwj_join3_linear.  Aggregates: I = J = 1, the plan in
 // which S's weight table and T's table are held whole in the L2 and nothing
-// is partitioned.  Rows: the partitioned plan above (the row output needs the
-// a-lists of R's buckets in shared memory).
+// is partitioned.  Rows: the partitioned plan above (a call without shares
+// takes it when its workspace has no room for R's and T's lists).
 mwj_status linear_default_shares(mwj_ctx *ctx, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T,
                                  mwj_mode mode, mwj_shares *sh) {
     if (mode == MWJ_MATERIALIZE) return plan_linear_default(ctx, R, S, T, sh);
@@ -385,12 +385,12 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
         Arena A(workspace, ws_bytes);
         LinRowsLayout L;
         lin_rows_layout(A, R, S, T, ctx->dev.num_sms, L);
-        if (A.overflow || !workspace)
-            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
-        const cudaError_t er =
-            lin_rows_run(L, R, S, T, ctx->seeds, (int4 *)out->rows, out->capacity, (long long *)out->n_rows,
-                         (unsigned long long *)out->total, ctx->status, ctx->dev.num_sms, st);
-        return er == cudaSuccess ? MWJ_OK : cuda_fail(ctx, er, "linear rows");
+        if (!A.overflow && workspace) {   // else the partitioned plan, which takes less
+            const cudaError_t er =
+                lin_rows_run(L, R, S, T, ctx->seeds, (int4 *)out->rows, out->capacity, (long long *)out->n_rows,
+                             (unsigned long long *)out->total, ctx->status, ctx->dev.num_sms, st);
+            return er == cudaSuccess ? MWJ_OK : cuda_fail(ctx, er, "linear rows");
+        }
     }
     mwj_shares sh;
     if (shares) sh = *shares; else linear_default_shares(ctx, R, S, T, out->mode, &sh);

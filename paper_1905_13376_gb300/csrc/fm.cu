@@ -700,11 +700,12 @@ extern "C" mwj_status mwj_fm_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel 
     if (fm_one(S, T, shares)) {
         FmOneLayout L;
         fm_one_layout(A, S, T, sms, sd, L);
-        if (A.overflow || !workspace)
-            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
-        if ((e = fm_one_run(L, R, S, T, a_domain, sketches, ctx->status, sms, st)) != cudaSuccess)
-            return cuda_fail(ctx, e, "fm one bucket");
-        return estimate();
+        if (!A.overflow && workspace) {   // else the partitioned plan, which takes less
+            if ((e = fm_one_run(L, R, S, T, a_domain, sketches, ctx->status, sms, st)) != cudaSuccess)
+                return cuda_fail(ctx, e, "fm one bucket");
+            return estimate();
+        }
+        A = Arena(workspace, ws_bytes);
     }
     uint32_t I;
     mwj_status s = fm_buckets(ctx, S, shares, &I);

@@ -194,21 +194,26 @@ extern "C" mwj_status mwj_join4_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
     if (s != MWJ_OK) return s;
     if (out->mode != MWJ_COUNT && out->mode != MWJ_COUNT_GROUP_BY_A)
         return fail(ctx, MWJ_ERR_INVALID_ARG, "4-relation chain: COUNT or COUNT GROUP BY A only");
-    Arena A(workspace, ws_bytes);
+    mwj_shares sh;
     if (!shares) {
         const mwj_rel rel[4] = {R, S, T, U};
         OneBucket L;
+        Arena A(workspace, ws_bytes);
         j4_one_layout(A, rel, ctx->dev.num_sms, L);
-        if (A.overflow || !workspace)
-            return fail(ctx, MWJ_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", ws_bytes, A.used);
-        const cudaError_t eo =
-            one_bucket_run(L, rel, 4, ctx->seeds, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
-                           (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
-                           ctx->dev.num_sms, (cudaStream_t)stream);
-        return eo == cudaSuccess ? MWJ_OK : cuda_fail(ctx, eo, "chain of four, one bucket");
+        if (!A.overflow && workspace) {   // else the partitioned plan, which may take less
+            const cudaError_t eo =
+                one_bucket_run(L, rel, 4, ctx->seeds, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
+                               (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
+                               ctx->dev.num_sms, (cudaStream_t)stream);
+            return eo == cudaSuccess ? MWJ_OK : cuda_fail(ctx, eo, "chain of four, one bucket");
+        }
+        plan_linear_default(ctx, R, S, T, &sh);
+    } else {
+        sh = *shares;
     }
+    Arena A(workspace, ws_bytes);
     uint32_t I, cap_log2;
-    if ((s = j4_shares(ctx, *shares, &I, &cap_log2)) != MWJ_OK) return s;
+    if ((s = j4_shares(ctx, sh, &I, &cap_log2)) != MWJ_OK) return s;
     J4Layout L;
     j4_layout(A, I, R, S, T, U, ctx->dev.num_sms, L);
     if (A.overflow || !workspace)

@@ -24,6 +24,7 @@
 // B values instead of S's (star_bucket_run): R is the small relation, so its
 // column is the cheap one to size, and S tuples whose b is not R's are
 // skipped.
+#include <algorithm>
 #include <type_traits>
 
 #include "group_table.cuh"
@@ -1074,8 +1075,11 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
 }
 
 void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, OneBucket &L) {
-    // the weights are R's, not S's, except in a small call (a chain like any other)
-    const mwj_rel rel[3] = {R, S.n <= kMediumMax && S.n > R.n ? S : R, T};
+    // the weights are R's, not S's, except in a small call (a chain like any
+    // other): room for either, so that what a call asks for grows with its sizes
+    mwj_rel w = R;
+    w.n = std::max(R.n, std::min(S.n, kMediumMax));
+    const mwj_rel rel[3] = {R, w, T};
     one_bucket_layout(A, rel, 3, num_sms, L);
 }
 
