@@ -131,11 +131,17 @@ mwj_status mwj_workspace_size(mwj_ctx *ctx, int kind, mwj_rel R, mwj_rel S, mwj_
 /* Linear 3-way join R(A,B) S(B,C) T(C,D) in one step (Algorithm 1, Section 4).
  * Shares s[0] = s[1] = 1 with COUNT or GROUP BY A (the default for those
  * modes when shares == NULL): one bucket per side, nothing partitioned, the
- * held tables kept whole in the L2: T's table c -> deg_T(c) is built (on a
- * context stream) while S's weight table b -> w(b) is sized, a pass over S
- * adds w(b) += deg_T(c), and a pass over R adds cnt[a] += w(b) and
- * total += w(b).  Both tables are sized from HyperLogLog estimates of the
- * distinct keys; w(b) is exact to 2^64.
+ * held tables kept whole in the L2: T's table c -> deg_T(c), a pass over S
+ * that adds w(b) += deg_T(c) into S's weight table, and a pass over R that
+ * adds cnt[a] += w(b) and total += w(b).  A table is an array indexed by
+ * key - min when the column's key range fits what is reserved for it, else a
+ * hash table sized from a HyperLogLog estimate of the distinct keys; w(b) is
+ * exact to 2^64.  Relations of at most 2^19 tuples use hash tables of two
+ * slots per tuple in four launches, of at most 2^14 in one.
+ * MATERIALIZE with shares == NULL: R grouped by B and T by C as lists in
+ * global memory, S streamed past them once, the rows of a chunk of S at the
+ * place that one atomic on *n_rows reserves; rows beyond the capacity are
+ * counted and not written.
  * Otherwise R is partitioned by H(B), S by (H(B), g(C)), T by g(C); each CTA holds one
  * H(B) bucket's B values as an on-chip hash table while the other side of
  * that bucket streams past it, and T's tables are probed (its bucket images
@@ -156,17 +162,23 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
 /* Cyclic 3-way join R(A,B) S(B,C) T(C,A) in one step (Section 5): tile
  * (i,j,k) of the share cube holds R_ij (H(a)=i, G(b)=j) and T_ki
  * (F(c)=k, H(a)=i) on chip while S_jk streams past them.  T's columns are
- * (c, a). */
+ * (c, a).  With x = y = 1 (the default) R is grouped by B as a whole; when T's
+ * columns are R's exchanged (T.x == R.y and T.y == R.x, as in triangle
+ * counting over one edge list) each wedge of an S tuple is taken from its
+ * shorter list, given a workspace sized for these relations.  MATERIALIZE may
+ * write rows[0, capacity) also when there are more rows than that. */
 mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
                             const mwj_shares *shares, const mwj_out *out,
                             void *workspace, size_t ws_bytes, void *stream);
 
 /* Star 3-way join R(A,B) S(B,C) T(C,D) (Section 6, "linear star 3-way
  * join"): the same query and outputs as mwj_join3_linear, planned for small
- * dimension relations R and T and a large fact relation S.  R is grouped by
- * h(B) and T by g(C) into bucket tables that stay on chip (L2 and L1); S is
- * read once, unpartitioned, each tuple looked up in both tables (twice for
- * MATERIALIZE: a counting pass, then the rows).  shares: s[0] = h(B) buckets
+ * dimension relations R and T and a large fact relation S.  S is read once,
+ * unpartitioned.  COUNT and GROUP BY A: T's degree table and a weight table
+ * with R's keys in the L2 (as in mwj_join3_linear); each S tuple whose b is a
+ * key of R adds deg_T(c) to w(b), and R's groups are added at the end; shares
+ * are not used.  MATERIALIZE: R is grouped by h(B) and T by g(C) into bucket
+ * tables, S read twice (a counting pass, then the rows).  shares: s[0] = h(B) buckets
  * of R, s[1] = g(C) buckets of T (0 or shares == NULL: about 2048 tuples per
  * bucket); s[2] is ignored.  GROUP BY A checks the domain of A while it adds
  * R's groups (MWJ_ERR_DOMAIN from mwj_stream_status).
@@ -181,7 +193,8 @@ mwj_status mwj_join3_star(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T, const m
  * on B as in mwj_join3_linear with w_T(c) in place of T's degree; no
  * intermediate relation is materialised.  shares: s[0] = H(B) buckets,
  * s[1] must be 1, s[2] = log2 of the on-chip table slots (as for the linear
- * join); NULL = the linear join's default.  MATERIALIZE is not offered
+ * join); NULL: one bucket per side, w_T(c) and w(b) whole in the L2 and a
+ * pass over each relation.  MATERIALIZE is not offered
  * (MWJ_ERR_INVALID_ARG).  workspace: >= mwj_join4_workspace_size(...). */
 mwj_status mwj_join4_workspace_size(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T, mwj_rel U,
                                     const mwj_shares *shares, mwj_mode mode, size_t *bytes);
@@ -201,7 +214,9 @@ mwj_status mwj_join4_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T, mwj_r
  * a_domain floats, or NULL: (16 / 0.77351) * 2^(mean over bitmaps of the
  * index of their lowest 0 bit).  Every a of R must lie in [0, a_domain)
  * (MWJ_ERR_DOMAIN from mwj_stream_status otherwise).  shares: s[0] = H(B)
- * buckets (NULL: ~16K S tuples per bucket); the other entries are ignored.
+ * buckets; the other entries are ignored.  NULL: one bucket while S and T have
+ * at most 2^28 tuples each (a 64-byte row of bitmaps per key of T's C and S's
+ * B, a pass over each relation), else ~16K S tuples per bucket.
  * workspace: device, >= mwj_fm_workspace_size(...). */
 mwj_status mwj_fm_workspace_size(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
                                  const mwj_shares *shares, size_t *bytes);
@@ -310,10 +325,11 @@ mwj_status mwj_batch_set_rules(mwj_ctx *ctx, const mwj_batch_rule *rules, int32_
 mwj_status mwj_batch_set_launch(mwj_ctx *ctx, int32_t prep_ctas_per_sm, int32_t join_ctas_per_sm);
 
 /* The shares the planner would choose for these relations (host result in
- * *shares), the ones a call with shares == NULL uses.  kind = MWJ_LINEAR,
+ * *shares).  kind = MWJ_LINEAR,
  * MWJ_CYCLIC or MWJ_STAR.  Linear: {1, 1, 1} for COUNT and GROUP BY A (the
- * one-bucket plan), H(B) buckets from |R| for MATERIALIZE.  Synchronises
- * `stream`. */
+ * one-bucket plan).  For MATERIALIZE, linear, the H(B) buckets of the
+ * partitioned plan, which a call with these shares runs; one with
+ * shares == NULL takes the lists described there.  Synchronises `stream`. */
 mwj_status mwj_plan_shares(mwj_ctx *ctx, int kind, mwj_rel R, mwj_rel S, mwj_rel T,
                            mwj_mode mode, mwj_shares *shares, void *stream);
 

@@ -65,7 +65,7 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
 // with one bit per pair 0.8 and 2.3 %).  On the 2^22-vertex graph (2.79e10
 // wedges, one GB300) the probe took 122 ms when it looked every wedge up in the
 // set, 38 with one bit, 24.4 from the shorter lists, and 21.2 with 16-byte
-// loads and the second bit.  Issue slots bound it (70 % taken), and the 3.5
+// loads and the second bit.  Issue slots bound it (73 % taken), and the 3.5
 // shared-memory wavefronts of a divergent load.
 constexpr uint32_t CC_NB = CC_TSLOTS / 2;
 constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); one region each

@@ -639,19 +639,20 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
 //  * up to kMediumMax: four launches, one that empties the tables and says how
 //    large they are, then the general passes on the whole GPU.
 //
-// Device time of a call with uniform keys, GROUP BY A (2^20 groups), and in
-// brackets of calls queued back to back by the binding, us:
+// Device time of a call with uniform keys, GROUP BY A (2^20 groups; a replayed
+// graph of ten), and in brackets of calls queued back to back by the binding, us:
 //
 //   tuples per relation   nine launches   four launches   one cluster
-//   2^10                  28 (53)         12 (36)         20 (27)
-//   2^14                  30 (51)         14 (36)         22 (27)
-//   2^16                  30 (53)         16 (37)         40 (42)
-//   2^18                  35 (57)         22 (37)         102 (106)
-//   2^19                  42 (64)         32 (42)
-//   2^20                  55 (77)         56 (66)
+//   2^10                  26 (41)         11 (26)         20 (23)
+//   2^14                  27 (38)         13 (25)         22 (24)
+//   2^16                  28 (39)         15 (26)         40 (41)
+//   2^18                  34 (39)         20 (26)         102 (104)
+//   2^19                  41 (42)         31 (32)
+//   2^20                  56 (56)         56 (55)
 //
-// (id keys, nine against four launches: 66 against 37 at 2^18, 109 against 75 at
-// 2^20; Zipf 1.5: 36 against 29, 48 against 53.)
+// Up to 2^14 what a queue of calls waits for is the host, and the cluster's one
+// launch is the cheapest there.  (id keys at 2^20, before launches overlapped:
+// nine 109, four 75.)
 constexpr int CT = 1024;              // threads per CTA
 constexpr int kSmallCtas = 16;        // CTAs of the largest cluster
 constexpr int64_t kSmallMax = 1 << 14;      // tuples per relation
