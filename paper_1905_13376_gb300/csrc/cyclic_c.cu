@@ -36,7 +36,10 @@ constexpr uint32_t CC_FWORDS = 8192;     // words of the filter in front of it (
 constexpr int RG_T = 512;                // threads of the grouping kernels
 constexpr uint32_t CC_QCAP = 768;        // long R lists queued per work item
 constexpr uint32_t CC_CH = 1024;         // wedges of a list per warp step (32 per lane, one mask word)
-constexpr uint32_t kQueueMin = 512;      // lists this long go to the item's queue
+// lists this long go to the item's queue, so that a hub is shared by the CTA's warps
+// (probe of the 2^22-vertex graph, lists up to 4096: 21.0 ms from 512 on, 20.7 from
+// 1024, 20.4 from 2048 or none)
+constexpr uint32_t kQueueMin = 2048;
 constexpr uint32_t CC_STAGE = 32;        // rows that a warp of the row pass stages
 constexpr uint32_t CC_QCAP_ROWS = 384;   // its queue's places: the rest hold the staged rows
 constexpr uint32_t kTurned = 0x80000000u;   // row output: mark of a turned tuple, in its list's start
@@ -64,8 +67,8 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
 // passes (2048 pairs leave 0.1 % of the open wedges standing, 6144 pairs 0.5 %;
 // with one bit per pair 0.8 and 2.3 %).  On the 2^22-vertex graph (2.79e10
 // wedges, one GB300) the probe took 122 ms when it looked every wedge up in the
-// set, 38 with one bit, 24.4 from the shorter lists, and 21.2 with 16-byte
-// loads and the second bit.  Issue slots bound it (73 % taken), and the 3.5
+// set, 38 with one bit, 24.4 from the shorter lists, 21.2 with 16-byte
+// loads and the second bit, and 20.4 with fewer lists queued.  Issue slots bound it (73 % taken), and the 3.5
 // shared-memory wavefronts of a divergent load.
 constexpr uint32_t CC_NB = CC_TSLOTS / 2;
 constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); one region each
