@@ -67,9 +67,9 @@ __device__ __forceinline__ unsigned long long cpack(uint32_t c, uint32_t a) {
 // passes (2048 pairs leave 0.1 % of the open wedges standing, 6144 pairs 0.5 %;
 // with one bit per pair 0.8 and 2.3 %).  On the 2^22-vertex graph (2.79e10
 // wedges, one GB300) the probe took 122 ms when it looked every wedge up in the
-// set, 38 with one bit, 24.4 from the shorter lists, 21.2 with 16-byte
-// loads and the second bit, and 20.4 with fewer lists queued.  Issue slots bound it (73 % taken), and the 3.5
-// shared-memory wavefronts of a divergent load.
+// set, 38 with one bit, 24.4 from the shorter lists, 21.2 with 16-byte loads and
+// the second bit, and 20.4 with fewer lists queued.  Issue slots bound it (73 %
+// taken), and the 3.5 shared-memory wavefronts of a divergent load.
 constexpr uint32_t CC_NB = CC_TSLOTS / 2;
 constexpr int CC_MAX_CTAS_PER_SM = 2;   // probe CTAs per SM (shared memory); one region each
 // two probe CTAs per SM: each keeps below half of the SM's 228 KB of shared
