@@ -1,7 +1,8 @@
 // scan.cu -- exclusive prefix sums (bucket offsets, output positions).
 //
 // Three launches, no inter-CTA waiting: per-tile totals, one CTA scanning the
-// tile totals, per-tile scan plus the tile's base.
+// tile totals, per-tile scan plus the tile's base.  Up to kOneCta tiles one CTA
+// takes them in turn, in one launch.
 #include "internal.h"
 
 namespace mwj {
@@ -64,10 +65,10 @@ __global__ void k_scan_sums(T *sums, size_t m) {
     }
 }
 
+// One tile's scan, `before` the sum of the tiles before it; returns its total.
 template <typename T>
-__global__ void k_tile_scan(const T *in, T *out, size_t n, const T *sums, bool with_total) {
-    after_previous();
-    size_t base = (size_t)blockIdx.x * SC_TILE + (size_t)threadIdx.x * SC_ITEMS;
+__device__ __forceinline__ T scan_tile(const T *in, T *out, size_t n, size_t tile, T before, bool with_total) {
+    size_t base = tile * SC_TILE + (size_t)threadIdx.x * SC_ITEMS;
     T v[SC_ITEMS];
     T local = 0;
 #pragma unroll
@@ -98,7 +99,7 @@ __global__ void k_tile_scan(const T *in, T *out, size_t n, const T *sums, bool w
     }
     __syncthreads();
     unsigned long long wb = (w > 0) ? wt[w - 1] : 0ull;
-    T run = (T)((unsigned long long)sums[blockIdx.x] + wb + x - (unsigned long long)local);
+    T run = (T)((unsigned long long)before + wb + x - (unsigned long long)local);
 #pragma unroll
     for (int k = 0; k < SC_ITEMS; ++k) {
         size_t i = base + k;
@@ -106,6 +107,26 @@ __global__ void k_tile_scan(const T *in, T *out, size_t n, const T *sums, bool w
         run += v[k];
     }
     if (with_total && base < n && base + SC_ITEMS >= n) out[n] = run;
+    const T total = (T)wt[31];
+    __syncthreads();   // wt is the next tile's
+    return total;
+}
+
+template <typename T>
+__global__ void k_tile_scan(const T *in, T *out, size_t n, const T *sums, bool with_total) {
+    after_previous();
+    scan_tile(in, out, n, blockIdx.x, sums[blockIdx.x], with_total);
+}
+
+// tiles (triangles of graphs of 1.2e5 and 2.2e5 edges: 206 and 246 us with three
+// launches for each scan, 194 and 237 this way; up to 16 tiles the same, but a
+// 1024-query batch, whose item counts are 16 tiles, 4.05 instead of 4.03 ms)
+constexpr size_t kOneCta = 4;
+template <typename T>
+__global__ void k_scan_one(const T *in, T *out, size_t n, bool with_total) {
+    after_previous();
+    T before = 0;
+    for (size_t t = 0; t * SC_TILE < n; ++t) before += scan_tile(in, out, n, t, before, with_total);
 }
 
 template <typename T>
@@ -116,6 +137,10 @@ cudaError_t scan_impl(const T *in, T *out, size_t n, bool with_total, void *scra
         return cudaSuccess;
     }
     size_t tiles = (n + SC_TILE - 1) / SC_TILE;
+    if (tiles <= kOneCta) {
+        ProfScope ps_("scan_one", st);
+        return launch_after(k_scan_one<T>, 1, SC_THREADS, st, in, out, n, with_total);
+    }
     T *sums = (T *)scratch;
     {
         ProfScope ps_("scan_tile_sums", st);

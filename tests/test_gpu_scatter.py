@@ -30,8 +30,10 @@ def relations(n, seed, dom):
     return (a, some()), (some(), hot()), (hot(), a[::-1].copy())
 
 
-# edges of a tile (4096 tuples), a CTA's several tiles, and the first bucket count of this path
-@pytest.mark.parametrize("z,n", [(4097, 1), (4097, 4095), (5000, 4097), (4097, 12289), (20011, 300001)])
+# edges of a tile (4096 tuples), a CTA's several tiles, the first bucket count of this
+# path, and the counts up to which one CTA scans them (4096 and 4 x 4096)
+@pytest.mark.parametrize("z,n", [(4097, 1), (4097, 4095), (5000, 4097), (4097, 12289), (20011, 300001),
+                                 (4096, 4000), (16383, 900), (16384, 900), (16385, 900)])
 @pytest.mark.parametrize("self_join", [False, True])
 def test_many_buckets(ctx, z, n, self_join):
     R, S, T = relations(n, z + n, n // 8 if self_join else n)
