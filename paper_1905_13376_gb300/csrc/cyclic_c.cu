@@ -530,8 +530,31 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
             const unsigned some = __ballot_sync(0xffffffffu, m != 0u);
             if (!some) return;
+            const int32_t rb = (int32_t)(turned ? c : b), rc = (int32_t)(turned ? b : c);
+            // not staged: this lane's m rows, after the `ex` of the lanes before it of `all`
+            auto write = [&](unsigned long long ex, unsigned long long all) {
+                unsigned long long p = 0;
+                if (lane == 0) p = atomicAdd(n_rows, all);
+                p = __shfl_sync(0xffffffffu, p, 0) + ex;
+                for (uint32_t e = 0; e < m && p < capacity; ++e, ++p) {
+                    rows[3 * p] = (int32_t)a;
+                    rows[3 * p + 1] = rb;
+                    rows[3 * p + 2] = rc;
+                }
+            };
+            if (__any_sync(0xffffffffu, m > CC_STAGE)) {
+                // a pair of T may occur |T| times: the step's rows are added in 64 bits
+                unsigned long long incl = m;
+#pragma unroll 1
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if ((int)lane >= o) incl += y;
+                }
+                write(incl - m, __shfl_sync(0xffffffffu, incl, 31));
+                return;
+            }
             uint32_t ex = __popc(some & ((1u << lane) - 1u)), tot = __popc(some);
-            if (__any_sync(0xffffffffu, m > 1u)) {
+            if (__any_sync(0xffffffffu, m > 1u)) {   // (at most 32 x CC_STAGE rows from here on)
                 uint32_t incl = m;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -541,16 +564,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 tot = __shfl_sync(0xffffffffu, incl, 31);
                 ex = incl - m;
             }
-            const int32_t rb = (int32_t)(turned ? c : b), rc = (int32_t)(turned ? b : c);
-            if (tot > CC_STAGE) {   // many copies: not staged
-                unsigned long long p = 0;
-                if (lane == 0) p = atomicAdd(n_rows, (unsigned long long)tot);
-                p = __shfl_sync(0xffffffffu, p, 0) + ex;
-                for (uint32_t e = 0; e < m && p < capacity; ++e, ++p) {
-                    rows[3 * p] = (int32_t)a;
-                    rows[3 * p + 1] = rb;
-                    rows[3 * p + 2] = rc;
-                }
+            if (tot > CC_STAGE) {
+                write(ex, tot);
                 return;
             }
             if (staged + tot > CC_STAGE) flush();
