@@ -15,12 +15,19 @@ struct LinRowsArgs {
     DevStatus *st;
 };
 
+// S tuples that make many rows: entry e is S tuple i[e], its rows go to p[e] and
+// its first piece is number s[e].
+struct BigTuples {
+    unsigned long long *n;   // entries << 32 | pieces
+    uint32_t *i, *s;
+    unsigned long long *p;
+};
+
 struct LinRowsLayout {
     RGroup r, t;
     uint32_t *rmeta, *tmeta;
     unsigned int *hll, *bump;
-    uint32_t *big_i;               // S tuples with many rows, and where they go
-    unsigned long long *big_p;
+    BigTuples big;
 };
 void lin_rows_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, LinRowsLayout &L);
 // rows (a, b, c, d) into rows[0, min(n_rows, capacity)); *total = n_rows; more rows than the capacity is an error.
