@@ -174,10 +174,11 @@ mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
 /* Star 3-way join R(A,B) S(B,C) T(C,D) (Section 6, "linear star 3-way
  * join"): the same query and outputs as mwj_join3_linear, planned for small
  * dimension relations R and T and a large fact relation S.  S is read once,
- * unpartitioned.  COUNT and GROUP BY A: T's degree table and a weight table
- * with R's keys in the L2 (as in mwj_join3_linear); each S tuple whose b is a
- * key of R adds deg_T(c) to w(b), and R's groups are added at the end; shares
- * are not used.  MATERIALIZE: R is grouped by h(B) and T by g(C) into bucket
+ * unpartitioned.  COUNT: R's and T's degree tables in the L2, the sum of
+ * deg_R(b) deg_T(c) over S.  GROUP BY A: T's degree table and a weight table
+ * with R's keys (as in mwj_join3_linear); each S tuple whose b is a key of R
+ * adds deg_T(c) to w(b), and R's groups are added at the end.  Neither uses the
+ * shares (relations of at most 2^19 tuples run as a linear join does).  MATERIALIZE: R is grouped by h(B) and T by g(C) into bucket
  * tables, S read twice (a counting pass, then the rows).  shares: s[0] = h(B) buckets
  * of R, s[1] = g(C) buckets of T (0 or shares == NULL: about 2048 tuples per
  * bucket); s[2] is ignored.  GROUP BY A checks the domain of A while it adds

@@ -20,10 +20,10 @@
 // summed inside each warp before they reach the L2; the R pass only reads
 // the table and adds each run of equal a once.
 //
-// A star join is the same three passes with the weight table laid out for R's
-// B values instead of S's (star_bucket_run): R is the small relation, so its
-// column is the cheap one to size, and S tuples whose b is not R's are
-// skipped.
+// A star join's GROUP BY is the same three passes with the weight table laid
+// out for R's B values instead of S's (star_bucket_run): R is the small
+// relation, so its column is the cheap one to size, and S tuples whose b is not
+// R's are skipped.  Its COUNT needs no weights: deg_R(b) deg_T(c) summed over S.
 #include <algorithm>
 #include <type_traits>
 
@@ -112,32 +112,34 @@ __device__ __forceinline__ void deg_add(unsigned long long *slots, uint32_t mask
 // atomics whose results are not needed (exact modulo 2^64, no carry word).
 // FILTER: a key outside the table's range is no error but a tuple that joins
 // nothing (star joins, whose table holds R's keys).
+// wshift: the sum of key k is at W[(k - min) << wshift] (kMetaShift; star joins only).
 template <bool FILTER>
 __device__ __forceinline__ void w_add_direct(unsigned long long *__restrict__ W, uint32_t wmin, uint32_t wspan,
-                                             uint32_t b, unsigned long long x, DevStatus *st) {
+                                             uint32_t wshift, uint32_t b, unsigned long long x, DevStatus *st) {
     if (b - wmin < wspan)
-        atomicAdd(W + (b - wmin), x);
+        atomicAdd(W + ((b - wmin) << (FILTER ? wshift : 0u)), x);
     else if (!FILTER)
         set_status(st, MWJ_ERR_CHECK, 9);   // a key outside the range the sizing pass saw
 }
 
 // w(k[q]) for the lane's tuples q < m (0 for the others) from a weight table
 // in either layout; hashed: the key groups are loaded together, then the sums.
-template <bool WD>
+template <bool WD, bool STAR = false>
 struct WLookup {
     const WTable &w;
-    uint32_t mask, min, span;
+    uint32_t mask, min, span, shift;
     __device__ explicit WLookup(const WTable &w_) : w(w_) {
         mask = __ldg(w.meta);
         min = WD ? __ldg(w.meta + kMetaMin) : 0u;
         span = WD ? __ldg(w.meta + kMetaSpan) : 0u;
+        shift = WD && STAR ? __ldg(w.meta + kMetaShift) : 0u;
     }
     __device__ __forceinline__ void operator()(const int32_t (&k)[WQ], uint32_t m, unsigned long long (&x)[WQ]) const {
         if constexpr (WD) {
 #pragma unroll
             for (int q = 0; q < WQ; ++q) {
                 const uint32_t i = (uint32_t)k[q] - min;
-                x[q] = ((uint32_t)q < m && i < span) ? __ldg(w.W + i) : 0ull;
+                x[q] = ((uint32_t)q < m && i < span) ? __ldg(w.W + (STAR ? i << shift : i)) : 0ull;
             }
         } else {
             uint32_t s[WQ];
@@ -236,13 +238,14 @@ struct SPass {
     DevStatus *st;
     const uint32_t *hs;
     HeavySums &hacc;
-    uint32_t wmin, wspan;
+    uint32_t wmin, wspan, wshift;
 
     __device__ SPass(const Source &src, const WTable &w_, DevStatus *st_, const uint32_t *hs_,
                      HeavySums &hacc_)
         : look(make_lookup<SW>(src)), w(w_), st(st_), hs(hs_), hacc(hacc_) {
         wmin = __ldg(w.meta + kMetaMin);
         wspan = __ldg(w.meta + kMetaSpan);
+        wshift = FILTER ? __ldg(w.meta + kMetaShift) : 0u;
     }
 
     __device__ __forceinline__ void round(const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) {
@@ -260,7 +263,7 @@ struct SPass {
             }
         }
         warp_runs(b, x, m, [&](int32_t key, unsigned long long sum) {
-            w_add_direct<FILTER>(w.W, wmin, wspan, (uint32_t)key, sum, st);
+            w_add_direct<FILTER>(w.W, wmin, wspan, wshift, (uint32_t)key, sum, st);
         });
     }
 
@@ -269,7 +272,7 @@ struct SPass {
         if (!hs) return;
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < kHeavySlots; i += nthreads)
-            if (heavy_sum(hacc, i)) w_add_direct<FILTER>(w.W, wmin, wspan, hs[i], heavy_sum(hacc, i), st);
+            if (heavy_sum(hacc, i)) w_add_direct<FILTER>(w.W, wmin, wspan, wshift, hs[i], heavy_sum(hacc, i), st);
     }
 };
 
@@ -332,6 +335,10 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
                    sspan = sd ? __ldg(smeta + kMetaSpan) : 0u;
     const uint32_t wmask = __ldg(w.meta + kMetaMask), wmin = wd ? __ldg(w.meta + kMetaMin) : 0u,
                    wspan = wd ? __ldg(w.meta + kMetaSpan) : 0u;
+    const uint32_t wshift = wd && FILTER ? __ldg(w.meta + kMetaShift) : 0u;
+    auto group = [&](uint32_t s) {   // four keys of the table (FILTER: none is added in this kernel)
+        return FILTER ? __ldg((const uint4 *)(w.keys + s)) : __ldcg((const uint4 *)(w.keys + s));
+    };
     auto value = [&](uint32_t c) -> unsigned long long {
         if (sd) {
             const uint32_t i = c - smin;
@@ -350,7 +357,7 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
     };
     auto add = [&](uint32_t b, uint32_t s, uint4 v, unsigned long long x) {
         if (wd) {
-            w_add_direct<FILTER>(w.W, wmin, wspan, b, x, st);
+            w_add_direct<FILTER>(w.W, wmin, wspan, wshift, b, x, st);
             return;
         }
         const uint32_t at = b == kEmptyKey ? wmask + 1
@@ -379,7 +386,7 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (!wd) {   // the target's key group, with the source's slot
             s = w_home((uint32_t)b, w.seed, wmask);
-            v = __ldcg((const uint4 *)(w.keys + s));
+            v = group(s);
         }
         unsigned long long x = has ? value((uint32_t)c) : 0ull;
         if (hs && x) {
@@ -400,7 +407,7 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
         const unsigned long long x = heavy_sum(hacc, j);
         if (!x) continue;
         const uint32_t s = wd ? 0u : w_home(hs[j], w.seed, wmask);
-        add(hs[j], s, wd ? make_uint4(0u, 0u, 0u, 0u) : __ldcg((const uint4 *)(w.keys + s)), x);
+        add(hs[j], s, wd ? make_uint4(0u, 0u, 0u, 0u) : group(s), x);
     }
 }
 
@@ -418,6 +425,79 @@ __global__ void __launch_bounds__(WT) k_w_build_direct(const int32_t *__restrict
     rounds_plain(Sb, Sc, 0u, n, warp, warps,
                  [&](const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) { P.round(b, c, m); });
     P.flush_heavy(WT);
+}
+
+// Star joins, COUNT: the sum of deg_R(b) deg_T(c) over S, two lookups a tuple and
+// no add.  With R's weights, as GROUP BY has them, hot keys in no order cost many
+// times as much: a call of 2^26 facts on 1000 uniform keys 2.03 ms, 2^24 on 1000
+// Zipf keys 0.58, now 0.128 and 0.055 (where no key is hot, 2^26 facts on 2^20
+// uniform keys, 0.45 and 0.49).  DIRECT: both tables direct-address; the call
+// launches both kernels.
+template <bool DIRECT>
+struct Deg32 {
+    const DegTable &t;
+    const uint32_t mask, min, span;
+    const bool dense;
+    __device__ explicit Deg32(const DegTable &t_)
+        : t(t_), mask(__ldg(t_.meta + kMetaMask)), min(__ldg(t_.meta + kMetaMin)), span(__ldg(t_.meta + kMetaSpan)),
+          dense(DIRECT || __ldg(t_.meta + kMetaDense) != 0u) {}
+    // deg(k[q]) of the lane's keys q < m, 0 for the others; hashed: the four home
+    // pairs are loaded together, as key, degree, key, degree
+    __device__ __forceinline__ void operator()(const int32_t (&k)[WQ], uint32_t m, uint32_t (&x)[WQ]) const {
+        if (DIRECT || dense) {
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) {
+                const uint32_t i = (uint32_t)k[q] - min;
+                x[q] = ((uint32_t)q < m && i < span) ? __ldg((const uint32_t *)t.slots + i) : 0u;
+            }
+            return;
+        }
+        uint4 v[WQ];
+        uint32_t more = 0;
+#pragma unroll
+        for (int q = 0; q < WQ; ++q) {
+            v[q] = make_uint4(0u, 0u, kEmptyKey, kEmptyKey);
+            if ((uint32_t)q < m) v[q] = __ldg((const uint4 *)(t.slots + deg_home((uint32_t)k[q], t.seed, mask)));
+        }
+#pragma unroll
+        for (int q = 0; q < WQ; ++q) {
+            const uint32_t c = (uint32_t)k[q];
+            x[q] = v[q].x == c ? v[q].y : v[q].z == c ? v[q].w : 0u;
+            if (x[q] == 0u && v[q].w != kEmptyKey && (uint32_t)q < m) more |= 1u << q;   // the pair is full
+            if (x[q] == kEmptyKey || (uint32_t)q >= m) x[q] = 0u;   // (key -1 against a free slot)
+        }
+        while (more) {   // rare: the pairs after the home pair
+            const uint32_t q = (uint32_t)__ffs((int)more) - 1u;
+            more &= more - 1u;
+            const uint32_t c = (uint32_t)(q == 0u ? k[0] : q == 1u ? k[1] : q == 2u ? k[2] : k[3]);
+            const uint32_t s = (deg_home(c, t.seed, mask) + 2u) & mask;
+            const uint32_t d = (uint32_t)deg_get(t.slots, mask, c, s, __ldg((const ulonglong2 *)(t.slots + s)));
+#pragma unroll
+            for (uint32_t u = 0; u < WQ; ++u)
+                if (u == q) x[u] = d;
+        }
+    }
+};
+
+template <bool DIRECT>
+__global__ void __launch_bounds__(WT) k_star_total(const int32_t *__restrict__ Sb, const int32_t *__restrict__ Sc,
+                                                   uint32_t n, DegTable r, DegTable t,
+                                                   unsigned long long *__restrict__ total) {
+    after_previous();
+    if ((__ldg(r.meta + kMetaDense) && __ldg(t.meta + kMetaDense)) != DIRECT) return;
+    __shared__ unsigned long long red[32];
+    const Deg32<DIRECT> lr(r), lt(t);
+    unsigned long long acc = 0;
+    const uint32_t warp = (blockIdx.x * WT + threadIdx.x) >> 5, warps = (gridDim.x * WT) >> 5;
+    rounds_plain(Sb, Sc, 0u, n, warp, warps, [&](const int32_t (&b)[WQ], const int32_t (&c)[WQ], uint32_t m) {
+        uint32_t x[WQ], y[WQ];
+        lr(b, m, x);
+        lt(c, m, y);
+#pragma unroll
+        for (int q = 0; q < WQ; ++q) acc += (unsigned long long)x[q] * y[q];
+    });
+    acc = block_sum_u64(acc, red);
+    if (threadIdx.x == 0 && acc) atomicAdd(total, acc);
 }
 
 // Star joins, hashed layout: R's keys into the weight table, so that the S pass
@@ -440,9 +520,9 @@ __global__ void __launch_bounds__(WT) k_w_keys(const int32_t *__restrict__ Rb, u
 // One warp round of the R pass: x = w(b) for the lane's tuples (a[q], b[q]),
 // q < m, added to the thread's total and (GROUP BY A) per run of equal a to
 // cnt[a].
-template <int MODE, bool WD>
+template <int MODE, bool WD, bool STAR>
 struct RPass {
-    const WLookup<WD> look;
+    const WLookup<WD, STAR> look;
     int32_t a_domain;
     unsigned long long *cnt;
     DevStatus *st;
@@ -467,13 +547,13 @@ struct RPass {
     }
 };
 
-template <int MODE, bool WD>
+template <int MODE, bool WD, bool STAR = false>
 __device__ __forceinline__ void w_probe_pass(const int32_t *__restrict__ Ra, const int32_t *__restrict__ Rb,
                                              uint32_t n, const WTable &w, int32_t a_domain,
                                              unsigned long long *__restrict__ cnt,
                                              unsigned long long *__restrict__ total, DevStatus *st,
                                              unsigned long long *red) {
-    RPass<MODE, WD> P(w, a_domain, cnt, st);
+    RPass<MODE, WD, STAR> P(w, a_domain, cnt, st);
     const uint32_t warp = (blockIdx.x * WT + threadIdx.x) >> 5, warps = (gridDim.x * WT) >> 5;
     rounds_plain(Ra, Rb, 0u, n, warp, warps,
                  [&](const int32_t (&a)[WQ], const int32_t (&b)[WQ], uint32_t m) { P.round(a, b, m); });
@@ -493,7 +573,7 @@ __global__ void __launch_bounds__(WT) k_w_probe(const int32_t *__restrict__ Ra, 
     w_probe_pass<MODE, false>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
 }
 
-template <int MODE>
+template <int MODE, bool STAR>
 __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict__ Ra,
                                                        const int32_t *__restrict__ Rb, uint32_t n, WTable w,
                                                        int32_t a_domain, unsigned long long *__restrict__ cnt,
@@ -501,7 +581,7 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
     after_previous();
     if (!__ldg(w.meta + kMetaDense)) return;
     __shared__ unsigned long long red[32];
-    w_probe_pass<MODE, true>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
+    w_probe_pass<MODE, true, STAR>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
 }
 
 // T pass: the degrees of the last relation's key column.
@@ -919,13 +999,13 @@ size_t w_table_slots(int64_t nS) { return single_table_slots(nS); }
 
 namespace {
 
-cudaError_t deg_build(const mwj_rel &T, const DegTable &t, DevStatus *status, int num_sms, cudaStream_t st,
-                      const HeavyArgs &heavy = HeavyArgs{}) {
-    const uint32_t n = (uint32_t)T.n;
+cudaError_t deg_build(const int32_t *keys, int64_t nkeys, const DegTable &t, DevStatus *status, int num_sms,
+                      cudaStream_t st, const HeavyArgs &heavy = HeavyArgs{}) {
+    const uint32_t n = (uint32_t)nkeys;
     if (n + heavy.n == 0) return cudaSuccess;
     const uint32_t groups = (n + WQ * DT - 1) / (WQ * DT), full = (uint32_t)num_sms * 3;
     ProfScope ps_("t_insert", st);
-    return launch_after(k_deg_build, heavy.n + (groups < full ? (groups ? groups : 1u) : full), DT, st, T.x, n, t, heavy,
+    return launch_after(k_deg_build, heavy.n + (groups < full ? (groups ? groups : 1u) : full), DT, st, keys, n, t, heavy,
                         status);
 }
 
@@ -955,10 +1035,10 @@ cudaError_t w_table_build(const mwj_rel &S, const Source &src, Pass pass, const 
 
 cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a_domain, unsigned long long *cnt,
                           unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st,
-                          bool hashed_only = false) {
+                          bool hashed_only = false, bool star = false) {
     if (R.n <= 0) return cudaSuccess;
     const uint32_t n = (uint32_t)R.n;
-    auto direct = mode == 1 ? k_w_probe_direct<1> : k_w_probe_direct<0>;
+    auto direct = star ? k_w_probe_direct<1, true> : mode == 1 ? k_w_probe_direct<1, false> : k_w_probe_direct<0, false>;
     auto hashed = mode == 1 ? k_w_probe<1> : k_w_probe<0>;
     if (!hashed_only) {
         ProfScope ps_(mode == 1 ? "w_probe_groupby" : "w_probe_count", st);
@@ -994,7 +1074,7 @@ bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32
         if (r.n > kMediumHeavy)
             heavy.h[heavy.n++] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)L.w[k].heavy};
     }
-    if ((*e = deg_build(rel[nrel - 1], L.deg, status, num_sms, st, heavy)) != cudaSuccess) return true;
+    if ((*e = deg_build(rel[nrel - 1].x, rel[nrel - 1].n, L.deg, status, num_sms, st, heavy)) != cudaSuccess) return true;
     Source src{};
     src.t = L.deg;
     for (int k = 0; k < nrel - 2; ++k) {
@@ -1065,7 +1145,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     if ((e = tables_clear(clear, (uint32_t)nrel - 1u, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull,
                           total, num_sms, st)) != cudaSuccess)
         return e;
-    if ((e = deg_build(last, L.deg, status, num_sms, st)) != cudaSuccess) return e;
+    if ((e = deg_build(last.x, last.n, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     Source src{};
     src.t = L.deg;
     for (int k = 0; k < nrel - 2; ++k) {
@@ -1075,14 +1155,42 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     return w_table_probe(rel[0], L.w[nrel - 3], mode, a_domain, cnt, total, status, num_sms, st);
 }
 
+// The weights are R's, not S's, except in a small call (a chain like any other):
+// room for either, so that what a call asks for grows with its sizes.
+static int64_t star_weights(const mwj_rel &R, const mwj_rel &S) { return std::max(R.n, std::min(S.n, kMediumMax)); }
+
 void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, OneBucket &L) {
-    // the weights are R's, not S's, except in a small call (a chain like any
-    // other): room for either, so that what a call asks for grows with its sizes
     mwj_rel w = R;
-    w.n = std::max(R.n, std::min(S.n, kMediumMax));
+    w.n = star_weights(R, S);
     const mwj_rel rel[3] = {R, w, T};
     one_bucket_layout(A, rel, 3, num_sms, L);
 }
+
+namespace {
+
+// COUNT: R's degrees in the place of the weight table.
+cudaError_t star_count(const OneBucket &L, const SizeCol (&cols)[2], const mwj_rel &R, const mwj_rel &S, const mwj_rel &T,
+                       unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st) {
+    cudaError_t e;
+    const DegTable r{L.w[0].W, L.w[0].meta, L.w[0].seed};
+    const ClearTable clear[2] = {ClearTable{L.deg.slots, nullptr, L.deg.meta}, ClearTable{r.slots, nullptr, r.meta}};
+    if ((e = size_columns(cols, 2, nullptr, 0, true, num_sms, st)) != cudaSuccess) return e;
+    if ((e = tables_clear(clear, 2, nullptr, 0ull, total, num_sms, st)) != cudaSuccess) return e;
+    if ((e = deg_build(T.x, T.n, L.deg, status, num_sms, st)) != cudaSuccess) return e;
+    if ((e = deg_build(R.y, R.n, r, status, num_sms, st)) != cudaSuccess) return e;
+    if (S.n <= 0) return cudaSuccess;
+    const uint32_t n = (uint32_t)S.n;
+    {
+        ProfScope ps_("star_count", st);
+        e = launch_after(k_star_total<true>, pass_grid(n, num_sms, kDirectCtas, WCHUNK), WT, st, S.x, S.y, n, r, L.deg, total);
+        if (e != cudaSuccess) return e;
+    }
+    ProfScope ps_("star_count_hashed", st);
+    return launch_after(k_star_total<false>, pass_grid(n, num_sms, kHashedProbeCtas, WCHUNK), WT, st, S.x, S.y, n, r, L.deg,
+                        total);
+}
+
+}  // namespace
 
 cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd, int mode,
                             int32_t a_domain, unsigned long long *cnt, unsigned long long *total, DevStatus *status,
@@ -1093,8 +1201,10 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     const mwj_rel rel[3] = {R, S, T};
     if (small_run(L, rel, 3, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
     const uint64_t tr = single_table_slots(T.n), rr = w_table_slots(R.n);
+    const uint64_t rw = w_table_slots(star_weights(R, S));   // what is reserved
     const SizeCol cols[2] = {SizeCol{T.x, (uint32_t)T.n, sd.slot2, L.hll[0], {L.deg.meta}, {tr}, {tr}, 1u},
-                             SizeCol{R.y, (uint32_t)R.n, sd.slot, L.hll[1], {L.w[0].meta}, {rr}, {rr}, 1u}};
+                             SizeCol{R.y, (uint32_t)R.n, sd.slot, L.hll[1], {L.w[0].meta}, {rr}, {rr}, 1u, mode == 1 ? rw : 0ull}};
+    if (mode == 0) return star_count(L, cols, R, S, T, total, status, num_sms, st);
     const HeavyCol heavy{S.x, (uint32_t)S.n, kWHeavyBuckets, (uint32_t *)L.w[0].heavy};
     const ClearTable clear[2] = {ClearTable{L.deg.slots, nullptr, L.deg.meta},
                                  ClearTable{L.w[0].W, L.w[0].keys, L.w[0].meta}};
@@ -1102,7 +1212,7 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     if ((e = tables_clear(clear, 2, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull, total, num_sms,
                           st)) != cudaSuccess)
         return e;
-    if ((e = deg_build(T, L.deg, status, num_sms, st)) != cudaSuccess) return e;
+    if ((e = deg_build(T.x, T.n, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     if (R.n > 0) {
         ProfScope ps_("star_keys", st);
         if ((e = launch_after(k_w_keys, pass_grid((uint32_t)R.n, num_sms, 8, 32), WT, st, R.y, (uint32_t)R.n, L.w[0],
@@ -1112,7 +1222,7 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     Source src{};
     src.t = L.deg;
     if ((e = w_table_build(S, src, PASS_STAR, L.w[0], status, num_sms, st)) != cudaSuccess) return e;
-    return w_table_probe(R, L.w[0], mode, a_domain, cnt, total, status, num_sms, st);
+    return w_table_probe(R, L.w[0], mode, a_domain, cnt, total, status, num_sms, st, false, true);
 }
 
 }  // namespace mwj

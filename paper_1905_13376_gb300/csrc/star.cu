@@ -7,12 +7,17 @@
 // loads R and T into the units first and then routes every S tuple to the
 // unit of its pair.  On this GPU the on-chip memory that every SM can reach
 // is the L2 (with the L1 in front of it).  The two aggregates are passes of
-// the one-bucket plan (linear_l2.cu, star_bucket_run): T's degrees, then
+// the one-bucket plan (linear_l2.cu, star_bucket_run): T's degrees, then for
+// COUNT R's degrees and
+//
+//   total += deg_R(b) deg_T(c)          per S tuple
+//
+// and for GROUP BY A
 //
 //   w[b] += deg_T(c)                    per S tuple whose b is R's
 //   cnt[a] += w[b], total += w[b]       per (a, b) of R
 //
-// with both tables direct-address arrays when the dimension keys are compact.
+// with the tables direct-address arrays when the dimension keys are compact.
 // Row output groups R by h(B) and T by g(C) into bucket tables that also hold
 // the lists b -> [a] and c -> [d]; every CTA streams its own contiguous
 // stretch of S straight from the input columns, looking each tuple up in both:

@@ -497,6 +497,20 @@ __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
     }
 }
 
+// A star join's weights (SizeCol::spread): many tuples add to few keys, and adds
+// that meet in an L2 line wait for one another.  Direct-address entries are set
+// apart, up to a line of 16 for each, while the table takes at most 2^18 entries
+// (2 MB): 2^26 facts on 1000, 3000 and 10,000 keys in no order take 2.03, 0.80 and
+// 0.46 ms packed, 0.65, 0.58 and 0.36 a sector apart, 0.48, 0.35 and 0.29 a line
+// apart.  Hashed tables get 16 slots a key up to 2^16 slots.
+constexpr uint64_t kSpreadEntries = 1u << 18, kSpreadSlots = 1u << 16;
+__device__ __forceinline__ uint32_t spread_shift(uint64_t span, uint64_t room) {
+    uint32_t sh = 0;
+    const uint64_t most = room < kSpreadEntries ? room : kSpreadEntries;
+    while (sh < 4 && (span << (sh + 1)) <= most) ++sh;
+    return sh;
+}
+
 // HyperLogLog registers (Flajolet, Fusy, Gandouet, Meunier 2007): register
 // h >> (32 - HLL_BITS) keeps the largest rank (position of the first 1 bit)
 // of the remaining bits.  mix32 is a bijection of 32-bit keys, so distinct
@@ -550,6 +564,7 @@ __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(SizeArgs g) {
                     c.meta[q][kMetaMask] = 15u;
                     c.meta[q][kMetaMin] = (uint32_t)lo;
                     c.meta[q][kMetaSpan] = (uint32_t)((int64_t)hi - (int64_t)lo + 1);
+                    c.meta[q][kMetaShift] = spread_shift((uint64_t)((int64_t)hi - (int64_t)lo + 1), c.spread);
                 }
             }
         }
@@ -699,6 +714,7 @@ __global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(SizeArgs g) {
         uint64_t cap = 16;
         while ((double)cap < factor * E && cap < res) cap <<= 1;
         if (cap > res) cap = res;
+        while ((double)cap < 16.0 * E && 2 * cap <= kSpreadSlots && 2 * cap <= c.spread) cap <<= 1;
         mt[kMetaMask] = (uint32_t)(cap - 1);
         mt[kMetaEst] = (uint32_t)E;
     }
@@ -732,7 +748,7 @@ __global__ void __launch_bounds__(BT) k_tables_clear(ClearArgs g) {
         return;
     }
     // weights: zero sums (hashed: of slot mask + 1, key -1, too), free keys
-    const uint64_t sums = dense ? (uint64_t)t.meta[kMetaSpan] : (uint64_t)t.meta[kMetaMask] + 2;
+    const uint64_t sums = dense ? (uint64_t)t.meta[kMetaSpan] << t.meta[kMetaShift] : (uint64_t)t.meta[kMetaMask] + 2;
     for (uint64_t s = i0; s < (sums + 1) / 2; s += stride) ((ulonglong2 *)t.tbl)[s] = make_ulonglong2(0ull, 0ull);
     if (dense) return;
     const uint4 free4 = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);

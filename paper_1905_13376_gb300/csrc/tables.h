@@ -6,10 +6,11 @@
 namespace mwj {
 
 // Words of a single table's meta array: mask of the hashed slots, distinct
-// estimate, an unused word, and, when the sizing pass chose the direct-address layout (kMetaDense = 1), the smallest
-// key and the span of the keys: the entry of key k is then at k - min,
+// estimate, and, when the sizing pass chose the direct-address layout
+// (kMetaDense = 1), the smallest key, the span of the keys and a shift: the entry
+// of key k is then at (k - min) << shift (0 for all but a star join's weights),
 // nothing is hashed and no key is stored.
-constexpr int kMetaMask = 0, kMetaEst = 1, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5;
+constexpr int kMetaMask = 0, kMetaEst = 1, kMetaShift = 2, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5;
 constexpr int kMetaWords = 8;
 
 // J == 0: one table of (meta[0] + 1) packed (deg << 32 | c) slots, home slot
@@ -96,6 +97,9 @@ struct SizeCol {
     uint32_t *meta[kSizeCols];
     uint64_t reserve[kSizeCols], range[kSizeCols];
     uint32_t ntargets;
+    // > 0: the direct-address entries of the (one) table are spread out over this
+    // many at most, so that adds to neighbouring keys meet in no L2 sector
+    uint64_t spread = 0;
 };
 // A column whose heavy keys (sampled share at least 1 / (2 x buckets)) are
 // named by the first of these launches (allow_dense only) in `heavy`
