@@ -40,6 +40,12 @@ constexpr uint32_t CC_CH = 1024;         // wedges of a list per warp step (32 p
 // (probe of the 2^22-vertex graph, lists up to 4096: 21.0 ms from 512 on, 20.7 from
 // 1024, 20.4 from 2048 or none)
 constexpr uint32_t kQueueMin = 2048;
+// An item of few S tuples (no more than the queue has places) has about as many
+// batches as warps or fewer: there lists of kFewMin entries go to the queue
+// already, and are shared in pieces of kFewStep.  Three relations of 1e4 tuples,
+// Zipf 1.1 (lists of 1300 in items of 32 tuples): 0.63 ms with one limit of 2048,
+// 0.17 with the two; 6e4 tuples on 300 keys (lists of 200) 0.47 and 0.18.
+constexpr uint32_t kFewMin = 128, kFewStep = 256;
 constexpr uint32_t CC_STAGE = 32;        // rows that a warp of the row pass stages
 constexpr uint32_t CC_QCAP_ROWS = 384;   // its queue's places: the rest hold the staged rows
 constexpr uint32_t kTurned = 0x80000000u;   // row output: mark of a turned tuple, in its list's start
@@ -447,6 +453,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
         const uint32_t li = item - item_off[lo];
         const uint32_t tci = li / sch, sci = li - tci * sch;
         const uint32_t s0 = g.offS[k] + sci * g.schunk, s1 = min(g.offS[k + 1], s0 + g.schunk);
+        const bool few = s1 - s0 <= QCAP;
+        const uint32_t qmin = few ? kFewMin : kQueueMin, qstep = few ? kFewStep : CC_CH;
         // T_k's set: the item's chunk on chip, or for a big bucket its region
         // of the workspace, built before this kernel
         bool big = cc_big(g.offT[k + 1] - g.offT[k]);
@@ -593,7 +601,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             return 0u;
         };
         // walk one list of the warp's: entries [lo, hi) from alist[jst & ~3] on,
-        // those before jst left out, lo a multiple of CC_CH.  In steps of CC_CH
+        // those before jst left out, lo a multiple of four.  In steps of CC_CH
         // entries: first the filter bits, 16 bytes of the list per lane and load
         // (a lane's 32 bits in the order of its entries, the first one on top),
         // then the set for those that passed, whose a is read again.  Every lane
@@ -642,7 +650,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
         };
         // phase 1: warps take batches of 32 S tuples as they come free;
-        // lists of kQueueMin or more entries go to the item's queue (walked at
+        // lists of qmin or more entries go to the item's queue (walked at
         // once when it is full), lists of 32 or more are walked by the warp,
         // shorter ones are spread over the warp's lanes, wedge wi going to
         // the first lane whose inclusive count exceeds it
@@ -666,7 +674,7 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 }
             }
             bool spill = false;
-            if (n >= kQueueMin) {
+            if (n >= qmin) {
                 const uint32_t qs = atomicAdd(&qn, 1u);
                 if (qs < QCAP)
                     queue[qs] = make_uint4(b, c, st, n);
@@ -681,8 +689,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                      __shfl_sync(0xffffffffu, st, j), 0u,
                      __shfl_sync(0xffffffffu, n + (st & 3u), j));
             }
-            // lists of 32 .. kQueueMin - 1 entries: the warp walks each one
-            unsigned mid_ = __ballot_sync(0xffffffffu, n >= 32u && n < kQueueMin);
+            // lists of 32 .. qmin - 1 entries: the warp walks each one
+            unsigned mid_ = __ballot_sync(0xffffffffu, n >= 32u && n < qmin);
             while (mid_) {
                 const int j = __ffs(mid_) - 1;
                 mid_ &= mid_ - 1u;
@@ -723,12 +731,12 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
             }
         }
         __syncthreads();
-        // phase 2: the queued lists in chunks of CC_CH entries, taken by the
+        // phase 2: the queued lists in chunks of qstep entries, taken by the
         // warps as they come free (a hub's long list is shared by all of them)
         const uint32_t nq = min(qn, QCAP);
         for (uint32_t q0 = 0; q0 <= nq; q0 += CC_T) {
             const uint32_t q = q0 + threadIdx.x;
-            const uint32_t d = q < nq ? ((queue[q].z & 3u) + queue[q].w + CC_CH - 1) / CC_CH : 0u;
+            const uint32_t d = q < nq ? ((queue[q].z & 3u) + queue[q].w + qstep - 1) / qstep : 0u;
             uint32_t tot;
             const uint32_t ex = block_excl_scan_u32(d, scan_scratch, &tot);
             if (q <= nq) cpre[q] = carry + ex;
@@ -748,8 +756,8 @@ __global__ void __launch_bounds__(CC_T, CC_MAX_CTAS_PER_SM) k_cc_probe(CycCArgs 
                 if (cpre[mid] <= ci) lo = mid; else hi = mid;
             }
             const uint4 L = queue[lo];
-            const uint32_t first = (ci - cpre[lo]) * CC_CH;
-            walk(L.x, L.y, L.z, first, min(first + CC_CH, (L.z & 3u) + L.w));
+            const uint32_t first = (ci - cpre[lo]) * qstep;
+            walk(L.x, L.y, L.z, first, min(first + qstep, (L.z & 3u) + L.w));
         }
         acc_all += acc;
         __syncthreads();
