@@ -45,7 +45,8 @@ constexpr uint32_t kQueueMin = 2048;
 // already, and are shared in pieces of kFewStep.  Three relations of 1e4 tuples,
 // Zipf 1.1 (lists of 1300 in items of 32 tuples): 0.63 ms with one limit of 2048,
 // 0.17 with the two; 6e4 tuples on 300 keys (lists of 200) 0.47 and 0.18.
-constexpr uint32_t kFewMin = 128, kFewStep = 256;
+constexpr uint32_t kFewMin = 128, kFewStep = 512;
+static_assert((uint64_t)CC_QCAP * ((1ull << 31) / kFewStep + 1) < 1ull << 32, "the queue's pieces are counted in 32 bits");
 constexpr uint32_t CC_STAGE = 32;        // rows that a warp of the row pass stages
 constexpr uint32_t CC_QCAP_ROWS = 384;   // its queue's places: the rest hold the staged rows
 constexpr uint32_t kTurned = 0x80000000u;   // row output: mark of a turned tuple, in its list's start
