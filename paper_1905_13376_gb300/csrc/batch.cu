@@ -710,7 +710,8 @@ uint32_t pow2_ge(uint64_t v) {
 struct Rule {
     uint32_t tpb;    // linear: R tuples per bucket
     uint32_t tfac;   // linear: T table slots per tuple
-    double fit;      // cyclic: fraction of a tile's capacity R_ij and T_ki may fill
+    double fit;      // cyclic: fraction of a tile's capacity R_ij and T_ki may fill,
+    double fine;     // and in a batch of few tiles
 };
 
 Rule batch_rule(const mwj_ctx *ctx, const mwj_query &q) {
@@ -720,10 +721,10 @@ Rule batch_rule(const mwj_ctx *ctx, const mwj_query &q) {
     const int k = q.kind == MWJ_LINEAR ? 0 : 1;
     // (fit: a tile above its capacity is only taken in two items; the cyclic half
     // of a 1024-query batch takes 3.98 ms at 0.5, 3.42 at 0.75, 3.17 at 0.95)
-    Rule r{8192u, 2u, 0.95};
+    Rule r{8192u, 2u, 0.95, 0.5};
     if (ctx->batch_tpb[k][c] > 0) r.tpb = (uint32_t)ctx->batch_tpb[k][c];
     if (ctx->batch_tfac[k][c] > 0) r.tfac = (uint32_t)ctx->batch_tfac[k][c];
-    if (ctx->batch_fit[k][c] > 0) r.fit = ctx->batch_fit[k][c] / 100.0;
+    if (ctx->batch_fit[k][c] > 0) r.fit = r.fine = ctx->batch_fit[k][c] / 100.0;
     return r;
 }
 
@@ -746,12 +747,19 @@ int cyc_rotation(const mwj_query &q) {
 // read (1024-query batch, cyclic half: 5.24 ms at 0, 4.97 at 1024, 4.87 at 4096,
 // another 0.07 less at 16384).
 constexpr double kTileCost = 16384.0;
+// A batch whose tiles, cut that way, are fewer than the persistent launch's CTAs
+// takes finer shares instead, without the tile cost and at half the fit: what counts
+// there is that the wedges are spread over the GPU.  One query of 1e4 tuples a
+// relation on 101 keys 276 us (8 tiles) -> 63, 16 of 5000 on 71 keys 204 -> 76, 16
+// of 2e4 on 142 keys 527 -> 287.  Where few tuples meet the tiles are what costs:
+// 16 of 2e4 on 2501 keys 88 -> 116 us.
 constexpr uint64_t kLinS = 16384;
 
 // shares of one batched query from its sizes: linear: about rule.tpb R
-// tuples per bucket; cyclic: the cost-model choice (z|R| + x|S| + y|T| + kTileCost xyz)
-// under the chunk fit, with every relation's bucket count at most kSegMaxP
-void batch_shares(const mwj_query &q, const Rule &rule, mwj_shares *sh) {
+// tuples per bucket; cyclic: the cost-model choice (z|R| + x|S| + y|T| + kTileCost xyz,
+// fine: without the last) under the chunk fit, with every relation's bucket count at
+// most kSegMaxP
+void batch_shares(const mwj_query &q, const Rule &rule, bool fine, mwj_shares *sh) {
     if (q.kind == MWJ_LINEAR) {
         // (and no more than kLinS S tuples per item on average: one CTA streams
         // a bucket's S alone, and a small R with a large S was the batch's tail)
@@ -765,14 +773,15 @@ void batch_shares(const mwj_query &q, const Rule &rule, mwj_shares *sh) {
         return;
     }
     const double nR = (double)q.R.n, nS = (double)q.S.n, nT = (double)q.T.n;
+    const double fit = fine ? rule.fine : rule.fit, tile_cost = fine ? 0.0 : kTileCost;
     double best = INFINITY;
     uint32_t bx = 1, by = 1, bz = 1;
     for (uint32_t x = 1; x <= 64; x <<= 1)
         for (uint32_t y = 1; y <= 64; y <<= 1)
             for (uint32_t z = 1; z <= 64; z <<= 1) {
                 if (x * y > kSegMaxP || y * z > kSegMaxP || z * x > kSegMaxP) continue;
-                if (nR / (x * y) > rule.fit * CRCAP || nT / (z * x) > rule.fit * CTCAP) continue;
-                const double cost = z * nR + x * nS + y * nT + kTileCost * x * y * z;
+                if (nR / (x * y) > fit * CRCAP || nT / (z * x) > fit * CTCAP) continue;
+                const double cost = z * nR + x * nS + y * nT + tile_cost * x * y * z;
                 if (cost < best) {
                     best = cost;
                     bx = x;
@@ -817,23 +826,36 @@ mwj_status mwj_batch_create(mwj_ctx *ctx, const mwj_query *queries, int32_t n, m
         A.take<char>(bytes);
         return reinterpret_cast<char *>(static_cast<uintptr_t>(off));
     };
-    uint32_t tiles = 0;
+    auto turned = [](mwj_query q, int rot) {   // the query from another corner (cyc_rotation)
+        const mwj_rel rel[3] = {q.R, q.S, q.T};
+        q.R = rel[rot];
+        q.S = rel[(rot + 1) % 3];
+        q.T = rel[(rot + 2) % 3];
+        return q;
+    };
+    uint64_t coarse = 0;   // cyclic tiles
     for (int32_t qi = 0; qi < n; ++qi) {
-        mwj_query q = queries[qi];
+        const mwj_query &q = queries[qi];
         if ((q.kind != MWJ_LINEAR && q.kind != MWJ_CYCLIC) || !rel_ok(q.R) || !rel_ok(q.S) ||
             !rel_ok(q.T)) {
             delete b;
             return fail(ctx, MWJ_ERR_INVALID_ARG, "query %d: bad kind or relation", qi);
         }
+        if (q.kind != MWJ_CYCLIC) continue;
+        mwj_shares sh = q.shares;
+        if (sh.s[0] <= 0) batch_shares(turned(q, cyc_rotation(q)), batch_rule(ctx, q), false, &sh);
+        if (sh.s[1] > 0 && sh.s[2] > 0) coarse += (uint64_t)sh.s[0] * (uint64_t)sh.s[1] * (uint64_t)sh.s[2];
+    }
+    const bool fine = coarse < 2u * (uint64_t)ctx->dev.num_sms;
+    uint32_t tiles = 0;
+    for (int32_t qi = 0; qi < n; ++qi) {
+        mwj_query q = queries[qi];
         mwj_shares sh = q.shares;
         const Rule rule = batch_rule(ctx, q);
         if (sh.s[0] <= 0) {
             const int rot = q.kind == MWJ_CYCLIC ? cyc_rotation(q) : 0;
-            const mwj_rel rel[3] = {q.R, q.S, q.T};
-            q.R = rel[rot];
-            q.S = rel[(rot + 1) % 3];
-            q.T = rel[(rot + 2) % 3];
-            batch_shares(q, rule, &sh);
+            q = turned(q, rot);
+            batch_shares(q, rule, fine, &sh);
             // reported for the query's own A, B, C: the rotated query's k-th is its (k + rot)-th
             mwj_shares own = sh;
             for (int k = 0; q.kind == MWJ_CYCLIC && k < 3; ++k) own.s[(k + rot) % 3] = sh.s[k];
