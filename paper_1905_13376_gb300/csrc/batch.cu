@@ -113,11 +113,17 @@ __device__ __forceinline__ void ttab_insert(unsigned long long *tbl, uint32_t ma
 }
 
 // ---- persistent segment kernel --------------------------------------------
-// A thread keeps PU tuples in flight: one CTA reads a whole relation twice, so
-// the largest one's latency is the kernel's (1.38 ms for the 1024-query batch
-// with one tuple in flight, 1.03 ms with eight).
-constexpr uint32_t PU = 8;
-__global__ void __launch_bounds__(BTH) k_batch_prep(BatchDev b, unsigned int *counter, DevStatus *st) {
+// A thread keeps PU tuples in flight.  One CTA reads a whole relation twice, so
+// the largest one's latency is the kernel's: 1.38 ms for the 1024-query batch with
+// one tuple in flight, 1.03 ms with eight, which take the registers of three CTAs.
+// Where no relation is large and there are several for every SM the CTAs hide each
+// other's latency instead, and one tuple is enough (linear batches of 256 queries,
+// 500, 5000 and 10,000 tuples a relation, whole call: 28, 85 and 158 us with eight,
+// 20, 74 and 149 with one; 20,000: 304 and 327; 64 queries of 5000: 51 and 58).
+constexpr uint32_t kPrepMany = 8;
+constexpr uint32_t kPrepSmall = 16384;   // tuples of the largest relation
+template <uint32_t PU>
+__global__ void __launch_bounds__(BTH, PU == 1 ? 3 : 1) k_batch_prep(BatchDev b, unsigned int *counter, DevStatus *st) {
     __shared__ uint32_t hist[kSegMaxP + 1];
     __shared__ uint32_t scan_scratch[33];
     __shared__ uint32_t seg_s, carry;
@@ -1031,7 +1037,10 @@ mwj_status mwj_batch_launch(mwj_batch *b, int64_t *counts, void *workspace, size
         return cuda_fail(ctx, e, "memset counter");
     {
         ProfScope ps_("batch_prep", st);
-        k_batch_prep<<<sms * (b->prep_cps > 0 ? b->prep_cps : 3), BTH, 0, st>>>(b->dev, counter, ctx->status);
+        // (the segments are sorted by size)
+        const bool small = !b->segs.empty() && b->segs[0].n <= kPrepSmall && b->segs.size() > 2u * (size_t)sms;
+        auto prep = small ? k_batch_prep<1> : k_batch_prep<kPrepMany>;
+        prep<<<sms * (b->prep_cps > 0 ? b->prep_cps : 3), BTH, 0, st>>>(b->dev, counter, ctx->status);
     }
     if (b->ncyc_tiles) {
         {
