@@ -417,8 +417,12 @@ struct SizeArgs {
     bool ranged;   // k_range has run: a compact column gets the direct-address layout
 };
 
-__device__ __forceinline__ bool span_fits(int32_t lo, int32_t hi, uint64_t most) {
-    return lo <= hi && (uint64_t)((int64_t)hi - (int64_t)lo + 1) <= most;
+// Entries from lo to hi, 0 when there is none or they are more than `most` (or than
+// 32 bits hold: a table of 2^32 entries has no span).
+__device__ __forceinline__ uint32_t span_within(int32_t lo, int32_t hi, uint64_t most) {
+    if (lo > hi) return 0u;
+    const uint64_t span = (uint64_t)((int64_t)hi - (int64_t)lo + 1);
+    return span <= most && span <= 0xFFFFFFFFull ? (uint32_t)span : 0u;
 }
 
 // Key range of every column: `rows` CTAs per column, each leaving the
@@ -556,15 +560,16 @@ __global__ void __launch_bounds__(BT, HLL_CTAS_PER_SM) k_hll(SizeArgs g) {
         hi = shi;
         bool all = true;
         for (uint32_t q = 0; q < c.ntargets; ++q) {
-            const bool dense = span_fits(lo, hi, c.range[q]);
+            const uint32_t span = span_within(lo, hi, c.range[q]);
+            const bool dense = span != 0u;
             all = all && dense;
             if (first) {
                 c.meta[q][kMetaDense] = dense ? 1u : 0u;
                 if (dense) {
                     c.meta[q][kMetaMask] = 15u;
                     c.meta[q][kMetaMin] = (uint32_t)lo;
-                    c.meta[q][kMetaSpan] = (uint32_t)((int64_t)hi - (int64_t)lo + 1);
-                    c.meta[q][kMetaShift] = spread_shift((uint64_t)((int64_t)hi - (int64_t)lo + 1), c.spread);
+                    c.meta[q][kMetaSpan] = span;
+                    c.meta[q][kMetaShift] = spread_shift(span, c.spread);
                 }
             }
         }
@@ -710,7 +715,8 @@ __global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(SizeArgs g) {
     for (uint32_t t = 0; t < c.ntargets; ++t) {
         uint32_t *mt = c.meta[t];
         if (__ldcg(mt + kMetaDense)) continue;
-        const uint64_t res = c.reserve[t];
+        // 2^31 slots hold the keys of any relation; masks of 32 ones are none
+        const uint64_t res = c.reserve[t] < (1ull << 31) ? c.reserve[t] : 1ull << 31;
         uint64_t cap = 16;
         while ((double)cap < factor * E && cap < res) cap <<= 1;
         if (cap > res) cap = res;
