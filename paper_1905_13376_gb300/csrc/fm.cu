@@ -558,6 +558,13 @@ cudaError_t fm_one_run(const FmOneLayout &L, const mwj_rel &R, const mwj_rel &S,
         cols[1] = SizeCol{S.x, (uint32_t)S.n, g.s.seed, L.hll[1], {g.s.meta}, {single_table_slots(S.n)}, {(uint64_t)S.n}, 1u};
         ncols = 2;
     }
+    // entries of 64 bytes, half an L2 line (2^24 tuples, 2^20 keys over 2^24 places 2.60
+    // ms direct-address and 2.87 hashed, 2^16 keys 1.96 and 1.58; 2^23 tuples, 2^16 keys
+    // over 2^22 places 0.65 and 1.01)
+    for (uint32_t k = 0; k < ncols; ++k) {
+        cols[k].sure = 1ull << 22;
+        cols[k].per_key = 40.0;
+    }
     cudaError_t e;
     if ((e = size_columns(cols, ncols, nullptr, 0, true, sms, st)) != cudaSuccess) return e;
     const uint64_t most = (uint64_t)(T.n > S.n ? T.n : S.n);

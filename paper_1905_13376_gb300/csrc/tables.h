@@ -10,7 +10,8 @@ namespace mwj {
 // (kMetaDense = 1), the smallest key, the span of the keys and a shift: the entry
 // of key k is then at (k - min) << shift (0 for all but a star join's weights),
 // nothing is hashed and no key is stored.
-constexpr int kMetaMask = 0, kMetaEst = 1, kMetaShift = 2, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5;
+// kMetaTry: that layout is left to the distinct estimate.
+constexpr int kMetaMask = 0, kMetaEst = 1, kMetaShift = 2, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5, kMetaTry = 6;
 constexpr int kMetaWords = 8;
 
 // J == 0: one table of (meta[0] + 1) packed (deg << 32 | c) slots, home slot
@@ -100,6 +101,11 @@ struct SizeCol {
     // > 0: the direct-address entries of the (one) table are spread out over this
     // many at most, so that adds to neighbouring keys meet in no L2 sector
     uint64_t spread = 0;
+    // a range of at most `sure` entries is direct-address whatever the number of
+    // distinct keys, a larger one when it is at most `per_key` times the estimate
+    // or the keys are few (k_hll)
+    uint64_t sure = 1ull << 24;
+    double per_key = 8.0;
 };
 // A column whose heavy keys (sampled share at least 1 / (2 x buckets)) are
 // named by the first of these launches (allow_dense only) in `heavy`
