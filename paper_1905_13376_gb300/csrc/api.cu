@@ -344,7 +344,7 @@ mwj_status mwj_workspace_size(mwj_ctx *ctx, int kind, mwj_rel R, mwj_rel S, mwj_
     if (mode < MWJ_COUNT || mode > MWJ_MATERIALIZE) return fail(ctx, MWJ_ERR_INVALID_ARG, "bad mode");
     mwj_shares sh;
     if (kind == MWJ_LINEAR) {
-        if (!shares && mode == MWJ_MATERIALIZE) {
+        if (!shares && mode == MWJ_MATERIALIZE && lin_rows_takes(R, T)) {
             Arena A(nullptr, 0);
             LinRowsLayout L;
             lin_rows_layout(A, R, S, T, ctx->dev.num_sms, L);
@@ -381,7 +381,7 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
     mwj_status s = check_out(ctx, out, 4);
     if (s != MWJ_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if (!shares && out->mode == MWJ_MATERIALIZE) {   // rows: lists of R and T, S streamed past them
+    if (!shares && out->mode == MWJ_MATERIALIZE && lin_rows_takes(R, T)) {   // rows: lists of R and T, S streamed past them
         Arena A(workspace, ws_bytes);
         LinRowsLayout L;
         lin_rows_layout(A, R, S, T, ctx->dev.num_sms, L);

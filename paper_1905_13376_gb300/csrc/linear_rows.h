@@ -29,6 +29,9 @@ struct LinRowsLayout {
     unsigned int *hll, *bump;
     BigTuples big;
 };
+// Relations whose lists are numbered in 31 bits (a relation's entries, at most four
+// times its tuples, and one for key -1); larger ones run the partitioned plan.
+inline bool lin_rows_takes(const mwj_rel &R, const mwj_rel &T) { return R.n < 1ll << 29 && T.n < 1ll << 29; }
 void lin_rows_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, LinRowsLayout &L);
 // rows (a, b, c, d) into rows[0, min(n_rows, capacity)); *total = n_rows; more rows than the capacity is an error.
 cudaError_t lin_rows_run(LinRowsLayout &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd,
