@@ -1055,6 +1055,15 @@ cudaError_t w_table_probe(const mwj_rel &R, const WTable &w, int mode, int32_t a
 
 namespace {
 
+// Many groups are zeroed by a memset of their own: the CTAs that clear them beside
+// the tables do not reach memory speed (2^20 tuples a relation, 2^26, 2^27 and 2^28
+// groups 178, 288 and 499 us in all that way, 145, 214 and 353 with the memset).
+constexpr int32_t kMemsetGroups = 1 << 24;
+cudaError_t zero_groups(int mode, int32_t a_domain, unsigned long long *cnt, bool *zeroed, cudaStream_t st) {
+    *zeroed = mode == 1 && a_domain > kMemsetGroups;
+    return *zeroed ? cudaMemsetAsync(cnt, 0, sizeof(*cnt) * (size_t)a_domain, st) : cudaSuccess;
+}
+
 // The small plans; false when the call is larger.
 bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32_t a_domain, unsigned long long *cnt,
                unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st, cudaError_t *e) {
@@ -1142,8 +1151,11 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     }
     if (small_run(L, rel, nrel, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
     if ((e = size_columns(cols, ncols, heavy, (uint32_t)nrel - 2u, true, num_sms, st)) != cudaSuccess) return e;
-    if ((e = tables_clear(clear, (uint32_t)nrel - 1u, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull,
-                          total, num_sms, st)) != cudaSuccess)
+    bool zeroed;
+    if ((e = zero_groups(mode, a_domain, cnt, &zeroed, st)) != cudaSuccess) return e;
+    const bool zero = mode == 1 && !zeroed;
+    if ((e = tables_clear(clear, (uint32_t)nrel - 1u, zero ? cnt : nullptr, zero ? (uint64_t)a_domain : 0ull, total,
+                          num_sms, st)) != cudaSuccess)
         return e;
     if ((e = deg_build(last.x, last.n, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     Source src{};
@@ -1209,8 +1221,11 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     const ClearTable clear[2] = {ClearTable{L.deg.slots, nullptr, L.deg.meta},
                                  ClearTable{L.w[0].W, L.w[0].keys, L.w[0].meta}};
     if ((e = size_columns(cols, 2, &heavy, 1, true, num_sms, st)) != cudaSuccess) return e;
-    if ((e = tables_clear(clear, 2, mode == 1 ? cnt : nullptr, mode == 1 ? (uint64_t)a_domain : 0ull, total, num_sms,
-                          st)) != cudaSuccess)
+    bool zeroed;
+    if ((e = zero_groups(mode, a_domain, cnt, &zeroed, st)) != cudaSuccess) return e;
+    const bool zero = mode == 1 && !zeroed;
+    if ((e = tables_clear(clear, 2, zero ? cnt : nullptr, zero ? (uint64_t)a_domain : 0ull, total, num_sms, st)) !=
+        cudaSuccess)
         return e;
     if ((e = deg_build(T.x, T.n, L.deg, status, num_sms, st)) != cudaSuccess) return e;
     if (R.n > 0) {
