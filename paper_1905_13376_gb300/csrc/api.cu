@@ -232,6 +232,7 @@ mwj_status mwj_create(mwj_ctx **out, const mwj_config *cfg) {
     cudaDeviceGetAttribute(&ctx->dev.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&ctx->dev.cc_major, cudaDevAttrComputeCapabilityMajor, dev);
     cudaDeviceGetAttribute(&ctx->dev.cc_minor, cudaDevAttrComputeCapabilityMinor, dev);
+    ctx->dev.cluster = chain_cluster_limit();
     ctx->seed = c.seed;
     ctx->seeds = make_seeds(c.seed);
     ctx->smem_bytes = c.smem_bytes;
@@ -414,7 +415,7 @@ mwj_status mwj_join3_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
         const mwj_rel rel[3] = {R, S, T};
         e = one_bucket_run(L.one, rel, 3, sd, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
                            (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
-                           ctx->dev.num_sms, st);
+                           ctx->dev, st);
         return e == cudaSuccess ? MWJ_OK : cuda_fail(ctx, e, "one-bucket plan");
     }
     if ((e = cudaMemsetAsync(out->total, 0, sizeof(int64_t), st)) != cudaSuccess)

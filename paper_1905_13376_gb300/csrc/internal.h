@@ -59,6 +59,7 @@ struct DevInfo {
     int num_sms;
     int smem_optin;   // max dynamic shared memory per block (opt-in)
     int cc_major, cc_minor;
+    int cluster;      // CTAs of the largest cluster the small plan can launch (chain_cluster_limit)
 };
 
 // Round up to a multiple of 256 bytes.

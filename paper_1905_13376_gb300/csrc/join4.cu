@@ -204,7 +204,7 @@ extern "C" mwj_status mwj_join4_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_r
             const cudaError_t eo =
                 one_bucket_run(L, rel, 4, ctx->seeds, out->mode == MWJ_COUNT_GROUP_BY_A ? 1 : 0, out->a_domain,
                                (unsigned long long *)out->group_counts, (unsigned long long *)out->total, ctx->status,
-                               ctx->dev.num_sms, (cudaStream_t)stream);
+                               ctx->dev, (cudaStream_t)stream);
             return eo == cudaSuccess ? MWJ_OK : cuda_fail(ctx, eo, "chain of four, one bucket");
         }
         plan_linear_default(ctx, R, S, T, &sh);

@@ -935,8 +935,16 @@ bool chain_within(const mwj_rel *rel, int nrel, int64_t most) {
         if (rel[k].n > most) return false;
     return true;
 }
-bool chain_is_small(const mwj_rel *rel, int nrel, int mode, int32_t a_domain) {
-    return chain_within(rel, nrel, kSmallMax) && (mode != 1 || a_domain <= kSmallGroups);
+// CTAs of the cluster that takes the call: one per 1024 tuples (and per 16K groups to
+// zero), a power of two up to 16; 0: the call is too large for one.
+int chain_cluster(const mwj_rel *rel, int nrel, int mode, int32_t a_domain) {
+    if (!chain_within(rel, nrel, kSmallMax) || (mode == 1 && a_domain > kSmallGroups)) return 0;
+    int64_t most = 1;
+    for (int k = 0; k < nrel; ++k) most = rel[k].n > most ? rel[k].n : most;
+    const int64_t want = (most + CT - 1) / CT, wantg = mode == 1 ? ((int64_t)a_domain + 16383) / 16384 : 1;
+    int ctas = 1;
+    while (ctas < kSmallCtas && (ctas < want || ctas < wantg)) ctas <<= 1;
+    return ctas;
 }
 
 // Tables as one_bucket_layout laid them out (at least two slots per tuple).
@@ -959,29 +967,24 @@ SmallArgs small_args(const OneBucket &L, const mwj_rel *rel, int nrel, int mode,
     return g;
 }
 
-cudaError_t chain_small(const SmallArgs &g, cudaStream_t st) {
-    int64_t most = 1;
-    for (int k = 0; k < g.nrel; ++k) most = g.rel[k].n > most ? g.rel[k].n : most;
-    // a CTA per 1024 tuples (and per 16K groups to zero), a power of two up to a cluster's 16
-    const int64_t want = (most + CT - 1) / CT, wantg = g.mode == 1 ? ((int64_t)g.a_domain + 16383) / 16384 : 1;
-    int ctas = 1;
-    while (ctas < kSmallCtas && (ctas < want || ctas < wantg)) ctas <<= 1;
-    if (ctas > 8) {   // more than the portable cluster size
-        const cudaError_t e = cudaFuncSetAttribute(k_chain_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
+struct ClusterLaunch {
     cudaLaunchConfig_t c{};
-    c.gridDim = dim3(ctas);
-    c.blockDim = dim3(CT);
-    c.stream = st;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ctas;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    c.attrs = at;
-    c.numAttrs = 1;
+    ClusterLaunch(int ctas, cudaStream_t st) {
+        c.gridDim = dim3(ctas);
+        c.blockDim = dim3(CT);
+        c.stream = st;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = ctas;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        c.attrs = at;
+        c.numAttrs = 1;
+    }
+};
+cudaError_t chain_small(const SmallArgs &g, int ctas, cudaStream_t st) {
+    const ClusterLaunch l(ctas, st);
     ProfScope ps_("chain_small", st);
-    return cudaLaunchKernelEx(&c, k_chain_small, g);
+    return cudaLaunchKernelEx(&l.c, k_chain_small, g);
 }
 
 // CTAs of a grid-stride pass: per_sm of them on every SM (what the registers
@@ -996,6 +999,18 @@ constexpr uint32_t kDirectCtas = 5, kProbeCtas = 5, kHashedProbeCtas = 4;
 }  // namespace
 
 size_t w_table_slots(int64_t nS) { return single_table_slots(nS); }
+
+int chain_cluster_limit() {
+    for (int ctas = kSmallCtas; ctas > 1; ctas >>= 1) {
+        const ClusterLaunch l(ctas, nullptr);
+        int n = 0;
+        if ((ctas <= 8 || cudaFuncSetAttribute(k_chain_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+            cudaOccupancyMaxActiveClusters(&n, k_chain_small, &l.c) == cudaSuccess && n > 0)
+            return ctas;
+        cudaGetLastError();
+    }
+    return 1;
+}
 
 namespace {
 
@@ -1064,14 +1079,17 @@ cudaError_t zero_groups(int mode, int32_t a_domain, unsigned long long *cnt, boo
     return *zeroed ? cudaMemsetAsync(cnt, 0, sizeof(*cnt) * (size_t)a_domain, st) : cudaSuccess;
 }
 
-// The small plans; false when the call is larger.
+// The small plans; false when the call is larger.  A device, partition or stream
+// whose SMs have no room for the cluster gets the four launches.
 bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32_t a_domain, unsigned long long *cnt,
-               unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st, cudaError_t *e) {
+               unsigned long long *total, DevStatus *status, const DevInfo &dev, cudaStream_t st, cudaError_t *e) {
     if (!chain_within(rel, nrel, kMediumMax)) return false;
+    const int num_sms = dev.num_sms;
     SmallArgs g = small_args(L, rel, nrel, mode, a_domain, cnt, total, status);
-    if (chain_is_small(rel, nrel, mode, a_domain)) {
-        *e = chain_small(g, st);
-        return true;
+    const int ctas = chain_cluster(rel, nrel, mode, a_domain);
+    if (ctas > 0 && ctas <= dev.cluster) {
+        if ((*e = chain_small(g, ctas, st)) == cudaSuccess) return true;
+        cudaGetLastError();   // refused (nothing of it runs): not the call's error
     }
     {
         ProfScope ps_("chain_clear", st);
@@ -1115,9 +1133,10 @@ void one_bucket_layout(Arena &A, const mwj_rel *rel, int nrel, int num_sms, OneB
 }
 
 cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const Seeds &sd, int mode, int32_t a_domain,
-                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, int num_sms,
+                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, const DevInfo &dev,
                            cudaStream_t st) {
     cudaError_t e;
+    const int num_sms = dev.num_sms;
     const mwj_rel &last = rel[nrel - 1];
     const uint32_t seeds[kChainMax - 2] = {nrel == 3 ? sd.slot : sd.slot ^ sd.D, sd.slot};
     // the key columns (of every relation but R); a column that plays two
@@ -1149,7 +1168,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
         heavy[k] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)w.heavy};
         clear[k + 1] = ClearTable{w.W, w.keys, w.meta};
     }
-    if (small_run(L, rel, nrel, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
+    if (small_run(L, rel, nrel, mode, a_domain, cnt, total, status, dev, st, &e)) return e;
     if ((e = size_columns(cols, ncols, heavy, (uint32_t)nrel - 2u, true, num_sms, st)) != cudaSuccess) return e;
     bool zeroed;
     if ((e = zero_groups(mode, a_domain, cnt, &zeroed, st)) != cudaSuccess) return e;
@@ -1206,12 +1225,13 @@ cudaError_t star_count(const OneBucket &L, const SizeCol (&cols)[2], const mwj_r
 
 cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd, int mode,
                             int32_t a_domain, unsigned long long *cnt, unsigned long long *total, DevStatus *status,
-                            int num_sms, cudaStream_t st) {
+                            const DevInfo &dev, cudaStream_t st) {
     cudaError_t e;
+    const int num_sms = dev.num_sms;
     L.deg.seed = sd.slot2;
     L.w[0].seed = sd.slot;
     const mwj_rel rel[3] = {R, S, T};
-    if (small_run(L, rel, 3, mode, a_domain, cnt, total, status, num_sms, st, &e)) return e;
+    if (small_run(L, rel, 3, mode, a_domain, cnt, total, status, dev, st, &e)) return e;
     const uint64_t tr = single_table_slots(T.n), rr = w_table_slots(R.n);
     const uint64_t rw = w_table_slots(star_weights(R, S));   // what is reserved
     const SizeCol cols[2] = {SizeCol{T.x, (uint32_t)T.n, sd.slot2, L.hll[0], {L.deg.meta}, {tr}, {tr}, 1u},

@@ -47,15 +47,18 @@ struct OneBucket {
 };
 // rel[0] = R ... rel[nrel - 1]: the last (nrel 3 or 4).
 void one_bucket_layout(Arena &A, const mwj_rel *rel, int nrel, int num_sms, OneBucket &L);
+// Largest power of two of CTAs (at most 16) that the current device launches as one
+// cluster of the small plan; 1: none.  Also allows the sizes above 8.
+int chain_cluster_limit();
 // COUNT (mode 0: *total) or GROUP BY A (mode 1: cnt[0, a_domain) too); the
 // outputs are zeroed here.  a outside [0, a_domain) raises MWJ_ERR_DOMAIN.
 cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const Seeds &sd, int mode, int32_t a_domain,
-                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, int num_sms,
+                           unsigned long long *cnt, unsigned long long *total, DevStatus *status, const DevInfo &dev,
                            cudaStream_t st);
 // The same for a star join (small R and T, large S): w[0] holds R's keys.
 void star_bucket_layout(Arena &A, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, int num_sms, OneBucket &L);
 cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, const mwj_rel &T, const Seeds &sd, int mode,
                             int32_t a_domain, unsigned long long *cnt, unsigned long long *total, DevStatus *status,
-                            int num_sms, cudaStream_t st);
+                            const DevInfo &dev, cudaStream_t st);
 
 }  // namespace mwj

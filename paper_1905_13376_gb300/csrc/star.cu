@@ -341,7 +341,7 @@ extern "C" mwj_status mwj_join3_star(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel
     cudaError_t e;
     if (!p.rows) {
         e = star_bucket_run(L.one, R, S, T, sd, p.group ? 1 : 0, out->a_domain, (unsigned long long *)out->group_counts,
-                            (unsigned long long *)out->total, ctx->status, sms, st);
+                            (unsigned long long *)out->total, ctx->status, ctx->dev, st);
         return e == cudaSuccess ? MWJ_OK : cuda_fail(ctx, e, "star aggregates");
     }
     // row output: R as (b, a) pairs by h(B), T as (c, d) pairs by g(C),
