@@ -217,7 +217,10 @@ mwj_status mwj_join4_linear(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T, mwj_r
  * (MWJ_ERR_DOMAIN from mwj_stream_status otherwise).  shares: s[0] = H(B)
  * buckets; the other entries are ignored.  NULL: one bucket while S and T have
  * at most 2^28 tuples each (a 64-byte row of bitmaps per key of T's C and S's
- * B, a pass over each relation), else ~16K S tuples per bucket.
+ * B, a pass over each relation), else ~16K S tuples per bucket.  The number of
+ * keys is not known when the workspace is asked for: with NULL it has a row for
+ * every tuple of S and of T, 80 bytes and more each (explicit shares: of T
+ * only); a smaller one makes the call partition.
  * workspace: device, >= mwj_fm_workspace_size(...). */
 mwj_status mwj_fm_workspace_size(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
                                  const mwj_shares *shares, size_t *bytes);

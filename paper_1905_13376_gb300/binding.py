@@ -272,6 +272,19 @@ class Context:
             self._ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
         return self._ws
 
+    def _less(self, err, shares, full, size, partitioned):
+        """After running out of device memory for the workspace (of `full` bytes) of
+        the plan without shares: the partitioned plan's shares and its workspace, if
+        that takes less; otherwise the error stands."""
+        import torch
+        if shares is not None or not isinstance(err, torch.cuda.OutOfMemoryError):
+            raise err
+        sh = _shares(partitioned())
+        nb = size(sh)
+        if nb >= full:
+            raise err
+        return sh, self.workspace(nb)
+
     def workspace_size(self, kind, R, S, T, shares=None, mode=MWJ_COUNT) -> int:
         n = ctypes.c_size_t()
         self._check(self.lib.mwj_workspace_size(self.h, kind, _rel(R), _rel(S), _rel(T),
@@ -342,8 +355,17 @@ class Context:
         r, s, t, hs = _rel(R), _rel(S), _rel(T), self._stream(stream)
         sh = _shares(shares) if with_shares else None
         nb = ctypes.c_size_t()
-        self._check(self.lib.mwj_workspace_size(self.h, kind_ws, r, s, t, sh, mode, ctypes.byref(nb)))
-        ws = self.workspace(nb.value)
+
+        def size(sh):
+            self._check(self.lib.mwj_workspace_size(self.h, kind_ws, r, s, t, sh, mode, ctypes.byref(nb)))
+            return nb.value
+        size(sh)
+        try:
+            ws = self.workspace(nb.value)
+        except RuntimeError as e:
+            if kind_ws != MWJ_LINEAR or mode != MWJ_MATERIALIZE:
+                raise
+            sh, ws = self._less(e, sh, nb.value, size, lambda: self.plan_shares(MWJ_LINEAR, R, S, T, mode, stream))
         args = (self.h,) + tuple(extra) + (r, s, t)
         if with_shares:
             args = args + (sh,)
@@ -382,10 +404,18 @@ class Context:
         if isinstance(mode, str):
             mode = MODES[mode]
         o, res = self._outputs(mode, a_domain, 0, 4)
-        nb = ctypes.c_size_t(0)
         rels, sh = (_rel(R), _rel(S), _rel(T), _rel(U)), _shares(shares)
-        self._check(self.lib.mwj_join4_workspace_size(self.h, *rels, sh, int(mode), ctypes.byref(nb)))
-        ws = self.workspace(nb.value)
+        nb = ctypes.c_size_t(0)
+
+        def size(sh):
+            self._check(self.lib.mwj_join4_workspace_size(self.h, *rels, sh, int(mode), ctypes.byref(nb)))
+            return nb.value
+        size(sh)
+        try:
+            ws = self.workspace(nb.value)
+        except RuntimeError as e:
+            sh, ws = self._less(e, sh, nb.value, size,
+                                lambda: self.plan_shares(MWJ_LINEAR, R, S, T, MWJ_MATERIALIZE, stream))
         self._check(self.lib.mwj_join4_linear(self.h, *rels, sh, ctypes.byref(o), ws.data_ptr(), ws.numel(),
                                               self._stream(stream)))
         if sync:
@@ -400,10 +430,18 @@ class Context:
         import torch
         sk = torch.empty((int(a_domain), 16), dtype=torch.int32, device=self.device)
         est = torch.empty(int(a_domain), dtype=torch.float32, device=self.device) if estimates else None
-        nb = ctypes.c_size_t(0)
         rels, sh = (_rel(R), _rel(S), _rel(T)), _shares(shares)
-        self._check(self.lib.mwj_fm_workspace_size(self.h, *rels, sh, ctypes.byref(nb)))
-        ws = self.workspace(nb.value)
+        nb = ctypes.c_size_t(0)
+
+        def size(sh):
+            self._check(self.lib.mwj_fm_workspace_size(self.h, *rels, sh, ctypes.byref(nb)))
+            return nb.value
+        size(sh)
+        try:
+            ws = self.workspace(nb.value)
+        except RuntimeError as e:   # (about 16K S tuples per bucket)
+            sh, ws = self._less(e, sh, nb.value, size,
+                                lambda: (min(1 << max(10, (rels[1].n // 16384).bit_length()), 16384), 1, 1))
         self._check(self.lib.mwj_fm_linear(self.h, *rels, sh, int(a_domain), sk.data_ptr(),
                                            est.data_ptr() if est is not None else None,
                                            ws.data_ptr(), ws.numel(), self._stream(stream)))
