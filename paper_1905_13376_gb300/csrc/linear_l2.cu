@@ -593,6 +593,11 @@ __global__ void __launch_bounds__(WT) k_w_probe_direct(const int32_t *__restrict
 // are not needed, exact modulo 2^32): a lane needs only the keys beside its
 // own, no search for where a run ends, and a run inside one lane is one add.
 // Hashed slots: a key per lane, as in the general S pass.
+// In the direct-address layout heavy keys (sampled) are counted per CTA in shared
+// memory: keys that hold a large share in no order lie side by side there, and adds
+// that meet in an L2 sector wait for one another (this pass over 2^22 and 2^23 keys,
+// Zipf 1.1, the most frequent the smallest: 757 and 1500 us without, 392 and 790 with;
+// two keys in turn at random 880 and 18).
 // The first nheavy CTAs sample the heavy keys of the weight passes instead (the
 // medium plan, which has no range pass to do it in).
 constexpr int DT = 512;
@@ -612,7 +617,7 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
     const uint32_t cta = blockIdx.x - heavy.n, ctas = gridDim.x - heavy.n;
     const uint32_t mask = t.meta[kMetaMask];
     const bool dense = t.meta[kMetaDense] != 0u;
-    const uint32_t kmin = dense ? t.meta[kMetaMin] : 0u, span = dense ? t.meta[kMetaSpan] : 0u;
+    const uint32_t kmin = t.meta[kMetaMin], span = t.meta[kMetaSpan];   // (dense)
     uint32_t *deg = (uint32_t *)t.slots;
     const bool vec = ((uintptr_t)keys & 15) == 0;
     const uint64_t pol = l2_evict_first();
@@ -648,14 +653,31 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
         }
         return;
     }
-    auto add = [&](int32_t key, uint32_t x) {
-        const uint32_t k = (uint32_t)key - kmin;
+    // the first keys are on their way while the heavy ones are looked at
+    int32_t v[G][WQ];
+    uint32_t m[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) m[g] = load(warp * G + g, v[g]);
+    // heavy keys are counted in shared memory (in the sample's place)
+    uint32_t *const hbuf = hsm.key, *const hsum = hsm.cnt;
+    static_assert(HeavySample<1024>::slots >= kHeavySlots, "room for the table and its sums");
+    for (uint32_t i = threadIdx.x; i < kHeavySlots; i += DT) hsum[i] = 0u;
+    const uint32_t *const hs = heavy_to_smem(t.heavy, hbuf);   // (ends with a barrier when there are any)
+    auto heavy_counted = [&](uint32_t k, uint32_t x) -> bool {
+        const uint32_t s = slot_of(k, kHeavySeed, kHeavySlots - 1), q = hs[s];
+        if (q == kEmptyKey) return false;
+        const int i = q == k ? (int)s : heavy_slot(hs, k);
+        if (i >= 0) atomicAdd(hsum + i, x);
+        return i >= 0;
+    };
+    auto add_word = [&](uint32_t key, uint32_t x) {
+        const uint32_t k = key - kmin;
         if (k < span)
             atomicAdd(deg + k, x);
         else
             set_status(st, MWJ_ERR_CHECK, 8);   // a key outside the range the sizing pass saw
     };
-    auto block_dense = [&](const int32_t (&v)[WQ], uint32_t m, uint32_t valid) {
+    auto block_dense = [&](const int32_t (&v)[WQ], uint32_t m, uint32_t valid, auto &&add) {
         const int32_t prev = __shfl_up_sync(0xffffffffu, v[WQ - 1], 1);
         const int32_t next = __shfl_down_sync(0xffffffffu, v[0], 1);
         if (m == 0) return;
@@ -676,31 +698,39 @@ __global__ void __launch_bounds__(DT, 3) k_deg_build(const int32_t *__restrict__
         if (i0 + m == valid || cur != next) x += i0 + m;   // the run ends with this lane
         if (x) add(cur, x);
     };
-    const uint32_t rounds = (blocks + G - 1) / G;
-    int32_t v[G][WQ];
-    uint32_t m[G];
-    uint32_t r = warp;
+    auto blocks_in_turn = [&](auto &&add) {
+        const uint32_t rounds = (blocks + G - 1) / G;
+        uint32_t r = warp;
+        while (r < rounds) {
+            const uint32_t nr = r + warps;
+            int32_t nv[G][WQ];
+            uint32_t nm[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g) m[g] = load(r * G + g, v[g]);
-    while (r < rounds) {
-        const uint32_t nr = r + warps;
-        int32_t nv[G][WQ];
-        uint32_t nm[G];
+            for (int g = 0; g < G; ++g) nm[g] = load(nr * G + g, nv[g]);
 #pragma unroll
-        for (int g = 0; g < G; ++g) nm[g] = load(nr * G + g, nv[g]);
+            for (int g = 0; g < G; ++g) {
+                const uint32_t b0 = (r * G + g) * WCHUNK;
+                block_dense(v[g], m[g], b0 < n ? min(WCHUNK, n - b0) : 0u, add);
+            }
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const uint32_t b0 = (r * G + g) * WCHUNK;
-            block_dense(v[g], m[g], b0 < n ? min(WCHUNK, n - b0) : 0u);
+            for (int g = 0; g < G; ++g) {
+                m[g] = nm[g];
+#pragma unroll
+                for (int q = 0; q < WQ; ++q) v[g][q] = nv[g][q];
+            }
+            r = nr;
         }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            m[g] = nm[g];
-#pragma unroll
-            for (int q = 0; q < WQ; ++q) v[g][q] = nv[g][q];
-        }
-        r = nr;
+    };
+    if (!hs) {
+        blocks_in_turn([&](int32_t key, uint32_t x) { add_word((uint32_t)key, x); });
+        return;
     }
+    blocks_in_turn([&](int32_t key, uint32_t x) {
+        if (!heavy_counted((uint32_t)key, x)) add_word((uint32_t)key, x);
+    });
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < kHeavySlots; j += DT)
+        if (hsum[j]) add_word(hs[j], hsum[j]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1086,6 +1116,8 @@ bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32
     if (!chain_within(rel, nrel, kMediumMax)) return false;
     const int num_sms = dev.num_sms;
     SmallArgs g = small_args(L, rel, nrel, mode, a_domain, cnt, total, status);
+    DegTable deg = L.deg;
+    deg.heavy = nullptr;   // (not sampled)
     const int ctas = chain_cluster(rel, nrel, mode, a_domain);
     if (ctas > 0 && ctas <= dev.cluster) {
         if ((*e = chain_small(g, ctas, st)) == cudaSuccess) return true;
@@ -1101,9 +1133,9 @@ bool small_run(const OneBucket &L, const mwj_rel *rel, int nrel, int mode, int32
         if (r.n > kMediumHeavy)
             heavy.h[heavy.n++] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)L.w[k].heavy};
     }
-    if ((*e = deg_build(rel[nrel - 1].x, rel[nrel - 1].n, L.deg, status, num_sms, st, heavy)) != cudaSuccess) return true;
+    if ((*e = deg_build(rel[nrel - 1].x, rel[nrel - 1].n, deg, status, num_sms, st, heavy)) != cudaSuccess) return true;
     Source src{};
-    src.t = L.deg;
+    src.t = deg;
     for (int k = 0; k < nrel - 2; ++k) {
         WTable w = L.w[k];
         if (rel[nrel - 2 - k].n <= kMediumHeavy) w.heavy = nullptr;
@@ -1130,6 +1162,7 @@ void one_bucket_layout(Arena &A, const mwj_rel *rel, int nrel, int num_sms, OneB
         L.w[k].heavy = A.take<uint32_t>(kHeavyTableWords);
     }
     for (int k = 0; k < nrel - 1; ++k) L.hll[k] = A.take<unsigned int>(hll_scratch_registers(num_sms));
+    L.deg.heavy = A.take<uint32_t>(kHeavyTableWords);
 }
 
 cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const Seeds &sd, int mode, int32_t a_domain,
@@ -1158,6 +1191,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
     HeavyCol heavy[kSizeCols];
     ClearTable clear[kSizeCols];
     L.deg.seed = sd.slot2;
+    const uint32_t *const own = L.deg.heavy;
     add(last, L.deg.seed, L.deg.meta, single_table_slots(last.n));
     clear[0] = ClearTable{L.deg.slots, nullptr, L.deg.meta};
     for (int k = 0; k < nrel - 2; ++k) {
@@ -1166,10 +1200,14 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
         w.seed = seeds[k];
         add(r, w.seed, w.meta, w_table_slots(r.n));
         heavy[k] = HeavyCol{r.x, (uint32_t)r.n, kWHeavyBuckets, (uint32_t *)w.heavy};
+        if (r.x == last.x && r.n == last.n) L.deg.heavy = w.heavy;   // one sample does
         clear[k + 1] = ClearTable{w.W, w.keys, w.meta};
     }
     if (small_run(L, rel, nrel, mode, a_domain, cnt, total, status, dev, st, &e)) return e;
-    if ((e = size_columns(cols, ncols, heavy, (uint32_t)nrel - 2u, true, num_sms, st)) != cudaSuccess) return e;
+    uint32_t nheavy = (uint32_t)nrel - 2u;
+    if (L.deg.heavy == own)
+        heavy[nheavy++] = HeavyCol{last.x, (uint32_t)last.n, kWHeavyBuckets, (uint32_t *)own, true};
+    if ((e = size_columns(cols, ncols, heavy, nheavy, true, num_sms, st)) != cudaSuccess) return e;
     bool zeroed;
     if ((e = zero_groups(mode, a_domain, cnt, &zeroed, st)) != cudaSuccess) return e;
     const bool zero = mode == 1 && !zeroed;
@@ -1203,7 +1241,7 @@ namespace {
 cudaError_t star_count(const OneBucket &L, const SizeCol (&cols)[2], const mwj_rel &R, const mwj_rel &S, const mwj_rel &T,
                        unsigned long long *total, DevStatus *status, int num_sms, cudaStream_t st) {
     cudaError_t e;
-    const DegTable r{L.w[0].W, L.w[0].meta, L.w[0].seed};
+    const DegTable r{L.w[0].W, L.w[0].meta, L.w[0].seed, nullptr};
     const ClearTable clear[2] = {ClearTable{L.deg.slots, nullptr, L.deg.meta}, ClearTable{r.slots, nullptr, r.meta}};
     if ((e = size_columns(cols, 2, nullptr, 0, true, num_sms, st)) != cudaSuccess) return e;
     if ((e = tables_clear(clear, 2, nullptr, 0ull, total, num_sms, st)) != cudaSuccess) return e;
@@ -1229,6 +1267,7 @@ cudaError_t star_bucket_run(OneBucket &L, const mwj_rel &R, const mwj_rel &S, co
     cudaError_t e;
     const int num_sms = dev.num_sms;
     L.deg.seed = sd.slot2;
+    L.deg.heavy = nullptr;   // (a dimension's keys hardly repeat)
     L.w[0].seed = sd.slot;
     const mwj_rel rel[3] = {R, S, T};
     if (small_run(L, rel, 3, mode, a_domain, cnt, total, status, dev, st, &e)) return e;

@@ -17,6 +17,7 @@ struct DegTable {
     unsigned long long *slots;   // single_table_slots(n)
     uint32_t *meta;              // kMetaWords entries
     uint32_t seed;
+    const uint32_t *heavy;       // heavy keys of the column (skew.h's table), or null
 };
 
 // Weights b -> w(b), exact modulo 2^64: the direct-address sums W[b - min], or

@@ -436,7 +436,10 @@ __global__ void __launch_bounds__(BT, RANGE_CTAS_PER_SM) k_range(SizeArgs g) {
     __shared__ HeavySample<2048> hsm;
     if (blockIdx.x < g.nheavy) {
         const HeavyCol &h = g.h[blockIdx.x];
-        heavy_sample_cta<BT, 2048>(h.keys, h.n, h.buckets, h.heavy, hsm);
+        if (h.coarse)
+            heavy_sample_cta<BT, 1024>(h.keys, h.n, h.buckets, h.heavy, reinterpret_cast<HeavySample<1024> &>(hsm));
+        else
+            heavy_sample_cta<BT, 2048>(h.keys, h.n, h.buckets, h.heavy, hsm);
         return;
     }
     const uint32_t cta = (blockIdx.x - g.nheavy) % g.range_rows;

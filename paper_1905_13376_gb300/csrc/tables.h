@@ -114,6 +114,7 @@ struct HeavyCol {
     const int32_t *keys;
     uint32_t n, buckets;
     uint32_t *heavy;
+    bool coarse = false;   // from half as large a sample
 };
 cudaError_t size_columns(const SizeCol *cols, uint32_t ncols, const HeavyCol *heavy, uint32_t nheavy, bool allow_dense,
                          int num_sms, cudaStream_t st, const char *hll_name = "t_hll",
