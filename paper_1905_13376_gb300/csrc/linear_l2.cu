@@ -122,14 +122,66 @@ __device__ __forceinline__ void w_add_direct(unsigned long long *__restrict__ W,
         set_status(st, MWJ_ERR_CHECK, 9);   // a key outside the range the sizing pass saw
 }
 
+// Packed slots: the slot at which the search for key k starts (key -1: its sum's).
+__device__ __forceinline__ uint32_t packed_home(uint32_t k, uint32_t seed, uint32_t mask) {
+    return k == kEmptyKey ? mask + 1 : slot_of(k, seed, mask);
+}
+// w(k) from the first slot (s, value v); 0 when k has none.
+__device__ __forceinline__ unsigned long long packed_get(const WTable &w, uint32_t mask, uint32_t packed, uint32_t k,
+                                                         uint32_t s, unsigned long long v) {
+    if (k == kEmptyKey) return v;
+    for (uint32_t it = 0; it < mask && v != kEmpty64 && (uint32_t)v != k; ++it) {
+        s = (s + 1) & mask;
+        v = __ldg(w.W + s);
+    }
+    if (v == kEmpty64 || (uint32_t)v != k) return 0ull;
+    return (v >> 32) | (packed & 2u ? (unsigned long long)__ldg(w.keys + s) << 32 : 0ull);
+}
+// w(k) += x (x > 0) from the first slot (s, value v, possibly read before other
+// threads claimed it).  A claim stores the key and x's lower word; later adds go to
+// the upper half of the slot, and what they carry out of it goes to keys[s].
+__device__ __forceinline__ void packed_add(const WTable &w, uint32_t mask, uint32_t k, uint32_t s, unsigned long long v,
+                                           unsigned long long x, DevStatus *st) {
+    if (k == kEmptyKey) {
+        atomicAdd(w.W + mask + 1, x);
+        return;
+    }
+    const unsigned long long lo = x & 0xFFFFFFFFull;
+    const uint32_t hx = (uint32_t)(x >> 32);
+    for (uint32_t it = 0; it <= mask; ++it) {
+        uint32_t h = hx;
+        bool mine = false;
+        if (v == kEmpty64) {
+            v = atomicCAS(w.W + s, kEmpty64, (lo << 32) | k);
+            mine = v == kEmpty64;
+        }
+        if (!mine && (uint32_t)v == k) {
+            const unsigned long long old = atomicAdd(w.W + s, lo << 32);
+            h += (uint32_t)(((old >> 32) + lo) >> 32);
+            mine = true;
+        }
+        if (mine) {
+            if (h) {
+                atomicAdd(w.keys + s, h);
+                atomicOr(w.meta + kMetaPacked, 2u);
+            }
+            return;
+        }
+        s = (s + 1) & mask;
+        v = __ldcg(w.W + s);
+    }
+    set_status(st, MWJ_ERR_CHECK, 7);   // table full: the sizing step under-estimated
+}
+
 // w(k[q]) for the lane's tuples q < m (0 for the others) from a weight table
 // in either layout; hashed: the key groups are loaded together, then the sums.
-template <bool WD, bool STAR = false>
+template <bool WD, bool STAR = false, bool PACKED = false>
 struct WLookup {
     const WTable &w;
-    uint32_t mask, min, span, shift;
+    uint32_t mask, min, span, shift, packed;
     __device__ explicit WLookup(const WTable &w_) : w(w_) {
         mask = __ldg(w.meta);
+        packed = PACKED ? __ldg(w.meta + kMetaPacked) : 0u;
         min = WD ? __ldg(w.meta + kMetaMin) : 0u;
         span = WD ? __ldg(w.meta + kMetaSpan) : 0u;
         shift = WD && STAR ? __ldg(w.meta + kMetaShift) : 0u;
@@ -141,6 +193,17 @@ struct WLookup {
                 const uint32_t i = (uint32_t)k[q] - min;
                 x[q] = ((uint32_t)q < m && i < span) ? __ldg(w.W + (STAR ? i << shift : i)) : 0ull;
             }
+        } else if constexpr (PACKED) {
+            uint32_t s[WQ];
+            unsigned long long v[WQ];
+#pragma unroll
+            for (int q = 0; q < WQ; ++q) {
+                s[q] = packed_home((uint32_t)k[q], w.seed, mask);
+                v[q] = (uint32_t)q < m ? __ldg(w.W + s[q]) : 0ull;
+            }
+#pragma unroll
+            for (int q = 0; q < WQ; ++q)
+                x[q] = (uint32_t)q < m ? packed_get(w, mask, packed, (uint32_t)k[q], s[q], v[q]) : 0ull;
         } else {
             uint32_t s[WQ];
             uint4 v[WQ];
@@ -336,6 +399,8 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
     const uint32_t wmask = __ldg(w.meta + kMetaMask), wmin = wd ? __ldg(w.meta + kMetaMin) : 0u,
                    wspan = wd ? __ldg(w.meta + kMetaSpan) : 0u;
     const uint32_t wshift = wd && FILTER ? __ldg(w.meta + kMetaShift) : 0u;
+    const bool wp = !FILTER && !wd && (__ldg(w.meta + kMetaPacked) & 1u);
+    const uint32_t sp = SW && !sd ? __ldg(smeta + kMetaPacked) : 0u;
     auto group = [&](uint32_t s) {   // four keys of the table (FILTER: none is added in this kernel)
         return FILTER ? __ldg((const uint4 *)(w.keys + s)) : __ldcg((const uint4 *)(w.keys + s));
     };
@@ -346,6 +411,10 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
             return SW ? __ldg(src.w.W + i) : (unsigned long long)__ldg((const uint32_t *)src.t.slots + i);
         }
         if constexpr (SW) {
+            if (sp) {
+                const uint32_t s = packed_home(c, src.w.seed, smask);
+                return packed_get(src.w, smask, sp, c, s, __ldg(src.w.W + s));
+            }
             if (c == kEmptyKey) return __ldg(src.w.W + smask + 1);
             const uint32_t s = w_home(c, src.w.seed, smask);
             const uint32_t at = w_find(src.w.keys, smask, c, s, __ldg((const uint4 *)(src.w.keys + s)));
@@ -368,44 +437,63 @@ __global__ void __launch_bounds__(WT, GC) k_w_build(const int32_t *__restrict__ 
         else if (!FILTER)
             set_status(st, MWJ_ERR_CHECK, 7);   // table full: the sizing step under-estimated
     };
-    const uint32_t T = gridDim.x * WT, lane = threadIdx.x & 31;
-    uint64_t i = (uint64_t)blockIdx.x * WT + threadIdx.x;
-    int32_t b = 0, c = 0;
-    if (i < n) {
-        b = __ldg(Sb + i);
-        c = __ldg(Sc + i);
-    }
-    for (; i - lane < n; i += T) {
-        int32_t nb = 0, nc = 0;
-        if (i + T < n) {
-            nb = __ldg(Sb + i + T);
-            nc = __ldg(Sc + i + T);
+    auto tuples_in_turn = [&](auto packed) {
+        constexpr bool PACKED = decltype(packed)::value;
+        const uint32_t T = gridDim.x * WT, lane = threadIdx.x & 31;
+        uint64_t i = (uint64_t)blockIdx.x * WT + threadIdx.x;
+        int32_t b = 0, c = 0;
+        if (i < n) {
+            b = __ldg(Sb + i);
+            c = __ldg(Sc + i);
         }
-        const bool has = i < n;
-        uint32_t s = 0;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (!wd) {   // the target's key group, with the source's slot
-            s = w_home((uint32_t)b, w.seed, wmask);
-            v = group(s);
-        }
-        unsigned long long x = has ? value((uint32_t)c) : 0ull;
-        if (hs && x) {
-            const int hsl = heavy_slot(hs, (uint32_t)b);
-            if (hsl >= 0) {
-                heavy_add(hacc, hsl, x);
-                x = 0ull;
+        for (; i - lane < n; i += T) {
+            int32_t nb = 0, nc = 0;
+            if (i + T < n) {
+                nb = __ldg(Sb + i + T);
+                nc = __ldg(Sc + i + T);
             }
+            const bool has = i < n;
+            uint32_t s = 0;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            unsigned long long p = 0;
+            if (PACKED) {   // the target's slot or key group, with the source's slot
+                s = slot_of((uint32_t)b, w.seed, wmask);
+                p = __ldcg(w.W + s);
+            } else if (!wd) {
+                s = w_home((uint32_t)b, w.seed, wmask);
+                v = group(s);
+            }
+            unsigned long long x = has ? value((uint32_t)c) : 0ull;
+            if (hs && x) {
+                const int hsl = heavy_slot(hs, (uint32_t)b);
+                if (hsl >= 0) {
+                    heavy_add(hacc, hsl, x);
+                    x = 0ull;
+                }
+            }
+            const unsigned long long sum = warp_run_sum1(b, x, has);
+            if (sum && PACKED)
+                packed_add(w, wmask, (uint32_t)b, s, p, sum, st);
+            else if (sum)
+                add((uint32_t)b, s, v, sum);
+            b = nb;
+            c = nc;
         }
-        const unsigned long long sum = warp_run_sum1(b, x, has);
-        if (sum) add((uint32_t)b, s, v, sum);
-        b = nb;
-        c = nc;
-    }
+    };
+    if (wp)
+        tuples_in_turn(std::integral_constant<bool, !FILTER>{});
+    else
+        tuples_in_turn(std::false_type{});
     if (!hs) return;
     __syncthreads();
     for (uint32_t j = threadIdx.x; j < kHeavySlots; j += WT) {
         const unsigned long long x = heavy_sum(hacc, j);
         if (!x) continue;
+        if (wp) {
+            const uint32_t s = slot_of(hs[j], w.seed, wmask);
+            packed_add(w, wmask, hs[j], s, __ldcg(w.W + s), x, st);
+            continue;
+        }
         const uint32_t s = wd ? 0u : w_home(hs[j], w.seed, wmask);
         add(hs[j], s, wd ? make_uint4(0u, 0u, 0u, 0u) : group(s), x);
     }
@@ -520,9 +608,9 @@ __global__ void __launch_bounds__(WT) k_w_keys(const int32_t *__restrict__ Rb, u
 // One warp round of the R pass: x = w(b) for the lane's tuples (a[q], b[q]),
 // q < m, added to the thread's total and (GROUP BY A) per run of equal a to
 // cnt[a].
-template <int MODE, bool WD, bool STAR>
+template <int MODE, bool WD, bool STAR, bool PACKED>
 struct RPass {
-    const WLookup<WD, STAR> look;
+    const WLookup<WD, STAR, PACKED> look;
     int32_t a_domain;
     unsigned long long *cnt;
     DevStatus *st;
@@ -547,13 +635,13 @@ struct RPass {
     }
 };
 
-template <int MODE, bool WD, bool STAR = false>
+template <int MODE, bool WD, bool STAR = false, bool PACKED = false>
 __device__ __forceinline__ void w_probe_pass(const int32_t *__restrict__ Ra, const int32_t *__restrict__ Rb,
                                              uint32_t n, const WTable &w, int32_t a_domain,
                                              unsigned long long *__restrict__ cnt,
                                              unsigned long long *__restrict__ total, DevStatus *st,
                                              unsigned long long *red) {
-    RPass<MODE, WD, STAR> P(w, a_domain, cnt, st);
+    RPass<MODE, WD, STAR, PACKED> P(w, a_domain, cnt, st);
     const uint32_t warp = (blockIdx.x * WT + threadIdx.x) >> 5, warps = (gridDim.x * WT) >> 5;
     rounds_plain(Ra, Rb, 0u, n, warp, warps,
                  [&](const int32_t (&a)[WQ], const int32_t (&b)[WQ], uint32_t m) { P.round(a, b, m); });
@@ -570,7 +658,10 @@ __global__ void __launch_bounds__(WT) k_w_probe(const int32_t *__restrict__ Ra, 
     after_previous();
     if (__ldg(w.meta + kMetaDense)) return;
     __shared__ unsigned long long red[32];
-    w_probe_pass<MODE, false>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
+    if (__ldg(w.meta + kMetaPacked) & 1u)
+        w_probe_pass<MODE, false, false, true>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
+    else
+        w_probe_pass<MODE, false>(Ra, Rb, n, w, a_domain, cnt, total, st, red);
 }
 
 template <int MODE, bool STAR>
@@ -835,6 +926,7 @@ __global__ void __launch_bounds__(WT) k_chain_clear(SmallArgs g) {
         for (int k = 0; k < g.nrel - 2; ++k) {
             g.w[k].meta[kMetaMask] = g.wmask[k];
             g.w[k].meta[kMetaDense] = 0u;
+            g.w[k].meta[kMetaPacked] = 0u;
         }
     }
 }
@@ -1186,6 +1278,7 @@ cudaError_t one_bucket_run(OneBucket &L, const mwj_rel *rel, int nrel, const See
             }
         }
         cols[ncols] = SizeCol{r.x, (uint32_t)r.n, seed, L.hll[ncols], {meta}, {reserve}, {reserve}, 1u};
+        cols[ncols].weights = true;
         ++ncols;
     };
     HeavyCol heavy[kSizeCols];

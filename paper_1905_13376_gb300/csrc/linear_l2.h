@@ -23,7 +23,10 @@ struct DegTable {
 // Weights b -> w(b), exact modulo 2^64: the direct-address sums W[b - min], or
 // 2^k slots, keys and sums apart: keys[s] in groups of four (one 16-byte load),
 // W[s] the sum, added to with 64-bit adds whose results are not needed.  Key -1,
-// the mark of a free slot, has its sum in W[mask + 1].
+// the mark of a free slot, has its sum in W[mask + 1].  A table larger than the L2
+// (from kPackedSlots slots on, tables.cu) has packed slots instead, W[s] = lower
+// word of the sum << 32 | key and keys[s] the upper word: a new key is claimed and
+// added with one atomic, and out there every atomic moves a sector from and to memory.
 struct WTable {
     unsigned long long *W;   // w_table_slots(n) + 2 entries reserved
     uint32_t *keys;          // w_table_slots(n) entries reserved

@@ -10,8 +10,10 @@ namespace mwj {
 // (kMetaDense = 1), the smallest key, the span of the keys and a shift: the entry
 // of key k is then at (k - min) << shift (0 for all but a star join's weights),
 // nothing is hashed and no key is stored.
-// kMetaTry: that layout is left to the distinct estimate.
-constexpr int kMetaMask = 0, kMetaEst = 1, kMetaShift = 2, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5, kMetaTry = 6;
+// kMetaTry: that layout is left to the distinct estimate.  kMetaPacked: hashed
+// weights in packed slots (bit 0; bit 1: some sum has an upper word, linear_l2.h).
+constexpr int kMetaMask = 0, kMetaEst = 1, kMetaShift = 2, kMetaDense = 3, kMetaMin = 4, kMetaSpan = 5, kMetaTry = 6,
+              kMetaPacked = 7;
 constexpr int kMetaWords = 8;
 
 // J == 0: one table of (meta[0] + 1) packed (deg << 32 | c) slots, home slot
@@ -104,6 +106,7 @@ struct SizeCol {
     // a range of at most `sure` entries is direct-address whatever the number of
     // distinct keys, a larger one when it is at most `per_key` times the estimate
     // or the keys are few (k_hll)
+    bool weights = false;   // the table may take packed slots (linear_l2.h)
     uint64_t sure = 1ull << 24;
     double per_key = 8.0;
 };
