@@ -10,6 +10,7 @@ loaded.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -272,18 +273,18 @@ class Context:
             self._ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
         return self._ws
 
-    def _less(self, err, shares, full, size, partitioned):
-        """After running out of device memory for the workspace (of `full` bytes) of
-        the plan without shares: the partitioned plan's shares and its workspace, if
-        that takes less; otherwise the error stands."""
+    def _less(self, err, shares, nb, size, partitioned):
+        """After running out of device memory for the workspace (of nb bytes) of the
+        plan without shares: the partitioned plan's shares and its workspace, if that
+        takes less; otherwise the error stands.  size(shares): the call that writes nb."""
         import torch
         if shares is not None or not isinstance(err, torch.cuda.OutOfMemoryError):
             raise err
-        sh = _shares(partitioned())
-        nb = size(sh)
-        if nb >= full:
+        full, sh = nb.value, _shares(partitioned())
+        self._check(size(sh))
+        if nb.value >= full:
             raise err
-        return sh, self.workspace(nb)
+        return sh, self.workspace(nb.value)
 
     def workspace_size(self, kind, R, S, T, shares=None, mode=MWJ_COUNT) -> int:
         n = ctypes.c_size_t()
@@ -346,6 +347,9 @@ class Context:
             res["n_rows"] = n_rows
         return o, res
 
+    def _rows_size(self, nb, r, s, t, sh):
+        return self.lib.mwj_workspace_size(self.h, MWJ_LINEAR, r, s, t, sh, MWJ_MATERIALIZE, ctypes.byref(nb))
+
     def _run(self, fn, kind_ws, R, S, T, mode, shares, a_domain, capacity, arity, stream, sync,
              extra=(), out=None):
         if isinstance(mode, str):
@@ -355,17 +359,14 @@ class Context:
         r, s, t, hs = _rel(R), _rel(S), _rel(T), self._stream(stream)
         sh = _shares(shares) if with_shares else None
         nb = ctypes.c_size_t()
-
-        def size(sh):
-            self._check(self.lib.mwj_workspace_size(self.h, kind_ws, r, s, t, sh, mode, ctypes.byref(nb)))
-            return nb.value
-        size(sh)
+        self._check(self.lib.mwj_workspace_size(self.h, kind_ws, r, s, t, sh, mode, ctypes.byref(nb)))
         try:
             ws = self.workspace(nb.value)
         except RuntimeError as e:
             if kind_ws != MWJ_LINEAR or mode != MWJ_MATERIALIZE:
                 raise
-            sh, ws = self._less(e, sh, nb.value, size, lambda: self.plan_shares(MWJ_LINEAR, R, S, T, mode, stream))
+            sh, ws = self._less(e, sh, nb, functools.partial(self._rows_size, nb, r, s, t),
+                                functools.partial(self.plan_shares, MWJ_LINEAR, R, S, T, mode, stream))
         args = (self.h,) + tuple(extra) + (r, s, t)
         if with_shares:
             args = args + (sh,)
@@ -382,8 +383,9 @@ class Context:
                      stream=None, sync=True, out=None):
         """Linear 3-way join R(A,B) S(B,C) T(C,D).  shares = (H(B) buckets,
         g(C) buckets[, log2 on-chip table slots]); None: one bucket per side
-        for "count" and "group_by_a" (T's and S's tables in L2), H(B)
-        buckets from |R| for "rows".  out: the result dict of an earlier
+        for "count" and "group_by_a" (T's and S's tables in L2), R and T as
+        lists for "rows" (the H(B) buckets of plan_shares where memory is
+        short or R or T has 2^29 tuples).  out: the result dict of an earlier
         aggregate call with the same mode and a_domain, whose tensors are
         written again instead of new ones."""
         return self._run(self.lib.mwj_join3_linear, MWJ_LINEAR, R, S, T, mode, shares, a_domain,
@@ -393,7 +395,8 @@ class Context:
                    stream=None, sync=True):
         """Star 3-way join: small R(A,B) and T(C,D) held on chip, S(B,C)
         streamed once.  shares = (h(B) buckets of R, g(C) buckets of T), 0 or
-        None for the default."""
+        None for the default; they apply to "rows", the aggregates have one
+        bucket per side whatever they are."""
         return self._run(self.lib.mwj_join3_star, MWJ_STAR, R, S, T, mode, shares, a_domain,
                          capacity, 4, stream, sync)
 
@@ -406,15 +409,12 @@ class Context:
         o, res = self._outputs(mode, a_domain, 0, 4)
         rels, sh = (_rel(R), _rel(S), _rel(T), _rel(U)), _shares(shares)
         nb = ctypes.c_size_t(0)
-
-        def size(sh):
-            self._check(self.lib.mwj_join4_workspace_size(self.h, *rels, sh, int(mode), ctypes.byref(nb)))
-            return nb.value
-        size(sh)
+        self._check(self.lib.mwj_join4_workspace_size(self.h, *rels, sh, int(mode), ctypes.byref(nb)))
         try:
             ws = self.workspace(nb.value)
         except RuntimeError as e:
-            sh, ws = self._less(e, sh, nb.value, size,
+            sh, ws = self._less(e, sh, nb, lambda q: self.lib.mwj_join4_workspace_size(self.h, *rels, q, int(mode),
+                                                                                        ctypes.byref(nb)),
                                 lambda: self.plan_shares(MWJ_LINEAR, R, S, T, MWJ_MATERIALIZE, stream))
         self._check(self.lib.mwj_join4_linear(self.h, *rels, sh, ctypes.byref(o), ws.data_ptr(), ws.numel(),
                                               self._stream(stream)))
@@ -432,15 +432,11 @@ class Context:
         est = torch.empty(int(a_domain), dtype=torch.float32, device=self.device) if estimates else None
         rels, sh = (_rel(R), _rel(S), _rel(T)), _shares(shares)
         nb = ctypes.c_size_t(0)
-
-        def size(sh):
-            self._check(self.lib.mwj_fm_workspace_size(self.h, *rels, sh, ctypes.byref(nb)))
-            return nb.value
-        size(sh)
+        self._check(self.lib.mwj_fm_workspace_size(self.h, *rels, sh, ctypes.byref(nb)))
         try:
             ws = self.workspace(nb.value)
         except RuntimeError as e:   # (about 16K S tuples per bucket)
-            sh, ws = self._less(e, sh, nb.value, size,
+            sh, ws = self._less(e, sh, nb, lambda q: self.lib.mwj_fm_workspace_size(self.h, *rels, q, ctypes.byref(nb)),
                                 lambda: (min(1 << max(10, (rels[1].n // 16384).bit_length()), 16384), 1, 1))
         self._check(self.lib.mwj_fm_linear(self.h, *rels, sh, int(a_domain), sk.data_ptr(),
                                            est.data_ptr() if est is not None else None,
