@@ -563,6 +563,7 @@ cudaError_t fm_one_run(const FmOneLayout &L, const mwj_rel &R, const mwj_rel &S,
     // over 2^22 places 0.65 and 1.01)
     for (uint32_t k = 0; k < ncols; ++k) {
         cols[k].sure = 1ull << 22;
+        cols[k].near = 0;
         cols[k].per_key = 40.0;
     }
     cudaError_t e;

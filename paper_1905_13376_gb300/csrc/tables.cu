@@ -523,7 +523,10 @@ __device__ __forceinline__ uint32_t spread_shift(uint64_t span, uint64_t room) {
 // keys take 0.87 and 2.20 ms with keys and sums apart, 0.66 and 1.62 packed; 6e6
 // tuples (2^23 slots) 0.50 apart and, in packed slots of another load, 0.52.
 constexpr uint64_t kPackedSlots = 1ull << 24;
-constexpr double kFewKeys = 8192.0;   // distinct keys up to which a large range is direct-address
+// Distinct keys up to which a large range is direct-address, and one of up to `near`
+// entries: 2^18 keys a line each are 32 MB a table (2.5e7 tuples over as many places,
+// 2^16 and 2^18 keys 0.82 and 0.84 ms direct-address, 1.03 and 1.07 hashed).
+constexpr double kFewKeys = 8192.0, kNearKeys = 1 << 18;
 
 // HyperLogLog registers (Flajolet, Fusy, Gandouet, Meunier 2007): register
 // h >> (32 - HLL_BITS) keeps the largest rank (position of the first 1 bit)
@@ -731,7 +734,8 @@ __global__ void __launch_bounds__(HLL_MW * 32) k_hll_merge_size(SizeArgs g) {
     for (uint32_t t = 0; t < c.ntargets; ++t) {
         uint32_t *mt = c.meta[t];
         if (__ldcg(mt + kMetaDense)) continue;
-        if (g.ranged && __ldcg(mt + kMetaTry) && ((double)__ldcg(mt + kMetaSpan) <= c.per_key * E || E <= kFewKeys)) {
+        const uint32_t span = g.ranged && __ldcg(mt + kMetaTry) ? __ldcg(mt + kMetaSpan) : 0u;
+        if (span && ((double)span <= c.per_key * E || E <= kFewKeys || (span <= c.near && E <= kNearKeys))) {
             mt[kMetaDense] = 1u;   // (the other words are there)
             continue;
         }

@@ -108,6 +108,7 @@ struct SizeCol {
     // or the keys are few (k_hll)
     bool weights = false;   // the table may take packed slots (linear_l2.h)
     uint64_t sure = 1ull << 24;
+    uint64_t near = 3ull << 23;   // the same for up to 2^18 keys
     double per_key = 8.0;
 };
 // A column whose heavy keys (sampled share at least 1 / (2 x buckets)) are
