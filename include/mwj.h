@@ -134,14 +134,17 @@ mwj_status mwj_workspace_size(mwj_ctx *ctx, int kind, mwj_rel R, mwj_rel S, mwj_
  * held tables kept whole in the L2: T's table c -> deg_T(c), a pass over S
  * that adds w(b) += deg_T(c) into S's weight table, and a pass over R that
  * adds cnt[a] += w(b) and total += w(b).  A table is an array indexed by
- * key - min when the column's key range fits what is reserved for it, else a
- * hash table sized from a HyperLogLog estimate of the distinct keys; w(b) is
+ * key - min when the column's key range fits what is reserved for it and is
+ * either at most 2^24 places or not large for its number of distinct keys,
+ * else a hash table sized from a HyperLogLog estimate of that number; w(b) is
  * exact to 2^64.  Relations of at most 2^19 tuples use hash tables of two
- * slots per tuple in four launches, of at most 2^14 in one.
+ * slots per tuple in four launches, of at most 2^14 in one (in four where the
+ * device takes no cluster of 16 CTAs).
  * MATERIALIZE with shares == NULL: R grouped by B and T by C as lists in
  * global memory, S streamed past them once, the rows of a chunk of S at the
  * place that one atomic on *n_rows reserves; rows beyond the capacity are
- * counted and not written.
+ * counted and not written.  Relations R or T of 2^29 tuples and more, and
+ * calls given only the workspace of the partitioned plan, run that plan.
  * Otherwise R is partitioned by H(B), S by (H(B), g(C)), T by g(C); each CTA holds one
  * H(B) bucket's B values as an on-chip hash table while the other side of
  * that bucket streams past it, and T's tables are probed (its bucket images
@@ -178,9 +181,10 @@ mwj_status mwj_join3_cyclic(mwj_ctx *ctx, mwj_rel R, mwj_rel S, mwj_rel T,
  * deg_R(b) deg_T(c) over S.  GROUP BY A: T's degree table and a weight table
  * with R's keys (as in mwj_join3_linear); each S tuple whose b is a key of R
  * adds deg_T(c) to w(b), and R's groups are added at the end.  Neither uses the
- * shares (relations of at most 2^19 tuples run as a linear join does).  MATERIALIZE: R is grouped by h(B) and T by g(C) into bucket
- * tables, S read twice (a counting pass, then the rows).  shares: s[0] = h(B) buckets
- * of R, s[1] = g(C) buckets of T (0 or shares == NULL: about 2048 tuples per
+ * shares (relations of at most 2^19 tuples run as a linear join does).
+ * MATERIALIZE: R is grouped by h(B) and T by g(C) into bucket tables, S read
+ * twice (a counting pass, then the rows).  shares: s[0] = h(B) buckets of R,
+ * s[1] = g(C) buckets of T (0 or shares == NULL: about 2048 tuples per
  * bucket); s[2] is ignored.  GROUP BY A checks the domain of A while it adds
  * R's groups (MWJ_ERR_DOMAIN from mwj_stream_status).
  * workspace: device, >= mwj_workspace_size(ctx, MWJ_STAR, ...). */
@@ -312,7 +316,9 @@ mwj_status mwj_batch_destroy(mwj_batch *batch);
  *   fit_pct            cyclic: R_ij and T_ki may fill this percentage of a
  *                      tile's on-chip capacity when the cube shares are
  *                      searched (Section 5.2's z|R| + x|S| + y|T|), 10 .. 100.
- * A field <= 0 keeps the library's rule (8192 tuples, factor 2, 95 %).
+ * A field <= 0 keeps the library's rule (8192 tuples, factor 2, 95 %; cyclic
+ * queries whose tiles at 95 % are fewer than two per SM over the whole batch
+ * are searched at 50 %, for more tiles).
  * mwj_batch_set_rules replaces the context's rules (n == 0 restores the
  * library's); mwj_batch_set_launch sets the CTAs per SM of the batch's
  * persistent partitioning and join launches (0: the library's choice, 3 and

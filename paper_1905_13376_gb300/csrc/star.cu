@@ -27,7 +27,7 @@
 //
 // 2^26 fact tuples sorted by B, dimensions of 2^20 unique keys, GROUP BY A: the
 // aggregates as two hashed lookups per tuple (8-byte slots, 32 MB a table) took
-// 0.56 ms, 0.455 of it that pass; 0.34 ms now, 0.275 of it the S pass, at one
+// 0.56 ms, 0.455 of it that pass; 0.32 ms now, 0.27 of it the S pass, at one
 // L1 tag per tuple (0.96 -> 0.64 ms with S in random order).
 #include "api_internal.h"
 #include "linear_l2.h"

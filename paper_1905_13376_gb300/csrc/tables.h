@@ -103,10 +103,10 @@ struct SizeCol {
     // > 0: the direct-address entries of the (one) table are spread out over this
     // many at most, so that adds to neighbouring keys meet in no L2 sector
     uint64_t spread = 0;
+    bool weights = false;   // the table may take packed slots (linear_l2.h)
     // a range of at most `sure` entries is direct-address whatever the number of
     // distinct keys, a larger one when it is at most `per_key` times the estimate
     // or the keys are few (k_hll)
-    bool weights = false;   // the table may take packed slots (linear_l2.h)
     uint64_t sure = 1ull << 24;
     uint64_t near = 3ull << 23;   // the same for up to 2^18 keys
     double per_key = 8.0;
