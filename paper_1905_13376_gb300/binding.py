@@ -448,8 +448,9 @@ class Context:
     def join3_cyclic(self, R, S, T, mode="count", shares=None, a_domain=None, capacity=0,
                      stream=None, sync=True, out=None):
         """Cyclic 3-way join R(A,B) S(B,C) T(C,A), T given as (c, a) columns.
-        shares = (H(A), G(B), F(C)) bucket counts; None: the library's cube
-        shares.  out: as for join3_linear."""
+        shares = (H(A), G(B), F(C)) bucket counts; None: (1, 1, z), R whole
+        as lists, S and T by C in the z buckets of plan_shares.  out: as for
+        join3_linear."""
         return self._run(self.lib.mwj_join3_cyclic, MWJ_CYCLIC, R, S, T, mode, shares, a_domain,
                          capacity, 3, stream, sync, out=out)
 
